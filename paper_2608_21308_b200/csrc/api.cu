@@ -77,9 +77,20 @@ int pick_impl(const e2ttt_params* p, bool save_states, int* impl) {
     return E2TTT_OK;
 }
 
-size_t simt_bytes(const e2ttt_params* p, bool save_states, bool backward, bool normed) {
+// The block-tiled kernels serve the any-shape calls of bf16 I/O up to d = 128 (a head dimension in one accumulator tile);
+// wider heads and fp32 I/O run on the SIMT kernels.
+bool can_tile(const e2ttt_params* p) { return p->io_dtype == E2TTT_BF16 && p->d <= kTileMaxD; }
+
+// A buffer with saved states has the block-tiled region whatever `impl` says: the forward and the backward of one training step may
+// be given different ones.
+SimtLayout layout_of(const e2ttt_params* p, bool save_states, bool backward, bool normed, bool allow_tile = true) {
     const int nchunks = (p->L + p->C - 1) / p->C;
-    SimtLayout l = simt_layout(p->d, p->h, p->C, nmat_of(p->kind), nchunks, save_states, backward, normed ? 0 : segment_chunks(p));
+    const bool tile = allow_tile && can_tile(p) && (save_states || backward || p->impl != E2TTT_IMPL_SIMT);
+    return simt_layout(p->d, p->h, p->C, nmat_of(p->kind), nchunks, save_states, backward, normed ? 0 : segment_chunks(p), tile, p->B * p->H);
+}
+
+size_t simt_bytes(const e2ttt_params* p, bool save_states, bool backward, bool normed, bool allow_tile = true) {
+    SimtLayout l = layout_of(p, save_states, backward, normed, allow_tile);
     const size_t elem = (p->io_dtype == E2TTT_F32) ? sizeof(double) : sizeof(float);
     return kStatusBytes + l.per_seq * elem * (size_t)p->B * p->H;
 }
@@ -146,7 +157,7 @@ static int fwd_common(const e2ttt_params* p, const void* q, const void* k, const
                       const float* beta, const float* gamma, const float* const* W_init, const float* const* M_init,
                       const float* const* row_norm, float norm_eps,
                       void* o, float* const* W_final, float* const* M_final, void* workspace, size_t workspace_bytes,
-                      int save_states, void* stream) {
+                      int save_states, void* stream, bool allow_tile = true) {
     int rc = check_params(p);
     if (rc) return rc;
     if (!q || !k || !v || !eta || !beta || !gamma || !W_init || !o || !W_final || !M_final) return E2TTT_ERR_NULL;
@@ -166,8 +177,7 @@ static int fwd_common(const e2ttt_params* p, const void* q, const void* k, const
             if (!row_norm[i]) return E2TTT_ERR_NULL;
         need = simt_bytes(p, save_states != 0, save_states != 0, true);  // the size e2ttt_workspace_bytes_normed reports
     } else {
-        rc = e2ttt_workspace_bytes(p, save_states, &need);
-        if (rc) return rc;
+        need = impl == E2TTT_IMPL_TCGEN05 && !save_states ? kStatusBytes : simt_bytes(p, save_states != 0, save_states != 0, false, allow_tile);
     }
     if (!workspace || workspace_bytes < need) return E2TTT_ERR_WORKSPACE;
     if (!aligned(workspace, 256)) return E2TTT_ERR_ALIGN;
@@ -192,7 +202,7 @@ static int fwd_common(const e2ttt_params* p, const void* q, const void* k, const
         t.status = static_cast<int*>(workspace);
         if (save_states) {
             const int seg = segment_chunks(p);
-            const SimtLayout lay = simt_layout(p->d, p->h, p->C, nmat, (p->L + p->C - 1) / p->C, true, true, seg);
+            const SimtLayout lay = layout_of(p, true, true, false);
             t.ckpt = reinterpret_cast<float*>(static_cast<char*>(workspace) + kStatusBytes) + (seg ? lay.cck : lay.ckpt);
             t.ckpt_seq_stride = lay.per_seq;
             t.ckpt_every = seg;
@@ -212,7 +222,7 @@ static int fwd_common(const e2ttt_params* p, const void* q, const void* k, const
         if (row_norm) { t.norm1 = row_norm[0]; t.norm2 = row_norm[1]; t.norm_eps = norm_eps; }
         if (save_states) {
             const int seg = row_norm ? 0 : segment_chunks(p);
-            const SimtLayout lay = simt_layout(p->d, p->h, p->C, nmat, (p->L + p->C - 1) / p->C, true, true, seg);
+            const SimtLayout lay = layout_of(p, true, true, row_norm != nullptr);
             t.ckpt = reinterpret_cast<float*>(static_cast<char*>(workspace) + kStatusBytes) + (seg ? lay.cck : lay.ckpt);
             t.ckpt_seq_stride = lay.per_seq;
             t.ckpt_every = seg;
@@ -245,8 +255,9 @@ static int fwd_common(const e2ttt_params* p, const void* q, const void* k, const
         a.row_norm[i] = row_norm ? row_norm[i] : nullptr;
     }
     a.norm_eps = norm_eps;
-    a.lay = simt_layout(p->d, p->h, p->C, nmat, a.nchunks, save_states != 0, save_states != 0, seg);
-    return simt_fwd_launch(a, p->kind, p->io_dtype, stream) == 0 ? E2TTT_OK : E2TTT_ERR_CUDA;
+    a.lay = layout_of(p, save_states != 0, save_states != 0, row_norm != nullptr, allow_tile);
+    const bool tile = impl == E2TTT_IMPL_TILED && can_tile(p) && allow_tile;
+    return (tile ? tile_fwd_launch(a, p->kind, stream) : simt_fwd_launch(a, p->kind, p->io_dtype, stream)) == 0 ? E2TTT_OK : E2TTT_ERR_CUDA;
 }
 
 int e2ttt_chunk_fwd(const e2ttt_params* p, const void* q, const void* k, const void* v, const float* eta,
@@ -256,6 +267,26 @@ int e2ttt_chunk_fwd(const e2ttt_params* p, const void* q, const void* k, const v
     return fwd_common(p, q, k, v, eta, beta, gamma, W_init, M_init, nullptr, 0.0f, o, W_final, M_final, workspace,
                       workspace_bytes, save_states, stream);
 }
+
+// e2ttt_chunk_fwd_noalloc (noalloc.cu): the forward in a scratch area of fixed size.  A shape whose block-tiled layout is the
+// larger one and does not fit still runs, on the SIMT kernels.
+}  // extern "C"
+namespace e2ttt {
+size_t fixed_scratch_need(const e2ttt_params* p, size_t have) {  // of valid parameters
+    size_t need = 0;
+    if (e2ttt_workspace_bytes(p, 0, &need) == E2TTT_OK && need > have && p->impl != E2TTT_IMPL_TCGEN05) need = simt_bytes(p, false, false, false, false);
+    return need;
+}
+int fwd_fixed_scratch(const e2ttt_params* p, const void* q, const void* k, const void* v, const float* eta, const float* beta,
+                      const float* gamma, const float* const* W_init, const float* const* M_init, void* o, float* const* W_final,
+                      float* const* M_final, void* scratch, size_t have, void* stream) {
+    size_t need = 0;
+    const int rc = e2ttt_workspace_bytes(p, 0, &need);
+    if (rc) return rc;
+    return fwd_common(p, q, k, v, eta, beta, gamma, W_init, M_init, nullptr, 0.0f, o, W_final, M_final, scratch, have, 0, stream, need <= have);
+}
+}  // namespace e2ttt
+extern "C" {
 
 int e2ttt_chunk_fwd_normed(const e2ttt_params* p, const void* q, const void* k, const void* v, const float* eta,
                            const float* beta, const float* gamma, const float* const* W_init,
@@ -305,7 +336,9 @@ static int bwd_common(const e2ttt_params* p, const void* q, const void* k, const
 
     const int nchunks = (p->L + p->C - 1) / p->C;
     const int seg = row_norm ? 0 : segment_chunks(p);
-    const SimtLayout lay = simt_layout(p->d, p->h, p->C, nmat, nchunks, true, true, seg);
+    const SimtLayout lay = layout_of(p, true, true, row_norm != nullptr);
+    const bool tile = impl != E2TTT_IMPL_SIMT && can_tile(p);
+
     void* ws_data = static_cast<char*>(workspace) + kStatusBytes;
     if (cudaMemsetAsync(workspace, 0, sizeof(int), reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -394,7 +427,7 @@ static int bwd_common(const e2ttt_params* p, const void* q, const void* k, const
             f.row_norm[i] = row_norm ? row_norm[i] : nullptr;
         }
         f.norm_eps = norm_eps;
-        return simt_fwd_launch(f, p->kind, p->io_dtype, stream);
+        return tile ? tile_fwd_launch(f, p->kind, stream) : simt_fwd_launch(f, p->kind, p->io_dtype, stream);
     };
     // The reverse sweep over chunks [first_chunk, first_chunk + n), whose start states sit in lay.ckpt slots 0 .. n-1.
     auto reverse = [&](int first_chunk, int n, bool carry_in, bool carry_out) -> int {

@@ -42,6 +42,10 @@ int scratch_for_current_device(void** out) {
 }  // namespace
 
 namespace e2ttt {
+size_t fixed_scratch_need(const e2ttt_params* p, size_t have);  // api.cu
+int fwd_fixed_scratch(const e2ttt_params* p, const void* q, const void* k, const void* v, const float* eta, const float* beta,
+                      const float* gamma, const float* const* W_init, const float* const* M_init, void* o, float* const* W_final,
+                      float* const* M_final, void* scratch, size_t have, void* stream);
 // Device address of the scratch array on the current device, or nullptr before the first call there.  Its first
 // word is the device status word of the calls that used it (read by e2ttt_device_status(NULL, ...)).
 const void* noalloc_scratch_if_known() {
@@ -60,10 +64,11 @@ extern "C" E2TTT_API int e2ttt_chunk_fwd_noalloc(const e2ttt_params* p, const vo
     size_t need = 0;
     int rc = e2ttt_workspace_bytes(p, 0, &need);
     if (rc != E2TTT_OK) return rc;
+    need = e2ttt::fixed_scratch_need(p, (size_t)E2TTT_NOALLOC_SCRATCH_BYTES);
     if (need > (size_t)E2TTT_NOALLOC_SCRATCH_BYTES) return E2TTT_ERR_WORKSPACE;
     void* scratch = nullptr;
     rc = scratch_for_current_device(&scratch);
     if (rc != E2TTT_OK) return rc;
-    return e2ttt_chunk_fwd(p, q, k, v, eta, beta, gamma, W_init, M_init, o, W_final, M_final, scratch,
-                           (size_t)E2TTT_NOALLOC_SCRATCH_BYTES, 0, stream);
+    return e2ttt::fwd_fixed_scratch(p, q, k, v, eta, beta, gamma, W_init, M_init, o, W_final, M_final, scratch,
+                                    (size_t)E2TTT_NOALLOC_SCRATCH_BYTES, stream);
 }

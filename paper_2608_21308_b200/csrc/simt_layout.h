@@ -4,6 +4,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "tile_layout.h"
+
 namespace e2ttt {
 
 struct SimtLayout {
@@ -25,21 +27,34 @@ struct SimtLayout {
     size_t cck;          // seg > 0: [nseg + 1][2][nmat][d*h] chunk-start states of every seg-th chunk (the checkpoints)
     int seg;             // chunks per segment (e2ttt_params.ckpt_every >= 2); 0 = the state of every chunk is kept
     size_t per_seq;      // elements per sequence
+    TileLayout tl;       // region of the block-tiled kernels, when `tile`
 };
 
-inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool save_states, bool backward, int seg = 0) {
+// tile != 0: a call may run on the block-tiled kernels (bf16 I/O, d <= 128): their region shares the space of the SIMT
+// kernels' intermediates (a call uses one of the two), behind the state that both kinds leave for each other.
+inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool save_states, bool backward, int seg = 0, int tile = 0, int N = 1) {
     SimtLayout l{};
     size_t o = 0;
     const size_t dh = (size_t)d * h;
     auto take = [&](size_t n) { size_t r = o; o += (n + 31) / 32 * 32; return r; };
     for (int i = 0; i < 3; ++i) { l.W[i] = take(i < nmat ? dh : 0); l.M[i] = take(i < nmat ? dh : 0); }
+    l.seg = save_states ? seg : 0;
+    if (backward)
+        for (int i = 0; i < 3; ++i) { l.T[i] = take(i < nmat ? dh : 0); l.S[i] = take(i < nmat ? dh : 0); }
+    l.rown = take(save_states && l.seg == 0 ? (size_t)nchunks * 3 * (size_t)(d > h ? d : h) : 0);
+    if (l.seg > 0) {
+        l.ckpt = take((size_t)(l.seg + 1) * 2 * nmat * dh);
+        l.cck = take((size_t)((nchunks + l.seg - 1) / l.seg + 1) * 2 * nmat * dh);
+    } else {
+        l.ckpt = take(save_states ? (size_t)(nchunks + 1) * 2 * nmat * dh : 0);
+        l.cck = 0;
+    }
+    const size_t begin = o;
     l.Z1 = take((size_t)2 * C * h); l.Z2 = take((size_t)2 * C * h); l.A = take((size_t)2 * C * h);
     l.U = take((size_t)2 * C * d); l.Pu = take((size_t)C * d);
     l.Pz1 = take((size_t)C * h); l.Pz2 = take((size_t)C * h);
     if (backward) {
-        for (int i = 0; i < 3; ++i) {
-            l.T[i] = take(i < nmat ? dh : 0); l.S[i] = take(i < nmat ? dh : 0); l.Wb[i] = take(i < nmat ? dh : 0);
-        }
+        for (int i = 0; i < 3; ++i) l.Wb[i] = take(i < nmat ? dh : 0);
         l.Pa = take((size_t)C * h); l.E = take((size_t)C * d);
         l.XY2 = take((size_t)C * 2 * d); l.XY1 = take((size_t)C * 2 * h);
         l.Pub = take((size_t)C * d); l.Pzb = take((size_t)C * h); l.Zkb = take((size_t)C * h);
@@ -51,14 +66,9 @@ inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool s
         l.kWb = take(C); l.kMb = take(C);
     }
     l.splitk = take((size_t)2 * 8 * 128 * 64);
-    l.rown = take(save_states ? (size_t)nchunks * 3 * (size_t)(d > h ? d : h) : 0);
-    l.seg = save_states ? seg : 0;
-    if (l.seg > 0) {
-        l.ckpt = take((size_t)(l.seg + 1) * 2 * nmat * dh);
-        l.cck = take((size_t)((nchunks + l.seg - 1) / l.seg + 1) * 2 * nmat * dh);
-    } else {
-        l.ckpt = take(save_states ? (size_t)(nchunks + 1) * 2 * nmat * dh : 0);
-        l.cck = 0;
+    if (tile) {
+        const size_t end = tile_layout(l.tl, begin, N, d, h, C, nmat, backward);
+        if (end > o) o = end;
     }
     l.per_seq = o;
     return l;
@@ -122,5 +132,8 @@ inline int simt_cluster_size(int N) {
 // launchers (simt_fwd.cu / simt_bwd.cu); return a cudaError_t value as int
 int simt_fwd_launch(const SimtFwdArgs& a, int kind, int io_dtype, void* stream);
 int simt_bwd_launch(const SimtBwdArgs& a, int kind, int io_dtype, void* stream);
+// the same calls on the block-tiled kernels (tile_fwd.cu / tile_bwd.cu); the layout must have been made with `tile`
+int tile_fwd_launch(const SimtFwdArgs& a, int kind, void* stream);
+int tile_bwd_launch(const SimtBwdArgs& a, int kind, void* stream);
 
 }  // namespace e2ttt
