@@ -455,7 +455,7 @@ static int bwd_common(const e2ttt_params* p, const void* q, const void* k, const
             b.d_row_norm[i] = (row_norm && d_row_norm) ? d_row_norm[i] : nullptr;
         }
         b.norm_eps = norm_eps;
-        return simt_bwd_launch(b, p->kind, p->io_dtype, stream);
+        return tile ? tile_bwd_launch(b, p->kind, stream) : simt_bwd_launch(b, p->kind, p->io_dtype, stream);
     };
 
     if (seg == 0) {
