@@ -92,6 +92,11 @@ struct Engine {
     __device__ void teardown() {
         tc_fence_before_sync();
         __syncthreads();
+        if (*wc.dead) {  // a wait has given up: copies nobody waited for may still be under way to this CTA's shared memory
+            const long long t0 = clock64();
+            while (clock64() - t0 < 8000000) {}
+            __syncthreads();
+        }
         if (warp == 0) tmem_dealloc(tmem, 512);
     }
 
@@ -302,6 +307,17 @@ __device__ __forceinline__ void st_tok4(__nv_bfloat16* row, int c, int d, const 
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             if (c + j < d) row[c + j] = __float2bfloat16_rn(v[j]);
+    }
+}
+// v += p[0] + p[stride] + .., in that order, four loads in flight
+__device__ __forceinline__ void add_parts(const float* p, int n, size_t stride, float (&v)[4]) {
+    for (int i0 = 0; i0 < n; i0 += 4) {
+        float4 x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            x[i] = i0 + i < n ? *reinterpret_cast<const float4*>(p + (size_t)(i0 + i) * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { v[0] += x[i].x; v[1] += x[i].y; v[2] += x[i].z; v[3] += x[i].w; }
     }
 }
 __device__ __forceinline__ float sum4(const float (&a)[4]) { return (a[0] + a[1]) + (a[2] + a[3]); }

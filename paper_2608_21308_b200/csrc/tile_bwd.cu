@@ -330,12 +330,9 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_rev_kern
         __nv_bfloat16* dkc = reinterpret_cast<__nv_bfloat16*>(a.dk) + ((size_t)seq * a.Ls + s) * d;
         for (int t = rank * kEpiWarps + warp; t < len; t += CL * kEpiWarps) {
             if (ci >= dp) continue;
-            float4 x = *reinterpret_cast<const float4*>(ws + tl.bEb[buf] + (size_t)t * dp + ci);
-            for (int r = 0; r < 2 * CL; ++r) {
-                const float4 p = *reinterpret_cast<const float4*>(ws + tl.bdk[buf] + ((size_t)r * tb * 64 + t) * dp + ci);
-                x.x += p.x; x.y += p.y; x.z += p.z; x.w += p.w;
-            }
-            const float o[4] = {x.x, x.y, x.z, x.w};
+            const float4 x = *reinterpret_cast<const float4*>(ws + tl.bEb[buf] + (size_t)t * dp + ci);
+            float o[4] = {x.x, x.y, x.z, x.w};
+            add_parts(ws + tl.bdk[buf] + (size_t)t * dp + ci, 2 * CL, (size_t)tb * 64 * dp, o);
             st_tok4(dkc + (size_t)t * d, ci, d, o);
         }
     };
@@ -428,39 +425,52 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_rev_kern
                         const size_t e0 = ok ? (((size_t)bl * tb + tk) * 64 + tok) * 64 + (row & 63) : 0;
                         const float* kw = sh.kw + tk * 64 + tok;
                         const float* km = sh.km + tk * 64 + tok;
-                        float x[16], y[16], phb[16];
+                        float x[16], y[16], phb[16], z0[16], ph[16], cv[16];
+                        auto ld_col = [&](size_t src, float (&v)[16]) {
 #pragma unroll
-                        for (int i = 0; i < LAST; ++i) {
-                            acc16(t + 128 * i + tok, x);
-                            acc16(t + 128 * i + 64 + tok, y);
-                            if (ok) {
-                                float ph[16], c1[16];
+                            for (int j = 0; j < 16; ++j) v[j] = ok ? sl[src + e0 + 64 * j] : 0.0f;
+                        };
+                        ld_col(tl.sph, ph);
+                        ld_col(tl.sc1, cv);
+                        ld_col(tl.sc4, z0);
+                        acc16(t + tok, x);
+                        acc16(t + 64 + tok, y);
 #pragma unroll
-                                for (int j = 0; j < 16; ++j) {
-                                    ph[j] = sl[tl.sph + e0 + 64 * j];
-                                    c1[j] = sl[(i ? tl.sc2 : tl.sc1) + e0 + 64 * j];
-                                }
+                        for (int j = 0; j < 16; ++j) {
+                            const float pz = ph[j] * cv[j], pzb = -(kw[j] * x[j] + km[j] * y[j]);
+                            x[j] = ok ? x[j] * pz : 0.0f;
+                            y[j] = ok ? y[j] * pz : 0.0f;
+                            phb[j] = pzb * cv[j];
+                            z0[j] *= pzb;
+                            if (SW) cv[j] = pzb;
+                        }
+                        kwb -= reduce16(x, lane);
+                        kmb -= reduce16(y, lane);
+                        if (SW) {
+                            ld_col(tl.sg1, x);
 #pragma unroll
-                                for (int j = 0; j < 16; ++j) {
-                                    const float pz = ph[j] * c1[j], pzb = -(kw[j] * x[j] + km[j] * y[j]);
-                                    x[j] *= pz;
-                                    y[j] *= pz;
-                                    if (i == 0) {
-                                        phb[j] = pzb * c1[j];
-                                        ws[tl.bz0[0] + e0 + 64 * j] = pzb * sl[tl.sc4 + e0 + 64 * j];
-                                        if (SW) ws[tl.bz0[LAST - 1] + e0 + 64 * j] = pzb * ph[j] * sl[tl.sg1 + e0 + 64 * j];
-                                    } else {
-                                        phb[j] += pzb * c1[j];
-                                        ws[tl.bz0[0] + e0 + 64 * j] += pzb * ph[j] * sl[tl.sg1 + e0 + 64 * j];
-                                    }
-                                }
-                            } else {
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) x[j] = y[j] = 0.0f;
+                            for (int j = 0; j < 16; ++j) {
+                                x[j] *= ph[j];  // ph silu'(z1)
+                                if (ok) ws[tl.bz0[LAST - 1] + e0 + 64 * j] = cv[j] * x[j];
                             }
-                            kwb -= reduce16(x, lane);
+                            ld_col(tl.sc2, cv);
+                            float x2[16];
+                            acc16(t + 128 + tok, x2);
+                            acc16(t + 192 + tok, y);
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                const float pz = ph[j] * cv[j], pzb = -(kw[j] * x2[j] + km[j] * y[j]);
+                                x2[j] = ok ? x2[j] * pz : 0.0f;
+                                y[j] = ok ? y[j] * pz : 0.0f;
+                                phb[j] += pzb * cv[j];
+                                z0[j] += pzb * x[j];
+                            }
+                            kwb -= reduce16(x2, lane);
                             kmb -= reduce16(y, lane);
                         }
+                        if (ok)
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) ws[tl.bz0[0] + e0 + 64 * j] = z0[j];
                         if (ok) st_split16(blk(tl.bPhb) + ((size_t)bl * tb + tk) * B, row & 63, tok, phb);
                     });
                 }
@@ -570,10 +580,7 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_rev_kern
                         const float4 p4 = *reinterpret_cast<const float4*>(sl + tl.spu + (size_t)t * dp + ci);
                         y[0] = y4.x; y[1] = y4.y; y[2] = y4.z; y[3] = y4.w;
                         pu[0] = p4.x; pu[1] = p4.y; pu[2] = p4.z; pu[3] = p4.w;
-                        for (int i = 0; i < 2 * CL; ++i) {
-                            const float4 p = *reinterpret_cast<const float4*>(ws + tl.bslot + ((size_t)i * tb * 64 + t) * dp + ci);
-                            pub[0] += p.x; pub[1] += p.y; pub[2] += p.z; pub[3] += p.w;
-                        }
+                        add_parts(ws + tl.bslot + (size_t)t * dp + ci, 2 * CL, (size_t)tb * 64 * dp, pub);
                     }
                     const float sx = warp_sum(sum4(pub)) * inv, mpy = warp_sum(dot4(pub, y)) * inv, spp = warp_sum(dot4(pub, pu));
 #pragma unroll
@@ -605,17 +612,34 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_rev_kern
                 G.term<1>(db, false, uk, p, {0u});
                 G.job_end([&](uint32_t t) {
                     const int bl = b0 + (row >> 6), tok = 16 * grp;
-                    float x[16], z[16];
-                    acc16(t + tok, x);
-                    if (row >= 64 && !two) return;
+                    float x[16], z[16], cv[16], ab[16];
+                    const bool ok = row < 64 || two;
                     const size_t e0 = (((size_t)bl * tb + tk) * 64 + tok) * 64 + (row & 63);
+                    if (ok)
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) x[j] += ws[tl.bakb + e0 + 64 * j];
+                        for (int j = 0; j < 16; ++j) {
+                            ab[j] = ws[tl.bakb + e0 + 64 * j];
+                            z[j] = ws[tl.bz0[0] + e0 + 64 * j];
+                            cv[j] = sl[tl.sc1 + e0 + 64 * j];
+                        }
+                    acc16(t + tok, x);
+                    if (!ok) return;
 #pragma unroll
-                    for (int i = 0; i < LAST; ++i) {
+                    for (int j = 0; j < 16; ++j) {
+                        x[j] += ab[j];
+                        z[j] += x[j] * cv[j];
+                    }
+                    if (SW)
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) z[j] = ws[tl.bz0[i] + e0 + 64 * j] + x[j] * sl[(i ? tl.sc2 : tl.sc1) + e0 + 64 * j];
-                        st_split16(blk(tl.bZk[i]) + ((size_t)bl * tb + tk) * B, row & 63, tok, z);
+                        for (int j = 0; j < 16; ++j) {
+                            ab[j] = ws[tl.bz0[LAST - 1] + e0 + 64 * j];
+                            cv[j] = sl[tl.sc2 + e0 + 64 * j];
+                        }
+                    st_split16(blk(tl.bZk[0]) + ((size_t)bl * tb + tk) * B, row & 63, tok, z);
+                    if (SW) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) ab[j] += x[j] * cv[j];
+                        st_split16(blk(tl.bZk[LAST - 1]) + ((size_t)bl * tb + tk) * B, row & 63, tok, ab);
                     }
                 });
             }
@@ -755,7 +779,7 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_rev_kern
 // One thread walks the chunk (a 3-term linear recurrence, ~10 flop per token) over operands in shared memory; the chunks are
 // independent.
 __global__ void __launch_bounds__(128) tile_gate_kernel(const GroupArgs ga) {
-    __shared__ float in[5][kMaxC], res[3][kMaxC];
+    __shared__ float in[8][kMaxC], res[3][kMaxC];
     const SimtBwdArgs& a = ga.a;
     const TileLayout& tl = a.lay.tl;
     const int seq = blockIdx.x / ga.ng, g = blockIdx.x % ga.ng, c = ga.c0 + g, s = c * a.C, len = min(a.C, a.L - s), CL = a.cl;
@@ -764,6 +788,7 @@ __global__ void __launch_bounds__(128) tile_gate_kernel(const GroupArgs ga) {
     const size_t t0 = (size_t)seq * a.Ls + s;
     for (int t = threadIdx.x; t < len; t += blockDim.x) {
         in[0][t] = a.beta[t0 + t]; in[1][t] = a.gamma[t0 + t]; in[2][t] = a.eta[t0 + t];
+        in[5][t] = sc.S[t + 1]; in[6][t] = sc.bt[t + 1]; in[7][t] = sc.gt[t + 1];
         float w = 0.0f, m = 0.0f;
         for (int r = 0; r < CL; ++r) {
             w += sl[tl.skwb + (size_t)r * tl.tb * 64 + t];
@@ -778,7 +803,7 @@ __global__ void __launch_bounds__(128) tile_gate_kernel(const GroupArgs ga) {
         for (int t = 0; t < len; ++t) {
             // index t: state t; token t + 1 lives at array index t
             const float b1 = in[0][t], g1 = in[1][t], e1 = in[2][t], kWb = in[3][t], kMb = in[4][t];
-            const float S1 = sc.S[t + 1], bt1 = sc.bt[t + 1], gt1 = sc.gt[t + 1];
+            const float S1 = in[5][t], bt1 = in[6][t], gt1 = in[7][t];
             // S_t = beta_{t+1} S_{t+1} + gt_t ; bt_t = beta_{t+1} bt_{t+1} ; gt_t = gamma_{t+1} gt_{t+1}
             gtb += Sb;
             float bb = Sb * S1 + btb * bt1, Sn = Sb * b1, bn = btb * b1;

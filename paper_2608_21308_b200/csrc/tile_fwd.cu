@@ -166,11 +166,7 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_fwd_kern
                 if (live) {
                     ld_tok4((key ? kc : qc) + (size_t)t * d, ci, d, x);
                     if (key) ld_tok4(vc + (size_t)t * d, ci, d, vv);
-                    if (ci < dp)
-                        for (int r = 0; r < CL; ++r) {
-                            const float4 p = *reinterpret_cast<const float4*>(ws + tl.fslot + ((size_t)(r * tb + tk) * 128 + (rr & 127)) * dp + ci);
-                            u[0] += p.x; u[1] += p.y; u[2] += p.z; u[3] += p.w;
-                        }
+                    if (ci < dp) add_parts(ws + tl.fslot + ((size_t)tk * 128 + (rr & 127)) * dp + ci, CL, (size_t)tb * 128 * dp, u);
                     const float mu = warp_sum(sum4(u)) / (float)d;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) u[j] = ci + j < d ? u[j] - mu : 0.0f;

@@ -28,9 +28,10 @@ struct TileLayout {
     size_t sK, sQ, sW[3], sAk, sAq, sZq[2], sPz[2], sPu, sUq, sph, sc1, sc2, sg1, sc4, sc1q, sc2q, sU, sy, spu, sr, smey, ssc, skwb, sdots;
 };
 
-// CTAs per sequence for N sequences: as many as keep every cluster resident at one CTA per SM, at most one per 64 hidden units
+// CTAs per sequence for N sequences: as many as keep every cluster resident at one CTA per SM (the driver's occupancy calculator:
+// GPU processing clusters do not divide evenly into larger clusters), at most one per 64 hidden units
 inline int tile_cluster_size(int N, int hb) {
-    static const int fit[9] = {0, 148, 74, 46, 33, 26, 22, 18, 16};  // clusters of 1..8 CTAs that fit the GPU together
+    static const int fit[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};  // clusters of 1..8 CTAs that fit the GPU together
     int cl = 1;
     for (int c = 2; c <= kTileMaxCl; ++c)
         if (N <= fit[c]) cl = c;
