@@ -134,37 +134,57 @@ def _io_torch_dtype(p):
     return torch.float32 if p.io_dtype == E2TTT_F32 else torch.bfloat16
 
 
+# A decode step is one 5-10 us kernel per layer, so what a call costs on the host counts: shapes of the matrices and the
+# ctypes table types are looked up once per (kind, d, h), pointers travel as plain integers, and the current stream
+# is asked for by its handle.  The checks of every argument stay (about 0.4 us per tensor).
+_F32 = torch.float32
+_shape_cache = {}
+
+
+def _state_shapes(p):
+    """((rows, cols) of every matrix, ctypes array type of a pointer table) of a call's network."""
+    key = (p.kind, p.d, p.h)
+    got = _shape_cache.get(key)
+    if got is None:
+        n = e2ttt_num_matrices(p.kind)
+        got = (tuple(e2ttt_matrix_shape(p.kind, p.d, p.h, i) for i in range(n)), ctypes.c_void_p * n)
+        if len(_shape_cache) >= 256:
+            _shape_cache.clear()
+        _shape_cache[key] = got
+    return got
+
+
 def _ptr(t, dtype, shape, name):
     if t is None:
         return None
+    try:
+        if t.is_cuda and t.dtype is dtype and t.is_contiguous() and (shape is None or t.shape == shape):
+            return t.data_ptr()
+    except AttributeError:
+        pass
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name}: expected a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name}: expected dtype {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name}: must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
-        raise ValueError(f"{name}: expected shape {tuple(shape)}, got {tuple(t.shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    raise ValueError(f"{name}: expected shape {tuple(shape)}, got {tuple(t.shape)}")
 
 
 def _table(ts, p, name):
     if ts is None:
         return None
-    n = e2ttt_num_matrices(p.kind)
-    if len(ts) != n:
-        raise ValueError(f"{name}: expected {n} matrices")
-    arr = (ctypes.c_void_p * n)()
-    for i, t in enumerate(ts):
-        r, c = e2ttt_matrix_shape(p.kind, p.d, p.h, i)
-        arr[i] = _ptr(t, torch.float32, (p.B, p.H, r, c), f"{name}[{i}]")
-    return arr
+    shapes, array = _state_shapes(p)
+    if len(ts) != len(shapes):
+        raise ValueError(f"{name}: expected {len(shapes)} matrices")
+    B, H = p.B, p.H
+    return array(*[_ptr(t, _F32, (B, H, *rc), f"{name}[{i}]") for i, (t, rc) in enumerate(zip(ts, shapes))])
 
 
 def _stream_ptr(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if isinstance(stream, torch.cuda.Stream) else int(stream))
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if isinstance(stream, torch.cuda.Stream) else int(stream)
 
 
 def e2ttt_chunk_fwd(p, q, k, v, eta, beta, gamma, W_init, M_init, o, W_final, M_final, workspace,
@@ -188,14 +208,10 @@ def _row_table(ts, p, name):
     """nmat pointers to [B, H, rows_i] fp32 tensors (row targets of the post-chunk normalisation, or their adjoints)."""
     if ts is None:
         return None
-    n = e2ttt_num_matrices(p.kind)
-    if len(ts) != n:
-        raise ValueError(f"{name}: expected {n} tensors")
-    arr = (ctypes.c_void_p * n)()
-    for i, t in enumerate(ts):
-        r, _ = e2ttt_matrix_shape(p.kind, p.d, p.h, i)
-        arr[i] = _ptr(t, torch.float32, (p.B, p.H, r), f"{name}[{i}]")
-    return arr
+    shapes, array = _state_shapes(p)
+    if len(ts) != len(shapes):
+        raise ValueError(f"{name}: expected {len(shapes)} tensors")
+    return array(*[_ptr(t, _F32, (p.B, p.H, rc[0]), f"{name}[{i}]") for i, (t, rc) in enumerate(zip(ts, shapes))])
 
 
 def e2ttt_chunk_fwd_normed(p, q, k, v, eta, beta, gamma, W_init, M_init, row_norm, norm_eps, o, W_final, M_final,
@@ -275,8 +291,8 @@ def e2ttt_apply(p, q, W, o, stream=None):
     """int e2ttt_apply(...) of include/e2ttt.h: o = f_W(q) for p.L tokens per sequence, no update.  Raises on error."""
     io = _io_torch_dtype(p)
     s4 = (p.B, p.H, p.L, p.d)
-    st = lib().e2ttt_apply(ctypes.byref(p), _ptr(q, io, s4, "q"), _table(W, p, "W"), _ptr(o, io, s4, "o"),
-                           _stream_ptr(stream))
+    st = (_lib or lib()).e2ttt_apply(ctypes.byref(p), _ptr(q, io, s4, "q"), _table(W, p, "W"), _ptr(o, io, s4, "o"),
+                                     _stream_ptr(stream))
     if st != E2TTT_OK:
         raise E2TTTError(st, "e2ttt_apply")
     return st
