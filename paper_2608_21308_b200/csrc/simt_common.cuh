@@ -11,6 +11,7 @@ constexpr int kSimtThreads = 256;
 constexpr int kMaxC = 512;  // the paper trains with chunks of 512 tokens
 constexpr int kMaxMat = 3;
 constexpr int kBM = 64, kBN = 64, kBK = 16;
+constexpr int kSM = 16, kSK = 64, kSplit = 4;  // the small tiling of the FMA GEMM
 
 // ---- I/O conversion -------------------------------------------------------------------------
 template <typename Real> __device__ __forceinline__ Real ld_io(const float* p, size_t i) { return (Real)p[i]; }
@@ -96,11 +97,9 @@ template <typename Real> struct ChunkScalars {
     Real cw, cm, cb;    // gt_0, bt_0 R_1 = beta_1 S_1, bt_0
 };
 
-// Executed by warp 0 only.  eta/beta/gamma point at the chunk's first token; len <= kMaxC tokens.
-template <typename Real>
-__device__ void chunk_scalars_warp(const float* eta, const float* beta, const float* gamma, int len,
-                                   ChunkScalars<Real>* out) {
-    constexpr int EPL = kMaxC / 32; // tokens per lane
+// Executed by one warp.  eta/beta/gamma point at the chunk's first token; len <= 32 EPL tokens, EPL per lane.
+template <typename Real, int EPL>
+__device__ void chunk_scalars_scan(const float* eta, const float* beta, const float* gamma, int len, ChunkScalars<Real>* out) {
     const int lane = threadIdx.x & 31;
     ScanMap<Real> local[EPL + 1];
     local[EPL].B = 1; local[EPL].G = 1; local[EPL].X = 0;
@@ -148,6 +147,12 @@ __device__ void chunk_scalars_warp(const float* eta, const float* beta, const fl
         out->cm = (Real)beta[0] * out->S[1];
     }
 }
+// A lane's own tokens are a serial chain in front of the shuffles, so short chunks take fewer per lane.
+template <typename Real>
+__device__ void chunk_scalars_warp(const float* eta, const float* beta, const float* gamma, int len, ChunkScalars<Real>* out) {
+    if (len <= 64) chunk_scalars_scan<Real, 2>(eta, beta, gamma, len, out);
+    else chunk_scalars_scan<Real, kMaxC / 32>(eta, beta, gamma, len, out);
+}
 
 // ---- elementwise pass with batched loads ---------------------------------------------------------
 // for e = begin, begin + stride, ... < end:  store(e, load(e)).  `load` returns everything element e needs from
@@ -180,6 +185,7 @@ __device__ __forceinline__ void phase_sync(int nranks) {
     if (nranks == 1) {
         __syncthreads();
     } else {
+        __syncwarp();  // .aligned: the warp's threads execute the instruction together, whatever branches came before
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
@@ -190,17 +196,109 @@ __device__ __forceinline__ void phase_sync(int nranks) {
 //   fa(m, k, a0, a1) writes the A value(s); fb(n, k) returns the B value; pre(m, n) loads what a result combines
 //   with; epi(m, n, acc0, acc1, loaded) consumes a result.
 // A_KFAST / B_KFAST say which index is contiguous in memory, so that neighbouring threads read neighbouring words.
-// 64x64 output tiles (dealt round-robin to the `nranks` CTAs of the sequence's cluster), 16-deep k slices through
-// shared memory, 4x4 results per thread.  Ends with phase_sync().
+// Two tilings, both ending with phase_sync(); the tiles are dealt round-robin to the `nranks` CTAs of the sequence's cluster:
+//   64x64 tiles, 16-deep k slices, 4x4 results per thread: fewest loads per product, where there is a tile for every CTA;
+//   16x16 tiles, 64-deep k slices cut four ways inside the CTA, 2x2 results per thread, the next slice's loads in flight while one
+//   is multiplied: for the few tokens of a small problem.  A [32 x 64] result with 256 terms is one 64x64 tile - one CTA of
+//   eight, half of its rows unused, 16 exposed round trips to L2 (14 us in fp64) - but 8 small ones with 4 slices each.
 template <typename Real> struct GemmSmem {
-    Real A[2][kBK][kBM + 4];
-    Real B[kBK][kBN + 4];
+    union {
+        struct {
+            Real A[2][kBK][kBM + 4];
+            Real B[kBK][kBN + 4];
+        };
+        struct {
+            Real a[2][kSK][kSM + 2];
+            Real b[kSK][kSM + 2];
+            Real part[2][kSplit][kSM * kSM];
+        } s;
+    };
 };
+
+template <typename Real, int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FP, typename FE>
+__device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, GemmSmem<Real>* sm, int rank, int nranks) {
+    const int tid = threadIdx.x;
+    const int grp = tid / (kSimtThreads / kSplit), tx = tid & 7, ty = (tid >> 3) & 7;
+    const int tn = (N + kSM - 1) / kSM, tiles = tn * ((M + kSM - 1) / kSM), slices = (K + kSK - 1) / kSK;
+    const int items = rank < tiles ? ((tiles - rank + nranks - 1) / nranks) * slices : 0;  // (tile, slice) in order
+    constexpr int PER = kSM * kSK / kSimtThreads;
+    Real ra0[PER], ra1[PER], rb[PER];
+    auto fetch = [&](int item) {
+        const int tile = rank + (item / slices) * nranks, k0 = (item % slices) * kSK;
+        const int m0 = (tile / tn) * kSM, n0 = (tile % tn) * kSM;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int idx = tid + r * kSimtThreads;
+            const int am = A_KFAST ? idx / kSK : idx % kSM, ak = A_KFAST ? idx % kSK : idx / kSM;
+            const int bn = B_KFAST ? idx / kSK : idx % kSM, bk = B_KFAST ? idx % kSK : idx / kSM;
+            ra0[r] = ra1[r] = rb[r] = 0;
+            if (m0 + am < M && k0 + ak < K) fa(m0 + am, k0 + ak, ra0[r], ra1[r]);
+            if (n0 + bn < N && k0 + bk < K) rb[r] = fb(n0 + bn, k0 + bk);
+        }
+    };
+    if (items > 0) fetch(0);
+    Real acc[NACC][2][2];
+    for (int item = 0; item < items; ++item) {
+        const int slice = item % slices;
+        if (slice == 0)
+#pragma unroll
+            for (int a = 0; a < NACC; ++a) acc[a][0][0] = acc[a][0][1] = acc[a][1][0] = acc[a][1][1] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int idx = tid + r * kSimtThreads;
+            const int am = A_KFAST ? idx / kSK : idx % kSM, ak = A_KFAST ? idx % kSK : idx / kSM;
+            const int bn = B_KFAST ? idx / kSK : idx % kSM, bk = B_KFAST ? idx % kSK : idx / kSM;
+            sm->s.a[0][ak][am] = ra0[r];
+            if (NACC == 2) sm->s.a[1][ak][am] = ra1[r];
+            sm->s.b[bk][bn] = rb[r];
+        }
+        __syncthreads();
+        if (item + 1 < items) fetch(item + 1);
+#pragma unroll 4
+        for (int i = 0; i < kSK / kSplit; ++i) {
+            const int kk = grp * (kSK / kSplit) + i;
+            const Real b0 = sm->s.b[kk][2 * tx], b1 = sm->s.b[kk][2 * tx + 1];
+#pragma unroll
+            for (int a = 0; a < NACC; ++a) {
+                const Real a0 = sm->s.a[a][kk][2 * ty], a1 = sm->s.a[a][kk][2 * ty + 1];
+                acc[a][0][0] += a0 * b0; acc[a][0][1] += a0 * b1;
+                acc[a][1][0] += a1 * b0; acc[a][1][1] += a1 * b1;
+            }
+        }
+        if (slice == slices - 1) {
+            const int tile = rank + (item / slices) * nranks;
+            const int m = (tile / tn) * kSM + tid / kSM, n = (tile % tn) * kSM + tid % kSM;
+            using P = decltype(pre(0, 0));
+            P p;
+            if (m < M && n < N) p = pre(m, n);
+#pragma unroll
+            for (int a = 0; a < NACC; ++a)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) sm->s.part[a][grp][(2 * ty + i) * kSM + 2 * tx + j] = acc[a][i][j];
+            __syncthreads();
+            Real s[2] = {0, 0};
+#pragma unroll
+            for (int a = 0; a < NACC; ++a)
+#pragma unroll
+                for (int g = 0; g < kSplit; ++g) s[a] += sm->s.part[a][g][tid];
+            if (m < M && n < N) epi(m, n, s[0], s[NACC - 1], p);
+        }
+    }
+}
 
 template <typename Real, int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FP, typename FE>
 __device__ void block_gemm(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, GemmSmem<Real>* sm, int rank, int nranks) {
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
+    // fewer large tiles than CTAs, or a lone tile's row that is mostly padding: the small tiling keeps the cluster busy
+    if (((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN) < nranks || 2 * M <= kBM || 2 * N <= kBN) {
+        block_gemm_small<Real, NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, pre, epi, sm, rank, nranks);
+        phase_sync(nranks);
+        return;
+    }
     int tile = 0;
     for (int m0 = 0; m0 < M; m0 += kBM) {
         for (int n0 = 0; n0 < N; n0 += kBN, ++tile) {
