@@ -7,6 +7,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <initializer_list>
+
 #include "simt_common.cuh"
 #include "sm100.cuh"
 
@@ -130,6 +132,60 @@ static __device__ void tc_chunk_tails(const float* beta, const float* gamma, int
         }
     }
     __syncwarp();
+}
+
+// 16 consecutive values of a state row <-> global memory.  Every lane has a row of its own (a TMEM lane), so an access of a warp
+// touches 32 sectors whatever its width: 32-byte accesses fill them, 16-byte ones take twice the transactions (saving every
+// every chunk's state at config 2: 2.48 ms with 16-byte stores, 1.88 ms with these).  WIDE: every state pointer is 32-byte aligned
+// (rows are 64-byte multiples apart); a template switch, because a second path inside the chunk loop costs the loop 5 %.
+template <bool WIDE> __device__ __forceinline__ void st_row16(float* p, const float* v) {
+    if (WIDE) {
+#pragma unroll
+        for (int j = 0; j < 16; j += 8)
+            asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p + j), "f"(v[j]), "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3]),
+                         "f"(v[j + 4]), "f"(v[j + 5]), "f"(v[j + 6]), "f"(v[j + 7])
+                         : "memory");
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(p + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    }
+}
+template <bool WIDE> __device__ __forceinline__ void st_row16(float* p, const uint32_t* v) {
+    float f[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
+    st_row16<WIDE>(p, f);
+}
+// `real` false: zeros.  (M_init has no alignment rule of its own: down to single words.)
+template <bool WIDE> __device__ __forceinline__ void ld_row16(const float* p, float* v, bool real) {
+    if (!real) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = 0.0f;
+    } else if (WIDE) {
+#pragma unroll
+        for (int j = 0; j < 16; j += 8)
+            asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                         : "=f"(v[j]), "=f"(v[j + 1]), "=f"(v[j + 2]), "=f"(v[j + 3]), "=f"(v[j + 4]), "=f"(v[j + 5]), "=f"(v[j + 6]), "=f"(v[j + 7])
+                         : "l"(p + j));
+    } else if ((reinterpret_cast<size_t>(p) & 15) == 0) {
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+            const float4 x = *reinterpret_cast<const float4*>(p + j);
+            v[j] = x.x; v[j + 1] = x.y; v[j + 2] = x.z; v[j + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = p[j];
+    }
+}
+
+// every state pointer of a call (nullptr entries aside) 32-byte aligned, and the sequences' strides multiples of 8 floats
+inline bool wide_rows(std::initializer_list<const void*> ptrs, std::initializer_list<size_t> strides) {
+    for (const void* p : ptrs)
+        if (reinterpret_cast<size_t>(p) & 31) return false;
+    for (size_t n : strides)
+        if (n & 7) return false;
+    return true;
 }
 
 __device__ __forceinline__ float fast_tanh(float x) {

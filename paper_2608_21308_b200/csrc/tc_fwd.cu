@@ -123,7 +123,8 @@ __device__ __forceinline__ float gelu_d1_fast(float z) {
 // spans the 4 CTAs, so its sum of squares crosses the cluster once per chunk.
 // MULTI: chunks of several 64-token blocks (128, 256, 512 tokens); a compile-time switch, so that the single-block
 // instantiations are exactly the code they were without it
-template <bool PAD, bool NORM, bool MULTI = false>
+// WIDE: 32-byte accesses to the state (tc_common.cuh)
+template <bool PAD, bool NORM, bool MULTI, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ,
               const __grid_constant__ CUtensorMap tmV, const TcFwdArgs a) {
@@ -155,6 +156,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     const float* gamma = a.gamma + (size_t)seq * Ls;
 
     if (tid == 0) {
+        if (blockIdx.x == 0 && !a.keep_status) *a.status = 0;  // a wait that gives up does so a second later
         s.dead = 0;
         mbar_init(&s.bar_x, 1);
         mbar_init(&s.bar_v, 1);
@@ -404,53 +406,37 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             const float* w2 = a.W2_init + head + (size_t)row * he + HC * me + c0;
             const float* m2 = a.M2_init ? a.M2_init + head + (size_t)row * he + HC * me + c0 : nullptr;
             const bool real2 = cta_real && row < de;  // this thread's W2 row exists
+            float* ck = a.ckpt ? a.ckpt + (size_t)seq * a.ckpt_seq_stride : nullptr;  // chunk-start state of chunk 0
+            // the momentum's loads first, all in flight: a wave of CTAs starts with nothing else to do
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
-                float w[16];
+                ld_row16<WIDE>(m1 + 16 * b, M1 + 16 * b, m1 && cta_real && c0 + 16 * b < de);
+                ld_row16<WIDE>(m2 + 16 * b, M2 + 16 * b, m2 && real2);
+            }
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                float w[16], v[16];
                 uint32_t st[16];
                 const bool real1 = cta_real && c0 + 16 * b < de;  // these 16 columns of W1 exist
+                ld_row16<WIDE>(w1 + 16 * b, w, real1);
+                ld_row16<WIDE>(w2 + 16 * b, v, real2);
 #pragma unroll
-                for (int j = 0; j < 16; j += 4) {
-                    const float4 x = real1 ? *reinterpret_cast<const float4*>(w1 + 16 * b + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    w[j] = x.x; w[j + 1] = x.y; w[j + 2] = x.z; w[j + 3] = x.w;
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    M1[16 * b + j] = (m1 && real1) ? m1[16 * b + j] : 0.0f;
-                    st[j] = __float_as_uint(multi ? fmaf(cm0, M1[16 * b + j], cw0 * w[j]) : cw0 * w[j]);
-                }
+                for (int j = 0; j < 16; ++j) st[j] = __float_as_uint(multi ? fmaf(cm0, M1[16 * b + j], cw0 * w[j]) : cw0 * w[j]);
                 tmem_st16(lane_addr + T_W1 + c0 + 16 * b, st);
                 st_slab16(s.W1[(c0 + 16 * b) >> 6], row, (c0 + 16 * b) & 63, w);
-                float* ck = a.ckpt ? a.ckpt + (size_t)seq * a.ckpt_seq_stride : nullptr;  // chunk-start state of chunk 0
                 if (ck && real1) {
                     const size_t o1 = ((size_t)(HC * me) + row) * de + c0 + 16 * b;
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) {
-                        *reinterpret_cast<float4*>(ck + o1 + j) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
-                        *reinterpret_cast<float4*>(ck + 2 * dh + o1 + j) =
-                            make_float4(M1[16 * b + j], M1[16 * b + j + 1], M1[16 * b + j + 2], M1[16 * b + j + 3]);
-                    }
+                    st_row16<WIDE>(ck + o1, w);
+                    st_row16<WIDE>(ck + 2 * dh + o1, M1 + 16 * b);
                 }
 #pragma unroll
-                for (int j = 0; j < 16; j += 4) {
-                    const float4 x = real2 ? *reinterpret_cast<const float4*>(w2 + 16 * b + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    w[j] = x.x; w[j + 1] = x.y; w[j + 2] = x.z; w[j + 3] = x.w;
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    M2[16 * b + j] = (m2 && real2) ? m2[16 * b + j] : 0.0f;
-                    st[j] = __float_as_uint(multi ? fmaf(cm0, M2[16 * b + j], cw0 * w[j]) : cw0 * w[j]);
-                }
+                for (int j = 0; j < 16; ++j) st[j] = __float_as_uint(multi ? fmaf(cm0, M2[16 * b + j], cw0 * v[j]) : cw0 * v[j]);
                 tmem_st16(lane_addr + T_W2 + c0 + 16 * b, st);
-                st_slab16(s.W2[(c0 + 16 * b) >> 6], row, (c0 + 16 * b) & 63, w);
+                st_slab16(s.W2[(c0 + 16 * b) >> 6], row, (c0 + 16 * b) & 63, v);
                 if (ck && real2) {
                     const size_t o2 = (size_t)row * he + HC * me + c0 + 16 * b;
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) {
-                        *reinterpret_cast<float4*>(ck + dh + o2 + j) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
-                        *reinterpret_cast<float4*>(ck + 3 * dh + o2 + j) =
-                            make_float4(M2[16 * b + j], M2[16 * b + j + 1], M2[16 * b + j + 2], M2[16 * b + j + 3]);
-                    }
+                    st_row16<WIDE>(ck + dh + o2, v);
+                    st_row16<WIDE>(ck + 3 * dh + o2, M2 + 16 * b);
                 }
             }
             tmem_wait_st();
@@ -827,9 +813,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                         for (int j = 0; j < 16; ++j) M1[16 * b + j] = fmaf(cbk, M1[16 * b + j], __uint_as_float(ma[j]));
                         if (wr && real1 && col < de) {
                             float* dst = (last ? a.M1_final + head : ck2 + 2 * dh) + off0 + col;
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4)
-                                *reinterpret_cast<float4*>(dst + j) = make_float4(M1[16 * b + j], M1[16 * b + j + 1], M1[16 * b + j + 2], M1[16 * b + j + 3]);
+st_row16<WIDE>(dst, M1 + 16 * b);
                         }
                     }
                     if (final_block) {
@@ -847,9 +831,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                             st_slab16p(s.W1[col >> 6], row, col & 63, p);
                             if (wr && real1 && col < de) {
                                 float* dst = (last ? a.W1_final + head : ck2) + off0 + col;
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4)
-                                    *reinterpret_cast<uint4*>(dst + j) = make_uint4(wa[j], wa[j + 1], wa[j + 2], wa[j + 3]);
+st_row16<WIDE>(dst, wa);
                             }
 #pragma unroll
                             for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(fmaf(cmn2, M1[16 * b + j], cwn2 * __uint_as_float(wa[j])));
@@ -874,9 +856,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                         for (int j = 0; j < 16; ++j) M2[16 * b + j] = fmaf(cbk, M2[16 * b + j], __uint_as_float(ma[j]));
                         if (wr && real2) {
                             float* dst = (last ? a.M2_final + head : ck2 + 3 * dh) + off0 + col;
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4)
-                                *reinterpret_cast<float4*>(dst + j) = make_float4(M2[16 * b + j], M2[16 * b + j + 1], M2[16 * b + j + 2], M2[16 * b + j + 3]);
+st_row16<WIDE>(dst, M2 + 16 * b);
                         }
                         if (final_block) {
                             uint32_t wa[16];
@@ -888,9 +868,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                             st_slab16p(s.W2[col >> 6], row, col & 63, p);
                             if (wr && real2) {
                                 float* dst = (last ? a.W2_final + head : ck2 + dh) + off0 + col;
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4)
-                                    *reinterpret_cast<uint4*>(dst + j) = make_uint4(wa[j], wa[j + 1], wa[j + 2], wa[j + 3]);
+st_row16<WIDE>(dst, wa);
                             }
 #pragma unroll
                             for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(fmaf(cmn2, M2[16 * b + j], cwn2 * __uint_as_float(wa[j])));
@@ -928,9 +906,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                         st_slab16p(s.W1[col >> 6], row, col & 63, p);
                         if (real1 && col < de && (last || save_ck)) {
                             float* dst = (last ? a.W1_final + head : ckn) + off0 + col;
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4)
-                                *reinterpret_cast<uint4*>(dst + j) = make_uint4(wa[j], wa[j + 1], wa[j + 2], wa[j + 3]);
+st_row16<WIDE>(dst, wa);
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(cwn * __uint_as_float(wa[j]));
@@ -964,14 +940,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                         st_slab16(s.W1[col >> 6], row, col & 63, wn);
                         if (real1 && col < de) {
                             if (last) {
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4)
-                                    *reinterpret_cast<float4*>(a.W1_final + head + off0 + col + j) = make_float4(wn[j], wn[j + 1], wn[j + 2], wn[j + 3]);
+st_row16<WIDE>(a.W1_final + head + off0 + col, wn);
                             }
                             if (save_ck) {
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4)
-                                    *reinterpret_cast<float4*>(ckn + off0 + col + j) = make_float4(wn[j], wn[j + 1], wn[j + 2], wn[j + 3]);
+st_row16<WIDE>(ckn + off0 + col, wn);
                             }
                         }
                     }
@@ -993,16 +965,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                     for (int j = 0; j < 16; ++j) M1[16 * b + j] = fmaf(cb, M1[16 * b + j], __uint_as_float(ma[j]));
                     if (real1 && col < de) {
                         if (last) {
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4)
-                                *reinterpret_cast<float4*>(a.M1_final + head + off0 + col + j) =
-                                    make_float4(M1[16 * b + j], M1[16 * b + j + 1], M1[16 * b + j + 2], M1[16 * b + j + 3]);
+st_row16<WIDE>(a.M1_final + head + off0 + col, M1 + 16 * b);
                         }
                         if (save_ck) {
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4)
-                                *reinterpret_cast<float4*>(ckn + 2 * dh + off0 + col + j) =
-                                    make_float4(M1[16 * b + j], M1[16 * b + j + 1], M1[16 * b + j + 2], M1[16 * b + j + 3]);
+st_row16<WIDE>(ckn + 2 * dh + off0 + col, M1 + 16 * b);
                         }
                     }
                 }
@@ -1039,9 +1005,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                             st_slab16p(s.W2[col >> 6], row, col & 63, p);
                             if (real2 && (last || save_ck)) {
                                 float* dst = (last ? a.W2_final + head : ckn + dh) + off0 + col;
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4)
-                                    *reinterpret_cast<uint4*>(dst + j) = make_uint4(wa[j], wa[j + 1], wa[j + 2], wa[j + 3]);
+st_row16<WIDE>(dst, wa);
                             }
 #pragma unroll
                             for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(cwn * __uint_as_float(wa[j]));
@@ -1057,16 +1021,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                     }
                     if (real2) {
                         if (last) {
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4)
-                                *reinterpret_cast<float4*>(a.M2_final + head + off0 + col + j) =
-                                    make_float4(M2[16 * b + j], M2[16 * b + j + 1], M2[16 * b + j + 2], M2[16 * b + j + 3]);
+st_row16<WIDE>(a.M2_final + head + off0 + col, M2 + 16 * b);
                         }
                         if (save_ck) {
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4)
-                                *reinterpret_cast<float4*>(ckn + 3 * dh + off0 + col + j) =
-                                    make_float4(M2[16 * b + j], M2[16 * b + j + 1], M2[16 * b + j + 2], M2[16 * b + j + 3]);
+st_row16<WIDE>(ckn + 3 * dh + off0 + col, M2 + 16 * b);
                         }
                     }
                 }
@@ -1122,14 +1080,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                         st_slab16(s.W2[col >> 6], row, col & 63, wn);
                         if (real2) {
                             if (last) {
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4)
-                                    *reinterpret_cast<float4*>(a.W2_final + head + off0 + col + j) = make_float4(wn[j], wn[j + 1], wn[j + 2], wn[j + 3]);
+st_row16<WIDE>(a.W2_final + head + off0 + col, wn);
                             }
                             if (save_ck) {
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4)
-                                    *reinterpret_cast<float4*>(ckn + dh + off0 + col + j) = make_float4(wn[j], wn[j + 1], wn[j + 2], wn[j + 3]);
+st_row16<WIDE>(ckn + dh + off0 + col, wn);
                             }
                         }
                     }
@@ -1178,26 +1132,11 @@ int tc_fwd_launch(const TcFwdArgs& a_in, void* stream) {
     if (!make_token_map(&tmK, a.k, rows, box_rows, a.d) || !make_token_map(&tmQ, a.q, rows, box_rows, a.d) ||
         !make_token_map(&tmV, a.v, rows, 16, a.d))
         return (int)cudaErrorInvalidValue;
-    static bool attr_done[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return (int)cudaGetLastError();
-    const int smem = (int)tc_fwd_smem_bytes();
-    if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(tc_fwd_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_fwd_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_fwd_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_fwd_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_fwd_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_fwd_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return (int)e;
-        if (dev >= 0 && dev < 64) attr_done[dev] = true;
-    }
-    cudaError_t e = a.keep_status ? cudaSuccess : cudaMemsetAsync(a.status, 0, sizeof(int), st);
-    if (e != cudaSuccess) return (int)e;
+    cudaError_t e = cudaSuccess;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(a.N * NC));
     cfg.blockDim = dim3(NTHREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.dynamicSmemBytes = tc_fwd_smem_bytes();
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1207,19 +1146,29 @@ int tc_fwd_launch(const TcFwdArgs& a_in, void* stream) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     const bool native = a.d == D && a.h == NC * HC;
-    if (a.norm1 && a.norm2) {
-        if (a.ckpt && !a.rown) return (int)cudaErrorInvalidValue;
-        if (a.ckpt_every > 1) return (int)cudaErrorInvalidValue;
-        e = native ? cudaLaunchKernelEx(&cfg, tc_fwd_kernel<false, true>, tmK, tmQ, tmV, a)
-                   : cudaLaunchKernelEx(&cfg, tc_fwd_kernel<true, true>, tmK, tmQ, tmV, a);
-    } else {
-        if (a.C > 64)
-            e = native ? cudaLaunchKernelEx(&cfg, tc_fwd_kernel<false, false, true>, tmK, tmQ, tmV, a)
-                       : cudaLaunchKernelEx(&cfg, tc_fwd_kernel<true, false, true>, tmK, tmQ, tmV, a);
-        else
-            e = native ? cudaLaunchKernelEx(&cfg, tc_fwd_kernel<false, false>, tmK, tmQ, tmV, a)
-                       : cudaLaunchKernelEx(&cfg, tc_fwd_kernel<true, false>, tmK, tmQ, tmV, a);
-    }
+    const bool norm = a.norm1 && a.norm2;
+    if (norm && ((a.ckpt && !a.rown) || a.ckpt_every > 1)) return (int)cudaErrorInvalidValue;
+    const bool wide = wide_rows({a.W1_init, a.W2_init, a.M1_init, a.M2_init, a.W1_final, a.W2_final, a.M1_final, a.M2_final, a.ckpt},
+                                {a.init_seq_stride, a.final_seq_stride, a.ckpt_seq_stride});
+    auto go = [&](auto kernel, bool (&attr_done)[64]) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess && (dev < 0 || dev >= 64 || !attr_done[dev])) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_fwd_smem_bytes());
+            if (e == cudaSuccess && dev >= 0 && dev < 64) attr_done[dev] = true;
+        }
+        return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, kernel, tmK, tmQ, tmV, a) : e;
+    };
+    static bool done[12][64];
+#define E2TTT_TC_FWD(i, PAD, NORM, MULTI)                                                     \
+    e = wide ? go(tc_fwd_kernel<PAD, NORM, MULTI, true>, done[i]) : go(tc_fwd_kernel<PAD, NORM, MULTI, false>, done[6 + i])
+    if (norm && native) E2TTT_TC_FWD(0, false, true, false);
+    else if (norm) E2TTT_TC_FWD(1, true, true, false);
+    else if (a.C > 64 && native) E2TTT_TC_FWD(2, false, false, true);
+    else if (a.C > 64) E2TTT_TC_FWD(3, true, false, true);
+    else if (native) E2TTT_TC_FWD(4, false, false, false);
+    else E2TTT_TC_FWD(5, true, false, false);
+#undef E2TTT_TC_FWD
     if (e != cudaSuccess) return (int)e;
     return (int)cudaGetLastError();
 }

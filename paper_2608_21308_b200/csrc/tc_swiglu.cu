@@ -92,7 +92,7 @@ __device__ __forceinline__ void st_two_term(uint8_t* hi_slab, uint8_t* lo_slab, 
 __device__ __forceinline__ float fast_sigmoid(float z) { return fmaf(0.5f, fast_tanh(0.5f * z), 0.5f); }
 
 // MULTI: chunks of several 64-token blocks (128, 256, 512 tokens), a compile-time switch
-template <bool MULTI>
+template <bool MULTI, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ,
                  const __grid_constant__ CUtensorMap tmV, const TcSwigluArgs a) {
@@ -121,6 +121,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const float* gamma = a.gamma + (size_t)seq * Ls;
 
     if (tid == 0) {
+        if (blockIdx.x == 0 && !a.keep_status) *a.status = 0;  // a wait that gives up does so a second later
         s.dead = 0;
         mbar_init(&s.bar_x, 1);
         mbar_init(&s.bar_v, 1);
@@ -326,20 +327,19 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             const float* w12 = (row < 64 ? a.W1_init : a.W2_init) + head0 + off12;
             const float* m12p = row < 64 ? a.M1_init : a.M2_init;
             const float* m12 = m12p ? m12p + head0 + off12 : nullptr;
+            const float* m3 = a.M3_init ? a.M3_init + head0 + off3 : nullptr;
+            ld_row16<WIDE>(m12, M12, m12 != nullptr);  // the momentum's loads first, all in flight
+            ld_row16<WIDE>(m12 + 16, M12 + 16, m12 != nullptr);
+            ld_row16<WIDE>(m3, M3, m3 != nullptr);
+            float w3[16];
+            ld_row16<WIDE>(a.W3_init + head0 + off3, w3, true);
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
                 float w[16];
                 uint32_t st[16];
+                ld_row16<WIDE>(w12 + 16 * b, w, true);
 #pragma unroll
-                for (int j = 0; j < 16; j += 4) {
-                    const float4 x = *reinterpret_cast<const float4*>(w12 + 16 * b + j);
-                    w[j] = x.x; w[j + 1] = x.y; w[j + 2] = x.z; w[j + 3] = x.w;
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    M12[16 * b + j] = m12 ? m12[16 * b + j] : 0.0f;
-                    st[j] = __float_as_uint(multi ? fmaf(cm0, M12[16 * b + j], cw0 * w[j]) : cw0 * w[j]);
-                }
+                for (int j = 0; j < 16; ++j) st[j] = __float_as_uint(multi ? fmaf(cm0, M12[16 * b + j], cw0 * w[j]) : cw0 * w[j]);
                 const int col = 32 * g + 16 * b;
                 tmem_st16(lane_addr + T_W12 + col, st);
                 uint32_t wu[16];
@@ -347,38 +347,19 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 for (int j = 0; j < 16; ++j) wu[j] = __float_as_uint(w[j]);
                 st_two_term(s.W12[col >> 6], s.W12lo[col >> 6], row, col & 63, wu);
                 if (ck0) {
-                    float* cw = ck0 + (row < 64 ? 0 : dh) + off12 + 16 * b;       // W1 | W2
-                    float* cm_ = ck0 + (row < 64 ? 3 : 4) * dh + off12 + 16 * b;   // M1 | M2
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) {
-                        *reinterpret_cast<float4*>(cw + j) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
-                        *reinterpret_cast<float4*>(cm_ + j) = make_float4(M12[16 * b + j], M12[16 * b + j + 1], M12[16 * b + j + 2], M12[16 * b + j + 3]);
-                    }
+                    st_row16<WIDE>(ck0 + (row < 64 ? 0 : dh) + off12 + 16 * b, w);                   // W1 | W2
+                    st_row16<WIDE>(ck0 + (row < 64 ? 3 : 4) * dh + off12 + 16 * b, M12 + 16 * b);    // M1 | M2
                 }
             }
             {
-                const float* w3 = a.W3_init + head0 + off3;
-                const float* m3 = a.M3_init ? a.M3_init + head0 + off3 : nullptr;
-                float w[16];
                 uint32_t st[16];
 #pragma unroll
-                for (int j = 0; j < 16; j += 4) {
-                    const float4 x = *reinterpret_cast<const float4*>(w3 + j);
-                    w[j] = x.x; w[j + 1] = x.y; w[j + 2] = x.z; w[j + 3] = x.w;
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    M3[j] = m3 ? m3[j] : 0.0f;
-                    st[j] = __float_as_uint(multi ? fmaf(cm0, M3[j], cw0 * w[j]) : cw0 * w[j]);
-                }
+                for (int j = 0; j < 16; ++j) st[j] = __float_as_uint(multi ? fmaf(cm0, M3[j], cw0 * w3[j]) : cw0 * w3[j]);
                 tmem_st16(lane_addr + T_W3 + 16 * g, st);
-                st_slab16(s.W3, row, 16 * g, w);
+                st_slab16(s.W3, row, 16 * g, w3);
                 if (ck0) {
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) {
-                        *reinterpret_cast<float4*>(ck0 + 2 * dh + off3 + j) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
-                        *reinterpret_cast<float4*>(ck0 + 5 * dh + off3 + j) = make_float4(M3[j], M3[j + 1], M3[j + 2], M3[j + 3]);
-                    }
+                    st_row16<WIDE>(ck0 + 2 * dh + off3, w3);
+                    st_row16<WIDE>(ck0 + 5 * dh + off3, M3);
                 }
             }
             tmem_wait_st();
@@ -693,9 +674,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     for (int j = 0; j < 16; ++j) M12[16 * b + j] = fmaf(cbk, M12[16 * b + j], __uint_as_float(ma[j]));
                     if (wr) {
                         float* dst = (last ? (row < 64 ? a.M1_final : a.M2_final) + head : ck2 + (row < 64 ? 3 : 4) * dh) + off12 + 16 * b;
-#pragma unroll
-                        for (int j = 0; j < 16; j += 4)
-                            *reinterpret_cast<float4*>(dst + j) = make_float4(M12[16 * b + j], M12[16 * b + j + 1], M12[16 * b + j + 2], M12[16 * b + j + 3]);
+st_row16<WIDE>(dst, M12 + 16 * b);
                     }
                 }
                 if (final_block) {
@@ -710,8 +689,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         st_two_term(s.W12[col >> 6], s.W12lo[col >> 6], row, col & 63, wa);
                         if (wr) {
                             float* dst = (last ? (row < 64 ? a.W1_final : a.W2_final) + head : ck2 + (row < 64 ? 0 : dh)) + off12 + 16 * b;
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4) *reinterpret_cast<uint4*>(dst + j) = make_uint4(wa[j], wa[j + 1], wa[j + 2], wa[j + 3]);
+st_row16<WIDE>(dst, wa);
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(fmaf(cmn2, M12[16 * b + j], cwn2 * __uint_as_float(wa[j])));
@@ -730,8 +708,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     for (int j = 0; j < 16; ++j) M3[j] = fmaf(cbk, M3[j], __uint_as_float(ma[j]));
                     if (wr) {
                         float* dst = (last ? a.M3_final + head : ck2 + 5 * dh) + off3;
-#pragma unroll
-                        for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(dst + j) = make_float4(M3[j], M3[j + 1], M3[j + 2], M3[j + 3]);
+st_row16<WIDE>(dst, M3);
                     }
                     if (final_block) {
                         uint32_t wa[16];
@@ -743,8 +720,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         st_slab16p(s.W3, row, 16 * g, p);
                         if (wr) {
                             float* dst = (last ? a.W3_final + head : ck2 + 2 * dh) + off3;
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4) *reinterpret_cast<uint4*>(dst + j) = make_uint4(wa[j], wa[j + 1], wa[j + 2], wa[j + 3]);
+st_row16<WIDE>(dst, wa);
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(fmaf(cmn2, M3[j], cwn2 * __uint_as_float(wa[j])));
@@ -768,8 +744,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 st_two_term(s.W12[col >> 6], s.W12lo[col >> 6], row, col & 63, wa);
                 if (last || save_ck) {
                     float* dst = (last ? (row < 64 ? a.W1_final : a.W2_final) + head : ckn + (row < 64 ? 0 : dh)) + off12 + 16 * b;
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) *reinterpret_cast<uint4*>(dst + j) = make_uint4(wa[j], wa[j + 1], wa[j + 2], wa[j + 3]);
+st_row16<WIDE>(dst, wa);
                 }
 #pragma unroll
                 for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(cwn * __uint_as_float(wa[j]));
@@ -786,9 +761,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 for (int j = 0; j < 16; ++j) M12[16 * b + j] = fmaf(cb, M12[16 * b + j], __uint_as_float(ma[j]));
                 if (last || save_ck) {
                     float* dst = (last ? (row < 64 ? a.M1_final : a.M2_final) + head : ckn + (row < 64 ? 3 : 4) * dh) + off12 + 16 * b;
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4)
-                        *reinterpret_cast<float4*>(dst + j) = make_float4(M12[16 * b + j], M12[16 * b + j + 1], M12[16 * b + j + 2], M12[16 * b + j + 3]);
+st_row16<WIDE>(dst, M12 + 16 * b);
                 }
             }
             tmem_wait_st();
@@ -809,8 +782,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 st_slab16p(s.W3, row, 16 * g, p);
                 if (last || save_ck) {
                     float* dst = (last ? a.W3_final + head : ckn + 2 * dh) + off3;
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) *reinterpret_cast<uint4*>(dst + j) = make_uint4(wa[j], wa[j + 1], wa[j + 2], wa[j + 3]);
+st_row16<WIDE>(dst, wa);
                 }
 #pragma unroll
                 for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(cwn * __uint_as_float(wa[j]));
@@ -822,8 +794,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 for (int j = 0; j < 16; ++j) M3[j] = fmaf(cb, M3[j], __uint_as_float(ma[j]));
                 if (last || save_ck) {
                     float* dst = (last ? a.M3_final + head : ckn + 5 * dh) + off3;
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(dst + j) = make_float4(M3[j], M3[j + 1], M3[j + 2], M3[j + 3]);
+st_row16<WIDE>(dst, M3);
                 }
             }
             tmem_wait_st();
@@ -858,22 +829,11 @@ int tc_swiglu_launch(const TcSwigluArgs& a_in, void* stream) {
     const unsigned box_rows = (unsigned)(Cc < 64 ? Cc : 64);
     if (!make_token_map(&tmK, a.k, rows, box_rows, D) || !make_token_map(&tmQ, a.q, rows, box_rows, D) || !make_token_map(&tmV, a.v, rows, 16, D))
         return (int)cudaErrorInvalidValue;
-    static bool attr_done[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return (int)cudaGetLastError();
-    const int smem = (int)tc_swiglu_smem_bytes();
-    if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(tc_swiglu_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_swiglu_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return (int)e;
-        if (dev >= 0 && dev < 64) attr_done[dev] = true;
-    }
-    cudaError_t e = a.keep_status ? cudaSuccess : cudaMemsetAsync(a.status, 0, sizeof(int), st);
-    if (e != cudaSuccess) return (int)e;
+    cudaError_t e = cudaSuccess;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(a.N * NC));
     cfg.blockDim = dim3(NTHREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.dynamicSmemBytes = tc_swiglu_smem_bytes();
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -882,8 +842,20 @@ int tc_swiglu_launch(const TcSwigluArgs& a_in, void* stream) {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    e = a.C > 64 ? cudaLaunchKernelEx(&cfg, tc_swiglu_kernel<true>, tmK, tmQ, tmV, a)
-                 : cudaLaunchKernelEx(&cfg, tc_swiglu_kernel<false>, tmK, tmQ, tmV, a);
+    const bool wide = wide_rows({a.W1_init, a.W2_init, a.W3_init, a.M1_init, a.M2_init, a.M3_init, a.W1_final, a.W2_final, a.W3_final, a.M1_final,
+                                 a.M2_final, a.M3_final, a.ckpt}, {a.init_seq_stride, a.final_seq_stride, a.ckpt_seq_stride});
+    auto go = [&](auto kernel, bool (&attr_done)[64]) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess && (dev < 0 || dev >= 64 || !attr_done[dev])) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_swiglu_smem_bytes());
+            if (e == cudaSuccess && dev >= 0 && dev < 64) attr_done[dev] = true;
+        }
+        return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, kernel, tmK, tmQ, tmV, a) : e;
+    };
+    static bool done[4][64];
+    if (a.C > 64) e = wide ? go(tc_swiglu_kernel<true, true>, done[0]) : go(tc_swiglu_kernel<true, false>, done[1]);
+    else e = wide ? go(tc_swiglu_kernel<false, true>, done[2]) : go(tc_swiglu_kernel<false, false>, done[3]);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaGetLastError();
 }
