@@ -238,7 +238,7 @@ static int fwd_common(const e2ttt_params* p, const void* q, const void* k, const
     SimtFwdArgs a{};
     a.N = p->B * p->H; a.L = p->L; a.d = p->d; a.h = p->h; a.C = p->C;
     a.nchunks = (p->L + p->C - 1) / p->C;
-    a.cl = simt_cluster_size(a.N);
+    a.cl = simt_cluster_size(a.N, p->io_dtype);
     a.tc = impl == E2TTT_IMPL_TILED;
     a.status = static_cast<int*>(workspace);
     const int seg = row_norm ? 0 : segment_chunks(p);
@@ -412,7 +412,7 @@ static int bwd_common(const e2ttt_params* p, const void* q, const void* k, const
         f.N = p->B * p->H; f.d = p->d; f.h = p->h; f.C = p->C; f.nchunks = n;
         f.L = (int)((size_t)p->L - t0 < (size_t)n * p->C ? (size_t)p->L - t0 : (size_t)n * p->C);
         f.Ls = p->L; f.init_slot = init_slot;
-        f.save_states = mode; f.eps = p->ln_eps; f.cl = simt_cluster_size(f.N);
+        f.save_states = mode; f.eps = p->ln_eps; f.cl = simt_cluster_size(f.N, p->io_dtype);
         f.tc = impl != E2TTT_IMPL_SIMT; f.status = static_cast<int*>(workspace);
         f.q = static_cast<const char*>(q) + t0 * p->d * esz;
         f.k = static_cast<const char*>(k) + t0 * p->d * esz;
@@ -438,7 +438,7 @@ static int bwd_common(const e2ttt_params* p, const void* q, const void* k, const
         b.N = p->B * p->H; b.d = p->d; b.h = p->h; b.C = p->C; b.nchunks = n; b.eps = p->ln_eps;
         b.L = (int)((size_t)p->L - t0 < (size_t)n * p->C ? (size_t)p->L - t0 : (size_t)n * p->C);
         b.Ls = p->L; b.carry_in = carry_in; b.carry_out = carry_out;
-        b.cl = simt_cluster_size(b.N);
+        b.cl = simt_cluster_size(b.N, p->io_dtype);
         b.tc = impl != E2TTT_IMPL_SIMT; b.status = static_cast<int*>(workspace);
         b.q = static_cast<const char*>(q) + tok; b.k = static_cast<const char*>(k) + tok;
         b.v = static_cast<const char*>(v) + tok; b.d_o = static_cast<const char*>(d_o) + tok;

@@ -1,4 +1,4 @@
-// Any-shape backward: the adjoint of the chunk program, chunks in reverse order, a cluster of 1-8 CTAs per sequence,
+// Any-shape backward: the adjoint of the chunk program, chunks in reverse order, a cluster of 1-16 CTAs per sequence,
 // for both fast-weight networks, on the same two GEMM engines as the forward (tc_gemm.cuh).  Per chunk it re-runs the chunk's forward from the saved chunk-start state, then reverses,
 // in matrix form over the whole chunk,
 //   (i)   the outputs o = f_{W0}(q),
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
         }
 
         auto load_x = [&](int m, int kk, Real& a0, Real& a1) {
-            a0 = (m < len) ? ld_io<Real>(kc, (size_t)m * d + kk) : ld_io<Real>(qc, (size_t)(m - len) * d + kk);
+            a0 = ld_io<Real>(m < len ? kc + (size_t)m * d : qc + (size_t)(m - len) * d, (size_t)kk);
         };
         auto load_k = [&](int m, int kk, Real& a0, Real& a1) { a0 = ld_io<Real>(kc, (size_t)m * d + kk); };
 
@@ -286,9 +286,9 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
         G.template run<1, true, false>(
             len, d, SW ? 2 * h : h,
             [&](int m, int kk, Real& a0, Real& a1) {
-                a0 = kk < h ? Zqb[(size_t)m * h + kk] : Zqb2[(size_t)m * h + kk - h];
+                a0 = (kk < h ? Zqb + kk : Zqb2 + (kk - h))[(size_t)m * h];
             },
-            [&](int n, int kk) { return kk < h ? W1[(size_t)kk * d + n] : W2[(size_t)(kk - h) * d + n]; },
+            [&](int n, int kk) { return (kk < h ? W1 + (size_t)kk * d : W2 + (size_t)(kk - h) * d)[n]; },
             [&](int m, int n, Real acc, Real) {
                 const size_t e = (size_t)m * d + n;
                 st_io(dq + (size_t)s * d, e, ld_io<Real>(doc, e) + acc);
@@ -341,18 +341,18 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
         BPROF(12);
         G.template run<1, true, true>( // XY2 = Ak [Tl; Sl]^T
             len, 2 * d, h, [&](int m, int kk, Real& a0, Real& a1) { a0 = A[(size_t)m * h + kk]; },
-            [&](int n, int kk) { return n < d ? T[LAST][(size_t)n * h + kk] : S[LAST][(size_t)(n - d) * h + kk]; },
+            [&](int n, int kk) { return (n < d ? T[LAST] + (size_t)n * h : S[LAST] + (size_t)(n - d) * h)[kk]; },
             [&](int m, int n, Real acc, Real) { XY2[(size_t)m * 2 * d + n] = acc; });
         BPROF(13);
         G.template run<1, true, true>( // XY1 = K [T1; S1]^T
             len, 2 * h, d, load_k,
-            [&](int n, int kk) { return n < h ? T[0][(size_t)n * d + kk] : S[0][(size_t)(n - h) * d + kk]; },
+            [&](int n, int kk) { return (n < h ? T[0] + (size_t)n * d : S[0] + (size_t)(n - h) * d)[kk]; },
             [&](int m, int n, Real acc, Real) { XY1[(size_t)m * 2 * h + n] = acc; });
         BPROF(14);
         if (SW)
             G.template run<1, true, true>( // XY1b = K [T2; S2]^T
                 len, 2 * h, d, load_k,
-                [&](int n, int kk) { return n < h ? T[1][(size_t)n * d + kk] : S[1][(size_t)(n - h) * d + kk]; },
+                [&](int n, int kk) { return (n < h ? T[1] + (size_t)n * d : S[1] + (size_t)(n - h) * d)[kk]; },
                 [&](int m, int n, Real acc, Real) { XY1b[(size_t)m * 2 * h + n] = acc; });
         BPROF(15);
         for (int t = warp + rank * (NT / 32); t < len; t += (NT / 32) * CL) {
@@ -388,26 +388,26 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
         G.template run<1, true, false>( // Akb = -[kW Pu | kM Pu] [Tl; Sl]
             len, h, 2 * d,
             [&](int m, int kk, Real& a0, Real& a1) {
-                a0 = kk < d ? sc.kW[m] * Pu[(size_t)m * d + kk] : sc.kM[m] * Pu[(size_t)m * d + kk - d];
+                a0 = (kk < d ? sc.kW[m] : sc.kM[m]) * Pu[(size_t)m * d + (kk < d ? kk : kk - d)];
             },
-            [&](int n, int kk) { return kk < d ? T[LAST][(size_t)kk * h + n] : S[LAST][(size_t)(kk - d) * h + n]; },
+            [&](int n, int kk) { return (kk < d ? T[LAST] + (size_t)kk * h : S[LAST] + (size_t)(kk - d) * h)[n]; },
             [&](int m, int n, Real acc, Real) { Akb[(size_t)m * h + n] = -acc; });
         BPROF(18);
         G.template run<1, true, false>( // Kb = -[kW Pz1 | kM Pz1] [T1; S1]
             len, d, 2 * h,
             [&](int m, int kk, Real& a0, Real& a1) {
-                a0 = kk < h ? sc.kW[m] * Pz1[(size_t)m * h + kk] : sc.kM[m] * Pz1[(size_t)m * h + kk - h];
+                a0 = (kk < h ? sc.kW[m] : sc.kM[m]) * Pz1[(size_t)m * h + (kk < h ? kk : kk - h)];
             },
-            [&](int n, int kk) { return kk < h ? T[0][(size_t)kk * d + n] : S[0][(size_t)(kk - h) * d + n]; },
+            [&](int n, int kk) { return (kk < h ? T[0] + (size_t)kk * d : S[0] + (size_t)(kk - h) * d)[n]; },
             [&](int m, int n, Real acc, Real) { Kb[(size_t)m * d + n] = -acc; });
         BPROF(19);
         if (SW)
             G.template run<1, true, false>( // Kb -= [kW Pz2 | kM Pz2] [T2; S2]
                 len, d, 2 * h,
                 [&](int m, int kk, Real& a0, Real& a1) {
-                    a0 = kk < h ? sc.kW[m] * Pz2[(size_t)m * h + kk] : sc.kM[m] * Pz2[(size_t)m * h + kk - h];
+                    a0 = (kk < h ? sc.kW[m] : sc.kM[m]) * Pz2[(size_t)m * h + (kk < h ? kk : kk - h)];
                 },
-                [&](int n, int kk) { return kk < h ? T[1][(size_t)kk * d + n] : S[1][(size_t)(kk - h) * d + n]; },
+                [&](int n, int kk) { return (kk < h ? T[1] + (size_t)kk * d : S[1] + (size_t)(kk - h) * d)[n]; },
                 [&](int m, int n, Real acc, Real) { Kb[(size_t)m * d + n] -= acc; });
         // back through pz: Pzb becomes the adjoint of ph; Zkb (Zkb2) start with the second-order terms
         BPROF(20);
@@ -494,9 +494,9 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
         G.template run<1, true, false>(
             len, d, SW ? 2 * h : h,
             [&](int m, int kk, Real& a0, Real& a1) {
-                a0 = kk < h ? Zkb[(size_t)m * h + kk] : Zkb2[(size_t)m * h + kk - h];
+                a0 = (kk < h ? Zkb + kk : Zkb2 + (kk - h))[(size_t)m * h];
             },
-            [&](int n, int kk) { return kk < h ? W1[(size_t)kk * d + n] : W2[(size_t)(kk - h) * d + n]; },
+            [&](int n, int kk) { return (kk < h ? W1 + (size_t)kk * d : W2 + (size_t)(kk - h) * d)[n]; },
             [&](int m, int n, Real acc, Real) {
                 const size_t e = (size_t)m * d + n;
                 st_io(dk + (size_t)s * d, e, Kb[e] + acc);
@@ -604,6 +604,7 @@ static int launch_bwd(const SimtBwdArgs& a, cudaStream_t st) {
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
         cudaError_t e =
             cudaFuncSetAttribute(simt_bwd_kernel<Real, IO, KIND, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(simt_bwd_kernel<Real, IO, KIND, TC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return (int)e;
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }

@@ -201,15 +201,17 @@ __device__ __forceinline__ void phase_sync(int nranks) {
 //   16x16 tiles, 64-deep k slices cut four ways inside the CTA, 2x2 results per thread, the next slice's loads in flight while one
 //   is multiplied: for the few tokens of a small problem.  A [32 x 64] result with 256 terms is one 64x64 tile - one CTA of
 //   eight, half of its rows unused, 16 exposed round trips to L2 (14 us in fp64) - but 8 small ones with 4 slices each.
-template <typename Real> struct GemmSmem {
+template <typename Real> struct __align__(2 * sizeof(Real)) Real2 { Real x, y; };
+
+template <typename Real> struct __align__(16) GemmSmem {
     union {
         struct {
             Real A[2][kBK][kBM + 4];
             Real B[kBK][kBN + 4];
         };
         struct {
-            Real a[2][kSK][kSM + 2];
-            Real b[kSK][kSM + 2];
+            Real2<Real> a[2][kSK][kSM / 2 + 1];  // pairs: one access per two values
+            Real2<Real> b[kSK][kSM / 2 + 1];
             Real part[2][kSplit][kSM * kSM];
         } s;
     };
@@ -219,59 +221,71 @@ template <typename Real, int NACC, bool A_KFAST, bool B_KFAST, typename FA, type
 __device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, GemmSmem<Real>* sm, int rank, int nranks) {
     const int tid = threadIdx.x;
     const int grp = tid / (kSimtThreads / kSplit), tx = tid & 7, ty = (tid >> 3) & 7;
-    const int tn = (N + kSM - 1) / kSM, tiles = tn * ((M + kSM - 1) / kSM), slices = (K + kSK - 1) / kSK;
-    const int items = rank < tiles ? ((tiles - rank + nranks - 1) / nranks) * slices : 0;  // (tile, slice) in order
+    const int tn = (N + kSM - 1) / kSM, tiles = tn * ((M + kSM - 1) / kSM);
     constexpr int PER = kSM * kSK / kSimtThreads;
-    Real ra0[PER], ra1[PER], rb[PER];
-    auto fetch = [&](int item) {
-        const int tile = rank + (item / slices) * nranks, k0 = (item % slices) * kSK;
-        const int m0 = (tile / tn) * kSM, n0 = (tile % tn) * kSM;
+    Real ra0[PER], ra1[PER], rb[PER], acc[NACC][2][2];
+    // the slice whose loads are in flight (the next one) and the slice in shared memory; divisions once per tile only
+    int tile = rank, fm0 = (rank / tn) * kSM, fn0 = (rank % tn) * kSM, fk0 = 0;
+    for (bool first = true;; first = false) {
+        const int m0 = fm0, n0 = fn0, k0 = fk0;
+        if (first) {
+            if (tile >= tiles) break;
+        } else {
+            __syncthreads();
 #pragma unroll
-        for (int r = 0; r < PER; ++r) {
-            const int idx = tid + r * kSimtThreads;
-            const int am = A_KFAST ? idx / kSK : idx % kSM, ak = A_KFAST ? idx % kSK : idx / kSM;
-            const int bn = B_KFAST ? idx / kSK : idx % kSM, bk = B_KFAST ? idx % kSK : idx / kSM;
-            ra0[r] = ra1[r] = rb[r] = 0;
-            if (m0 + am < M && k0 + ak < K) fa(m0 + am, k0 + ak, ra0[r], ra1[r]);
-            if (n0 + bn < N && k0 + bk < K) rb[r] = fb(n0 + bn, k0 + bk);
-        }
-    };
-    if (items > 0) fetch(0);
-    Real acc[NACC][2][2];
-    for (int item = 0; item < items; ++item) {
-        const int slice = item % slices;
-        if (slice == 0)
-#pragma unroll
-            for (int a = 0; a < NACC; ++a) acc[a][0][0] = acc[a][0][1] = acc[a][1][0] = acc[a][1][1] = 0;
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < PER; ++r) {
-            const int idx = tid + r * kSimtThreads;
-            const int am = A_KFAST ? idx / kSK : idx % kSM, ak = A_KFAST ? idx % kSK : idx / kSM;
-            const int bn = B_KFAST ? idx / kSK : idx % kSM, bk = B_KFAST ? idx % kSK : idx / kSM;
-            sm->s.a[0][ak][am] = ra0[r];
-            if (NACC == 2) sm->s.a[1][ak][am] = ra1[r];
-            sm->s.b[bk][bn] = rb[r];
-        }
-        __syncthreads();
-        if (item + 1 < items) fetch(item + 1);
-#pragma unroll 4
-        for (int i = 0; i < kSK / kSplit; ++i) {
-            const int kk = grp * (kSK / kSplit) + i;
-            const Real b0 = sm->s.b[kk][2 * tx], b1 = sm->s.b[kk][2 * tx + 1];
-#pragma unroll
-            for (int a = 0; a < NACC; ++a) {
-                const Real a0 = sm->s.a[a][kk][2 * ty], a1 = sm->s.a[a][kk][2 * ty + 1];
-                acc[a][0][0] += a0 * b0; acc[a][0][1] += a0 * b1;
-                acc[a][1][0] += a1 * b0; acc[a][1][1] += a1 * b1;
+            for (int r = 0; r < PER; ++r) {
+                const int idx = tid + r * kSimtThreads;
+                const int am = A_KFAST ? idx / kSK : idx % kSM, ak = A_KFAST ? idx % kSK : idx / kSM;
+                const int bn = B_KFAST ? idx / kSK : idx % kSM, bk = B_KFAST ? idx % kSK : idx / kSM;
+                const bool ina = m0 + am < M && k0 + ak < K, inb = n0 + bn < N && k0 + bk < K;
+                reinterpret_cast<Real*>(sm->s.a[0][ak])[am] = ina ? ra0[r] : (Real)0;
+                if (NACC == 2) reinterpret_cast<Real*>(sm->s.a[1][ak])[am] = ina ? ra1[r] : (Real)0;
+                reinterpret_cast<Real*>(sm->s.b[bk])[bn] = inb ? rb[r] : (Real)0;
+            }
+            __syncthreads();
+            fk0 += kSK;
+            if (fk0 >= K) {
+                fk0 = 0;
+                tile += nranks;
+                fm0 = (tile / tn) * kSM;
+                fn0 = (tile % tn) * kSM;
             }
         }
-        if (slice == slices - 1) {
-            const int tile = rank + (item / slices) * nranks;
-            const int m = (tile / tn) * kSM + tid / kSM, n = (tile % tn) * kSM + tid % kSM;
-            using P = decltype(pre(0, 0));
-            P p;
-            if (m < M && n < N) p = pre(m, n);
+        if (tile < tiles) {
+#pragma unroll
+            for (int r = 0; r < PER; ++r) {
+                const int idx = tid + r * kSimtThreads;
+                const int am = A_KFAST ? idx / kSK : idx % kSM, ak = A_KFAST ? idx % kSK : idx / kSM;
+                const int bn = B_KFAST ? idx / kSK : idx % kSM, bk = B_KFAST ? idx % kSK : idx / kSM;
+                // indices are clamped and the values masked when they are stored: no branch may stand between the loads, and
+                // nothing may use a value before the multiplication that hides the loads
+                ra0[r] = ra1[r] = 0;
+                fa(min(fm0 + am, M - 1), min(fk0 + ak, K - 1), ra0[r], ra1[r]);
+                rb[r] = fb(min(fn0 + bn, N - 1), min(fk0 + bk, K - 1));
+            }
+        }
+        if (first) continue;
+        const bool last_slice = k0 + kSK >= K;
+        if (k0 == 0)
+#pragma unroll
+            for (int a = 0; a < NACC; ++a) acc[a][0][0] = acc[a][0][1] = acc[a][1][0] = acc[a][1][1] = 0;
+        // what the tile's results combine with: on its way while the last slice is multiplied
+        using P = decltype(pre(0, 0));
+        P p;
+        const int m = m0 + tid / kSM, n = n0 + tid % kSM;
+        if (last_slice) p = pre(min(m, M - 1), min(n, N - 1));
+        const int terms = min(kSK, K - k0);  // of this slice; dealt to the four groups in turn
+#pragma unroll 4
+        for (int kk = grp; kk < terms; kk += kSplit) {
+            const Real2<Real> b = sm->s.b[kk][tx];
+#pragma unroll
+            for (int a = 0; a < NACC; ++a) {
+                const Real2<Real> v = sm->s.a[a][kk][ty];
+                acc[a][0][0] += v.x * b.x; acc[a][0][1] += v.x * b.y;
+                acc[a][1][0] += v.y * b.x; acc[a][1][1] += v.y * b.y;
+            }
+        }
+        if (last_slice) {
 #pragma unroll
             for (int a = 0; a < NACC; ++a)
 #pragma unroll
@@ -285,6 +299,7 @@ __device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE e
 #pragma unroll
                 for (int g = 0; g < kSplit; ++g) s[a] += sm->s.part[a][g][tid];
             if (m < M && n < N) epi(m, n, s[0], s[NACC - 1], p);
+            if (tile >= tiles) break;
         }
     }
 }

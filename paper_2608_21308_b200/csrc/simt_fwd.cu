@@ -1,4 +1,4 @@
-// Any-shape forward: Algorithm 1 applied chunk after chunk for any d, h, C and both networks.  A cluster of 1-8 CTAs
+// Any-shape forward: Algorithm 1 applied chunk after chunk for any d, h, C and both networks.  A cluster of 1-16 CTAs
 // works on one sequence; the CTAs split every phase and share state and intermediates through the workspace, meeting
 // at the cluster barrier between phases.  The matrix products run on one of two engines (tc_gemm.cuh): CUDA-core FMAs
 // (fp64 for fp32 I/O - the GPU-side reference of the tensor-core paths - or fp32), or tcgen05 MMAs for bf16 I/O.
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_fwd_ke
         SPROF(1);
         // Algorithm 1 line 1: the network on the chunk's keys (rows 0..len-1) and queries (rows len..2len-1)
         auto load_x = [&](int m, int kk, Real& a0, Real& a1) {
-            a0 = (m < len) ? ld_io<Real>(kc, (size_t)m * d + kk) : ld_io<Real>(qc, (size_t)(m - len) * d + kk);
+            a0 = ld_io<Real>(m < len ? kc + (size_t)m * d : qc + (size_t)(m - len) * d, (size_t)kk);
         };
         G.template run<1, true, true>(
             2 * len, h, d, load_x, [&](int n, int kk) { return W[0][(size_t)n * d + kk]; },
@@ -275,6 +275,7 @@ static int launch_fwd(const SimtFwdArgs& a, cudaStream_t st) {
     if (cudaGetDevice(&dev) != cudaSuccess) return (int)cudaGetLastError();
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
         cudaError_t e = cudaFuncSetAttribute(simt_fwd_kernel<Real, IO, KIND, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(simt_fwd_kernel<Real, IO, KIND, TC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return (int)e;
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }

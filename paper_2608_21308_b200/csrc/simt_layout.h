@@ -122,8 +122,11 @@ struct SimtBwdArgs {
     SimtLayout lay;
 };
 
-// CTAs per sequence: the largest power of two <= 8 that keeps N * cl within one wave of the GPU's SMs
-inline int simt_cluster_size(int N) {
+// CTAs per sequence: the largest power of two <= 8 that keeps N * cl within one wave of the GPU's SMs.  The fp64 kernels take 16 for the
+// few sequences of a check (clusters above 8 are non-portable and at most 7 of 16 fit this GPU at one CTA per SM): their phases are
+// chains of small products, and with 8 CTAs a CTA has several tiles of most of them.
+inline int simt_cluster_size(int N, int io_dtype) {
+    if (io_dtype == 0 && N <= 7) return 16;
     int cl = 1;
     while (cl < 8 && (long long)N * (cl * 2) <= 148) cl *= 2;
     return cl;
