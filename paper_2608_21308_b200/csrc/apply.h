@@ -14,6 +14,9 @@ struct ApplyArgs {
     const void* q;   // [N, T, d] io dtype
     const float* W[3];
     void* o;         // [N, T, d] io dtype
+    // set by the launcher of the one-token kernel: hidden units per CTA, ring geometry
+    int per, nslots;
+    uint32_t slot_bytes, ring_at;
 };
 
 int apply_token_block(int T);
