@@ -50,6 +50,10 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
+// bytes and address multiples of 16
+__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
 struct Engine {
@@ -309,15 +313,15 @@ __device__ __forceinline__ void st_tok4(__nv_bfloat16* row, int c, int d, const 
             if (c + j < d) row[c + j] = __float2bfloat16_rn(v[j]);
     }
 }
-// v += p[0] + p[stride] + .., in that order, four loads in flight
-__device__ __forceinline__ void add_parts(const float* p, int n, size_t stride, float (&v)[4]) {
-    for (int i0 = 0; i0 < n; i0 += 4) {
-        float4 x[4];
+// v += p[0] + p[stride] + .., in that order, U loads in flight
+template <int U = 4> __device__ __forceinline__ void add_parts(const float* p, int n, size_t stride, float (&v)[4]) {
+    for (int i0 = 0; i0 < n; i0 += U) {
+        float4 x[U];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < U; ++i)
             x[i] = i0 + i < n ? *reinterpret_cast<const float4*>(p + (size_t)(i0 + i) * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { v[0] += x[i].x; v[1] += x[i].y; v[2] += x[i].z; v[3] += x[i].w; }
+        for (int i = 0; i < U; ++i) { v[0] += x[i].x; v[1] += x[i].y; v[2] += x[i].z; v[3] += x[i].w; }
     }
 }
 __device__ __forceinline__ float sum4(const float (&a)[4]) { return (a[0] + a[1]) + (a[2] + a[3]); }

@@ -11,25 +11,12 @@
 // Notation: T, S = adjoints of (W, M) at the chunk end; a trailing "b" marks an adjoint; the first matrices are [h x d], the
 // last one [d x h].
 #include "simt_layout.h"
-#include "tile.cuh"
+#include "tile_chain.h"
 
 namespace e2ttt {
 using namespace tile;
 
 namespace {
-
-constexpr uint32_t B = 2 * kHalf;  // bytes of an operand block
-
-struct GroupArgs {
-    SimtBwdArgs a;
-    int c0, ng;          // chunks [c0, c0 + ng) of the call
-    int first, last;     // first / last group of the call
-};
-
-__device__ __forceinline__ float* slot_of(const SimtBwdArgs& a, int seq, int g) {
-    return reinterpret_cast<float*>(a.ws) + (size_t)seq * a.lay.per_seq + a.lay.tl.slot + (size_t)g * a.lay.tl.slot_stride;
-}
-__device__ __forceinline__ unsigned char* bytes_of(float* p) { return reinterpret_cast<unsigned char*>(p); }
 
 // ---- operand blocks of the chunk-start weights and of the tokens; scalar kernels --------------------------------------------
 template <int NMAT> __global__ void __launch_bounds__(256) tile_prep_kernel(const GroupArgs ga) {
@@ -547,7 +534,7 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_rev_kern
             float x = 0.0f;
 #pragma unroll
             for (int i = 0; i < 4; ++i) x += sh.red[t >> 6][i][t & 63][w];
-            sl[tl.skwb + ((size_t)w * kTileMaxCl + rank) * tb * 64 + t] = x;
+            sl[tl.skwb + ((size_t)w * kTileShares + rank) * tb * 64 + t] = x;
         }
         // pub += W_last phb
         for (int tk = 0; tk < tbn; ++tk) {
@@ -790,9 +777,9 @@ __global__ void __launch_bounds__(128) tile_gate_kernel(const GroupArgs ga) {
         in[0][t] = a.beta[t0 + t]; in[1][t] = a.gamma[t0 + t]; in[2][t] = a.eta[t0 + t];
         in[5][t] = sc.S[t + 1]; in[6][t] = sc.bt[t + 1]; in[7][t] = sc.gt[t + 1];
         float w = 0.0f, m = 0.0f;
-        for (int r = 0; r < CL; ++r) {
+        for (int r = 0; r < ga.shares; ++r) {
             w += sl[tl.skwb + (size_t)r * tl.tb * 64 + t];
-            m += sl[tl.skwb + (size_t)(kTileMaxCl + r) * tl.tb * 64 + t];
+            m += sl[tl.skwb + (size_t)(kTileShares + r) * tl.tb * 64 + t];
         }
         in[3][t] = w; in[4][t] = m;
     }
@@ -829,6 +816,22 @@ __global__ void __launch_bounds__(128) tile_gate_kernel(const GroupArgs ga) {
 constexpr size_t kRecSmem = 1024 + (size_t)kUnits * kUnitBytes + sizeof(Sync);
 constexpr size_t kRevSmem = kRecSmem + sizeof(RevShared);
 
+template <int KIND> cudaError_t launch_rev(const GroupArgs& ga, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(ga.a.N * ga.a.cl));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kRevSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ga.a.cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, tile_rev_kernel<KIND>, ga);
+}
+
 template <int KIND> int launch(const SimtBwdArgs& a0, cudaStream_t st) {
     static bool attr_done[64];
     int dev = 0;
@@ -842,7 +845,8 @@ template <int KIND> int launch(const SimtBwdArgs& a0, cudaStream_t st) {
     GroupArgs ga{};
     ga.a = a0;
     const TileLayout& tl = a0.lay.tl;
-    ga.a.cl = tl.cl;
+    ga.a.cl = tile_chain_serves(tl) ? tile_chain_ctas(tl) : tl.cl;
+    ga.shares = tile_chain_serves(tl) ? 4 * ga.a.cl : tl.cl;
     for (int end = a0.nchunks; end > 0; end -= tl.G) {
         ga.c0 = end > tl.G ? end - tl.G : 0;
         ga.ng = end - ga.c0;
@@ -851,19 +855,7 @@ template <int KIND> int launch(const SimtBwdArgs& a0, cudaStream_t st) {
         const int chunks = a0.N * ga.ng, items = chunks * tl.tb;
         tile_prep_kernel<KIND == 0 ? 2 : 3><<<dim3(chunks, chunks >= 592 ? 1 : (592 + chunks - 1) / chunks), 256, 0, st>>>(ga);
         tile_rec_kernel<KIND><<<items < 148 ? items : 148, kThreads, kRecSmem, st>>>(ga);
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)(a0.N * tl.cl));
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = kRevSmem;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)tl.cl;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        cudaError_t e = cudaLaunchKernelEx(&cfg, tile_rev_kernel<KIND>, ga);
+        cudaError_t e = tile_chain_serves(tl) ? (cudaError_t)tile_chain_launch(ga, KIND, st) : launch_rev<KIND>(ga, st);
         if (e != cudaSuccess) return (int)e;
         tile_gate_kernel<<<chunks, 128, 0, st>>>(ga);
         e = cudaGetLastError();

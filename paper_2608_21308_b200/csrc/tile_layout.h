@@ -12,6 +12,7 @@ namespace e2ttt {
 constexpr size_t kTileBlk = 4096;  // floats per block (hi + lo)
 constexpr int kTileMaxD = 128;
 constexpr int kTileMaxCl = 8;
+constexpr int kTileShares = 4 * kTileMaxCl;
 
 struct TileLayout {
     int db, hb, tb;  // 64-blocks along d, h and the tokens of a chunk
@@ -80,9 +81,11 @@ inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, i
     t.bPhb = take(hb * tb * kTileBlk);
     for (int i = 0; i < nmat - 1; ++i) { t.bZk[i] = take(hb * tb * kTileBlk); t.bz0[i] = take(hb * tb * kTileBlk); }
     t.bUk = take(tb * db * kTileBlk); t.bakb = take(hb * tb * kTileBlk);
-    t.bslot = take((size_t)2 * t.cl * tb * 64 * db * 64);
+    const int ctas = (t.hb + 1) / 2;  // of the chain kernel, where it serves
+    const size_t parts = 2 * (size_t)(ctas <= kTileMaxCl && ctas > t.cl ? ctas : t.cl);
+    t.bslot = take(parts * tb * 64 * db * 64);
     for (int i = 0; i < 2; ++i) {
-        t.bdk[i] = take((size_t)2 * t.cl * tb * 64 * db * 64);
+        t.bdk[i] = take(parts * tb * 64 * db * 64);
         t.bEb[i] = take(tb * 64 * db * 64);
     }
     t.bred = take((size_t)kTileMaxCl * 128);
@@ -99,7 +102,7 @@ inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, i
     t.sy = take(tb * 64 * db * 64); t.spu = take(tb * 64 * db * 64);
     t.sr = take(tb * 64); t.smey = take(tb * 64);
     t.ssc = take(5 * 512 + 16);
-    t.skwb = take((size_t)2 * kTileMaxCl * tb * 64);
+    t.skwb = take((size_t)2 * kTileShares * tb * 64);
     t.sdots = take((size_t)4 * kTileMaxCl);
     t.slot_stride = o;
     o = t.slot + t.slot_stride * (size_t)t.G;
