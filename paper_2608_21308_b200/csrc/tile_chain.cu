@@ -340,25 +340,29 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
         };
         auto prefetch_late = [&](int g) {  // for the rest of the chunk
             float* sn = slot_of(a, seq, g);
-            const float* cn = ws + lay.ckpt + (size_t)(ga.c0 + g) * 2 * NMAT * dh;
             if (lane < 3) {
                 const size_t src[3] = {tl.sAq, tl.sZq[0], SW ? tl.sZq[LAST - 1] : tl.sAq};
                 pf(sn + src[lane] + own, own_bytes);
             } else if (lane >= 4 && lane < 4 + LAST) {
                 pf(sn + tl.sW[lane - 4] + (size_t)b0 * db * kTileBlk, (size_t)nb * db * B);
-            } else if (lane >= 8 && lane < 8 + 2 * LAST) {
-                const int i = (lane - 8) >> 1;
-                pf(cn + (size_t)(((lane & 1) ? NMAT : 0) + i) * dh + (size_t)h0 * d, (size_t)nh * d * 4);
-            } else if (lane >= 16 && lane < 19) {
+            } else if (lane >= 8 && lane < 11) {
                 const size_t src[3] = {tl.sQ, tl.sUq, tl.sy};
-                if ((lane - 16) % CL == rank) pf(sn + src[lane - 16], (size_t)tb * 64 * dp * (lane == 16 ? 2 : 4));
+                if ((lane - 8) % CL == rank) pf(sn + src[lane - 8], (size_t)tb * 64 * dp * (lane == 8 ? 2 : 4));
             }
-            // 512-byte pieces of the last matrix's rows: plain prefetches (the bulk engine takes as long for a small piece as for a
-            // large one, and the loads of the products queue behind it)
-            const char* wl = reinterpret_cast<const char*>(cn + (size_t)LAST * dh + h0);
+            __syncwarp();
+        };
+        // The saved W, M that the scaling of the masters reads: plain prefetches, which do not stand in the bulk engine's queue before
+        // the loads of the products
+        auto prefetch_state = [&](int g) {
+            const float* cn = ws + lay.ckpt + (size_t)(ga.c0 + g) * 2 * NMAT * dh;
+            auto line = [](const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); };
+            for (int i = 0; i < 2 * LAST; ++i) {
+                const float* p = cn + (size_t)((i & 1 ? NMAT : 0) + (i >> 1)) * dh + (size_t)h0 * d;
+                for (int r = 32 * lane; r < nh * d; r += 32 * 32) line(p + r);
+            }
+            const float* wl = cn + (size_t)LAST * dh + h0;
             for (int r = lane; r < 8 * d; r += 32)
-                if ((r & 3) * 128 < nh * 4)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(wl + ((size_t)(r & 4 ? NMAT : 0) * dh + (size_t)(r >> 3) * h) * 4 + (r & 3) * 128));
+                if ((r & 3) * 32 < nh) line(wl + (size_t)(r & 4 ? NMAT : 0) * dh + (size_t)(r >> 3) * h + (r & 3) * 32);
             __syncwarp();
         };
         uint32_t n = 0;
@@ -374,10 +378,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             auto tok_d = [&](const unsigned char* m) { return Opnd{m, db == 2 ? m + B : nullptr, (uint32_t)db * B, true, true}; };
             auto key_d = [&](const unsigned char* m) { return Opnd{m, db == 2 ? m + kHalf : nullptr, (uint32_t)db * kHalf, false, true}; };
 
-            if (G.copier()) {
-                if (n == 0) prefetch_early(g);
-                prefetch_late(g);
-            }
+            if (G.copier()) prefetch_state(g);
             if (NORMED) {
                 G.cluster_arrive_all();
                 G.cluster_wait_all();
@@ -403,6 +404,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 for (int i = 0; i < LAST; ++i) by_d(tok_h(sblk(tl.sPz[i]), tk), i, i > 0);
                 G.job_end();
             }
+            if (G.copier()) prefetch_late(g);
             for (int tk = 0; tk < tbn; ++tk) {  // pub += W_last phb
                 G.job_begin();
                 G.streamed(nb, w_by_d(sblk(tl.sW[LAST]), false), tok_h(blk(tl.bPhb), tk), G.acc(), false, [&] { G.await(&sh.phb, n, 406); });
@@ -431,12 +433,12 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 G.job_end();
             }
             // the keys' part
-            if (G.copier() && g > 0) prefetch_early(g - 1);
 #pragma unroll
             for (int i = 0; i < LAST; ++i) G.streamed(tbn, key_d(sblk(tl.sK)), h_tok(blk(tl.bZk[i])), 128 * i, true, nothing);
             G.streamed(tbn, h_tok(blk(tl.bPhb)), tok_d(sblk(tl.sPu)), 128 * LAST, true, nothing);
             G.streamed(tbn, h_tok(sblk(tl.sAk)), tok_d(blk(tl.bUk)), 128 * LAST, true, nothing);
             if (G.issuer()) umma_commit_elect(&sh.upd, lane == 0);
+            if (G.copier() && g > 0) prefetch_early(g - 1);
         }
         G.cluster_arrive_all();
         G.cluster_wait_all();
