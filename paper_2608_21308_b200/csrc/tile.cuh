@@ -291,6 +291,29 @@ __device__ __forceinline__ float reduce16(const float (&v)[16], int lane) {
     return s + __shfl_xor_sync(0xffffffffu, s, 1);
 }
 
+// ---- activations ---------------------------------------------------------------------------------------------------------------
+// The epilogues evaluate them for every token and hidden unit, and were bound by the instructions of erff, expf and the division.
+// Normal distribution function and density: erfc(x) = t exp(P(t) - x^2), t = 1 / (1 + x / 2), P a Chebyshev fit of degree 9 to
+// log(exp(x^2) erfc(x) / t) on t in [0.15, 1], error 6e-8 (beyond, at |z| > 16, the tail is 0 in fp32); the distribution function is
+// within 2.4e-7, where the products that follow round to 16 bits of mantissa.
+__device__ __forceinline__ void normal_dist(float z, float& cdf, float& pdf) {
+    const float x = 0.70710678118f * fabsf(z), x2 = x * x;
+    const float t = __fdividef(1.0f, fmaf(0.5f, x, 1.0f));
+    float p = fmaf(t, 0.154191726f, -0.731059300f);
+    p = fmaf(t, p, 1.274361592f);
+    p = fmaf(t, p, -0.851879440f);
+    p = fmaf(t, p, 0.047508604f);
+    p = fmaf(t, p, -0.066028275f);
+    p = fmaf(t, p, 0.057246348f);
+    p = fmaf(t, p, 0.381963899f);
+    p = fmaf(t, p, 0.999168800f);
+    p = fmaf(t, p, -1.265473900f);
+    const float q = 0.5f * t * __expf(p - x2);  // P(Z > |z|)
+    cdf = z < 0.0f ? q : 1.0f - q;
+    pdf = 0.39894228040f * __expf(-x2);
+}
+__device__ __forceinline__ float sigmoid_hw(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
+
 // ---- rows of the caller's bf16 token tensors: 4 values at column c (0 beyond d) -----------------------------------------
 __device__ __forceinline__ void ld_tok4(const __nv_bfloat16* row, int c, int d, float (&v)[4]) {
     if ((d & 3) == 0) {
@@ -324,6 +347,17 @@ template <int U = 4> __device__ __forceinline__ void add_parts(const float* p, i
         for (int i = 0; i < U; ++i) { v[0] += x[i].x; v[1] += x[i].y; v[2] += x[i].z; v[3] += x[i].w; }
     }
 }
+// warp-wide sums of R values, R independent shuffles in flight
+template <int R> __device__ __forceinline__ void warp_sums(float (&v)[R]) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        float o[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) o[i] = __shfl_xor_sync(0xffffffffu, v[i], off);
+#pragma unroll
+        for (int i = 0; i < R; ++i) v[i] += o[i];
+    }
+}
 __device__ __forceinline__ float sum4(const float (&a)[4]) { return (a[0] + a[1]) + (a[2] + a[3]); }
 __device__ __forceinline__ float dot4(const float (&a)[4], const float (&b)[4]) {
     return (a[0] * b[0] + a[1] * b[1]) + (a[2] * b[2] + a[3] * b[3]);
@@ -333,10 +367,19 @@ __device__ __forceinline__ float dot4(const float (&a)[4], const float (&b)[4]) 
 // pick the rows of the calling warp out of tb * 64.
 __device__ __forceinline__ void tokens_to_blocks(const __nv_bfloat16* src, int len, int d, int db, int tb, unsigned char* dst, int first, int step,
                                                  int lane) {
-    for (int t = first; t < tb * 64; t += step) {
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (t < len) ld_tok4(src + (size_t)t * d, 4 * lane, d, v);
-        if (4 * lane < db * 64) st_split4<false>(dst + (size_t)((t >> 6) * db + (lane >> 4)) * kHalf, t & 63, (4 * lane) & 63, v);
+    constexpr int R = 4;  // rows in flight
+    for (int t0 = first; t0 < tb * 64; t0 += R * step) {
+        float v[R][4];
+#pragma unroll
+        for (int i = 0; i < R; ++i) ld_tok4(src + (size_t)min(t0 + i * step, len - 1) * d, 4 * lane, d, v[i]);
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const int t = t0 + i * step;
+            if (t >= len)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[i][j] = 0.0f;
+            if (t < tb * 64 && 4 * lane < db * 64) st_split4<false>(dst + (size_t)((t >> 6) * db + (lane >> 4)) * kHalf, t & 63, (4 * lane) & 63, v[i]);
+        }
     }
 }
 
@@ -350,7 +393,10 @@ __device__ __forceinline__ void matrix_to_blocks(const float* src, int nfast, in
         const int f = fb0 * 64 + 32 * (e % nf) + lane, s0 = sb0 * 64 + 16 * (e / nf);
         float v[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = (f < nfast && s0 + j < nslow) ? src[(size_t)(s0 + j) * nfast + f] : 0.0f;
+        for (int j = 0; j < 16; ++j) v[j] = src[(size_t)min(s0 + j, nslow - 1) * nfast + min(f, nfast - 1)];
+        if (f >= nfast || s0 + 16 > nslow)
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = (f < nfast && s0 + j < nslow) ? v[j] : 0.0f;
         st_split16(dst + ((size_t)(f >> 6) * rs + (size_t)(s0 >> 6) * cs) * (2 * kHalf), f & 63, s0 & 63, v);
     }
 }

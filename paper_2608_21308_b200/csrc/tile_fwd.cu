@@ -117,11 +117,12 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_fwd_kern
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             if (!SW) {
-                                const float cdf = norm_cdf(z1[j]);
+                                float cdf, pdf;
+                                normal_dist(z1[j], cdf, pdf);
                                 act[j] = z1[j] * cdf;
-                                if (key) c1[64 * j] = cdf + z1[j] * norm_pdf(z1[j]);
+                                if (key) c1[64 * j] = cdf + z1[j] * pdf;
                             } else {
-                                const float sg = sigmoid_f(z1[j]), sl = z1[j] * sg;
+                                const float sg = sigmoid_hw(z1[j]), sl = z1[j] * sg;
                                 act[j] = sl * z2[j];
                                 if (key) {
                                     c1[64 * j] = z2[j] * (sg * (1.0f + z1[j] * (1.0f - sg)));
@@ -158,41 +159,84 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_fwd_kern
 
         // ---- rows: layer norm; outputs of the queries; pu = dL/du of the keys (Algorithm 1 line 3) ----------------------------
         if (G.epi()) {
-            const int ci = 4 * lane;
-            for (int rr = rank * kEpiWarps + warp; rr < tbn * 128; rr += CL * kEpiWarps) {
-                const int tk = rr >> 7, t = tk * 64 + (rr & 63);
-                const bool key = (rr & 127) < 64, live = t < len;
-                float u[4] = {0.f, 0.f, 0.f, 0.f}, x[4], vv[4];
-                if (live) {
-                    ld_tok4((key ? kc : qc) + (size_t)t * d, ci, d, x);
-                    if (key) ld_tok4(vc + (size_t)t * d, ci, d, vv);
-                    if (ci < dp) add_parts(ws + tl.fslot + ((size_t)tk * 128 + (rr & 127)) * dp + ci, CL, (size_t)tb * 128 * dp, u);
-                    const float mu = warp_sum(sum4(u)) / (float)d;
+            const int ci = 4 * lane, step = CL * kEpiWarps, nrows = tbn * 128;
+            constexpr int R = 2;  // rows of a warp in flight: a row is a chain of loads and five reductions
+            for (int r0 = rank * kEpiWarps + warp; r0 < nrows; r0 += R * step) {
+                float u[R][4], x[R][4], vv[R][4], mu[R], rs[R];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) u[j] = ci + j < d ? u[j] - mu : 0.0f;
-                    const float r = r_rsqrt(warp_sum(dot4(u, u)) / (float)d + a.eps);
+                for (int i = 0; i < R; ++i) {
+                    const int rr = min(r0 + i * step, nrows - 1), t = min((rr >> 7) * 64 + (rr & 63), len - 1);
+                    ld_tok4(((rr & 127) < 64 ? kc : qc) + (size_t)t * d, ci, d, x[i]);
+                    ld_tok4(vc + (size_t)t * d, ci, d, vv[i]);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) u[j] *= r;
-                    if (key) {
-                        float e[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) e[j] = x[j] + u[j] - vv[j];
-                        const float se = warp_sum(sum4(e)) / (float)d, sey = warp_sum(dot4(e, u)) / (float)d;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) u[j] = ci + j < d ? r * (e[j] - se - u[j] * sey) : 0.0f;
-                    } else if (a.o) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) u[j] += x[j];
-                        st_tok4(o + (size_t)(s + t) * d, ci, d, u);
-                    }
+                    for (int j = 0; j < 4; ++j) u[i][j] = 0.0f;
                 }
-                if (key && ci < dp) {
+                for (int r = 0; r < CL; ++r) {  // the CTAs' partial sums, in CTA order
+                    float4 p[R];
+#pragma unroll
+                    for (int i = 0; i < R; ++i)
+                        p[i] = *reinterpret_cast<const float4*>(ws + tl.fslot + ((size_t)r * tb * 128 + min(r0 + i * step, nrows - 1)) * dp + min(ci, dp - 4));
+#pragma unroll
+                    for (int i = 0; i < R; ++i) { u[i][0] += p[i].x; u[i][1] += p[i].y; u[i][2] += p[i].z; u[i][3] += p[i].w; }
+                }
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) u[i][j] = ci + j < d ? u[i][j] : 0.0f;
+                    mu[i] = sum4(u[i]);
+                }
+                warp_sums(mu);
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    const float m = mu[i] / (float)d;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) u[i][j] = ci + j < d ? u[i][j] - m : 0.0f;
+                    rs[i] = dot4(u[i], u[i]);
+                }
+                warp_sums(rs);
+                float se[R], sey[R];
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    rs[i] = r_rsqrt(rs[i] / (float)d + a.eps);
+                    float e[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        u[i][j] *= rs[i];
+                        e[j] = x[i][j] + u[i][j] - vv[i][j];
+                    }
+                    se[i] = sum4(e);
+                    sey[i] = dot4(e, u[i]);
+                }
+                warp_sums(se);
+                warp_sums(sey);
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    const int rr = r0 + i * step, tk = rr >> 7, t = tk * 64 + (rr & 63);
+                    if (rr >= nrows) continue;
+                    const bool live = t < len;
+                    if ((rr & 127) >= 64) {
+                        if (live && a.o) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) u[i][j] += x[i][j];
+                            st_tok4(o + (size_t)(s + t) * d, ci, d, u[i]);
+                        }
+                        continue;
+                    }
                     const float kw = live ? sc.kW[t] : 0.0f, km = live ? sc.kM[t] : 0.0f;
-                    const size_t off = (size_t)(tk * db + (lane >> 4)) * B;
-                    const float uw[4] = {kw * u[0], kw * u[1], kw * u[2], kw * u[3]}, um[4] = {km * u[0], km * u[1], km * u[2], km * u[3]};
-                    st_split4<true>(blk(tl.fPu) + off, t & 63, ci & 63, u);
-                    st_split4<true>(blk(tl.fPuW) + off, t & 63, ci & 63, uw);
-                    st_split4<true>(blk(tl.fPuM) + off, t & 63, ci & 63, um);
+                    float pu[4], uw[4], um[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float e = x[i][j] + u[i][j] - vv[i][j];
+                        pu[j] = live && ci + j < d ? rs[i] * (e - se[i] / (float)d - u[i][j] * (sey[i] / (float)d)) : 0.0f;
+                        uw[j] = kw * pu[j];
+                        um[j] = km * pu[j];
+                    }
+                    if (ci < dp) {
+                        const size_t off = (size_t)(tk * db + (lane >> 4)) * B;
+                        st_split4<true>(blk(tl.fPu) + off, t & 63, ci & 63, pu);
+                        st_split4<true>(blk(tl.fPuW) + off, t & 63, ci & 63, uw);
+                        st_split4<true>(blk(tl.fPuM) + off, t & 63, ci & 63, um);
+                    }
                 }
             }
             if (c + 1 < a.nchunks) {  // the next chunk's tokens
@@ -259,27 +303,42 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_fwd_kern
                 w_copy[i] = ck + (size_t)i * dh; m_copy[i] = ck + (size_t)(NMAT + i) * dh;
             }
         }
-        // 16 results of one lane: element e0 + j * es, weights' aggregate in aw, momentum's in am
-        auto transition = [&](int i, size_t e0, size_t es, bool lane_ok, int nj, uint32_t t, int col, unsigned char* wb, int brow) {
-            float aw[16], am[16], w[16], m[16];
-            acc16(t + col, aw);
-            acc16(t + 128 + col, am);
+        // 16 results of one lane: elements base + ln + j * es, j < nj, of lane index ln < nl; weights' aggregate in columns col..,
+        // momentum's 128 further.  Indices are clamped and values masked: with a branch at every load they were one round trip each
+        auto transition = [&](int i, size_t base, int ln, int nl, int es, int nj, uint32_t t, int col, unsigned char* wb, int brow) {
+            float acc[16], w[16], m[16];
+            const bool lane_ok = ln < nl;
+            if (nj > 0) {
+                const size_t b = base + min(ln, nl - 1);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const bool ok = lane_ok && j < nj;
-                w[j] = ok ? w_in[i][e0 + j * es] : 0.0f;
-                m[j] = ok && m_in[i] ? m_in[i][e0 + j * es] : 0.0f;
+                for (int j = 0; j < 16; ++j) w[j] = w_in[i][b + (size_t)(min(j, nj - 1) * es)];
+                if (m_in[i])
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) m[j] = m_in[i][b + (size_t)(min(j, nj - 1) * es)];
+                else
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) m[j] = 0.0f;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) w[j] = m[j] = 0.0f;
             }
+            acc16(t + 128 + col, acc);  // G_t = -grad: the aggregations enter with a minus sign
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-                const float wn = cw * w[j] + cm * m[j] - aw[j];  // G_t = -grad: the aggregations enter with a minus sign
-                const float mn = cb * m[j] - am[j];
+                const float mj = m[j];
+                m[j] = cb * mj - acc[j];
+                w[j] = cw * w[j] + cm * mj;
+            }
+            acc16(t + col, acc);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
                 const bool ok = lane_ok && j < nj;
+                w[j] = ok ? w[j] - acc[j] : 0.0f;
+                const size_t e = base + ln + (size_t)(j * es);
                 if (ok) {
-                    w_out[i][e0 + j * es] = wn; m_out[i][e0 + j * es] = mn;
-                    if (w_copy[i]) { w_copy[i][e0 + j * es] = wn; m_copy[i][e0 + j * es] = mn; }
+                    w_out[i][e] = w[j]; m_out[i][e] = m[j];
+                    if (w_copy[i]) { w_copy[i][e] = w[j]; m_copy[i][e] = m[j]; }
                 }
-                w[j] = ok ? wn : 0.0f;
             }
             if (wb && !normed) st_split16(wb, brow, col & 63, w);
         };
@@ -300,7 +359,7 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_fwd_kern
                     for (int half = 0; half < 2; ++half) {
                         const int col = 32 * grp + 16 * half, j0 = b0 * 64 + col, bl = b0 + (col >> 6);
                         if (col >= 64 && !two) break;
-                        transition(i, (size_t)j0 * d + row, d, row < d, h - j0, t, col,
+                        transition(i, (size_t)j0 * d, row, d, d, h - j0, t, col,
                                    row < dp ? blk(tl.Wb[i]) + ((size_t)bl * db + (row >> 6)) * B : nullptr, row & 63);
                     }
                 });
@@ -314,12 +373,12 @@ template <int KIND> __global__ void __launch_bounds__(kThreads, 1) tile_fwd_kern
                 G.job_begin();
                 G.term<2>(tbn, true, act, pu, {0u, 128u});
                 G.job_end([&](uint32_t t) {
-                    const int bl = b0 + (row >> 6), j = b0 * 64 + row;
+                    const int bl = b0 + (row >> 6);
 #pragma unroll 1
                     for (int half = 0; half < 2; ++half) {
                         const int col = 32 * grp + 16 * half;
                         if (col >= dp) break;
-                        transition(LAST, (size_t)col * h + j, h, (row < 64 || two) && j < h, d - col, t, col,
+                        transition(LAST, (size_t)col * h + b0 * 64, row, min(two ? 128 : 64, h - b0 * 64), h, d - col, t, col,
                                    row < 64 || two ? blk(tl.Wb[LAST]) + ((size_t)bl * db + (col >> 6)) * B : nullptr, row & 63);
                     }
                 });

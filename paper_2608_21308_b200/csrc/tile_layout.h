@@ -41,16 +41,20 @@ inline int tile_cluster_size(int N, int hb) {
     return (hb + sb - 1) / sb;
 }
 
-// Chunks prepared at a time: N * tb * G independent work items should fill whole waves of 148 CTAs; bounded, since a slot
-// costs about 30 bytes per token and hidden unit.
-inline int tile_group_chunks(int N, int tb) {
+// Chunks prepared at a time: N * tb * G independent work items should fill whole waves of 148 CTAs, and each group costs a launch of
+// every kernel.  At most 9 items per sequence, and 512 MB of slots for the whole call (a slot costs about 30 bytes per token and hidden
+// unit): the workspace of a checkpointed call is to stay a small part of what all chunks' states would take.
+inline int tile_group_chunks(int N, int tb, size_t slot_bytes) {
     int best = 1;
     double best_eff = 0.0;
     for (int g = 1; g <= 9; ++g) {
-        if (g > 1 && (size_t)g * tb > 9) break;
+        if (g > 1 && ((size_t)g * tb > 9 || slot_bytes * g * N > ((size_t)512 << 20))) break;
         const double items = (double)N * tb * g, waves = (double)(long long)((items + 147) / 148);
         const double eff = items / (148.0 * waves);
-        if (eff > best_eff + 0.03) { best_eff = eff; best = g; }
+        if (eff > best_eff - 0.01) {
+            best = g;
+            if (eff > best_eff) best_eff = eff;
+        }
     }
     return best;
 }
@@ -61,7 +65,6 @@ inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, i
     auto take = [&](size_t n) { size_t r = o; o += (n + 31) / 32 * 32; return r; };
     t.db = blocks(d); t.hb = blocks(h); t.tb = blocks(C);
     t.cl = tile_cluster_size(N, t.hb);
-    t.G = tile_group_chunks(N, t.tb);
     const size_t db = t.db, hb = t.hb, tb = t.tb;
     const int sw = nmat == 3;
     if (backward)
@@ -105,6 +108,7 @@ inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, i
     t.skwb = take((size_t)2 * kTileShares * tb * 64);
     t.sdots = take((size_t)4 * kTileMaxCl);
     t.slot_stride = o;
+    t.G = tile_group_chunks(N, t.tb, o * sizeof(float));
     o = t.slot + t.slot_stride * (size_t)t.G;
     return o > end_fwd ? o : end_fwd;
 }
