@@ -10,9 +10,10 @@
 //   shared memory : operand blocks (hi, lo) of T of as many matrices as fit 128 KB (two at d > 64), rows = the index on the
 //                   lanes: read K-major with that index on the lanes, MN-major with the other one there
 // S, and T blocks that do not fit, live in the workspace; 33 sequences' worth stays in L2.
-// In a chunk the products run on the operand blocks of the arriving T, S; then the masters are scaled by the carries
-// (T <- cw T, S <- cm T + cb S) while the cluster exchanges partial sums, the chunk's own contribution is accumulated onto T at the
-// end, and the operand blocks are written anew.  Everything else streams from the slots that tile_prep and tile_rec filled.
+// In a chunk the products run on the operand blocks of the arriving T, S; meanwhile, piece by piece between their epilogues, the
+// masters are scaled by the carries (T <- cw T, S <- cm T + cb S; the blocks of the new S go to the other of two buffers, by the
+// parity of the chunk), the chunk's own contribution is accumulated onto T, and T's operand blocks are written anew.  Everything else
+// streams from the slots that tile_prep and tile_rec filled.
 //
 // 18 warps: 0-15 epilogues (warp w: lanes 32 (w & 3).., group w >> 2 of the columns), 16 copies operand blocks, 17 issues MMAs.
 #include "tile_chain.h"
@@ -287,6 +288,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
     const int nb = two ? 2 : 1;
     float* ws = reinterpret_cast<float*>(a.ws) + (size_t)seq * lay.per_seq;
     auto blk = [&](size_t off) { return bytes_of(ws + off); };
+    const size_t sblks = (size_t)db * tl.hb * kTileBlk;  // between the two buffers of S blocks
     // resident T of matrix i at i * unit: hi blocks, then lo; blocks that share the index on their columns are neighbours
     const uint32_t half = 2u * db * kHalf, unit = 2 * half;
     const int nres = min(NMAT, (int)(kResident / unit));
@@ -303,18 +305,19 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             const unsigned char* p = m + (size_t)b0 * db * B;
             return Opnd{p, db == 2 ? p + B : nullptr, (uint32_t)db * B, true, !rows_d};
         };
+        size_t sbuf = 0;  // S blocks of the chunk at hand
         // products of a [tokens x ..] operand with T and S of matrix i, hidden units or d on the lanes
         auto by_h = [&](const Opnd& x, int i) {
             const bool f = i < LAST;
             G.pair(db, x, i < nres,
                    [&](int k) { return SOp{G.resident + i * unit + k * (f ? kHalf : 2 * kHalf), half, f ? db * kHalf : kHalf, f, false}; },
-                   w_by_h(blk(tl.Tb[i]), f), w_by_h(blk(tl.Sb[i]), f), false);
+                   w_by_h(blk(tl.Tb[i]), f), w_by_h(blk(tl.Sb[i] + sbuf), f), false);
         };
         auto by_d = [&](const Opnd& x, int i, bool acc) {
             const bool f = i < LAST;
             G.pair(nb, x, i < nres,
                    [&](int k) { return SOp{G.resident + i * unit + k * (f ? db * kHalf : kHalf), half, f ? kHalf : 2 * kHalf, !f, false}; },
-                   w_by_d(blk(tl.Tb[i]), f), w_by_d(blk(tl.Sb[i]), f), acc);
+                   w_by_d(blk(tl.Tb[i]), f), w_by_d(blk(tl.Sb[i] + sbuf), f), acc);
         };
         auto nothing = [] {};
         // What a chunk reads was written long ago and comes from HBM: into L2 half a chunk ahead (a whole chunk ahead would not fit
@@ -366,6 +369,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             __syncwarp();
         };
         uint32_t n = 0;
+        if (G.copier()) prefetch_state(ga.ng - 1);
         for (int g = ga.ng - 1; g >= 0; --g, ++n) {
             const int c = ga.c0 + g, len = min(a.C, a.L - c * a.C), tbn = (len + 63) / 64;
             float* sl = slot_of(a, seq, g);
@@ -378,13 +382,15 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             auto tok_d = [&](const unsigned char* m) { return Opnd{m, db == 2 ? m + B : nullptr, (uint32_t)db * B, true, true}; };
             auto key_d = [&](const unsigned char* m) { return Opnd{m, db == 2 ? m + kHalf : nullptr, (uint32_t)db * kHalf, false, true}; };
 
-            if (G.copier()) prefetch_state(g);
+            sbuf = (c & 1) * sblks;
             if (NORMED) {
                 G.cluster_arrive_all();
                 G.cluster_wait_all();
             }
             G.cluster_arrive_all();  // the first of the chunk's two barriers: nothing of these warps' is waited for
-            G.await(&sh.ops, n, 405);
+            // T in shared memory waits for the blocks written at the end of the chunk before; loads of S only for its scaling there
+            if (G.issuer() || n == 0) G.await(&sh.ops, n, 405);
+            else G.await(&sh.scaled, n - 1, 410);
             for (int tk = 0; tk < tbn; ++tk) {
                 const Opnd kt{sblk(tl.sK) + (size_t)tk * db * kHalf, nullptr, kHalf, false, false};
 #pragma unroll
@@ -393,6 +399,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                     by_h(kt, i);
                     G.job_end();
                 }
+                if (G.copier() && tk == 0 && nres < NMAT) G.await(&sh.ops, n, 411);
                 G.job_begin();
                 by_h(Opnd{sblk(tl.sPu) + (size_t)tk * db * B, nullptr, B, true, false}, LAST);
                 G.job_end();
@@ -404,17 +411,21 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 for (int i = 0; i < LAST; ++i) by_d(tok_h(sblk(tl.sPz[i]), tk), i, i > 0);
                 G.job_end();
             }
-            if (G.copier()) prefetch_late(g);
+            if (G.copier()) {
+                prefetch_late(g);
+                if (g > 0) prefetch_state(g - 1);
+            }
             for (int tk = 0; tk < tbn; ++tk) {  // pub += W_last phb
                 G.job_begin();
                 G.streamed(nb, w_by_d(sblk(tl.sW[LAST]), false), tok_h(blk(tl.bPhb), tk), G.acc(), false, [&] { G.await(&sh.phb, n, 406); });
                 G.job_end();
             }
-            // the queries' part of the chunk's contribution, onto the scaled masters
+            // the chunk's contribution, onto the scaled masters: the queries' part and whatever else there is before the rows
             if (G.issuer()) G.await(&sh.scaled, n, 407);
 #pragma unroll
             for (int i = 0; i < LAST; ++i) G.streamed(tbn, key_d(sblk(tl.sQ)), h_tok(sblk(tl.sZq[i])), 128 * i, true, nothing);
             G.streamed(tbn, h_tok(sblk(tl.sAq)), tok_d(sblk(tl.sUq)), 128 * LAST, true, nothing);
+            G.streamed(tbn, h_tok(blk(tl.bPhb)), tok_d(sblk(tl.sPu)), 128 * LAST, true, nothing);
             G.cluster_wait_all();
             G.cluster_arrive_all();
             if (G.issuer()) G.cluster_wait_all();
@@ -425,6 +436,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 });
                 G.job_end();
             }
+            G.streamed(tbn, h_tok(sblk(tl.sAk)), tok_d(blk(tl.bUk)), 128 * LAST, true, nothing);
             for (int tk = 0; tk < tbn; ++tk) {  // dk += W_first^T zb
                 G.job_begin();
 #pragma unroll
@@ -432,11 +444,9 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                     G.streamed(nb, w_by_d(sblk(tl.sW[i]), true), tok_h(blk(tl.bZk[i]), tk), G.acc(), i > 0, [&] { G.await(&sh.zb, n, 408); });
                 G.job_end();
             }
-            // the keys' part
+            // what waits for zb
 #pragma unroll
             for (int i = 0; i < LAST; ++i) G.streamed(tbn, key_d(sblk(tl.sK)), h_tok(blk(tl.bZk[i])), 128 * i, true, nothing);
-            G.streamed(tbn, h_tok(blk(tl.bPhb)), tok_d(sblk(tl.sPu)), 128 * LAST, true, nothing);
-            G.streamed(tbn, h_tok(sblk(tl.sAk)), tok_d(blk(tl.bUk)), 128 * LAST, true, nothing);
             if (G.issuer()) umma_commit_elect(&sh.upd, lane == 0);
             if (G.copier() && g > 0) prefetch_early(g - 1);
         }
@@ -462,19 +472,25 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = row < lane_lim(i) && j < nc ? v[j] : 0.0f;
     };
-    // operand blocks of T (resident or not) and S: 16 values of row `row`
-    auto put = [&](bool is_T, int i, int col, const float (&v)[16]) {
+    // operand blocks of T (resident or not) and S (of the chunks of one parity): 16 values of row `row`
+    auto put = [&](bool is_T, int sbuf, int i, int col, const float (&v)[16]) {
         const int rb = row >> 6, cb = col >> 6;
         if (i < LAST ? (row >= dp || (cb && !two)) : (!on_h || col >= dp)) return;
         const uint32_t res = i < LAST ? (uint32_t)(cb * db + rb) : (uint32_t)(cb * 2 + rb);
         if (is_T && i < nres) sts_split16(G.resident + i * unit + res * kHalf, half, row & 63, col & 63, v);
         else {
             const int hblk = i < LAST ? cb : rb, dblk = i < LAST ? rb : cb;
-            st_split16(blk(is_T ? tl.Tb[i] : tl.Sb[i]) + (size_t)((b0 + hblk) * db + dblk) * B, row & 63, col & 63, v);
+            st_split16(blk(is_T ? tl.Tb[i] : tl.Sb[i] + sbuf * sblks) + (size_t)((b0 + hblk) * db + dblk) * B, row & 63, col & 63, v);
         }
     };
-    // a piece of a state-shaped fp32 array (row-major [h x d], the last matrix [d x h]); 0 outside.  Indices are clamped and the
-    // values masked: with a branch at every load they were one round trip each
+    // A piece of a state-shaped fp32 array (row-major [h x d], the last matrix [d x h]); 0 outside.  At the edges indices are clamped
+    // and the values masked: with a branch at every load they were one round trip each.  The strides are opaque to the compiler, which
+    // otherwise keeps sixteen offsets per stride in registers, and spills: with 227 KB of shared memory in use hardly any L1 is left,
+    // so that a spilled value comes from L2
+    auto opaque = [](int x) {
+        asm volatile("" : "+r"(x));
+        return x;
+    };
     auto ld_state = [&](int i, const float* p, int col, float (&v)[16]) {
         const int nc = col_lim(i) - col;
         if (!p || nc <= 0) {
@@ -482,19 +498,24 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             for (int j = 0; j < 16; ++j) v[j] = 0.0f;
             return;
         }
-        const int ld = i < LAST ? d : h;
+        const int ld = opaque(i < LAST ? d : h);
         const float* q = p + (i < LAST ? (size_t)(h0 + col) * d : (size_t)col * h + h0) + min(row, lane_lim(i) - 1);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = q[(size_t)(min(j, nc - 1) * ld)];
+        for (int j = 0; j < 16; ++j) {
+            v[j] = *q;
+            if (j + 1 < nc) q += ld;
+        }
         mask(i, col, v);
     };
     auto st_state = [&](int i, float* p, int col, const float (&v)[16]) {
-        const int nc = col_lim(i) - col, ld = i < LAST ? d : h;
+        const int nc = col_lim(i) - col, ld = opaque(i < LAST ? d : h);
         float* q = p + (i < LAST ? (size_t)(h0 + col) * d : (size_t)col * h + h0) + row;
         if (row < lane_lim(i))
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if (j < nc) q[(size_t)(j * ld)] = v[j];
+            for (int j = 0; j < 16; ++j) {
+                if (j < nc) *q = v[j];
+                q += ld;
+            }
     };
 
     // ---- T -> tensor memory; T, S -> operand blocks; S -> the workspace
@@ -509,11 +530,9 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             ld_state(i, tf, col, t);
             ld_state(i, sf, col, s);
             acc_st16(lanes + 128 * i + col, t);
-            if (!NORMED) put(true, i, col, t);
-            if (given) {  // otherwise the launch before this one left them
-                put(false, i, col, s);
-                st_state(i, ws + lay.S[i], col, s);
-            }
+            if (!NORMED) put(true, 0, i, col, t);
+            if (ga.first) put(false, (ga.c0 + ga.ng - 1) & 1, i, col, s);  // otherwise the launch before this one left them
+            if (given) st_state(i, ws + lay.S[i], col, s);
         }
         tmem_wait_st();
         if (!NORMED) G.signal(&sh.ops);
@@ -590,12 +609,42 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
 #pragma unroll
                     for (int j = 0; j < 16; ++j) t[j] = __shfl_sync(0xffffffffu, f, j) * t[j] - y[j] * __shfl_sync(0xffffffffu, gy, j);
                     acc_st16(lanes + 128 * i + col_of(pc), t);
-                    put(true, i, col_of(pc), t);
+                    put(true, 0, i, col_of(pc), t);
                 }
                 G.epi_sync();
             }
             tmem_wait_st();
             G.signal(&sh.ops);
+        }
+
+        // The carries' adjoints <T, W>, <T, M>, <S, M>; T <- cw T, S <- cm T + cb S, while
+        // the first products run
+        {
+            float pw = 0.0f, pm = 0.0f, pb = 0.0f;
+            const float cw = sc.cw, cm = sc.cm, cb = sc.cb;
+#pragma unroll 1
+            for (int e = 0; e < 2 * NMAT; ++e) {
+                const int i = e >> 1, col = col_of(e & 1);
+                float w[16], m[16], t[16], sv[16];
+                ld_state(i, ck + (size_t)i * dh, col, w);
+                ld_state(i, ck + (size_t)(NMAT + i) * dh, col, m);
+                ld_state(i, ws + lay.S[i], col, sv);
+                acc16(lanes + 128 * i + col, t);
+                mask(i, col, t);  // lanes past the matrix collect whatever the MMAs read past the operands
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    pw += t[j] * w[j]; pm += t[j] * m[j]; pb += sv[j] * m[j];
+                    sv[j] = cm * t[j] + cb * sv[j];
+                    t[j] *= cw;
+                }
+                acc_st16(lanes + 128 * i + col, t);
+                st_state(i, ws + lay.S[i], col, sv);
+                put(false, buf ^ 1, i, col, sv);
+            }
+            tmem_wait_st();
+            pw = warp_sum(pw); pm = warp_sum(pm); pb = warp_sum(pb);
+            if (lane == 0) { sh.dots[warp][0] = pw; sh.dots[warp][1] = pm; sh.dots[warp][2] = pb; }
+            G.signal(&sh.scaled);
         }
 
         // ---- everything that meets (T, S) directly.  G_t enters W_C with K^W_t and M_C with K^M_t: its adjoint is K^W_t T + K^M_t S
@@ -685,9 +734,9 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             float pv[16];
             {
                 const float* p = sl + tl.spu + (size_t)(tk * 64 + 16 * grp) * dp + min(row, dp - 1);
-                const int nt = len - tk * 64 - 16 * grp;
+                const int nt = len - tk * 64 - 16 * grp, ld = opaque(dp);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) pv[j] = p[(size_t)j * dp];
+                for (int j = 0; j < 16; ++j, p += ld) pv[j] = *p;
 #pragma unroll
                 for (int j = 0; j < 16; ++j) pv[j] = row < dp && j < nt ? pv[j] : 0.0f;
             }
@@ -697,9 +746,11 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 acc16(t + 16 * grp, x);
                 acc16(t + 64 + 16 * grp, y);
                 float* out = partial(tl.bslot, 0, tk);
+                const int ld = opaque(dp);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
-                    if (row < dp) out[(size_t)j * dp] = -(kb[j] * x[j] + kb[16 + j] * y[j]);
+                    if (row < dp) *out = -(kb[j] * x[j] + kb[16 + j] * y[j]);
+                    out += ld;
                     x[j] = row < dp ? x[j] * pv[j] : 0.0f;
                     y[j] = row < dp ? y[j] * pv[j] : 0.0f;
                 }
@@ -717,9 +768,10 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 acc16(t + 16 * grp, x);
                 acc16(t + 64 + 16 * grp, y);
                 float* out = partial(tl.bdk[buf], 0, tk);
+                const int ld = opaque(dp);
                 if (row < dp)
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) out[(size_t)j * dp] = -(kb[j] * x[j] + kb[16 + j] * y[j]);
+                    for (int j = 0; j < 16; ++j, out += ld) *out = -(kb[j] * x[j] + kb[16 + j] * y[j]);
             });
         }
         auto plain_share = [&](size_t base) {
@@ -729,43 +781,15 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                     float x[16];
                     acc16(t + 16 * grp, x);
                     float* out = partial(base, 1, tk);
+                    const int ld = opaque(dp);
                     if (row < dp)
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) out[(size_t)j * dp] = x[j];
+                        for (int j = 0; j < 16; ++j, out += ld) *out = x[j];
                 });
         };
         plain_share(tl.bslot);  // pub += W_last phb
         G.cluster_arrive_all();
 
-        // ---- while the shares meet: the carries' adjoints <T, W>, <T, M>, <S, M>; T <- cw T, S <- cm T + cb S (every product with
-        // the operand blocks of the old S is in: they are written anew here, T's when the chunk's contribution is in)
-        {
-            const float cw = sc.cw, cm = sc.cm, cb = sc.cb;
-            float pw = 0.0f, pm = 0.0f, pb = 0.0f;
-#pragma unroll 1
-            for (int e = 0; e < 2 * NMAT; ++e) {
-                const int i = e >> 1, col = col_of(e & 1);
-                float w[16], m[16], t[16], sv[16];
-                ld_state(i, ck + (size_t)i * dh, col, w);
-                ld_state(i, ck + (size_t)(NMAT + i) * dh, col, m);
-                ld_state(i, ws + lay.S[i], col, sv);
-                acc16(lanes + 128 * i + col, t);
-                mask(i, col, t);  // lanes past the matrix collect whatever the MMAs read past the operands
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    pw += t[j] * w[j]; pm += t[j] * m[j]; pb += sv[j] * m[j];
-                    sv[j] = cm * t[j] + cb * sv[j];
-                    t[j] *= cw;
-                }
-                acc_st16(lanes + 128 * i + col, t);
-                st_state(i, ws + lay.S[i], col, sv);
-                put(false, i, col, sv);
-            }
-            tmem_wait_st();
-            pw = warp_sum(pw); pm = warp_sum(pm); pb = warp_sum(pb);
-            if (lane == 0) { sh.dots[warp][0] = pw; sh.dots[warp][1] = pm; sh.dots[warp][2] = pb; }
-            G.signal(&sh.scaled);
-        }
         G.cluster_wait_all();
 
         // ---- rows, dealt to the cluster's warps.  Warps 0-7: pu = J(u) e, e = k + y - v, y = LN(u): adjoints of e and u; dv.
@@ -849,7 +873,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 float t[16];
                 acc16(lanes + 128 * (e >> 1) + col_of(e & 1), t);
                 mask(e >> 1, col_of(e & 1), t);
-                put(true, e >> 1, col_of(e & 1), t);
+                put(true, 0, e >> 1, col_of(e & 1), t);
             }
             G.signal(&sh.ops);
         }

@@ -67,8 +67,9 @@ inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, i
     t.cl = tile_cluster_size(N, t.hb);
     const size_t db = t.db, hb = t.hb, tb = t.tb;
     const int sw = nmat == 3;
+    const bool chain = (t.hb + 1) / 2 <= kTileMaxCl;  // tile_chain.h: S blocks of even and of odd chunks
     if (backward)
-        for (int i = 0; i < nmat; ++i) { t.Tb[i] = take(db * hb * kTileBlk); t.Sb[i] = take(db * hb * kTileBlk); }
+        for (int i = 0; i < nmat; ++i) { t.Tb[i] = take(db * hb * kTileBlk); t.Sb[i] = take((chain ? 2 : 1) * db * hb * kTileBlk); }
     const size_t begin = o;
     for (int i = 0; i < nmat; ++i) t.Wb[i] = take(db * hb * kTileBlk);
     for (int i = 0; i < 2; ++i) { t.fK[i] = take(tb * db * kTileBlk / 2); t.fQ[i] = take(tb * db * kTileBlk / 2); }
