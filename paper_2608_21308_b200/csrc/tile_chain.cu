@@ -172,7 +172,7 @@ template <int NSET> struct Chain {
     __device__ void mma(uint32_t d, const SOp& a, const SOp& b, bool acc) {
         const uint32_t idesc = make_idesc(128, b.wide ? 128 : 64, a.mn, b.mn);
         const uint32_t sa = a.mn ? 2048u : 32u, sb = b.mn ? 2048u : 32u;
-#pragma unroll
+#pragma unroll 1
         for (int ks = 0; ks < 4; ++ks) {
             const uint64_t ah = make_smem_desc(a.addr + ks * sa, a.lbo, 1024), bh = make_smem_desc(b.addr + ks * sb, b.lbo, 1024);
             bool c = acc || ks > 0;
@@ -196,12 +196,14 @@ template <int NSET> struct Chain {
     // resident (part(k)) or from the ring (p), Q from the ring.
     template <typename F> __device__ void pair(int nk, const Opnd& s, bool p_resident, F part, const Opnd& p, const Opnd& q, bool acc0) {
         if (copier())
+#pragma unroll 1
             for (int k = 0; k < nk; ++k) {
                 load(s, k, false);
                 if (!p_resident) load(p, k, true);
                 load(q, k, true);
             }
         else if (issuer())
+#pragma unroll 1
             for (int k = 0; k < nk; ++k) {
                 uint32_t bs, bp, bq;
                 const SOp b = take(s, bs, false);
@@ -219,12 +221,14 @@ template <int NSET> struct Chain {
     // the first of p
     template <typename F> __device__ void streamed(int nk, const Opnd& s, const Opnd& p, uint32_t col, bool acc0, F before) {
         if (copier())
+#pragma unroll 1
             for (int k = 0; k < nk; ++k) {
                 load(s, k, true);
                 if (k == 0) before();
                 load(p, k, false);
             }
         else if (issuer())
+#pragma unroll 1
             for (int k = 0; k < nk; ++k) {
                 uint32_t ba, bb;
                 const SOp a = take(s, ba, true), b = take(p, bb, false);
@@ -391,9 +395,10 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             // T in shared memory waits for the blocks written at the end of the chunk before; loads of S only for its scaling there
             if (G.issuer() || n == 0) G.await(&sh.ops, n, 405);
             else G.await(&sh.scaled, n - 1, 410);
+#pragma unroll 1
             for (int tk = 0; tk < tbn; ++tk) {
                 const Opnd kt{sblk(tl.sK) + (size_t)tk * db * kHalf, nullptr, kHalf, false, false};
-#pragma unroll
+#pragma unroll 1
                 for (int i = 0; i < LAST; ++i) {
                     G.job_begin();
                     by_h(kt, i);
@@ -407,7 +412,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 by_d(tok_h(sblk(tl.sAk), tk), LAST, false);
                 G.job_end();
                 G.job_begin();
-#pragma unroll
+#pragma unroll 1
                 for (int i = 0; i < LAST; ++i) by_d(tok_h(sblk(tl.sPz[i]), tk), i, i > 0);
                 G.job_end();
             }
@@ -415,6 +420,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 prefetch_late(g);
                 if (g > 0) prefetch_state(g - 1);
             }
+#pragma unroll 1
             for (int tk = 0; tk < tbn; ++tk) {  // pub += W_last phb
                 G.job_begin();
                 G.streamed(nb, w_by_d(sblk(tl.sW[LAST]), false), tok_h(blk(tl.bPhb), tk), G.acc(), false, [&] { G.await(&sh.phb, n, 406); });
@@ -422,13 +428,14 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             }
             // the chunk's contribution, onto the scaled masters: the queries' part and whatever else there is before the rows
             if (G.issuer()) G.await(&sh.scaled, n, 407);
-#pragma unroll
+#pragma unroll 1
             for (int i = 0; i < LAST; ++i) G.streamed(tbn, key_d(sblk(tl.sQ)), h_tok(sblk(tl.sZq[i])), 128 * i, true, nothing);
             G.streamed(tbn, h_tok(sblk(tl.sAq)), tok_d(sblk(tl.sUq)), 128 * LAST, true, nothing);
             G.streamed(tbn, h_tok(blk(tl.bPhb)), tok_d(sblk(tl.sPu)), 128 * LAST, true, nothing);
             G.cluster_wait_all();
             G.cluster_arrive_all();
             if (G.issuer()) G.cluster_wait_all();
+#pragma unroll 1
             for (int tk = 0; tk < tbn; ++tk) {  // adjoint of u back through W_last
                 G.job_begin();
                 G.streamed(db, w_by_h(sblk(tl.sW[LAST]), false), Opnd{blk(tl.bUk) + (size_t)tk * db * B, nullptr, B, true, false}, G.acc(), false, [&] {
@@ -437,15 +444,16 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
                 G.job_end();
             }
             G.streamed(tbn, h_tok(sblk(tl.sAk)), tok_d(blk(tl.bUk)), 128 * LAST, true, nothing);
+#pragma unroll 1
             for (int tk = 0; tk < tbn; ++tk) {  // dk += W_first^T zb
                 G.job_begin();
-#pragma unroll
+#pragma unroll 1
                 for (int i = 0; i < LAST; ++i)
                     G.streamed(nb, w_by_d(sblk(tl.sW[i]), true), tok_h(blk(tl.bZk[i]), tk), G.acc(), i > 0, [&] { G.await(&sh.zb, n, 408); });
                 G.job_end();
             }
             // what waits for zb
-#pragma unroll
+#pragma unroll 1
             for (int i = 0; i < LAST; ++i) G.streamed(tbn, key_d(sblk(tl.sK)), h_tok(blk(tl.bZk[i])), 128 * i, true, nothing);
             if (G.issuer()) umma_commit_elect(&sh.upd, lane == 0);
             if (G.copier() && g > 0) prefetch_early(g - 1);
