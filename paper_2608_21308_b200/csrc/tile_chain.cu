@@ -151,11 +151,10 @@ template <int NSET> struct Chain {
             const uint32_t dst = ring + at;
             const size_t off = (size_t)k * o.ks;
             mbar_expect_tx(full, kHalf * (o.p1 ? 2u : 1u) * (o.lo ? 2u : 1u));
-            bulk_g2s(dst, o.p0 + off, kHalf, full);
-            if (o.p1) bulk_g2s(dst + kHalf, o.p1 + off, kHalf, full);
-            if (o.lo) {
-                bulk_g2s(dst + lo_of(o), o.p0 + off + kHalf, kHalf, full);
-                if (o.p1) bulk_g2s(dst + lo_of(o) + kHalf, o.p1 + off + kHalf, kHalf, full);
+#pragma unroll 1
+            for (int part = 0; part < (o.lo ? 2 : 1); ++part) {
+                bulk_g2s(dst + part * lo_of(o), o.p0 + off + part * kHalf, kHalf, full);
+                if (o.p1) bulk_g2s(dst + part * lo_of(o) + kHalf, o.p1 + off + part * kHalf, kHalf, full);
             }
         }
         __syncwarp();
@@ -192,50 +191,48 @@ template <int NSET> struct Chain {
         if (issuer()) umma_commit_elect(&sh->acc_full[job % NSET], lane == 0);
         ++job;
     }
-    // A column-side operand from the ring with two lane-side partners: D[0] += P S^T, D[64] += Q S^T over nk slices.  P is
-    // resident (part(k)) or from the ring (p), Q from the ring.
-    template <typename F> __device__ void pair(int nk, const Opnd& s, bool p_resident, F part, const Opnd& p, const Opnd& q, bool acc0) {
-        if (copier())
+    // One product over nk slices of 64, copy and MMA warps.  Paired: the column-side operand x with two lane-side partners,
+    // D[col] += Y X^T and D[col + 64] += Z X^T, where Y is resident or from the ring; else D[col] += X Z^T with x on the lane side.
+    // All products of a chunk go through the one copy of this code: with a copy for each, the two warps pushed the epilogues out of
+    // the instruction cache in every chunk (a quarter of all warps' time).
+    struct Product {
+        int nk;
+        Opnd x, y, z;
+        SOp part;             // Y, where it is resident (x ring otherwise), and its step per slice
+        uint32_t part_step, col;
+        bool paired, resident, acc0;
+        uint64_t* before;     // what the copy warp waits for between the first load of x and the first of z
+        bool before_cluster;  // the cluster barrier instead
+    };
+    __device__ void run(const Product& P, uint32_t phase) {
+        if (copier()) {
 #pragma unroll 1
-            for (int k = 0; k < nk; ++k) {
-                load(s, k, false);
-                if (!p_resident) load(p, k, true);
-                load(q, k, true);
+            for (int k = 0; k < P.nk; ++k) {
+                load(P.x, k, !P.paired);
+                if (k == 0 && P.before) await(P.before, phase, 406);
+                if (k == 0 && P.before_cluster) cluster_wait_all();
+                if (P.paired && !P.resident) load(P.y, k, true);
+                load(P.z, k, P.paired);
             }
-        else if (issuer())
+        } else if (issuer()) {
 #pragma unroll 1
-            for (int k = 0; k < nk; ++k) {
-                uint32_t bs, bp, bq;
-                const SOp b = take(s, bs, false);
-                if (p_resident) mma(tmem + acc(), part(k), b, acc0 || k > 0);
-                else {
-                    mma(tmem + acc(), take(p, bp, true), b, acc0 || k > 0);
-                    umma_commit_elect(&sh->empty[bp], lane == 0);
+            for (int k = 0; k < P.nk; ++k) {
+                uint32_t bx, by, bz;
+                const bool c = P.acc0 || k > 0;
+                const SOp x = take(P.x, bx, !P.paired);
+                if (P.paired) {
+                    SOp y = P.part;
+                    y.addr += k * P.part_step;
+                    if (!P.resident) y = take(P.y, by, true);
+                    mma(P.col, y, x, c);
+                    if (!P.resident) umma_commit_elect(&sh->empty[by], lane == 0);
                 }
-                mma(tmem + acc() + 64, take(q, bq, true), b, acc0 || k > 0);
-                umma_commit_elect(&sh->empty[bs], lane == 0);
-                umma_commit_elect(&sh->empty[bq], lane == 0);
+                const SOp z = take(P.z, bz, P.paired);
+                mma(P.col + (P.paired ? 64 : 0), P.paired ? z : x, P.paired ? x : z, c);
+                umma_commit_elect(&sh->empty[bx], lane == 0);
+                umma_commit_elect(&sh->empty[bz], lane == 0);
             }
-    }
-    // both operands from the ring; `s` is on the lane side.  `before`: what the copy warp waits for between the first load of s and
-    // the first of p
-    template <typename F> __device__ void streamed(int nk, const Opnd& s, const Opnd& p, uint32_t col, bool acc0, F before) {
-        if (copier())
-#pragma unroll 1
-            for (int k = 0; k < nk; ++k) {
-                load(s, k, true);
-                if (k == 0) before();
-                load(p, k, false);
-            }
-        else if (issuer())
-#pragma unroll 1
-            for (int k = 0; k < nk; ++k) {
-                uint32_t ba, bb;
-                const SOp a = take(s, ba, true), b = take(p, bb, false);
-                mma(tmem + col, a, b, acc0 || k > 0);
-                umma_commit_elect(&sh->empty[ba], lane == 0);
-                umma_commit_elect(&sh->empty[bb], lane == 0);
-            }
+        }
     }
     template <typename F> __device__ void job_out(F f) {  // epilogue warps
         mbar_wait(&sh->acc_full[job % NSET], (job / NSET) & 1, wc, 404);
@@ -310,20 +307,35 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             return Opnd{p, db == 2 ? p + B : nullptr, (uint32_t)db * B, true, !rows_d};
         };
         size_t sbuf = 0;  // S blocks of the chunk at hand
+        using Product = typename Chain<SW ? 1 : 2>::Product;
         // products of a [tokens x ..] operand with T and S of matrix i, hidden units or d on the lanes
-        auto by_h = [&](const Opnd& x, int i) {
+        auto by_h = [&](Product& P, const Opnd& x, int i) {
             const bool f = i < LAST;
-            G.pair(db, x, i < nres,
-                   [&](int k) { return SOp{G.resident + i * unit + k * (f ? kHalf : 2 * kHalf), half, f ? db * kHalf : kHalf, f, false}; },
-                   w_by_h(blk(tl.Tb[i]), f), w_by_h(blk(tl.Sb[i] + sbuf), f), false);
+            P.nk = db;
+            P.x = x;
+            P.paired = true;
+            P.resident = i < nres;
+            P.part = SOp{G.resident + i * unit, half, f ? db * kHalf : kHalf, f, false};
+            P.part_step = f ? kHalf : 2 * kHalf;
+            P.y = w_by_h(blk(tl.Tb[i]), f);
+            P.z = w_by_h(blk(tl.Sb[i] + sbuf), f);
         };
-        auto by_d = [&](const Opnd& x, int i, bool acc) {
+        auto by_d = [&](Product& P, const Opnd& x, int i) {
             const bool f = i < LAST;
-            G.pair(nb, x, i < nres,
-                   [&](int k) { return SOp{G.resident + i * unit + k * (f ? db * kHalf : kHalf), half, f ? kHalf : 2 * kHalf, !f, false}; },
-                   w_by_d(blk(tl.Tb[i]), f), w_by_d(blk(tl.Sb[i] + sbuf), f), acc);
+            P.nk = nb;
+            P.x = x;
+            P.paired = true;
+            P.resident = i < nres;
+            P.part = SOp{G.resident + i * unit, half, f ? kHalf : 2 * kHalf, !f, false};
+            P.part_step = f ? db * kHalf : kHalf;
+            P.y = w_by_d(blk(tl.Tb[i]), f);
+            P.z = w_by_d(blk(tl.Sb[i] + sbuf), f);
         };
-        auto nothing = [] {};
+        auto simple = [](Product& P, int nk, const Opnd& x, const Opnd& z) {
+            P.nk = nk;
+            P.x = x;
+            P.z = z;
+        };
         // What a chunk reads was written long ago and comes from HBM: into L2 half a chunk ahead (a whole chunk ahead would not fit
         // beside the state of 33 sequences)
         auto pf = [&](const void* p, size_t bytes) {
@@ -395,66 +407,62 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             // T in shared memory waits for the blocks written at the end of the chunk before; loads of S only for its scaling there
             if (G.issuer() || n == 0) G.await(&sh.ops, n, 405);
             else G.await(&sh.scaled, n - 1, 410);
+            // Steps of the chunk: phase, block of 64 tokens, product
+            //   0  everything with T, S          2  the chunk's contribution, as far as it waits for no rows      4  T_last += a_k u_k
+            //   1  pub += W_last phb             3  adjoint of u back through W_last                             5  dk += W_first^T zb
+            //   6  T_first += zb k
 #pragma unroll 1
-            for (int tk = 0; tk < tbn; ++tk) {
-                const Opnd kt{sblk(tl.sK) + (size_t)tk * db * kHalf, nullptr, kHalf, false, false};
-#pragma unroll 1
-                for (int i = 0; i < LAST; ++i) {
-                    G.job_begin();
-                    by_h(kt, i);
-                    G.job_end();
+            for (int ph = 0; ph < 7; ++ph) {
+                if (ph == 1 && G.copier()) {
+                    prefetch_late(g);
+                    if (g > 0) prefetch_state(g - 1);
                 }
-                if (G.copier() && tk == 0 && nres < NMAT) G.await(&sh.ops, n, 411);
-                G.job_begin();
-                by_h(Opnd{sblk(tl.sPu) + (size_t)tk * db * B, nullptr, B, true, false}, LAST);
-                G.job_end();
-                G.job_begin();
-                by_d(tok_h(sblk(tl.sAk), tk), LAST, false);
-                G.job_end();
-                G.job_begin();
+                if (ph == 2 && G.issuer()) G.await(&sh.scaled, n, 407);
+                if (ph == 3) {
+                    G.cluster_wait_all();
+                    G.cluster_arrive_all();
+                    if (G.issuer()) G.cluster_wait_all();
+                }
+                const bool jobs = ph < 2 || ph == 3 || ph == 5;
+                const int ntk = jobs ? tbn : 1;
+                const int nstep = ph == 0 ? 2 * LAST + 2 : ph == 2 ? LAST + 2 : ph >= 5 ? LAST : 1;
 #pragma unroll 1
-                for (int i = 0; i < LAST; ++i) by_d(tok_h(sblk(tl.sPz[i]), tk), i, i > 0);
-                G.job_end();
+                for (int e = 0, tk = 0, st = 0; e < ntk * nstep; ++e) {
+                    if (ph == 0 && st == LAST && tk == 0 && nres < NMAT && G.copier()) G.await(&sh.ops, n, 411);
+                    // the first matrices' dk products of phases 0 and 5 share a job
+                    const bool opens = jobs && (ph == 0 ? st <= LAST + 2 : ph == 5 ? st == 0 : true), closes = jobs && (ph == 0 ? st < LAST + 2 || st == 2 * LAST + 1 : st == nstep - 1);
+                    Product P{};
+                    P.col = jobs ? G.tmem + G.acc() : G.tmem + 128 * (ph == 6 ? st : ph == 2 ? min(st, LAST) : LAST);
+                    P.acc0 = jobs ? !opens : true;
+                    if (ph == 0) {
+                        if (st < LAST) by_h(P, Opnd{sblk(tl.sK) + (size_t)tk * db * kHalf, nullptr, kHalf, false, false}, st);
+                        else if (st == LAST) by_h(P, Opnd{sblk(tl.sPu) + (size_t)tk * db * B, nullptr, B, true, false}, LAST);
+                        else if (st == LAST + 1) by_d(P, tok_h(sblk(tl.sAk), tk), LAST);
+                        else by_d(P, tok_h(sblk(tl.sPz[st - LAST - 2]), tk), st - LAST - 2);
+                    } else if (ph == 1) {
+                        simple(P, nb, w_by_d(sblk(tl.sW[LAST]), false), tok_h(blk(tl.bPhb), tk));
+                        P.before = &sh.phb;
+                    } else if (ph == 2) {
+                        if (st < LAST) simple(P, tbn, key_d(sblk(tl.sQ)), h_tok(sblk(tl.sZq[st])));
+                        else if (st == LAST) simple(P, tbn, h_tok(sblk(tl.sAq)), tok_d(sblk(tl.sUq)));
+                        else simple(P, tbn, h_tok(blk(tl.bPhb)), tok_d(sblk(tl.sPu)));
+                    } else if (ph == 3) {
+                        simple(P, db, w_by_h(sblk(tl.sW[LAST]), false), Opnd{blk(tl.bUk) + (size_t)tk * db * B, nullptr, B, true, false});
+                        P.before_cluster = tk == 0;
+                    } else if (ph == 4) {
+                        simple(P, tbn, h_tok(sblk(tl.sAk)), tok_d(blk(tl.bUk)));
+                    } else if (ph == 5) {
+                        simple(P, nb, w_by_d(sblk(tl.sW[st]), true), tok_h(blk(tl.bZk[st]), tk));
+                        P.before = &sh.zb;
+                    } else {
+                        simple(P, tbn, key_d(sblk(tl.sK)), h_tok(blk(tl.bZk[st])));
+                    }
+                    if (opens) G.job_begin();
+                    G.run(P, n);
+                    if (closes) G.job_end();
+                    if (++st == nstep) { st = 0; ++tk; }
+                }
             }
-            if (G.copier()) {
-                prefetch_late(g);
-                if (g > 0) prefetch_state(g - 1);
-            }
-#pragma unroll 1
-            for (int tk = 0; tk < tbn; ++tk) {  // pub += W_last phb
-                G.job_begin();
-                G.streamed(nb, w_by_d(sblk(tl.sW[LAST]), false), tok_h(blk(tl.bPhb), tk), G.acc(), false, [&] { G.await(&sh.phb, n, 406); });
-                G.job_end();
-            }
-            // the chunk's contribution, onto the scaled masters: the queries' part and whatever else there is before the rows
-            if (G.issuer()) G.await(&sh.scaled, n, 407);
-#pragma unroll 1
-            for (int i = 0; i < LAST; ++i) G.streamed(tbn, key_d(sblk(tl.sQ)), h_tok(sblk(tl.sZq[i])), 128 * i, true, nothing);
-            G.streamed(tbn, h_tok(sblk(tl.sAq)), tok_d(sblk(tl.sUq)), 128 * LAST, true, nothing);
-            G.streamed(tbn, h_tok(blk(tl.bPhb)), tok_d(sblk(tl.sPu)), 128 * LAST, true, nothing);
-            G.cluster_wait_all();
-            G.cluster_arrive_all();
-            if (G.issuer()) G.cluster_wait_all();
-#pragma unroll 1
-            for (int tk = 0; tk < tbn; ++tk) {  // adjoint of u back through W_last
-                G.job_begin();
-                G.streamed(db, w_by_h(sblk(tl.sW[LAST]), false), Opnd{blk(tl.bUk) + (size_t)tk * db * B, nullptr, B, true, false}, G.acc(), false, [&] {
-                    if (tk == 0) G.cluster_wait_all();
-                });
-                G.job_end();
-            }
-            G.streamed(tbn, h_tok(sblk(tl.sAk)), tok_d(blk(tl.bUk)), 128 * LAST, true, nothing);
-#pragma unroll 1
-            for (int tk = 0; tk < tbn; ++tk) {  // dk += W_first^T zb
-                G.job_begin();
-#pragma unroll 1
-                for (int i = 0; i < LAST; ++i)
-                    G.streamed(nb, w_by_d(sblk(tl.sW[i]), true), tok_h(blk(tl.bZk[i]), tk), G.acc(), i > 0, [&] { G.await(&sh.zb, n, 408); });
-                G.job_end();
-            }
-            // what waits for zb
-#pragma unroll 1
-            for (int i = 0; i < LAST; ++i) G.streamed(tbn, key_d(sblk(tl.sK)), h_tok(blk(tl.bZk[i])), 128 * i, true, nothing);
             if (G.issuer()) umma_commit_elect(&sh.upd, lane == 0);
             if (G.copier() && g > 0) prefetch_early(g - 1);
         }
