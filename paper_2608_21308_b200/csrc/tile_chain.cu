@@ -507,7 +507,7 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
         asm volatile("" : "+r"(x));
         return x;
     };
-    auto ld_state = [&](int i, const float* p, int col, float (&v)[16]) {
+    auto ld_raw = [&](int i, const float* p, int col, float (&v)[16]) {
         const int nc = col_lim(i) - col;
         if (!p || nc <= 0) {
 #pragma unroll
@@ -521,6 +521,9 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             v[j] = *q;
             if (j + 1 < nc) q += ld;
         }
+    };
+    auto ld_state = [&](int i, const float* p, int col, float (&v)[16]) {
+        ld_raw(i, p, col, v);
         mask(i, col, v);
     };
     auto st_state = [&](int i, float* p, int col, const float (&v)[16]) {
@@ -633,27 +636,36 @@ template <int KIND, bool NORMED> __global__ void __launch_bounds__(kThreads, 1) 
             G.signal(&sh.ops);
         }
 
-        // The carries' adjoints <T, W>, <T, M>, <S, M>; T <- cw T, S <- cm T + cb S, while
-        // the first products run
+        // The carries' adjoints <T, W>, <T, M>, <S, M>; T <- cw T, S <- cm T + cb S, while the first products run.  The next piece's W, M
+        // are under way while this one's S is written (L1, what is left of it, holds 28 KB of loads in flight)
         {
-            float pw = 0.0f, pm = 0.0f, pb = 0.0f;
+            float pw = 0.0f, pm = 0.0f, pb = 0.0f, w[16], m[16];
+            auto ld_wm = [&](int e) {
+                ld_raw(e >> 1, ck + (size_t)(e >> 1) * dh, col_of(e & 1), w);
+                ld_raw(e >> 1, ck + (size_t)(NMAT + (e >> 1)) * dh, col_of(e & 1), m);
+            };
             const float cw = sc.cw, cm = sc.cm, cb = sc.cb;
+            ld_wm(0);
 #pragma unroll 1
             for (int e = 0; e < 2 * NMAT; ++e) {
                 const int i = e >> 1, col = col_of(e & 1);
-                float w[16], m[16], t[16], sv[16];
-                ld_state(i, ck + (size_t)i * dh, col, w);
-                ld_state(i, ck + (size_t)(NMAT + i) * dh, col, m);
-                ld_state(i, ws + lay.S[i], col, sv);
+                float t[16], sv[16];
+                ld_raw(i, ws + lay.S[i], col, sv);
+                mask(i, col, w);
+                mask(i, col, m);
                 acc16(lanes + 128 * i + col, t);
                 mask(i, col, t);  // lanes past the matrix collect whatever the MMAs read past the operands
 #pragma unroll
+                for (int j = 0; j < 16; ++j) { pw += t[j] * w[j]; pm += t[j] * m[j]; }
+                mask(i, col, sv);
+#pragma unroll
                 for (int j = 0; j < 16; ++j) {
-                    pw += t[j] * w[j]; pm += t[j] * m[j]; pb += sv[j] * m[j];
+                    pb += sv[j] * m[j];
                     sv[j] = cm * t[j] + cb * sv[j];
                     t[j] *= cw;
                 }
                 acc_st16(lanes + 128 * i + col, t);
+                if (e + 1 < 2 * NMAT) ld_wm(e + 1);
                 st_state(i, ws + lay.S[i], col, sv);
                 put(false, buf ^ 1, i, col, sv);
             }
