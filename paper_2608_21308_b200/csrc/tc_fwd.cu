@@ -50,7 +50,7 @@ __device__ long long g_tc_prof[16 * 32 * 24];
 
 namespace {
 
-constexpr int D = 128, HC = 128, NC = 4;
+constexpr int D = 128, HC = 128;
 constexpr int NG = 4;                    // column groups per TMEM lane quadrant
 constexpr int NEPI = 128 * NG;           // epilogue threads
 constexpr int NTHREADS = NEPI + 128;     // + one control warpgroup (issuer warp, loader warp, two idle warps)
@@ -124,7 +124,9 @@ __device__ __forceinline__ float gelu_d1_fast(float z) {
 // MULTI: chunks of several 64-token blocks (128, 256, 512 tokens); a compile-time switch, so that the single-block
 // instantiations are exactly the code they were without it
 // WIDE: 32-byte accesses to the state (tc_common.cuh)
-template <bool PAD, bool NORM, bool MULTI, bool WIDE>
+// NC: CTAs per cluster, 4, or 2 where the hidden units fill no more (the launch's rule).  A CTA owns 64 / NC key and query rows, in
+// groups of 16
+template <int NC, bool PAD, bool NORM, bool MULTI, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ,
               const __grid_constant__ CUtensorMap tmV, const TcFwdArgs a) {
@@ -137,6 +139,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t me = cluster_ctarank();
+    constexpr int RPC = 64 / NC, NPASS = RPC / 16;  // rows per CTA; groups of 16
+    constexpr uint32_t NP = NC - 1;                 // peers
     const int seq = blockIdx.x / NC;
     const int Cc = a.C;                     // chunk size
     const int Cr = min(Cc, C);              // tokens per block (<= C = 64, the tile's rows)
@@ -175,11 +179,11 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         mbar_init(&s.bar_w2, NEW);
         mbar_init(&s.bar_ksent, NEW / 2);
         mbar_init(&s.bar_go, 1);
-        mbar_init(&s.bar_partK, 1);  // + 3 x 8 KB of peer partial sums (key rows) per chunk
-        mbar_init(&s.bar_partQ, 1);  // + 3 x 4 KB (query rows, bf16)
-        mbar_init(&s.bar_pu, 2);     // + 12 KB of pu rows from the peers per chunk, one arrival for the own rows
-        mbar_init(&s.bar_credit, 3);
-        mbar_init(&s.bar_rs, 1);     // + 3 x 512 B of peer row sums per chunk (normalisation only)
+        mbar_init(&s.bar_partK, 1);  // + the peers' partial sums (key rows, fp32) per chunk
+        mbar_init(&s.bar_partQ, 1);  // + the same of the query rows, bf16
+        mbar_init(&s.bar_pu, 2);     // + the pu rows from the peers per chunk, one arrival for the own rows
+        mbar_init(&s.bar_credit, NP);
+        mbar_init(&s.bar_rs, 1);     // + 512 B of row sums per peer and chunk (normalisation only)
         fence_mbar_init();
         tma_prefetch_desc(&tmK);
         tma_prefetch_desc(&tmQ);
@@ -191,7 +195,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         tc_chunk_scalars(eta, beta, gamma, &s.sc[0], min(Cr, L), multi ? &s.tails[0] : nullptr);
     }
     if (de < 128)  // the padded half of the token tile is never loaded: zero it once
-        for (int i = tid; i < 16384 / 16; i += NTHREADS) reinterpret_cast<uint4*>(s.X[1])[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = tid; i < 16384 / 16; i += NTHREADS) {
+            reinterpret_cast<uint4*>(s.X[1])[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (i < 8192 / 16) reinterpret_cast<uint4*>(s.Pu[1])[i] = make_uint4(0u, 0u, 0u, 0u);  // and that of pu never sent
+        }
     if (Cr < C)    // short chunks: the key and query rows past the chunk are never loaded either (128-byte rows, 8 pieces each)
         for (int i = tid; i < 32768 / 16; i += NTHREADS)
             if (((i >> 3) & 63) >= Cr) reinterpret_cast<uint4*>(s.X[0])[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -230,7 +237,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 tc_fence_after_sync();
                 PROF(0);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) umma_bf16_elect(tb + T_R0, dk(sb + oX, 16384, k), dk(sb + oW1, 16384, k), id_kk, k > 0, el);
+                for (int k = 0; k < 8; ++k)
+                    if (!PAD || 16 * k < de) umma_bf16_elect(tb + T_R0, dk(sb + oX, 16384, k), dk(sb + oW1, 16384, k), id_kk, k > 0, el);
                 umma_commit_elect(&s.bar_g1, el);
                 PROF(1);
                 // G2: Upart = A W2c^T -> R1.  Needs gelu(Z) in A, the refreshed bf16 W2 and R1 read out (M2 aggregate).
@@ -252,7 +260,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 tc_fence_after_sync();
                 PROF(4);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) umma_bf16_elect(tb + T_R1, dk(sb + oPu, 8192, k), dmn(sb + oW2, 16384, k), id_kmn, k > 0, el);
+                for (int k = 0; k < 8; ++k)
+                    if (!PAD || 16 * k < de) umma_bf16_elect(tb + T_R1, dk(sb + oPu, 8192, k), dmn(sb + oW2, 16384, k), id_kmn, k > 0, el);
                 umma_commit_elect(&s.bar_g3, el);
                 PROF(5);
                 // W2 aggregation on top of the master
@@ -304,20 +313,22 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                     mbar_wait(&s.bar_w2, ph, wc, 100 + 20);
                 }
                 if (lane == 0) {
-                    mbar_expect_tx(&s.bar_partK, 3 * 8192);  // this chunk's incoming partial sums and pu rows
-                    mbar_expect_tx(&s.bar_partQ, 3 * 4096);
-                    mbar_expect_tx(&s.bar_pu, 12288);
-                    if (NORM) mbar_expect_tx(&s.bar_rs, 3 * 512);
+                    mbar_expect_tx(&s.bar_partK, NP * RPC * 4 * (uint32_t)de);  // this chunk's incoming partial sums and pu rows
+                    mbar_expect_tx(&s.bar_partQ, NP * RPC * 2 * (uint32_t)de);
+                    mbar_expect_tx(&s.bar_pu, NP * RPC * 2 * (uint32_t)de);
+                    if (NORM) mbar_expect_tx(&s.bar_rs, NP * 512);
                     if (r + 1 < nchunks) {
                         // the next chunk's tokens: into L2 now, so that the loads issued at the end of this chunk are short
                         const int y = seq * Ls + tok0 + Cr;
                         tma_prefetch_l2_2d(&tmK, 0, y);
                         tma_prefetch_l2_2d(&tmQ, 0, y);
-                        tma_prefetch_l2_2d(&tmV, 0, y + 16 * (int)me);
+#pragma unroll
+                        for (int p = 0; p < NPASS; ++p) tma_prefetch_l2_2d(&tmV, 0, y + RPC * (int)me + 16 * p);
                         if (de == 128) {
                             tma_prefetch_l2_2d(&tmK, 64, y);
                             tma_prefetch_l2_2d(&tmQ, 64, y);
-                            tma_prefetch_l2_2d(&tmV, 64, y + 16 * (int)me);
+#pragma unroll
+                            for (int p = 0; p < NPASS; ++p) tma_prefetch_l2_2d(&tmV, 64, y + RPC * (int)me + 16 * p);
                         }
                     }
                 }
@@ -335,13 +346,16 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&s.bar_sc);
                 }
-                // the 16 value rows this CTA needs for its key rows: into the gelu tile's first slab, dead once G2 is done
+                // the value rows this CTA needs for its key rows: into the gelu tile's first slab, dead once G2 is done
                 mbar_wait(&s.bar_g2, ph, wc, 100 + 21);
                 if (lane == 0) {
-                    mbar_expect_tx(&s.bar_v, de == 128 ? 4096u : 2048u);
-                    const int y = seq * Ls + tok0 + 16 * (int)me;
-                    tma_load_2d(s.A[0], &tmV, 0, y, &s.bar_v);
-                    if (de == 128) tma_load_2d(s.A[0] + 2048, &tmV, 64, y, &s.bar_v);
+                    mbar_expect_tx(&s.bar_v, RPC * 2 * (uint32_t)de);
+                    const int y = seq * Ls + tok0 + RPC * (int)me;
+#pragma unroll
+                    for (int p = 0; p < NPASS; ++p) {
+                        tma_load_2d(s.A[0] + 2048 * p, &tmV, 0, y + 16 * p, &s.bar_v);
+                        if (de == 128) tma_load_2d(s.A[0] + 128 * RPC + 2048 * p, &tmV, 64, y + 16 * p, &s.bar_v);
+                    }
                 }
                 if (r + 1 < nchunks) {
                     // the W1 / M1 aggregations were the last readers of the key tile: the next chunk's tokens may land in X
@@ -519,18 +533,22 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             }
             PROF(3);
 
-            // Row ownership: CTA c normalises key tokens 16c..16c+15 and query tokens 16c..16c+15, so every CTA carries
+            // Row ownership: CTA c normalises key tokens and query tokens RPC c .. RPC c + RPC - 1, so every CTA carries
             // the same mix of work.  TMEM lane 32q+l holds key token 32q+l (q < 2) or query token 32(q-2)+l.
             // Partial sums of the key rows travel as fp32 (they feed the state), those of the query rows as bf16 (they
             // only feed o, which is rounded to bf16 anyway).  The sender's own rows stay fp32 in the dead gelu tile.
-            const uint32_t owner = 2u * ((uint32_t)q & 1u) + ((uint32_t)lane >> 4);
-            const uint32_t srow = (uint32_t)lane & 15u;                 // row inside the owner's slot
-            const uint32_t slot = (me - owner - 1u) & 3u;               // where the owner keeps what comes from this CTA
+            // Staging holds groups of 16 rows: of the three peers one each, or two of the one peer.
+            const uint32_t owner = NC == 4 ? 2u * ((uint32_t)q & 1u) + ((uint32_t)lane >> 4) : (uint32_t)q & 1u;
+            const uint32_t srow = (uint32_t)lane & 15u;                                       // row inside the group
+            const uint32_t sgrp = NC == 4 ? 0u : (uint32_t)lane >> 4;                         // own group
+            const uint32_t slot = NC == 4 ? (me - owner - 1u) & 3u : sgrp;                    // where the owner keeps what comes from this CTA
+            // own query rows of a group: behind the own key rows, or (two groups) behind the value rows and the peer's query rows
+            auto own_q = [&](int grp) -> uint8_t* { return NC == 4 ? s.A[1] + 8192 : grp ? s.Stage2 + 8192 : s.A[0] + 8192; };
             auto send_k = [&]() {
                 const bool mine = owner == me;
                 uint32_t dst_base, dst_bar = 0;
                 if (mine) {
-                    dst_base = smem_u32(s.A[1]);  // the gelu tile is dead once G2 has completed
+                    dst_base = smem_u32(s.A[1]) + 8192u * sgrp;  // the gelu tile is dead once G2 has completed
                 } else {
                     const uint8_t* p = (slot == 0) ? s.PzW[0] : (slot == 1) ? s.PzW[1] : s.PzM[0];
                     dst_base = map_to_cta(smem_u32(p), owner);
@@ -538,6 +556,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 }
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
+                    if (PAD && c0 + 16 * b >= de) continue;
                     uint32_t u[16];
                     tmem_ld16(lane_addr + T_R1 + c0 + 16 * b, u);
                     tmem_wait_ld();
@@ -555,11 +574,12 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             };
             auto send_q = [&]() {
                 const bool mine = owner == me;
-                const uint32_t own_base = smem_u32(s.A[1]) + 8192u;
+                const uint32_t own_base = smem_u32(own_q((int)sgrp));
                 const uint32_t dst_base = map_to_cta(smem_u32(s.Stage2) + slot * 4096u, owner);
                 const uint32_t dst_bar = map_to_cta(smem_u32(&s.bar_partQ), owner);
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
+                    if (PAD && c0 + 16 * b >= de) continue;
                     uint32_t u[16];
                     tmem_ld16(lane_addr + T_R1 + c0 + 16 * b, u);
                     tmem_wait_ld();
@@ -582,14 +602,14 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 if (lane == 0) mbar_arrive(&s.bar_r1);
             };
 
-            // Layer norm on the 16 key rows (warps of quadrants 0/1) or the 16 query rows (quadrants 2/3) this CTA owns:
+            // Layer norm on 16 of the key rows (warps of quadrants 0/1) or of the query rows (quadrants 2/3) this CTA owns:
             // 16 threads per row, 8 columns each.
-            auto layer_norm = [&](const bool key_rows) {
+            auto layer_norm = [&](const bool key_rows, const int pass) {
                 constexpr int TPR = NEPI / 32, CPT = 128 / TPR;  // threads per row, columns per thread
                 static_assert(TPR == 16 && CPT == 8, "row mapping below assumes two rows per warp, one 16-byte piece per thread");
-                const int lrow = 2 * ((q & 1) + 2 * g) + (lane >> 4);   // row of the slot (0..15)
+                const int lrow = 2 * ((q & 1) + 2 * g) + (lane >> 4);   // row of the group (0..15)
                 const int cg = lane & 15;
-                const int t = 16 * (int)me + lrow;           // token inside the chunk
+                const int t = RPC * (int)me + 16 * pass + lrow;  // token inside the chunk
                 const int xrow = key_rows ? t : 64 + t;      // its row in the X tile
                 const int col0 = CPT * cg;
                 const size_t off = (size_t)(tok0 + t) * de + col0;
@@ -598,7 +618,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 const uint4 xraw = *reinterpret_cast<const uint4*>(s.X[col0 >> 6] + xrow * 128 + ((c ^ (xrow & 7)) << 4));
                 float u[CPT];
                 {   // own rows, fp32
-                    const uint8_t* p = s.A[1] + (key_rows ? 0 : 8192);
+                    const uint8_t* p = key_rows ? s.A[1] + 8192 * pass : own_q(pass);
                     const float4 x0 = *reinterpret_cast<const float4*>(p + stage_offset((uint32_t)(2 * cg), (uint32_t)lrow));
                     const float4 x1 = *reinterpret_cast<const float4*>(p + stage_offset((uint32_t)(2 * cg + 1), (uint32_t)lrow));
                     u[0] = x0.x; u[1] = x0.y; u[2] = x0.z; u[3] = x0.w; u[4] = x1.x; u[5] = x1.y; u[6] = x1.z; u[7] = x1.w;
@@ -606,10 +626,11 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 mbar_wait<true>(key_rows ? &s.bar_partK : &s.bar_partQ, ph, wc, 100 + 35);
                 PROF(15);
                 // the peers' pieces, added in a fixed order (slot 0, 1, 2 = the CTAs me+1, me+2, me+3): the sum does not
-                // depend on arrival order, and each CTA adds its four pieces in its own fixed order
+                // depend on arrival order, and each CTA adds its NC pieces in its own fixed order
                 if (key_rows) {
 #pragma unroll
-                    for (int sl = 0; sl < 3; ++sl) {
+                    for (int i = 0; i < (int)NP; ++i) {
+                        const int sl = NC == 4 ? i : pass;
                         const uint8_t* p = (sl == 0) ? s.PzW[0] : (sl == 1) ? s.PzW[1] : s.PzM[0];
                         const float4 x0 = *reinterpret_cast<const float4*>(p + stage_offset((uint32_t)(2 * cg), (uint32_t)lrow));
                         const float4 x1 = *reinterpret_cast<const float4*>(p + stage_offset((uint32_t)(2 * cg + 1), (uint32_t)lrow));
@@ -617,14 +638,15 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                     }
                 } else {
 #pragma unroll
-                    for (int sl = 0; sl < 3; ++sl) {
+                    for (int i = 0; i < (int)NP; ++i) {
+                        const int sl = NC == 4 ? i : pass;
                         const uint4 x = *reinterpret_cast<const uint4*>(s.Stage2 + sl * 4096 + stage_offset_q((uint32_t)cg, (uint32_t)lrow));
                         const __nv_bfloat162* x2 = reinterpret_cast<const __nv_bfloat162*>(&x);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float2 f = __bfloat1622float2(x2[i]);
-                            u[2 * i] += f.x;
-                            u[2 * i + 1] += f.y;
+                        for (int j = 0; j < 4; ++j) {
+                            const float2 f = __bfloat1622float2(x2[j]);
+                            u[2 * j] += f.x;
+                            u[2 * j + 1] += f.y;
                         }
                     }
                 }
@@ -642,7 +664,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                     //   mean(e y) = rstd (s4 - mu s3)/d + var rstd^2
                     mbar_wait(&s.bar_v, ph, wc, 100 + 36);
                     PROF(16);
-                    const uint4 vraw = real ? *reinterpret_cast<const uint4*>(s.A[0] + (col0 >> 6) * 2048 + lrow * 128 + ((c ^ (lrow & 7)) << 4))
+                    const uint4 vraw = real ? *reinterpret_cast<const uint4*>(s.A[0] + (col0 >> 6) * (128 * RPC) + 2048 * pass + lrow * 128 + ((c ^ (lrow & 7)) << 4))
                                             : make_uint4(0u, 0u, 0u, 0u);
                     const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&xraw);
                     const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&vraw);
@@ -680,17 +702,18 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
 #pragma unroll
                     for (int j = 0; j < CPT; j += 2)
                         pk[j / 2] = real ? pack_bf16(rstd * (e[j] - me_ - u[j] * mey), rstd * (e[j + 1] - me_ - u[j + 1] * mey)) : 0u;  // 0 in the padding
-                    // The bf16 pu rows go into this CTA's own pu tile; one bulk copy per peer and slab (2 KB: the 16 rows of a
+                    // The bf16 pu rows go into this CTA's own pu tile; one bulk copy per peer and slab (the CTA's rows of a
                     // slab are contiguous) then carries them to the peers' tiles.  Bulk copies write through the async proxy,
                     // the one the MMAs read through, so the receivers need no proxy fence.
                     *reinterpret_cast<uint4*>(s.Pu[col0 >> 6] + t * 128 + ((c ^ (t & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    if (pass + 1 < NPASS) return;
                     fence_proxy_async_smem();
                     named_sync(BAR_KOWN, NEPI / 2);
                     if (warp == 0) {
-                        if (lane < 6) {
-                            const uint32_t dst = (me + 1u + (uint32_t)(lane >> 1)) & 3u;
-                            const uint32_t src = smem_u32(s.Pu[lane & 1]) + 2048u * me;
-                            bulk_copy_to_cta(map_to_cta(src, dst), src, 2048u, map_to_cta(smem_u32(&s.bar_pu), dst));
+                        if (lane < 2 * (int)NP && (lane & 1) * 64 < de) {
+                            const uint32_t dst = (me + 1u + (uint32_t)(lane >> 1)) & (NC - 1u);
+                            const uint32_t src = smem_u32(s.Pu[lane & 1]) + 128u * RPC * me;
+                            bulk_copy_to_cta(map_to_cta(src, dst), src, 128u * RPC, map_to_cta(smem_u32(&s.bar_pu), dst));
                         }
                         if (lane == 0) mbar_arrive(&s.bar_pu);  // the own rows are in place
                     }
@@ -698,7 +721,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                     // query rows (not on the critical path): two-pass statistics, o = q + y
                     float sum = 0.0f;
 #pragma unroll
-                    for (int j = 0; j < CPT; ++j) sum += u[j];
+                    for (int j = 0; j < CPT; ++j) {
+                        if (!real) u[j] = 0.0f;  // columns never sent
+                        sum += u[j];
+                    }
                     const float mu = row_sum(sum) * inv_d;
                     float sq = 0.0f;
 #pragma unroll
@@ -735,7 +761,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 PROF(14);
                 named_sync(BAR_KOWN, NEPI / 2);  // this CTA's own key rows are staged
                 PROF(5);
-                layer_norm(true);
+#pragma unroll
+                for (int p = 0; p < NPASS; ++p) layer_norm(true, p);
                 PROF(6);
                 PROF(17);
                 // ---------------- G3 epilogue: Pz = Pa * gelu'(Zk), scaled by kW and kM into two bf16 tiles
@@ -770,7 +797,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 PROF(14);
                 named_sync(BAR_QOWN, NEPI / 2);  // own query rows staged
                 PROF(5);
-                layer_norm(false);
+#pragma unroll
+                for (int p = 0; p < NPASS; ++p) layer_norm(false, p);
                 PROF(6);
             }
 
@@ -1134,18 +1162,22 @@ int tc_fwd_launch(const TcFwdArgs& a_in, void* stream) {
         return (int)cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(a.N * NC));
+    // Two CTAs per cluster where they hold all hidden units (h <= 256), if the call then takes fewer waves: 74 clusters of 2 fit the
+    // GPU and 33 of 4 (half of whose CTAs had only padding).  With as many waves the four CTAs are kept: each normalises half as many
+    // rows per chunk.  96 sequences of 2048 tokens, d = 64, h = 256: 745 -> 510 us
+    const int nc = a.h <= 2 * HC && (a.N + 73) / 74 < (a.N + 32) / 33 ? 2 : 4;
+    cfg.gridDim = dim3((unsigned)(a.N * nc));
     cfg.blockDim = dim3(NTHREADS);
     cfg.dynamicSmemBytes = tc_fwd_smem_bytes();
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = NC;
+    at[0].val.clusterDim.x = (unsigned)nc;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const bool native = a.d == D && a.h == NC * HC;
+    const bool native = a.d == D && a.h == 4 * HC;
     const bool norm = a.norm1 && a.norm2;
     if (norm && ((a.ckpt && !a.rown) || a.ckpt_every > 1)) return (int)cudaErrorInvalidValue;
     const bool wide = wide_rows({a.W1_init, a.W2_init, a.M1_init, a.M2_init, a.W1_final, a.W2_final, a.M1_final, a.M2_final, a.ckpt},
@@ -1159,15 +1191,18 @@ int tc_fwd_launch(const TcFwdArgs& a_in, void* stream) {
         }
         return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, kernel, tmK, tmQ, tmV, a) : e;
     };
-    static bool done[12][64];
-#define E2TTT_TC_FWD(i, PAD, NORM, MULTI)                                                     \
-    e = wide ? go(tc_fwd_kernel<PAD, NORM, MULTI, true>, done[i]) : go(tc_fwd_kernel<PAD, NORM, MULTI, false>, done[6 + i])
-    if (norm && native) E2TTT_TC_FWD(0, false, true, false);
-    else if (norm) E2TTT_TC_FWD(1, true, true, false);
-    else if (a.C > 64 && native) E2TTT_TC_FWD(2, false, false, true);
-    else if (a.C > 64) E2TTT_TC_FWD(3, true, false, true);
-    else if (native) E2TTT_TC_FWD(4, false, false, false);
-    else E2TTT_TC_FWD(5, true, false, false);
+    static bool done[18][64];
+#define E2TTT_TC_FWD(i, NC, PAD, NORM, MULTI)                                                 \
+    e = wide ? go(tc_fwd_kernel<NC, PAD, NORM, MULTI, true>, done[i]) : go(tc_fwd_kernel<NC, PAD, NORM, MULTI, false>, done[9 + i])
+    if (norm && native) E2TTT_TC_FWD(0, 4, false, true, false);
+    else if (norm && nc == 2) E2TTT_TC_FWD(6, 2, true, true, false);
+    else if (norm) E2TTT_TC_FWD(1, 4, true, true, false);
+    else if (a.C > 64 && native) E2TTT_TC_FWD(2, 4, false, false, true);
+    else if (a.C > 64 && nc == 2) E2TTT_TC_FWD(7, 2, true, false, true);
+    else if (a.C > 64) E2TTT_TC_FWD(3, 4, true, false, true);
+    else if (native) E2TTT_TC_FWD(4, 4, false, false, false);
+    else if (nc == 2) E2TTT_TC_FWD(8, 2, true, false, false);
+    else E2TTT_TC_FWD(5, 4, true, false, false);
 #undef E2TTT_TC_FWD
     if (e != cudaSuccess) return (int)e;
     return (int)cudaGetLastError();
