@@ -1,0 +1,112 @@
+"""Every branch that the dispatch on sizes and alignment can take, at the sizes where its kernel can go wrong: block-tiled forward and
+reverse pass, two-CTA clusters of the fused MLP forward, narrow state accesses, streamed decode."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_21308_b200 import binding as E
+from paper_2608_21308_b200 import inputs
+from tests import util
+from tests.test_gpu_apply import gpu_apply, oracle_apply
+from tests.test_gpu_normed import gpu_backward_normed, gpu_forward_normed, oracle_bwd, oracle_fwd, targets
+from tests.test_gpu_parity import TOL_BF16, check_backward, check_forward
+
+pytestmark = pytest.mark.gpu
+MLP, SWIGLU = inputs.KIND_MLP, inputs.KIND_SWIGLU
+
+
+def _inputs(N, L, d, h, C, kind, **kw):
+    r = inputs.paper_regime(inputs.Recipe(B=N, H=1, L=L, d=d, h=h, C=C, kind=kind, io="bf16", seed=31, m_std=0.002))
+    return inputs.generate(r, **kw), dict(d=d, h=h, C=C, kind=kind, io="bf16")
+
+
+@pytest.mark.parametrize("normed", [False, True], ids=["plain", "normed"])
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("d,h,C,L", [
+    (8, 64, 24, 30),      # one block in every direction
+    (64, 72, 64, 65),     # a hidden block of 8 units; a chunk of one token
+    (72, 640, 65, 66),    # five CTAs in the reverse chain; two token blocks, the second of one token
+    (128, 1024, 16, 20),  # the most CTAs the chain takes
+    (128, 1088, 16, 20),  # more hidden units than it takes
+    (128, 136, 512, 520), # the longest chunks
+])
+def test_block_tiled_edges(d, h, C, L, kind, normed):
+    x, shape = _inputs(1, L, d, h, C, kind, with_d_o=True, with_dstate=True)
+    if normed:
+        tgt = targets(x)
+        got = gpu_forward_normed(x, tgt, impl=E.E2TTT_IMPL_TILED, **shape)
+        check_forward(got, oracle_fwd(x, tgt, C, kind), TOL_BF16, "block-tiled normed forward")
+        got = gpu_backward_normed(x, tgt, impl=E.E2TTT_IMPL_TILED, via_saved_states=True, **shape)
+        check_backward(got, oracle_bwd(x, tgt, C, kind), 2 * TOL_BF16, "block-tiled normed backward")
+    else:
+        got, hd = util.gpu_forward(x, impl=E.E2TTT_IMPL_TILED, **shape)
+        assert E.e2ttt_device_status(hd["ws"]) == 0
+        check_forward(got, util.oracle_forward(x, C, kind), TOL_BF16, "block-tiled forward")
+        check_backward(util.gpu_backward(x, impl=E.E2TTT_IMPL_TILED, **shape), util.oracle_backward(x, C, kind), 2 * TOL_BF16, "block-tiled backward")
+
+
+@pytest.mark.parametrize("N,ckpt", [(1, 0), (1, 5), (40, 0), (40, 5)])
+def test_block_tiled_reverse_over_groups_of_chunks(N, ckpt):
+    """23 chunks: groups of 9 of them per launch (of 3 or 4 with 40 sequences), the last shorter; segments of an odd number of chunks."""
+    x, shape = _inputs(N, 23 * 16 - 3, 64, 192, 16, MLP, with_d_o=True, with_dstate=True)
+    got = util.gpu_backward(x, impl=E.E2TTT_IMPL_TILED, via_saved_states=ckpt > 0, ckpt_every=ckpt, **shape)
+    ref = util.gpu_backward(x, impl=E.E2TTT_IMPL_SIMT, **shape)
+    check_backward(got, ref, TOL_BF16, f"groups N={N} ckpt={ckpt}")
+
+
+@pytest.mark.parametrize("normed", [False, True], ids=["plain", "normed"])
+@pytest.mark.parametrize("N,d,h,C,L", [(34, 64, 256, 64, 130), (74, 128, 256, 16, 50), (75, 64, 128, 32, 64), (34, 128, 128, 128, 300)])
+def test_two_cta_clusters_of_the_fused_forward(N, d, h, C, L, normed):
+    """Copies of two sequences: all copies equal, the first two against the oracle."""
+    if normed and C > 64:
+        pytest.skip("normalised chunks of several blocks run on the block-tiled kernels")
+    x, shape = _inputs(2, L, d, h, C, MLP)
+    rep = lambda a: np.concatenate([a] * ((N + 1) // 2))[:N]
+    xs = {n: [rep(w) for w in a] if isinstance(a, list) else rep(a) for n, a in x.items()}
+    if normed:
+        got = gpu_forward_normed(xs, targets(xs), impl=E.E2TTT_IMPL_TCGEN05, **shape)
+        ref = oracle_fwd(x, targets(x), C, MLP)
+    else:
+        got, hd = util.gpu_forward(xs, impl=E.E2TTT_IMPL_TCGEN05, **shape)
+        assert E.e2ttt_device_status(hd["ws"]) == 0
+        ref = util.oracle_forward(x, C, MLP)
+    cut = lambda a: [w[:2] for w in a] if isinstance(a, list) else a[:2]
+    for a in [got["o"]] + got["W"] + got["M"]:
+        assert all(np.array_equal(a[n], a[n % 2]) for n in range(N))
+    check_forward({n: cut(a) for n, a in got.items()}, ref, TOL_BF16, "two-CTA clusters")
+
+
+@pytest.mark.parametrize("kind,h", [(MLP, 512), (SWIGLU, 384)])
+def test_states_off_the_32_byte_grid_give_the_same_result(kind, h):
+    x, shape = _inputs(2, 100, 128, h, 64, kind)
+    ref, _ = util.gpu_forward(x, impl=E.E2TTT_IMPL_TCGEN05, **shape)
+    p = E.make_params(2, 1, 100, 128, h, 64, kind, E.E2TTT_BF16, 1e-5, E.E2TTT_IMPL_TCGEN05)
+    dev = lambda a, t=torch.float32: torch.tensor(a, dtype=torch.float32).to(t).cuda()
+    q, k, v = (dev(x[n], torch.bfloat16).view(2, 1, 100, 128) for n in ("q", "k", "v"))
+    gates = [dev(x[n]).view(2, 1, 100) for n in ("eta", "beta", "gamma")]
+
+    def off16(a):  # a copy 16 bytes past a 32-byte boundary
+        t = torch.empty(a.size + 4, dtype=torch.float32, device="cuda")[4:].view((2, 1) + a.shape[1:])
+        t.copy_(dev(a).view(t.shape))
+        return t
+
+    W, M = [off16(w) for w in x["W"]], [off16(m) for m in x["M"]]
+    Wf, Mf = [off16(w) for w in x["W"]], [off16(m) for m in x["M"]]
+    o = torch.empty_like(q)
+    ws = torch.empty(E.e2ttt_workspace_bytes(p, 0), dtype=torch.uint8, device="cuda")
+    E.e2ttt_chunk_fwd(p, q, k, v, *gates, W, M, o, Wf, Mf, ws, 0)
+    torch.cuda.synchronize()
+    assert np.array_equal(o.float().cpu().numpy()[:, 0], ref["o"])
+    for a, b in zip(Wf + Mf, ref["W"] + ref["M"]):
+        assert np.array_equal(a.cpu().numpy()[:, 0], b)
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("io", ["f32", "bf16"])
+@pytest.mark.parametrize("d,h,N", [(4, 4, 1), (8, 260, 3), (132, 256, 2), (256, 4096, 1), (256, 4100, 1), (128, 510, 2), (260, 64, 1), (64, 256, 300)])
+def test_one_token_decode(kind, io, d, h, N):
+    """Rows of less than a piece and of several, the widest that is streamed, and neighbours that are not."""
+    r = inputs.Recipe(B=N, H=1, L=1, d=d, h=h, C=1, kind=kind, io=io, seed=22, w_std=0.05)
+    x = inputs.generate(r)
+    got = gpu_apply(x["q"], x["W"], d=d, h=h, kind=kind, io=io)
+    assert util.rel_err(got, oracle_apply(x["q"], x["W"], kind)) <= (1e-5 if io == "f32" else TOL_BF16)
