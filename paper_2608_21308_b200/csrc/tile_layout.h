@@ -17,6 +17,8 @@ constexpr int kTileShares = 4 * kTileMaxCl;
 struct TileLayout {
     int db, hb, tb;  // 64-blocks along d, h and the tokens of a chunk
     int G;           // chunks the reverse pass prepares at a time
+    int sets;        // sets of G slots: 2 where the chain's launch takes the next group's independent part along
+    int spare;       // CTAs it has for that
     int cl;          // most CTAs per sequence
     // reverse pass, kept from launch to launch: operand blocks of the adjoints T, S of the chunk-end state
     size_t Tb[3], Sb[3];
@@ -31,26 +33,29 @@ struct TileLayout {
 
 // CTAs per sequence for N sequences: as many as keep every cluster resident at one CTA per SM (the driver's occupancy calculator:
 // GPU processing clusters do not divide evenly into larger clusters), at most one per 64 hidden units
+inline int tile_clusters_fit(int cl) {  // clusters of 1..8 CTAs that fit the GPU together
+    static const int fit[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+    return fit[cl];
+}
 inline int tile_cluster_size(int N, int hb) {
-    static const int fit[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};  // clusters of 1..8 CTAs that fit the GPU together
     int cl = 1;
     for (int c = 2; c <= kTileMaxCl; ++c)
-        if (N <= fit[c]) cl = c;
+        if (N <= tile_clusters_fit(c)) cl = c;
     if (cl > hb) cl = hb;
     const int sb = (hb + cl - 1) / cl;  // hidden blocks per CTA; drop CTAs that would have none
     return (hb + sb - 1) / sb;
 }
 
-// Chunks prepared at a time: N * tb * G independent work items should fill whole waves of 148 CTAs, and each group costs a launch of
-// every kernel.  At most 9 items per sequence, and 512 MB of slots for the whole call (a slot costs about 30 bytes per token and hidden
+// Chunks prepared at a time: N * tb * G independent work items should fill whole waves of `ctas` CTAs, and each group costs a launch of
+// every kernel.  At most 9 items per sequence, and 512 MB per set of slots for the whole call (a slot costs about 30 bytes per token and hidden
 // unit): the workspace of a checkpointed call is to stay a small part of what all chunks' states would take.
-inline int tile_group_chunks(int N, int tb, size_t slot_bytes) {
+inline int tile_group_chunks(int N, int tb, int ctas, size_t slot_bytes) {
     int best = 1;
     double best_eff = 0.0;
     for (int g = 1; g <= 9; ++g) {
         if (g > 1 && ((size_t)g * tb > 9 || slot_bytes * g * N > ((size_t)512 << 20))) break;
-        const double items = (double)N * tb * g, waves = (double)(long long)((items + 147) / 148);
-        const double eff = items / (148.0 * waves);
+        const double items = (double)N * tb * g, waves = (double)(long long)((items + ctas - 1) / ctas);
+        const double eff = items / (ctas * waves);
         if (eff > best_eff - 0.01) {
             best = g;
             if (eff > best_eff) best_eff = eff;
@@ -109,8 +114,12 @@ inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, i
     t.skwb = take((size_t)2 * kTileShares * tb * 64);
     t.sdots = take((size_t)4 * kTileMaxCl);
     t.slot_stride = o;
-    t.G = tile_group_chunks(N, t.tb, o * sizeof(float));
-    o = t.slot + t.slot_stride * (size_t)t.G;
+    // The chain takes a CTA per 128 hidden units and sequence.  A chunk costs it about as much time as an item of the independent part:
+    // with as many CTAs to spare as sequences that part is done when the chain is (chunks of one block; longer ones alike)
+    t.spare = chain && ctas <= kTileMaxCl ? (tile_clusters_fit(ctas) - N) * ctas : 0;
+    t.sets = t.spare >= N && o * sizeof(float) * N <= ((size_t)512 << 20) ? 2 : 1;
+    t.G = tile_group_chunks(N, t.tb, t.sets == 2 ? t.spare : 148, o * sizeof(float));
+    o = t.slot + t.slot_stride * (size_t)(t.sets * t.G);
     return o > end_fwd ? o : end_fwd;
 }
 
