@@ -38,7 +38,7 @@ struct ChainShared {
     uint64_t ops, phb, scaled, zb, upd;
     uint32_t tmem;
     int dead;
-    float dots[16][4];
+    float dots[2][16][4];  // by the parity of the launch's chunk: a warp may be a chunk's scaling ahead of the one that adds them up
     float kb[16][32];  // per epilogue warp: K^W then K^M of its 16 tokens of the current block of 64; normalisation: scratch
 };
 constexpr size_t kChainSmem = kResident + kRingBytes + sizeof(ChainShared);
@@ -680,7 +680,7 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
             }
             tmem_wait_st();
             pw = warp_sum(pw); pm = warp_sum(pm); pb = warp_sum(pb);
-            if (lane == 0) { sh.dots[warp][0] = pw; sh.dots[warp][1] = pm; sh.dots[warp][2] = pb; }
+            if (lane == 0) { sh.dots[n & 1][warp][0] = pw; sh.dots[n & 1][warp][1] = pm; sh.dots[n & 1][warp][2] = pb; }
             G.signal(&sh.scaled);
         }
 
@@ -901,7 +901,7 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
         G.await(&sh.upd, n, 409);
         if (threadIdx.x < 3) {  // (the issuer waited for every warp's share before the MMAs this wait is for)
             float x = 0.0f;
-            for (int w = 0; w < 16; ++w) x += sh.dots[w][threadIdx.x];
+            for (int w = 0; w < 16; ++w) x += sh.dots[n & 1][w][threadIdx.x];
             sl[tl.sdots + rank * 4 + threadIdx.x] = x;
         }
         if (!NORMED) {
