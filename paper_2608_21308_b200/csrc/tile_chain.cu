@@ -413,9 +413,9 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
                 G.cluster_wait_all();
             }
             G.cluster_arrive_all();  // the first of the chunk's two barriers: nothing of these warps' is waited for
-            // T in shared memory waits for the blocks written at the end of the chunk before; loads of S only for its scaling there
+            // T in shared memory waits for the blocks written at the end of the chunk before; loads of S only for its scaling there,
+            // which the copy warp waits for inside that chunk
             if (G.issuer() || n == 0) G.await(&sh.ops, n, 405);
-            else G.await(&sh.scaled, n - 1, 410);
             // Steps of the chunk: phase, block of 64 tokens, product
             //   0  everything with T, S          2  the chunk's contribution, as far as it waits for no rows      4  T_last += a_k u_k
             //   1  pub += W_last phb             3  adjoint of u back through W_last                             5  dk += W_first^T zb
@@ -428,6 +428,9 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
                 }
                 if (ph == 2 && G.issuer()) G.await(&sh.scaled, n, 407);
                 if (ph == 3) {
+                    // Taken before the loads that the chunk's end waits for: later, the epilogues could be through with the next chunk's
+                    // scaling, and a wait for this one's parity would be a wait for the one after
+                    if (G.copier()) G.await(&sh.scaled, n, 410);
                     G.cluster_wait_all();
                     G.cluster_arrive_all();
                     if (G.issuer()) G.cluster_wait_all();

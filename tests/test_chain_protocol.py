@@ -6,14 +6,16 @@ the barrier's current one - and again once the barrier has completed one phase m
 import pathlib
 import re
 
+import pytest
+
 SOURCE = pathlib.Path(__file__).resolve().parent.parent / "paper_2608_21308_b200" / "csrc" / "tile_chain.cu"
 CHUNKS = 4
 
 # The statements the programs below stand for, in the order of the source
 STATEMENTS = [
     "if (G.issuer() || n == 0) G.await(&sh.ops, n, 405);",
-    "else G.await(&sh.scaled, n - 1, 410);",
     "if (ph == 2 && G.issuer()) G.await(&sh.scaled, n, 407);",
+    "if (G.copier()) G.await(&sh.scaled, n, 410);",
     "if (ph == 0 && st == LAST && tk == 0 && nres < NMAT && G.copier()) G.await(&sh.ops, n, 411);",
     "P.before = &sh.phb;",
     "P.before = &sh.zb;",
@@ -35,7 +37,7 @@ def dots_slot(n):
 
 
 def scaled_wait(n, at):  # chunks whose `scaled` the copy warp waits for at this point of chunk n
-    return [n - 1] if at == "head" and n > 0 else []
+    return [n] if at == "rows" else []
 
 
 def programs(resident):
@@ -114,3 +116,8 @@ def test_the_model_is_of_this_source():
 
 def test_dot_products_of_two_chunks_do_not_meet():
     assert not [f for f in explore(programs(True)) if f.startswith("sum")]
+
+
+@pytest.mark.parametrize("resident", [True, False])
+def test_no_wait_is_overtaken(resident):
+    assert not explore(programs(resident))
