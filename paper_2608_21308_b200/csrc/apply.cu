@@ -133,6 +133,8 @@ __global__ void __launch_bounds__(kApThreads, 2) apply_kernel(const ApplyArgs a)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(Wl + (size_t)i * h + h0) + (size_t)c * 128));
         }
     }
+    // shared memory of another CTA may be touched only once that CTA runs: arrived here, waited for before the first store there
+    sm100::cluster_arrive();
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     for (int t0 = 0; t0 < T; t0 += TB) {
@@ -204,6 +206,8 @@ __global__ void __launch_bounds__(kApThreads, 2) apply_kernel(const ApplyArgs a)
             __syncthreads();
         }
         // hand the partial sums to the first CTA of the cluster
+        __syncwarp();
+        if (t0 == 0) sm100::cluster_wait();
         for (int e = tid; e < TB * d; e += kApThreads) slot0[(size_t)rank * TB * d + e] = up[e];
         cluster.sync();
         if (rank == 0) {
@@ -299,6 +303,7 @@ template <typename IO, int KIND> __global__ void __launch_bounds__(kDsWarps * 32
     for (int i = threadIdx.x; i < d; i += kDsWarps * 32) sh.up[i] = 0.0f;
     sm100::fence_mbar_init();
     __syncthreads();
+    sm100::cluster_arrive();  // waited for before the first store to another CTA, which has to run by then
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // this warp's groups, in order: 8 rows of every first matrix, then 8 rows x up to 256 columns of the last
@@ -393,6 +398,8 @@ template <typename IO, int KIND> __global__ void __launch_bounds__(kDsWarps * 32
     }
     __syncthreads();
     // hand the partial sums to the first CTA of the cluster
+    __syncwarp();
+    sm100::cluster_wait();
     float* slot0 = cluster.map_shared_rank(&sh.slots[0], 0);
     for (int i = threadIdx.x; i < d; i += kDsWarps * 32) slot0[(size_t)rank * d + i] = sh.up[i];
     cluster.sync();

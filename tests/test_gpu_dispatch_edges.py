@@ -110,3 +110,14 @@ def test_one_token_decode(kind, io, d, h, N):
     x = inputs.generate(r)
     got = gpu_apply(x["q"], x["W"], d=d, h=h, kind=kind, io=io)
     assert util.rel_err(got, oracle_apply(x["q"], x["W"], kind)) <= (1e-5 if io == "f32" else TOL_BF16)
+
+
+@pytest.mark.parametrize("io", ["f32", "bf16"])
+@pytest.mark.parametrize("T", [1, 3, 9])
+def test_decode_with_ctas_that_own_no_hidden_unit(T, io):
+    """Four hidden units in a cluster of eight: seven CTAs do nothing but store their zero partial sums."""
+    r = inputs.Recipe(B=3, H=1, L=T, d=4, h=4, C=T, kind=MLP, io=io, seed=23, w_std=0.5)
+    x = inputs.generate(r)
+    for _ in range(20):
+        got = gpu_apply(x["q"], x["W"], d=4, h=4, kind=MLP, io=io)
+        assert util.rel_err(got, oracle_apply(x["q"], x["W"], MLP)) <= (1e-5 if io == "f32" else TOL_BF16)
