@@ -514,7 +514,7 @@ int e2ttt_apply(const e2ttt_params* p, const void* q, const float* const* W, voi
     a.cl = apply_cluster_size(a.N);
     a.tb = apply_token_block(a.T);
     while (a.cl > 1 && apply_smem_bytes(a.d, a.cl, a.tb) > 40 * 1024) a.cl /= 2;  // room for two CTAs per SM
-    if (apply_smem_bytes(a.d, a.cl, a.tb) > 200 * 1024) return E2TTT_ERR_SHAPE;
+    if (apply_smem_bytes(a.d, a.cl, a.tb) > kApMaxSmem) return E2TTT_ERR_SHAPE;
     a.stage = apply_smem_bytes(a.d, a.cl, a.tb) <= 40 * 1024 && apply_can_stage(a.d, a.h, a.cl);
     a.q = q; a.o = o;
     for (int i = 0; i < nmat; ++i) a.W[i] = W[i];

@@ -14,6 +14,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "apply.h"
 #include "simt_common.cuh"
 #include "sm100.cuh"
@@ -234,10 +236,6 @@ __global__ void __launch_bounds__(kApThreads, 2) apply_kernel(const ApplyArgs a)
 // The rows of the last matrix do not depend on the activations: their copies are under way while the activations are
 // computed.  Eight dot products are reduced together (9 shuffles), which leaves one row per four lanes: the activation function
 // runs once per row.  128 sequences x SwiGLU d = 128, h = 384 (75.5 MB): 17.8 us with loads through registers.
-constexpr int kDsWarps = 8, kDsRows = 8, kDsMaxSlots = 8;
-constexpr int kDsCols = 256;                 // columns of the last matrix per piece, and the widest d this kernel takes
-constexpr uint32_t kDsRingBytes = 96 * 1024; // of all warps
-
 __device__ __forceinline__ void ds_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
@@ -271,6 +269,7 @@ struct __align__(128) DsShared {
     float up[kDsCols];                 // this CTA's partial sums
     float slots[8 * kDsCols];          // on the first CTA: every CTA's partial sums
 };
+static_assert(sizeof(DsShared) == kDsFixedBytes, "");
 
 template <typename IO, int KIND> __global__ void __launch_bounds__(kDsWarps * 32, 2) apply_stream_kernel(const ApplyArgs a) {
     constexpr int NFIRST = KIND == 0 ? 1 : 2, NMAT = NFIRST + 1;
@@ -418,33 +417,27 @@ template <typename IO, int KIND> __global__ void __launch_bounds__(kDsWarps * 32
     }
 }
 
+// A kernel's shared-memory limit, once per device.  The size varies from call to call; the limit is the largest of them, so that host
+// threads that come here together write the same value (a limit that followed the calls could be set back by a smaller one).
+template <typename K> cudaError_t allow_smem(K kernel, size_t most, std::atomic<bool> (&done)[64]) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev])) return e;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+    return e;
+}
+
 template <typename IO, int KIND> int launch_stream(const ApplyArgs& a_in, cudaStream_t st) {
     ApplyArgs a = a_in;
-    // as many CTAs per sequence as keep every cluster resident at two CTAs per SM (the occupancy calculator's numbers: GPU processing
-    // clusters do not divide evenly into larger clusters)
-    static const int fit[9] = {0, 296, 148, 93, 71, 56, 45, 37, 33};
-    a.cl = 1;
-    for (int c = 2; c <= 8; ++c)
-        if (a.N <= fit[c]) a.cl = c;
-    a.per = ((a.h + a.cl - 1) / a.cl + 3) & ~3;
-    const int cols = a.per < kDsCols ? a.per : kDsCols;
-    a.slot_bytes = (uint32_t)(kDsRows * 4 * (a.d > cols ? a.d : cols));
-    const uint32_t fit_slots = kDsRingBytes / (kDsWarps * a.slot_bytes);
-    a.nslots = (int)(fit_slots < 1 ? 1 : fit_slots > kDsMaxSlots ? kDsMaxSlots : fit_slots);
-    a.ring_at = (uint32_t)((sizeof(DsShared) + (size_t)a.per * 4 + 127) / 128 * 128);
-    const size_t smem = a.ring_at + (size_t)kDsWarps * a.nslots * a.slot_bytes;
-    static size_t attr_bytes[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return (int)cudaGetLastError();
-    if (dev < 0 || dev >= 64 || attr_bytes[dev] < smem) {
-        cudaError_t e = cudaFuncSetAttribute(apply_stream_kernel<IO, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return (int)e;
-        if (dev >= 0 && dev < 64) attr_bytes[dev] = smem;
-    }
+    const StreamGeometry g = apply_stream_geometry(a.N, a.d, a.h);
+    a.cl = g.cl; a.per = g.per; a.nslots = g.nslots; a.slot_bytes = g.slot_bytes; a.ring_at = g.ring_at;
+    static std::atomic<bool> done[64];
+    if (cudaError_t e = allow_smem(apply_stream_kernel<IO, KIND>, kDsMaxSmem, done)) return (int)e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(a.N * a.cl));
     cfg.blockDim = dim3(kDsWarps * 32);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = g.smem;
     cfg.stream = st;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -469,14 +462,8 @@ namespace {
 template <typename IO, int KIND, int TB, bool VEC>
 int launch_apply(const ApplyArgs& a, cudaStream_t st) {
     const size_t smem = apply_smem_bytes(a.d, a.cl, TB) + (a.stage ? (size_t)kApStageBytes : 0);
-    static size_t attr_bytes[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return (int)cudaGetLastError();
-    if (dev < 0 || dev >= 64 || attr_bytes[dev] < smem) {
-        cudaError_t e = cudaFuncSetAttribute(apply_kernel<IO, KIND, TB, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return (int)e;
-        if (dev >= 0 && dev < 64) attr_bytes[dev] = smem;
-    }
+    static std::atomic<bool> done[64];
+    if (cudaError_t e = allow_smem(apply_kernel<IO, KIND, TB, VEC>, kApMaxSmem, done)) return (int)e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(a.N * a.cl));
     cfg.blockDim = dim3(kApThreads);
@@ -520,7 +507,7 @@ int apply_launch(const ApplyArgs& a, int kind, int io_dtype, void* stream) {
     const int nmat = kind == 0 ? 2 : 3;
     for (int i = 0; i < nmat; ++i) vec = vec && (reinterpret_cast<uintptr_t>(a.W[i]) % 16 == 0);
     // one token per sequence, bulk copies of whole rows: same alignment, and a token that two 16-byte pieces per lane hold
-    if (vec && a.T == 1 && a.d <= kDsCols && a.h <= 4096) {
+    if (vec && a.T == 1 && a.d <= kDsCols && a.h <= kDsMaxHidden) {
         if (io_dtype == 0) return kind == 0 ? launch_stream<float, 0>(a, st) : launch_stream<float, 1>(a, st);
         return kind == 0 ? launch_stream<__nv_bfloat16, 0>(a, st) : launch_stream<__nv_bfloat16, 1>(a, st);
     }

@@ -1,6 +1,7 @@
 """What the decode kernels (csrc/apply.cu) rest on and a CPU can check."""
 import pathlib
 import re
+import subprocess
 
 import pytest
 
@@ -21,3 +22,32 @@ def test_the_cluster_has_started_before_its_shared_memory_is_written(name):
     store = re.search(r"\bslot0\[[^\]]*\] = ", body).start()
     arrive, wait = body.find("cluster_arrive();"), body.find("cluster_wait();")
     assert 0 <= arrive < wait < store
+
+
+SIZES = r"""
+#include "apply.h"
+#include <cstdio>
+#include <initializer_list>
+using namespace e2ttt;
+int main() {
+    int bad = 0;
+    for (int N : {1, 33, 34, 37, 45, 56, 71, 93, 94, 128, 148, 149, 296, 297, 5000})
+        for (int d = 4; d <= kDsCols; d += 4)
+            for (int h = 4; h <= kDsMaxHidden; h += 4) {
+                const StreamGeometry g = apply_stream_geometry(N, d, h);
+                const int cols = g.per < kDsCols ? g.per : kDsCols;
+                if (g.smem > kDsMaxSmem || g.nslots < 1 || g.per * g.cl < h || g.slot_bytes < 32u * (d > cols ? d : cols) || g.ring_at % 128 ||
+                    g.slot_bytes % 16 || g.ring_at < kDsFixedBytes + 4u * g.per)
+                    if (bad++ < 5) std::printf("N=%d d=%d h=%d: %zu bytes\n", N, d, h, g.smem);
+            }
+    return bad != 0;
+}
+"""
+
+
+def test_no_call_takes_more_shared_memory_than_the_limit_set_for_all(tmp_path):
+    """The limit is a kernel attribute, set once: a larger call later would be refused at its launch."""
+    (tmp_path / "sizes.cpp").write_text(SIZES)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", str(CSRC), str(tmp_path / "sizes.cpp"), "-o", str(tmp_path / "sizes")], check=True)
+    out = subprocess.run([str(tmp_path / "sizes")], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout

@@ -1,5 +1,9 @@
 """e2ttt_apply (outputs of fixed fast weights, the decode path) against the fp64 oracle, against the chunk forward's
 own outputs, and as a streaming decoder: apply per token + one chunk update every C tokens == the one-shot forward."""
+import pathlib
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -102,3 +106,43 @@ def test_apply_rejects_bad_arguments():
         E.e2ttt_apply(p, None, W, q)
     with pytest.raises(Exception):
         E.e2ttt_apply(p, q, W[:1], q)
+
+
+THREADS = """
+import threading, torch
+from paper_2608_21308_b200 import binding as E
+jobs = []
+for kind in (0, 1):
+    for io, dt in ((0, torch.float32), (1, torch.bfloat16)):
+        for h in (64, 512, 1024, 2048, 4096):
+            for T in (1, 2):
+                p = E.make_params(8, 1, T, 256, h, T, kind, io, 1e-5, 0)
+                W = [torch.full((8, 1, *E.e2ttt_matrix_shape(kind, 256, h, i)), 0.01, device="cuda") for i in range(2 + kind)]
+                q = torch.ones(8, 1, T, 256, device="cuda", dtype=dt)
+                jobs.append((p, q, W, torch.empty_like(q)))
+torch.cuda.synchronize()
+gate, failed = threading.Barrier(len(jobs)), []
+def go(job):
+    try:
+        gate.wait()
+        E.e2ttt_apply(*job)
+    except Exception as e:
+        failed.append(repr(e))
+threads = [threading.Thread(target=go, args=(j,)) for j in jobs]
+for t in threads: t.start()
+for t in threads: t.join()
+for j in jobs:
+    try:
+        E.e2ttt_apply(*j)
+    except Exception as e:
+        failed.append(repr(e))
+torch.cuda.synchronize()
+print(len(failed), failed[:3])
+raise SystemExit(bool(failed))
+"""
+
+
+def test_first_calls_of_many_sizes_from_many_threads():
+    """Every thread's call is the first of its size; afterwards every size still launches."""
+    out = subprocess.run([sys.executable, "-c", THREADS], capture_output=True, text=True, timeout=600, cwd=pathlib.Path(__file__).parent.parent)
+    assert out.returncode == 0, out.stdout + out.stderr
