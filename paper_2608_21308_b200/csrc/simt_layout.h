@@ -67,7 +67,7 @@ inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool s
     }
     l.splitk = take((size_t)2 * 8 * 128 * 64);
     if (tile) {
-        const size_t end = tile_layout(l.tl, begin, N, d, h, C, nmat, backward);
+        const size_t end = tile_layout(l.tl, begin, N, d, h, C, nmat, backward, l.seg > 0 && l.seg < nchunks ? l.seg : nchunks);
         if (end > o) o = end;
     }
     l.per_seq = o;

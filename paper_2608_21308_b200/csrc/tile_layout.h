@@ -47,8 +47,9 @@ inline int tile_cluster_size(int N, int hb) {
 }
 
 // Chunks prepared at a time: N * tb * G independent work items should fill whole waves of `ctas` CTAs, and each group costs a launch of
-// every kernel.  At most 9 items per sequence, and 512 MB per set of slots for the whole call (a slot costs about 30 bytes per token and hidden
-// unit): the workspace of a checkpointed call is to stay a small part of what all chunks' states would take.
+// every kernel.  At most 9 items per sequence, and 512 MB per set of slots for the whole call unless one slot per sequence takes more (a
+// slot costs about 30 bytes per token and hidden unit): the workspace of a checkpointed call is to stay a small part of what all chunks'
+// states would take.
 inline int tile_group_chunks(int N, int tb, int ctas, size_t slot_bytes) {
     int best = 1;
     double best_eff = 0.0;
@@ -64,8 +65,9 @@ inline int tile_group_chunks(int N, int tb, int ctas, size_t slot_bytes) {
     return best;
 }
 
-// Appends the region behind offset o (floats); returns the end.
-inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, int nmat, bool backward) {
+// Appends the region behind offset o (floats); returns the end.  `chunks`: the most that one reverse launch sequence covers (those of a
+// checkpointed segment, or of the call); no slot is laid out beyond them.
+inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, int nmat, bool backward, int chunks) {
     auto blocks = [](int n) { return (n + 63) / 64; };
     auto take = [&](size_t n) { size_t r = o; o += (n + 31) / 32 * 32; return r; };
     t.db = blocks(d); t.hb = blocks(h); t.tb = blocks(C);
@@ -119,6 +121,10 @@ inline size_t tile_layout(TileLayout& t, size_t o, int N, int d, int h, int C, i
     t.spare = chain && ctas <= kTileMaxCl ? (tile_clusters_fit(ctas) - N) * ctas : 0;
     t.sets = t.spare >= N && o * sizeof(float) * N <= ((size_t)512 << 20) ? 2 : 1;
     t.G = tile_group_chunks(N, t.tb, t.sets == 2 ? t.spare : 148, o * sizeof(float));
+    if (chunks <= t.G) {  // one group: no next one to prepare beside it
+        t.G = chunks;
+        t.sets = 1;
+    }
     o = t.slot + t.slot_stride * (size_t)(t.sets * t.G);
     return o > end_fwd ? o : end_fwd;
 }

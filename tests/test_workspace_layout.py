@@ -1,0 +1,48 @@
+"""The workspace of the block-tiled reverse pass (csrc/tile_layout.h): no more than the call can use, within the bound it states."""
+import pathlib
+import subprocess
+
+from paper_2608_21308_b200 import binding as E
+
+CSRC = pathlib.Path(__file__).resolve().parent.parent / "paper_2608_21308_b200" / "csrc"
+
+LAYOUTS = r"""
+#include "simt_layout.h"
+#include <cstdio>
+#include <initializer_list>
+using namespace e2ttt;
+int main() {
+    int bad = 0;
+    for (int N : {1, 4, 16, 32, 33, 34, 64, 150, 2048})
+        for (int d : {8, 64, 128})
+            for (int h : {8, 192, 512, 1024, 1088})
+                for (int C : {16, 64, 65, 512})
+                    for (int nmat : {2, 3})
+                        for (int nchunks : {1, 2, 3, 8, 23, 128})
+                            for (int seg : {0, 2, 4, 32}) {
+                                const SimtLayout l = simt_layout(d, h, C, nmat, nchunks, true, true, seg, 1, N);
+                                const TileLayout& t = l.tl;
+                                const int chunks = seg > 0 && seg < nchunks ? seg : nchunks;
+                                const size_t slots = (size_t)t.G * N * t.slot_stride * 4, one = (size_t)N * t.slot_stride * 4;
+                                const bool unused = t.G > chunks || (t.sets == 2 && chunks <= t.G);
+                                const bool over = slots > (one > ((size_t)512 << 20) ? one : (size_t)512 << 20);
+                                const bool outside = t.slot + (size_t)t.sets * t.G * t.slot_stride > l.per_seq;
+                                if ((unused || over || outside || t.G < 1) && bad++ < 5)
+                                    std::printf("N=%d d=%d h=%d C=%d nmat=%d chunks=%d: G=%d sets=%d\n", N, d, h, C, nmat, chunks, t.G, t.sets);
+                            }
+    return bad != 0;
+}
+"""
+
+
+def test_slots_of_the_reverse_pass_are_bounded_by_the_chunks_of_a_launch(tmp_path):
+    (tmp_path / "layouts.cpp").write_text(LAYOUTS)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", str(CSRC), str(tmp_path / "layouts.cpp"), "-o", str(tmp_path / "layouts")], check=True)
+    out = subprocess.run([str(tmp_path / "layouts")], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout
+
+
+def test_a_short_training_call_asks_for_one_chunks_slots():
+    """16 sequences of one chunk, d = 128, h = 512: 9.0 MB each, of which one slot is 1.83 MB (16 slots would make it 36.4 MB)."""
+    p = E.make_params(1, 16, 64, 128, 512, 64, E.E2TTT_MLP_GELU, E.E2TTT_BF16, 1e-5, E.E2TTT_IMPL_AUTO)
+    assert E.e2ttt_workspace_bytes(p, 1) < 16 * 9.5e6
