@@ -294,24 +294,21 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
                 st_io(dq + (size_t)s * d, e, ld_io<Real>(doc, e) + acc);
             });
         BPROF(8);
-        G.template run_rmw<1, false, false>( // Wbl += Uqb^T Aq
+        G.template run_add<1, false, false>( // Wbl += Uqb^T Aq
             d, h, len, [&](int m, int t, Real& a0, Real& a1) { a0 = Uqb[(size_t)t * d + m]; },
             [&](int n, int t) { return Aq[(size_t)t * h + n]; },
-            [&](int m, int n) { return Wb[LAST][(size_t)m * h + n]; },
-            [&](int m, int n, Real acc, Real, Real old) { Wb[LAST][(size_t)m * h + n] = old + acc; });
+            [&](int m, int n) -> Real& { return Wb[LAST][(size_t)m * h + n]; });
         BPROF(9);
-        G.template run_rmw<1, false, false>( // Wb1 += Zqb^T Q
+        G.template run_add<1, false, false>( // Wb1 += Zqb^T Q
             h, d, len, [&](int m, int t, Real& a0, Real& a1) { a0 = Zqb[(size_t)t * h + m]; },
             [&](int n, int t) { return ld_io<Real>(qc, (size_t)t * d + n); },
-            [&](int m, int n) { return Wb[0][(size_t)m * d + n]; },
-            [&](int m, int n, Real acc, Real, Real old) { Wb[0][(size_t)m * d + n] = old + acc; });
+            [&](int m, int n) -> Real& { return Wb[0][(size_t)m * d + n]; });
         BPROF(10);
         if (SW)
-            G.template run_rmw<1, false, false>( // Wb2 += Zqb2^T Q
+            G.template run_add<1, false, false>( // Wb2 += Zqb2^T Q
                 h, d, len, [&](int m, int t, Real& a0, Real& a1) { a0 = Zqb2[(size_t)t * h + m]; },
                 [&](int n, int t) { return ld_io<Real>(qc, (size_t)t * d + n); },
-                [&](int m, int n) { return Wb[1][(size_t)m * d + n]; },
-            [&](int m, int n, Real acc, Real, Real old) { Wb[1][(size_t)m * d + n] = old + acc; });
+                [&](int m, int n) -> Real& { return Wb[1][(size_t)m * d + n]; });
 
         BPROF(11);
         // ---------------- (ii) state transition: carries ----------------
@@ -436,11 +433,10 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
             [&](int n, int kk) { return Wl[(size_t)n * h + kk]; },
             [&](int m, int n, Real acc, Real) { Pub[(size_t)m * d + n] += acc; });
         BPROF(22);
-        G.template run_rmw<1, false, false>( // Wbl += Pu^T Phb
+        G.template run_add<1, false, false>( // Wbl += Pu^T Phb
             d, h, len, [&](int m, int t, Real& a0, Real& a1) { a0 = Pu[(size_t)t * d + m]; },
             [&](int n, int t) { return Phb[(size_t)t * h + n]; },
-            [&](int m, int n) { return Wb[LAST][(size_t)m * h + n]; },
-            [&](int m, int n, Real acc, Real, Real old) { Wb[LAST][(size_t)m * h + n] = old + acc; });
+            [&](int m, int n) -> Real& { return Wb[LAST][(size_t)m * h + n]; });
         // pu = J(u) e, e = k + y - v, y = LN(u)
         BPROF(23);
         for (int t = warp + rank * (NT / 32); t < len; t += (NT / 32) * CL) {
@@ -484,11 +480,10 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
                 }
             });
         BPROF(25);
-        G.template run_rmw<1, false, false>( // Wbl += Ukb^T Ak
+        G.template run_add<1, false, false>( // Wbl += Ukb^T Ak
             d, h, len, [&](int m, int t, Real& a0, Real& a1) { a0 = Ukb[(size_t)t * d + m]; },
             [&](int n, int t) { return A[(size_t)t * h + n]; },
-            [&](int m, int n) { return Wb[LAST][(size_t)m * h + n]; },
-            [&](int m, int n, Real acc, Real, Real old) { Wb[LAST][(size_t)m * h + n] = old + acc; });
+            [&](int m, int n) -> Real& { return Wb[LAST][(size_t)m * h + n]; });
         // z1 = W1 k (, z2 = W2 k)
         BPROF(26);
         G.template run<1, true, false>(
@@ -502,18 +497,16 @@ __global__ void __launch_bounds__(TC ? kTgThreads : kSimtThreads, 1) simt_bwd_ke
                 st_io(dk + (size_t)s * d, e, Kb[e] + acc);
             });
         BPROF(27);
-        G.template run_rmw<1, false, false>( // Wb1 += Zkb^T K
+        G.template run_add<1, false, false>( // Wb1 += Zkb^T K
             h, d, len, [&](int m, int t, Real& a0, Real& a1) { a0 = Zkb[(size_t)t * h + m]; },
             [&](int n, int t) { return ld_io<Real>(kc, (size_t)t * d + n); },
-            [&](int m, int n) { return Wb[0][(size_t)m * d + n]; },
-            [&](int m, int n, Real acc, Real, Real old) { Wb[0][(size_t)m * d + n] = old + acc; });
+            [&](int m, int n) -> Real& { return Wb[0][(size_t)m * d + n]; });
         BPROF(28);
         if (SW)
-            G.template run_rmw<1, false, false>( // Wb2 += Zkb2^T K
+            G.template run_add<1, false, false>( // Wb2 += Zkb2^T K
                 h, d, len, [&](int m, int t, Real& a0, Real& a1) { a0 = Zkb2[(size_t)t * h + m]; },
                 [&](int n, int t) { return ld_io<Real>(kc, (size_t)t * d + n); },
-                [&](int m, int n) { return Wb[1][(size_t)m * d + n]; },
-            [&](int m, int n, Real acc, Real, Real old) { Wb[1][(size_t)m * d + n] = old + acc; });
+                [&](int m, int n) -> Real& { return Wb[1][(size_t)m * d + n]; });
 
         BPROF(29);
         // ---------------- adjoints of the chunk-start state ----------------

@@ -7,7 +7,9 @@
 //   run_rmw: pre(m, n) returns what the result has to be combined with (anything loaded from memory), and
 //            epi(m, n, acc0, acc1, loaded) consumes it.  The engine calls pre for a batch of results before the
 //            batch's epi calls, so that the loads are in flight together instead of one memory round trip per result
-//            (the compiler cannot move a load of epi above the previous result's store: they may alias).
+//            (the compiler cannot move a load of epi above the previous result's store: they may alias);
+//   run_add: the result is added to at(m, n).  The FMA engine batches the loads (run_rmw); the tensor-core engine, whose kernels have
+//            128 registers per thread, does not: the batches made the reverse pass spill (d = 160: 5-10 % slower).
 // Output tiles are dealt round-robin to the `nranks` CTAs of the sequence's cluster; run() ends with phase_sync().
 //
 //   FmaGemm<Real> : CUDA-core FMAs in the kernel's own precision (fp64 for fp32 I/O, fp32 for bf16 I/O).
@@ -44,6 +46,11 @@ template <typename Real> struct FmaGemm {
     __device__ void run(int M, int N, int K, FA fa, FB fb, FE epi) {
         run_rmw<NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, [](int, int) { return 0; },
                                         [&](int m, int n, Real a0, Real a1, int) { epi(m, n, a0, a1); });
+    }
+    template <int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FT>
+    __device__ void run_add(int M, int N, int K, FA fa, FB fb, FT at) {
+        run_rmw<NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, [&](int m, int n) { return at(m, n); },
+                                        [&](int m, int n, Real acc, Real, Real old) { at(m, n) = old + acc; });
     }
 };
 
@@ -195,6 +202,10 @@ template <bool SPLITK> struct TcGemmT {
     __device__ void run(int M, int N, int K, FA fa, FB fb, FE epi) {
         run_rmw<NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, [](int, int) { return 0; },
                                         [&](int m, int n, float a0, float a1, int) { epi(m, n, a0, a1); });
+    }
+    template <int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FT>
+    __device__ void run_add(int M, int N, int K, FA fa, FB fb, FT at) {
+        run<NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, [&](int m, int n, float acc, float) { at(m, n) += acc; });
     }
 
     template <int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FP, typename FE>
