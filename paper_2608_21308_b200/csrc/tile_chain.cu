@@ -4,16 +4,16 @@
 // through the workspace that was 7 of 10.7 MB of memory traffic per chunk and sequence at d = 128, h = 512, C = 64, and with 64
 // sequences at once it does not fit L2.  Here a cluster has one CTA per 128 hidden units (33 clusters of 4 fit the GPU; one CTA per
 // 64 units was slower: 15 clusters of 8), and a CTA keeps its slices for the whole launch:
-//   tensor memory : fp32 masters of T, 128 x 128 per matrix; the aggregations' MMAs accumulate into them.  The contiguous index of
-//                   the matrix in memory is on the lanes (d for the first matrices, hidden units for the last), so that the state
-//                   (T, S, and the saved W, M of every chunk) is read and written whole lines at a time
+//   tensor memory : fp32 masters of T, 128 x 128 per matrix.  The contiguous index of the matrix in memory is on the lanes (d for the
+//                   first matrices, hidden units for the last), so that the state (T, S, and the saved W, M of every chunk) is read
+//                   and written whole lines at a time
 //   shared memory : operand blocks (hi, lo) of T of as many matrices as fit 128 KB (two at d > 64), rows = the index on the
 //                   lanes: read K-major with that index on the lanes, MN-major with the other one there
 // S, and T blocks that do not fit, live in the workspace; 33 sequences' worth stays in L2.
-// In a chunk the products run on the operand blocks of the arriving T, S; meanwhile, piece by piece between their epilogues, the
-// masters are scaled by the carries (T <- cw T, S <- cm T + cb S; the blocks of the new S go to the other of two buffers, by the
-// parity of the chunk), the chunk's own contribution is accumulated onto T, and T's operand blocks are written anew.  Everything else
-// streams from the slots that tile_prep and tile_rec filled.
+// A chunk starts with one pass over the masters (T <- cw T, S <- cm T + cb S; the blocks of the new S go to the other of two buffers,
+// by the parity of the chunk) while the first products run on the operand blocks of the arriving T, S.  Every product that contributes
+// to T has an epilogue of its own, which adds it to the master; after a matrix's last one T's operand blocks are written anew.
+// Everything else streams from the slots that tile_prep and tile_rec filled.
 //
 // 18 warps: 0-15 epilogues (warp w: lanes 32 (w & 3).., group w >> 2 of the columns), 16 copies operand blocks, 17 issues MMAs.
 #include <type_traits>
@@ -34,8 +34,8 @@ constexpr uint32_t kResident = 128 * 1024, kRingBytes = kCells * kCell;
 
 struct ChainShared {
     uint64_t full[kLoads], empty[kLoads], acc_full[2], acc_empty[2];
-    // once per chunk: operand blocks of T, S written; phb written; masters scaled; zb written; T accumulated
-    uint64_t ops, phb, scaled, zb, upd;
+    // once per chunk: operand blocks of T, S written; phb written; masters scaled; zb written
+    uint64_t ops, phb, scaled, zb;
     uint32_t tmem;
     int dead;
     float dots[2][16][4];  // by the parity of the launch's chunk: a warp may be a chunk's scaling ahead of the one that adds them up
@@ -79,7 +79,6 @@ template <int NSET> struct Chain {
             for (int i = 0; i < kLoads; ++i) { mbar_init(&s->full[i], 1); mbar_init(&s->empty[i], 1); }
             for (int i = 0; i < 2; ++i) { mbar_init(&s->acc_full[i], 1); mbar_init(&s->acc_empty[i], 16); }
             mbar_init(&s->ops, 16); mbar_init(&s->phb, 16); mbar_init(&s->scaled, 16); mbar_init(&s->zb, 16);
-            mbar_init(&s->upd, 1);
             s->dead = 0;
             fence_mbar_init();
         }
@@ -286,7 +285,8 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
         return;
     }
     const int CL = a.cl, seq = blockIdx.x / CL, rank = blockIdx.x % CL;
-    Chain<SW ? 1 : 2> G;
+    constexpr int EARLY = SW ? 1 : 2;  // accumulator sets
+    Chain<EARLY> G;
     G.setup(chain_smem, &sh, a.status, CL);
     const int warp = G.warp, lane = G.lane;
     const SimtLayout& lay = a.lay;
@@ -316,7 +316,7 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
             return Opnd{p, db == 2 ? p + B : nullptr, (uint32_t)db * B, true, !rows_d};
         };
         size_t sbuf = 0;  // S blocks of the chunk at hand
-        using Product = typename Chain<SW ? 1 : 2>::Product;
+        using Product = typename Chain<EARLY>::Product;
         // products of a [tokens x ..] operand with T and S of matrix i, hidden units or d on the lanes
         auto by_h = [&](Product& P, const Opnd& x, int i) {
             const bool f = i < LAST;
@@ -417,16 +417,16 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
             // which the copy warp waits for inside that chunk
             if (G.issuer() || n == 0) G.await(&sh.ops, n, 405);
             // Steps of the chunk: phase, block of 64 tokens, product
-            //   0  everything with T, S          2  the chunk's contribution, as far as it waits for no rows      4  T_last += a_k u_k
-            //   1  pub += W_last phb             3  adjoint of u back through W_last                             5  dk += W_first^T zb
-            //   6  T_first += zb k
+            //   0  everything with T, S          3  adjoint of u back through W_last
+            //   1  pub += W_last phb             5  dk += W_first^T zb
+            //   2, 4, 6  contributions to T: q zq (first matrices), aq uq, phb pu and ak uk (last), zb k (first).  The first ones wait for
+            //      no rows: as many as there are accumulator sets run while the rows do
 #pragma unroll 1
             for (int ph = 0; ph < 7; ++ph) {
                 if (ph == 1 && G.copier()) {
                     prefetch_late(g);
                     if (g > 0) prefetch_state(g - 1);
                 }
-                if (ph == 2 && G.issuer()) G.await(&sh.scaled, n, 407);
                 if (ph == 3) {
                     // Taken before the loads that the chunk's end waits for: later, the epilogues could be through with the next chunk's
                     // scaling, and a wait for this one's parity would be a wait for the one after
@@ -435,17 +435,16 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
                     G.cluster_arrive_all();
                     if (G.issuer()) G.cluster_wait_all();
                 }
-                const bool jobs = ph < 2 || ph == 3 || ph == 5;
-                const int ntk = jobs ? tbn : 1;
-                const int nstep = ph == 0 ? 2 * LAST + 2 : ph == 2 ? LAST + 2 : ph >= 5 ? LAST : 1;
+                const int ntk = ph == 2 || ph == 4 || ph == 6 ? 1 : tbn;
+                const int nstep = ph == 0 ? 2 * LAST + 2 : ph == 2 ? EARLY : ph == 4 ? LAST + 3 - EARLY : ph >= 5 ? LAST : 1;
 #pragma unroll 1
                 for (int e = 0, tk = 0, st = 0; e < ntk * nstep; ++e) {
                     if (ph == 0 && st == LAST && tk == 0 && nres < NMAT && G.copier()) G.await(&sh.ops, n, 411);
                     // the first matrices' dk products of phases 0 and 5 share a job
-                    const bool opens = jobs && (ph == 0 ? st <= LAST + 2 : ph == 5 ? st == 0 : true), closes = jobs && (ph == 0 ? st < LAST + 2 || st == 2 * LAST + 1 : st == nstep - 1);
+                    const bool opens = ph == 0 ? st <= LAST + 2 : ph == 5 ? st == 0 : true, closes = ph == 0 ? st < LAST + 2 || st == 2 * LAST + 1 : ph == 5 ? st == nstep - 1 : true;
                     Product P{};
-                    P.col = jobs ? G.tmem + G.acc() : G.tmem + 128 * (ph == 6 ? st : ph == 2 ? min(st, LAST) : LAST);
-                    P.acc0 = jobs ? !opens : true;
+                    P.col = G.tmem + G.acc();
+                    P.acc0 = !opens;
                     if (ph == 0) {
                         if (st < LAST) by_h(P, Opnd{sblk(tl.sK) + (size_t)tk * db * kHalf, nullptr, kHalf, false, false}, st);
                         else if (st == LAST) by_h(P, Opnd{sblk(tl.sPu) + (size_t)tk * db * B, nullptr, B, true, false}, LAST);
@@ -454,15 +453,15 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
                     } else if (ph == 1) {
                         simple(P, nb, w_by_d(sblk(tl.sW[LAST]), false), tok_h(blk(tl.bPhb), tk));
                         P.before = &sh.phb;
-                    } else if (ph == 2) {
-                        if (st < LAST) simple(P, tbn, key_d(sblk(tl.sQ)), h_tok(sblk(tl.sZq[st])));
-                        else if (st == LAST) simple(P, tbn, h_tok(sblk(tl.sAq)), tok_d(sblk(tl.sUq)));
-                        else simple(P, tbn, h_tok(blk(tl.bPhb)), tok_d(sblk(tl.sPu)));
+                    } else if (ph == 2 || ph == 4) {
+                        const int k = ph == 2 ? st : EARLY + st;
+                        if (k < LAST) simple(P, tbn, key_d(sblk(tl.sQ)), h_tok(sblk(tl.sZq[k])));
+                        else if (k == LAST) simple(P, tbn, h_tok(sblk(tl.sAq)), tok_d(sblk(tl.sUq)));
+                        else if (k == LAST + 1) simple(P, tbn, h_tok(blk(tl.bPhb)), tok_d(sblk(tl.sPu)));
+                        else simple(P, tbn, h_tok(sblk(tl.sAk)), tok_d(blk(tl.bUk)));
                     } else if (ph == 3) {
                         simple(P, db, w_by_h(sblk(tl.sW[LAST]), false), Opnd{blk(tl.bUk) + (size_t)tk * db * B, nullptr, B, true, false});
                         P.before_cluster = tk == 0;
-                    } else if (ph == 4) {
-                        simple(P, tbn, h_tok(sblk(tl.sAk)), tok_d(blk(tl.bUk)));
                     } else if (ph == 5) {
                         simple(P, nb, w_by_d(sblk(tl.sW[st]), true), tok_h(blk(tl.bZk[st]), tk));
                         P.before = &sh.zb;
@@ -475,7 +474,6 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
                     if (++st == nstep) { st = 0; ++tk; }
                 }
             }
-            if (G.issuer()) umma_commit_elect(&sh.upd, lane == 0);
             if (G.copier() && g > 0) prefetch_early(g - 1);
         }
         G.cluster_arrive_all();
@@ -869,6 +867,32 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
         }
         G.cluster_arrive_all();
 
+        // A product's contribution to T of matrix i, rounded to nearest onto the master; `done`: the last one, T's operand blocks follow.
+        // Accumulated onto the master itself, every MMA truncated T, chunk after chunk: 64 chunks of 64 tokens, d = 128, h = 512, error
+        // of the adjoints against 64 bits 3.1e-5 (first matrix) and 3.3e-5 (momentum of the last), this way 9.8e-6 and 7.0e-6; the
+        // step takes as long (15.2 ms for 64 sequences)
+        auto contribution = [&](int i, bool done) {
+            G.job_out([&](uint32_t t) {
+#pragma unroll 1
+                for (int pc = 0; pc < 2; ++pc) {
+                    const int col = col_of(pc);
+                    float x[16], m[16];
+                    acc16(t + col, x);
+                    acc16(lanes + 128 * i + col, m);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) m[j] += x[j];
+                    acc_st16(lanes + 128 * i + col, m);
+                    if (done && !NORMED) {
+                        mask(i, col, m);
+                        put(true, 0, i, col, m);
+                    }
+                }
+                tmem_wait_st();
+            });
+        };
+#pragma unroll 1
+        for (int k = 0; k < EARLY; ++k) contribution(min(k, LAST), false);
+
         // ---- u = W_last a ; a = act(z): adjoint of z
 #pragma unroll 1
         for (int tk = 0; tk < tbn; ++tk) {
@@ -898,25 +922,21 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
             });
         }
         G.signal(&sh.zb);
-        plain_share(tl.bdk[buf]);  // dk += W_first^T zb
-
-        // ---- T -> operand blocks, once the chunk's contribution is in
-        G.await(&sh.upd, n, 409);
-        if (threadIdx.x < 3) {  // (the issuer waited for every warp's share before the MMAs this wait is for)
-            float x = 0.0f;
-            for (int w = 0; w < 16; ++w) x += sh.dots[n & 1][w][threadIdx.x];
-            sl[tl.sdots + rank * 4 + threadIdx.x] = x;
-        }
-        if (!NORMED) {
 #pragma unroll 1
-            for (int e = 0; e < 2 * NMAT; ++e) {
-                float t[16];
-                acc16(lanes + 128 * (e >> 1) + col_of(e & 1), t);
-                mask(e >> 1, col_of(e & 1), t);
-                put(true, 0, e >> 1, col_of(e & 1), t);
+        for (int k = EARLY; k < LAST + 3; ++k) contribution(min(k, LAST), k == LAST + 2);
+        plain_share(tl.bdk[buf]);  // dk += W_first^T zb
+#pragma unroll 1
+        for (int i = 0; i < LAST; ++i) contribution(i, true);
+
+        if (warp == 0) {
+            G.await(&sh.scaled, n, 409);  // every warp's share of the dot products
+            if (lane < 3) {
+                float x = 0.0f;
+                for (int w = 0; w < 16; ++w) x += sh.dots[n & 1][w][lane];
+                sl[tl.sdots + rank * 4 + lane] = x;
             }
-            G.signal(&sh.ops);
         }
+        if (!NORMED) G.signal(&sh.ops);
     }
     G.cluster_arrive_all();
     G.cluster_wait_all();

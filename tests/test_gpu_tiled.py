@@ -100,3 +100,15 @@ def test_wide_networks_forward_and_backward(kind, io, impl):
     assert E.e2ttt_device_status(hd["ws"]) == 0
     check_forward(got, util.oracle_forward(x, r.C, kind), tol, "wide forward")
     check_backward(util.gpu_backward(x, impl=impl, **shape), util.oracle_backward(x, r.C, kind), tol, "wide backward")
+
+
+def test_reverse_chain_of_many_chunks_keeps_its_precision():
+    """64 chunks.  A two-term operand is off by 2^-17 of its value at most, a product of two by 1.1e-5 with both at their worst: the bound
+    of the last matrix's momentum adjoint, which one product feeds, and twice that of the first matrix's adjoint, which takes two in a
+    row.  (The other two amplify it and are left out.)  Summed up by the tensor cores over the chunks, both came to 3.5e-5."""
+    r = inputs.paper_regime(inputs.Recipe(B=2, H=1, L=4096, d=128, h=512, C=64, kind=MLP, io="bf16", seed=41))
+    x = inputs.generate(r, with_d_o=True)
+    got = util.gpu_backward(x, d=128, h=512, C=64, kind=MLP, io="bf16", impl=E.E2TTT_IMPL_TILED, use_M=False, use_dstate=False)
+    ref = util.oracle_backward(x, 64, MLP, use_M=False, use_dstate=False)
+    assert util.rel_l2(got["dM"][1], ref["dM"][1]) <= 1.1e-5
+    assert util.rel_l2(got["dW"][0], ref["dW"][0]) <= 2.2e-5
