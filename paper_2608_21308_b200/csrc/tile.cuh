@@ -146,8 +146,9 @@ struct Engine {
     }
 
     // sum over nk slices of 64 k:  D[col[i]] += S P[i]^T  for i < np, with S on the lane side (s_lane) or the column side.
-    // `col`: first column of the accumulator inside the job's set.
-    template <int NP> __device__ void term(int nk, bool s_lane, const Opnd& s, const Opnd (&p)[NP], const uint32_t (&col)[NP]) {
+    // `col`: first column of the accumulator inside the job's set.  SPLIT: the products with a lo part in the 128 columns behind it, for
+    // contractions of many slices (every MMA onto the sum truncates it; theirs are 2^-9 of it), added by the epilogue.
+    template <int NP, bool SPLIT = false> __device__ void term(int nk, bool s_lane, const Opnd& s, const Opnd (&p)[NP], const uint32_t (&col)[NP]) {
         if (warp == kEpiWarps) {
             for (int k = 0; k < nk; ++k) {
                 load(s, k);
@@ -177,8 +178,14 @@ struct Engine {
                         const uint64_t ah = make_smem_desc(ua + ks * sa, kHalf, 1024), bh = make_smem_desc(ub + ks * sb, kHalf, 1024);
                         const uint64_t al = ah + (2 * kHalf >> 4), bl = bh + (2 * kHalf >> 4);
                         bool acc = (started >> i & 1u) || ks > 0;
-                        if (a.lo) { umma_bf16_elect(d, al, bh, idesc, acc, issue); acc = true; }  // small terms first
-                        if (b.lo) { umma_bf16_elect(d, ah, bl, idesc, acc, issue); acc = true; }
+                        if constexpr (SPLIT) {
+                            bool acl = acc;
+                            if (a.lo) { umma_bf16_elect(d + 128, al, bh, idesc, acl, issue); acl = true; }
+                            if (b.lo) umma_bf16_elect(d + 128, ah, bl, idesc, acl, issue);
+                        } else {
+                            if (a.lo) { umma_bf16_elect(d, al, bh, idesc, acc, issue); acc = true; }  // small terms first
+                            if (b.lo) { umma_bf16_elect(d, ah, bl, idesc, acc, issue); acc = true; }
+                        }
                         umma_bf16_elect(d, ah, bh, idesc, acc, issue);
                     }
                     started |= 1u << i;

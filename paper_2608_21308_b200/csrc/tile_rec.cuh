@@ -115,20 +115,25 @@ template <int KIND> __device__ __forceinline__ void rec_items(const SimtBwdArgs&
         }
         G.sync_cta();
 
-        // u = W_last a
+        // u = W_last a.  One CTA contracts all hidden units: with the small terms apart the chain of truncating MMAs is a third as long
+        // (h = 1100, C = 16: error of the gate adjoints against 64 bits 1.17-1.33 -> 1.04-1.17 times that of fp32 sums over eight CTAs;
+        // d = 64, h = 1024: of dW 1.13 -> 0.95 times)
         float* U = sl + tl.sU + (size_t)tk * 128 * dp;
         {
             const unsigned char* pw = blk(tl.sW[LAST]);
             const Opnd act{blk(tl.sAk) + (size_t)tk * B, blk(tl.sAq) + (size_t)tk * B, (uint32_t)tb * B, true, true};
             const Opnd w[1] = {{pw, db == 2 ? pw + B : nullptr, (uint32_t)db * B, true, true}};
             G.job_begin();
-            G.term<1>(hb, false, act, w, {0u});
+            G.term<1, true>(hb, false, act, w, {0u});
             G.job_end([&](uint32_t t) {
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
                     const int col = 32 * grp + 16 * half;
-                    float u[16];
+                    float u[16], ul[16];
                     acc16(t + col, u);
+                    acc16(t + 128 + col, ul);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) u[j] += ul[j];
                     if (row < dp)
 #pragma unroll
                         for (int j = 0; j < 16; ++j) U[(size_t)(col + j) * dp + row] = u[j];
