@@ -81,6 +81,35 @@ int pick_impl(const e2ttt_params* p, bool save_states, int* impl) {
 // wider heads and fp32 I/O run on the SIMT kernels.
 bool can_tile(const e2ttt_params* p) { return p->io_dtype == E2TTT_BF16 && p->d <= kTileMaxD; }
 
+// Where they do not pay, the any-shape kernels with tensor-core products (simt_fwd.cu, simt_bwd.cu) keep the call.  Both lose their time
+// in phases that follow one another; these have fewer CTAs to spread a phase over where the hidden units are few (one per 64, in
+// the reverse chain per 128), those split the tokens as well, over clusters of 8 or 4 CTAs, as long as all of them fit the GPU at once.
+int other_cluster(const e2ttt_params* p) {  // CTAs per sequence there; 0 if the call's clusters do not fit together
+    const int N = p->B * p->H, cl = simt_cluster_size(N, E2TTT_BF16);
+    return N <= tile_clusters_fit(cl) ? cl : 0;
+}
+// Forward, GELU network.  At most 64 hidden units and long chunks: C = 512, d = 64, 8 sequences 0.77 of the block-tiled time, 32 sequences
+// 0.85 (C = 128: 0.99; 16 sequences, which take clusters of 8 in two waves, 1.0).  Short chunks of small states where the
+// others run without clusters, more than 74 sequences: a block of 64 tokens is then mostly padding (300 sequences, d = h = 64: C = 1 0.77,
+// C = 16 0.80, C = 32 0.96).  The SwiGLU network, with two more products per block, gains everywhere.
+bool tile_forward(const e2ttt_params* p) {
+    if (!can_tile(p)) return false;
+    if (p->kind != E2TTT_MLP_GELU) return true;
+    const int N = p->B * p->H, dh = p->d * p->h, cl = other_cluster(p);
+    if (p->h <= 64 && (cl == 8 ? p->C > 128 : cl == 4 && p->C > 384)) return false;
+    if (N > 148) return !((p->C <= 4 && dh <= 16384) || (p->C <= 16 && dh <= 12288) || (p->C <= 32 && dh <= 9216 && p->h <= 256));
+    return !(N > 74 && p->C <= 4 && dh <= 16384);
+}
+// Reverse pass.  At most 128 hidden units (one CTA per sequence in the chain) and long chunks: d = h = 64, 8 sequences, C = 512 0.60 of the
+// block-tiled time, C = 320 0.81 (256: 0.99); 15 sequences C = 448 0.70.  States of a few hundred values, up to 33 sequences: d = 16,
+// h = 8, 32 sequences, C = 512 0.78, C = 256 0.87.
+bool tile_backward(const e2ttt_params* p) {
+    if (!can_tile(p)) return false;
+    const int N = p->B * p->H;
+    if (p->h <= 128 && ((N <= 8 && p->C > 256) || (N <= 15 && p->C > 384))) return false;
+    return !(p->d * p->h <= 512 && p->C > 192 && other_cluster(p) >= 4);
+}
+
 // A buffer with saved states has the block-tiled region whatever `impl` says: the forward and the backward of one training step may
 // be given different ones.
 SimtLayout layout_of(const e2ttt_params* p, bool save_states, bool backward, bool normed, bool allow_tile = true) {
@@ -256,7 +285,7 @@ static int fwd_common(const e2ttt_params* p, const void* q, const void* k, const
     }
     a.norm_eps = norm_eps;
     a.lay = layout_of(p, save_states != 0, save_states != 0, row_norm != nullptr, allow_tile);
-    const bool tile = impl == E2TTT_IMPL_TILED && can_tile(p) && allow_tile;
+    const bool tile = impl == E2TTT_IMPL_TILED && tile_forward(p) && allow_tile;
     return (tile ? tile_fwd_launch(a, p->kind, stream) : simt_fwd_launch(a, p->kind, p->io_dtype, stream)) == 0 ? E2TTT_OK : E2TTT_ERR_CUDA;
 }
 
@@ -337,7 +366,7 @@ static int bwd_common(const e2ttt_params* p, const void* q, const void* k, const
     const int nchunks = (p->L + p->C - 1) / p->C;
     const int seg = row_norm ? 0 : segment_chunks(p);
     const SimtLayout lay = layout_of(p, true, true, row_norm != nullptr);
-    const bool tile = impl != E2TTT_IMPL_SIMT && can_tile(p);
+    const bool tile = impl != E2TTT_IMPL_SIMT && tile_backward(p);  // the recomputing forwards too: both keep blocks in one region
 
     void* ws_data = static_cast<char*>(workspace) + kStatusBytes;
     if (cudaMemsetAsync(workspace, 0, sizeof(int), reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) {

@@ -121,3 +121,26 @@ def test_decode_with_ctas_that_own_no_hidden_unit(T, io):
     for _ in range(20):
         got = gpu_apply(x["q"], x["W"], d=4, h=4, kind=MLP, io=io)
         assert util.rel_err(got, oracle_apply(x["q"], x["W"], MLP)) <= (1e-5 if io == "f32" else TOL_BF16)
+
+
+@pytest.mark.parametrize("N,d,h,C,L", [
+    (15, 64, 64, 129, 260), (16, 64, 64, 129, 260), (2, 72, 72, 129, 260),    # forward: 64 hidden units or more, 15 sequences or more
+    (33, 64, 64, 385, 400), (34, 64, 64, 385, 400),                           # forward: clusters of 4 that fit together, and not
+    (75, 64, 64, 4, 10), (149, 96, 128, 16, 20), (149, 64, 200, 16, 20),      # forward: many sequences of short chunks
+    (8, 64, 128, 257, 520), (9, 64, 128, 257, 520), (15, 48, 64, 385, 400),   # reverse pass: 8 and 15 sequences
+    (19, 16, 32, 193, 200),                                                   # reverse pass: small states
+])
+def test_few_hidden_units_or_tokens(N, d, h, C, L):
+    """Either side of the lines between the block-tiled kernels and the others, on copies of two sequences.  Forward and reverse pass
+    need not be on the same side, nor the reverse pass of a checkpointed call and the forward that saved its states."""
+    x, shape = _inputs(2, L, d, h, C, MLP, with_d_o=True, with_dstate=True)
+    rep = lambda a: np.concatenate([a] * ((N + 1) // 2))[:N]
+    xs = {n: [rep(w) for w in a] if isinstance(a, list) else rep(a) for n, a in x.items()}
+    cut = lambda a: [w[:2] for w in a] if isinstance(a, list) else a[:2]
+    got, hd = util.gpu_forward(xs, impl=E.E2TTT_IMPL_TILED, **shape)
+    assert E.e2ttt_device_status(hd["ws"]) == 0
+    check_forward({n: cut(a) for n, a in got.items()}, util.oracle_forward(x, C, MLP), TOL_BF16, "forward")
+    ref = util.oracle_backward(x, C, MLP)
+    for ckpt in (0, 2):
+        got = util.gpu_backward(xs, impl=E.E2TTT_IMPL_TILED, via_saved_states=True, ckpt_every=ckpt, **shape)
+        check_backward({n: cut(a) for n, a in got.items()}, ref, 2 * TOL_BF16, f"backward, checkpoints {ckpt}")
