@@ -160,7 +160,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     const float* gamma = a.gamma + (size_t)seq * Ls;
 
     if (tid == 0) {
-        if (blockIdx.x == 0 && !a.keep_status) *a.status = 0;  // a wait that gives up does so a second later
         s.dead = 0;
         mbar_init(&s.bar_x, 1);
         mbar_init(&s.bar_v, 1);
@@ -1160,7 +1159,9 @@ int tc_fwd_launch(const TcFwdArgs& a_in, void* stream) {
     if (!make_token_map(&tmK, a.k, rows, box_rows, a.d) || !make_token_map(&tmQ, a.q, rows, box_rows, a.d) ||
         !make_token_map(&tmV, a.v, rows, 16, a.d))
         return (int)cudaErrorInvalidValue;
-    cudaError_t e = cudaSuccess;
+    // Before the launch, not by one of its CTAs: nothing orders that one before a wait that gives up in another
+    cudaError_t e = a.keep_status ? cudaSuccess : cudaMemsetAsync(a.status, 0, sizeof(int), st);
+    if (e != cudaSuccess) return (int)e;
     cudaLaunchConfig_t cfg{};
     // Two CTAs per cluster where they hold all hidden units (h <= 256), if the call then takes fewer waves: 74 clusters of 2 fit the
     // GPU and 33 of 4 (half of whose CTAs had only padding).  With as many waves the four CTAs are kept: each normalises half as many

@@ -121,7 +121,6 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const float* gamma = a.gamma + (size_t)seq * Ls;
 
     if (tid == 0) {
-        if (blockIdx.x == 0 && !a.keep_status) *a.status = 0;  // a wait that gives up does so a second later
         s.dead = 0;
         mbar_init(&s.bar_x, 1);
         mbar_init(&s.bar_v, 1);
@@ -829,7 +828,9 @@ int tc_swiglu_launch(const TcSwigluArgs& a_in, void* stream) {
     const unsigned box_rows = (unsigned)(Cc < 64 ? Cc : 64);
     if (!make_token_map(&tmK, a.k, rows, box_rows, D) || !make_token_map(&tmQ, a.q, rows, box_rows, D) || !make_token_map(&tmV, a.v, rows, 16, D))
         return (int)cudaErrorInvalidValue;
-    cudaError_t e = cudaSuccess;
+    // Before the launch, not by one of its CTAs: nothing orders that one before a wait that gives up in another
+    cudaError_t e = a.keep_status ? cudaSuccess : cudaMemsetAsync(a.status, 0, sizeof(int), st);
+    if (e != cudaSuccess) return (int)e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(a.N * NC));
     cfg.blockDim = dim3(NTHREADS);
