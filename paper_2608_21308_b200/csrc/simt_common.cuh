@@ -5,6 +5,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
+#include "simt_layout.h"
+
 namespace e2ttt {
 
 constexpr int kSimtThreads = 256;
@@ -152,6 +156,54 @@ template <typename Real>
 __device__ void chunk_scalars_warp(const float* eta, const float* beta, const float* gamma, int len, ChunkScalars<Real>* out) {
     if (len <= 64) chunk_scalars_scan<Real, 2>(eta, beta, gamma, len, out);
     else chunk_scalars_scan<Real, kMaxC / 32>(eta, beta, gamma, len, out);
+}
+
+// ---- launch of an any-shape kernel: N clusters of a.cl CTAs -------------------------------------
+// `state`, per device: 0 nothing known, 1 the shared-memory limit is set, 8 or 16 the largest cluster the device grants
+template <typename K, typename A> int simt_launch(K kernel, A a, int threads, size_t smem, std::atomic<int> (&state)[64], cudaStream_t st) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return (int)e;
+    const bool keep = dev >= 0 && dev < 64;
+    int known = keep ? state[dev].load() : 0;
+    if (known == 0) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return (int)e;
+        known = 1;
+    }
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    auto of = [&](int cl) {
+        at[0].val.clusterDim.x = (unsigned)cl;
+        cfg.gridDim = dim3((unsigned)(a.N * cl));
+    };
+    if (a.cl > 8) {
+        if (known < 8)
+            known = simt_granted_cluster(16, [&](int cl) {
+                int n = 0;
+                of(cl);
+                if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+                    cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+                    (void)cudaGetLastError();
+                    return 0;
+                }
+                return n;
+            });
+        if (a.cl > known) a.cl = known;
+    }
+    if (keep && known > state[dev].load()) state[dev] = known;
+    of(a.cl);
+    e = cudaLaunchKernelEx(&cfg, kernel, a);
+    if (e != cudaSuccess) return (int)e;
+    return (int)cudaGetLastError();
 }
 
 // ---- elementwise pass with batched loads ---------------------------------------------------------

@@ -270,30 +270,8 @@ template <typename Real, typename IO, int KIND, bool TC>
 static int launch_fwd(const SimtFwdArgs& a, cudaStream_t st) {
     using Engine = typename std::conditional<TC, TcGemmT<false>, FmaGemm<Real>>::type;
     constexpr size_t smem = Engine::kBytes + sizeof(ChunkScalars<Real>) + (TC ? 1024 : 0);
-    static bool attr_done[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return (int)cudaGetLastError();
-    if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(simt_fwd_kernel<Real, IO, KIND, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(simt_fwd_kernel<Real, IO, KIND, TC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return (int)e;
-        if (dev >= 0 && dev < 64) attr_done[dev] = true;
-    }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(a.N * a.cl));
-    cfg.blockDim = dim3(Engine::kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)a.cl;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, simt_fwd_kernel<Real, IO, KIND, TC>, a);
-    if (e != cudaSuccess) return (int)e;
-    return (int)cudaGetLastError();
+    static std::atomic<int> state[64];
+    return simt_launch(simt_fwd_kernel<Real, IO, KIND, TC>, a, Engine::kThreads, smem, state, st);
 }
 
 int simt_fwd_launch(const SimtFwdArgs& a, int kind, int io_dtype, void* stream) {

@@ -132,6 +132,10 @@ inline int simt_cluster_size(int N, int io_dtype) {
     return cl;
 }
 
+// What of that a device grants: `active(cl)` tells how many clusters of cl CTAs it can run at once.  Above the portable 8 that may be none
+// (how the SMs are spread over processing clusters differs from board to board); every phase runs on any number of CTAs.
+template <typename Q> int simt_granted_cluster(int cl, Q active) { return cl > 8 && active(cl) < 1 ? 8 : cl; }
+
 // launchers (simt_fwd.cu / simt_bwd.cu); return a cudaError_t value as int
 int simt_fwd_launch(const SimtFwdArgs& a, int kind, int io_dtype, void* stream);
 int simt_bwd_launch(const SimtBwdArgs& a, int kind, int io_dtype, void* stream);
