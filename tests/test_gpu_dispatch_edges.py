@@ -144,3 +144,28 @@ def test_few_hidden_units_or_tokens(N, d, h, C, L):
     for ckpt in (0, 2):
         got = util.gpu_backward(xs, impl=E.E2TTT_IMPL_TILED, via_saved_states=True, ckpt_every=ckpt, **shape)
         check_backward({n: cut(a) for n, a in got.items()}, ref, 2 * TOL_BF16, f"backward, checkpoints {ckpt}")
+
+
+@pytest.mark.parametrize("kind,N,h,C,L", [(SWIGLU, 2, 384, 128, 200), (MLP, 2, 512, 96, 100), (SWIGLU, 2, 384, 256, 256)])
+def test_noalloc_forward_where_the_block_tiled_layout_does_not_fit(kind, N, h, C, L):
+    """The last one fits neither layout and is refused.  The others run on the kernels for wider heads: the same two-term products and fp32
+    sums in another order.  A product's operands are off by 2^-17 each at most, so both sides are within a few 1e-5 of the exact result;
+    1e-4 leaves room for the amplification over two chunks.  A lost term of an operand would show as 4e-3."""
+    x, shape = _inputs(N, L, 128, h, C, kind)
+    ref, hd = util.gpu_forward(x, impl=E.E2TTT_IMPL_AUTO, **shape)
+    p = hd["p"]
+    assert E.e2ttt_workspace_bytes(p, 0) > E.E2TTT_NOALLOC_SCRATCH_BYTES
+    o = torch.empty_like(hd["q"])
+    Wf, Mf = [torch.empty_like(w) for w in hd["W"]], [torch.empty_like(w) for w in hd["W"]]
+    args = (p, hd["q"], hd["k"], hd["v"], hd["eta"], hd["beta"], hd["gamma"], hd["W"], hd["M"], o, Wf, Mf)
+    simt = E.make_params(N, 1, L, 128, h, C, kind, E.E2TTT_BF16, 1e-5, E.E2TTT_IMPL_SIMT)
+    if E.e2ttt_workspace_bytes(simt, 0) > E.E2TTT_NOALLOC_SCRATCH_BYTES:
+        with pytest.raises(E.E2TTTError) as ei:
+            E.e2ttt_chunk_fwd_noalloc(*args)
+        assert ei.value.status == -5
+        return
+    E.e2ttt_chunk_fwd_noalloc(*args)
+    assert E.e2ttt_device_status(None) == 0
+    for a, b in zip(Wf + Mf, ref["W"] + ref["M"]):
+        assert util.rel_l2(a.cpu().numpy()[:, 0], b) <= 1e-4
+    assert util.rel_l2(o.float().cpu().numpy()[:, 0], ref["o"]) <= 1e-3  # bf16: a few values round to the other neighbour
