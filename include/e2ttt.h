@@ -218,6 +218,8 @@ E2TTT_API int e2ttt_chunk_bwd_normed(const e2ttt_params* p, const void* q, const
  *   W        in  (host array of device pointers)  the nmat fast-weight matrices, fp32, shapes as above
  *   o        out (device)  [B,H,L,d] io_dtype, 16-byte aligned
  * Needs no workspace; the work is enqueued on `stream`; nothing is allocated and the host is not synchronised.
+ * With no workspace there is no device status word: the bounded waits of the one-token kernel guard bulk loads, which
+ * cannot fail short of a device fault; should one give up all the same, every output of its sequence is NaN.
  * Arithmetic: fp32 throughout (weights are read as fp32, never rounded).  For a few tokens the call is bound
  * by reading W once: 4 * nmat * d * h bytes per (b, h).
  * Returns E2TTT_OK or E2TTT_ERR_NULL / _SHAPE / _DTYPE / _ALIGN / _ARCH / _CUDA. */

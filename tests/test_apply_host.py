@@ -24,6 +24,14 @@ def test_the_cluster_has_started_before_its_shared_memory_is_written(name):
     assert 0 <= arrive < wait < store
 
 
+def test_a_wait_that_gives_up_shows_in_the_outputs():
+    """The decode step has no status word.  The flag that such a wait leaves is looked at before the partial sums are handed over, and
+    again before the CTA gives up its shared memory to copies that may still be under way."""
+    body = kernel("apply_stream_kernel")
+    flag, store, drain = body.find("dead = *(volatile int*)&sh.dead"), body.find("= dead ? __int_as_float"), body.rfind("if (dead)")
+    assert 0 <= body.find("*dead = 1") < flag < store < drain
+
+
 SIZES = r"""
 #include "apply.h"
 #include <cstdio>
