@@ -232,10 +232,13 @@ __global__ void __launch_bounds__(kApThreads, 2) apply_kernel(const ApplyArgs a)
 // ---- one token per sequence: the decode step -----------------------------------------------------------------------------------
 // Bound by HBM (a step reads every weight once).  Every warp streams its own share of the CTA's rows through a ring of its own in
 // shared memory: groups of 8 rows by bulk copies (one for the first matrices, whose rows are contiguous, 8 for column slices of
-// the last), issued one ring ahead by lane 0, so ~100 KB per CTA and two CTAs per SM are in flight whatever the registers hold.
+// the last), issued one ring ahead by lane 0, so 64 to 96 KB per CTA and two CTAs per SM are in flight whatever the registers hold.
+// Pieces of 256 columns (or rows of more than 192 floats) leave room for one slot per warp: it is filled again once the warp has read
+// it, from L2, where the prefetch at the start has brought all of the CTA's weights.  Pieces of 128 columns in three slots were slower,
+// 11.7 -> 14.4 us at 94 sequences and 17.6 -> 22.3 us at 149 (GELU, d = 128, h = 512).
 // The rows of the last matrix do not depend on the activations: their copies are under way while the activations are
 // computed.  Eight dot products are reduced together (9 shuffles), which leaves one row per four lanes: the activation function
-// runs once per row.  128 sequences x SwiGLU d = 128, h = 384 (75.5 MB): 17.8 us with loads through registers.
+// runs once per row.  128 sequences x SwiGLU d = 128, h = 384 (75.5 MB): 20.9 us with loads through registers, 16.4 us.
 __device__ __forceinline__ void ds_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
