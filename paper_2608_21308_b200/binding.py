@@ -157,11 +157,8 @@ def _state_shapes(p):
 def _ptr(t, dtype, shape, name):
     if t is None:
         return None
-    try:
-        if t.is_cuda and t.dtype is dtype and t.is_contiguous() and (shape is None or t.shape == shape):
-            return t.data_ptr()
-    except AttributeError:
-        pass
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.is_contiguous() and (shape is None or t.shape == shape):
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name}: expected a CUDA tensor")
     if t.dtype != dtype:
