@@ -135,8 +135,8 @@ static __device__ void tc_chunk_tails(const float* beta, const float* gamma, int
 }
 
 // 16 consecutive values of a state row <-> global memory.  Every lane has a row of its own (a TMEM lane), so an access of a warp
-// touches 32 sectors whatever its width: 32-byte accesses fill them, 16-byte ones take twice the transactions (saving every
-// every chunk's state at config 2: 2.48 ms with 16-byte stores, 1.88 ms with these).  WIDE: every state pointer is 32-byte aligned
+// touches 32 sectors whatever its width: 32-byte accesses fill them, 16-byte ones take twice the transactions (saving
+// every chunk's state of 64 x 4096 tokens: 2.48 ms with 16-byte stores, 1.84 ms with these).  WIDE: every state pointer is 32-byte aligned
 // (rows are 64-byte multiples apart); a template switch, because a second path inside the chunk loop costs the loop 5 %.
 template <bool WIDE> __device__ __forceinline__ void st_row16(float* p, const float* v) {
     if (WIDE) {

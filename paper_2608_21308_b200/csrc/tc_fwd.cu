@@ -840,7 +840,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                         for (int j = 0; j < 16; ++j) M1[16 * b + j] = fmaf(cbk, M1[16 * b + j], __uint_as_float(ma[j]));
                         if (wr && real1 && col < de) {
                             float* dst = (last ? a.M1_final + head : ck2 + 2 * dh) + off0 + col;
-st_row16<WIDE>(dst, M1 + 16 * b);
+                            st_row16<WIDE>(dst, M1 + 16 * b);
                         }
                     }
                     if (final_block) {
@@ -858,7 +858,7 @@ st_row16<WIDE>(dst, M1 + 16 * b);
                             st_slab16p(s.W1[col >> 6], row, col & 63, p);
                             if (wr && real1 && col < de) {
                                 float* dst = (last ? a.W1_final + head : ck2) + off0 + col;
-st_row16<WIDE>(dst, wa);
+                                st_row16<WIDE>(dst, wa);
                             }
 #pragma unroll
                             for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(fmaf(cmn2, M1[16 * b + j], cwn2 * __uint_as_float(wa[j])));
@@ -883,7 +883,7 @@ st_row16<WIDE>(dst, wa);
                         for (int j = 0; j < 16; ++j) M2[16 * b + j] = fmaf(cbk, M2[16 * b + j], __uint_as_float(ma[j]));
                         if (wr && real2) {
                             float* dst = (last ? a.M2_final + head : ck2 + 3 * dh) + off0 + col;
-st_row16<WIDE>(dst, M2 + 16 * b);
+                            st_row16<WIDE>(dst, M2 + 16 * b);
                         }
                         if (final_block) {
                             uint32_t wa[16];
@@ -895,7 +895,7 @@ st_row16<WIDE>(dst, M2 + 16 * b);
                             st_slab16p(s.W2[col >> 6], row, col & 63, p);
                             if (wr && real2) {
                                 float* dst = (last ? a.W2_final + head : ck2 + dh) + off0 + col;
-st_row16<WIDE>(dst, wa);
+                                st_row16<WIDE>(dst, wa);
                             }
 #pragma unroll
                             for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(fmaf(cmn2, M2[16 * b + j], cwn2 * __uint_as_float(wa[j])));
@@ -933,7 +933,7 @@ st_row16<WIDE>(dst, wa);
                         st_slab16p(s.W1[col >> 6], row, col & 63, p);
                         if (real1 && col < de && (last || save_ck)) {
                             float* dst = (last ? a.W1_final + head : ckn) + off0 + col;
-st_row16<WIDE>(dst, wa);
+                            st_row16<WIDE>(dst, wa);
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(cwn * __uint_as_float(wa[j]));
@@ -967,10 +967,10 @@ st_row16<WIDE>(dst, wa);
                         st_slab16(s.W1[col >> 6], row, col & 63, wn);
                         if (real1 && col < de) {
                             if (last) {
-st_row16<WIDE>(a.W1_final + head + off0 + col, wn);
+                                st_row16<WIDE>(a.W1_final + head + off0 + col, wn);
                             }
                             if (save_ck) {
-st_row16<WIDE>(ckn + off0 + col, wn);
+                                st_row16<WIDE>(ckn + off0 + col, wn);
                             }
                         }
                     }
@@ -992,10 +992,10 @@ st_row16<WIDE>(ckn + off0 + col, wn);
                     for (int j = 0; j < 16; ++j) M1[16 * b + j] = fmaf(cb, M1[16 * b + j], __uint_as_float(ma[j]));
                     if (real1 && col < de) {
                         if (last) {
-st_row16<WIDE>(a.M1_final + head + off0 + col, M1 + 16 * b);
+                            st_row16<WIDE>(a.M1_final + head + off0 + col, M1 + 16 * b);
                         }
                         if (save_ck) {
-st_row16<WIDE>(ckn + 2 * dh + off0 + col, M1 + 16 * b);
+                            st_row16<WIDE>(ckn + 2 * dh + off0 + col, M1 + 16 * b);
                         }
                     }
                 }
@@ -1032,7 +1032,7 @@ st_row16<WIDE>(ckn + 2 * dh + off0 + col, M1 + 16 * b);
                             st_slab16p(s.W2[col >> 6], row, col & 63, p);
                             if (real2 && (last || save_ck)) {
                                 float* dst = (last ? a.W2_final + head : ckn + dh) + off0 + col;
-st_row16<WIDE>(dst, wa);
+                                st_row16<WIDE>(dst, wa);
                             }
 #pragma unroll
                             for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(cwn * __uint_as_float(wa[j]));
@@ -1048,10 +1048,10 @@ st_row16<WIDE>(dst, wa);
                     }
                     if (real2) {
                         if (last) {
-st_row16<WIDE>(a.M2_final + head + off0 + col, M2 + 16 * b);
+                            st_row16<WIDE>(a.M2_final + head + off0 + col, M2 + 16 * b);
                         }
                         if (save_ck) {
-st_row16<WIDE>(ckn + 3 * dh + off0 + col, M2 + 16 * b);
+                            st_row16<WIDE>(ckn + 3 * dh + off0 + col, M2 + 16 * b);
                         }
                     }
                 }
@@ -1107,10 +1107,10 @@ st_row16<WIDE>(ckn + 3 * dh + off0 + col, M2 + 16 * b);
                         st_slab16(s.W2[col >> 6], row, col & 63, wn);
                         if (real2) {
                             if (last) {
-st_row16<WIDE>(a.W2_final + head + off0 + col, wn);
+                                st_row16<WIDE>(a.W2_final + head + off0 + col, wn);
                             }
                             if (save_ck) {
-st_row16<WIDE>(ckn + dh + off0 + col, wn);
+                                st_row16<WIDE>(ckn + dh + off0 + col, wn);
                             }
                         }
                     }

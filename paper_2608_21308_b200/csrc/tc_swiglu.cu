@@ -673,7 +673,7 @@ tc_swiglu_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     for (int j = 0; j < 16; ++j) M12[16 * b + j] = fmaf(cbk, M12[16 * b + j], __uint_as_float(ma[j]));
                     if (wr) {
                         float* dst = (last ? (row < 64 ? a.M1_final : a.M2_final) + head : ck2 + (row < 64 ? 3 : 4) * dh) + off12 + 16 * b;
-st_row16<WIDE>(dst, M12 + 16 * b);
+                        st_row16<WIDE>(dst, M12 + 16 * b);
                     }
                 }
                 if (final_block) {
@@ -688,7 +688,7 @@ st_row16<WIDE>(dst, M12 + 16 * b);
                         st_two_term(s.W12[col >> 6], s.W12lo[col >> 6], row, col & 63, wa);
                         if (wr) {
                             float* dst = (last ? (row < 64 ? a.W1_final : a.W2_final) + head : ck2 + (row < 64 ? 0 : dh)) + off12 + 16 * b;
-st_row16<WIDE>(dst, wa);
+                            st_row16<WIDE>(dst, wa);
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(fmaf(cmn2, M12[16 * b + j], cwn2 * __uint_as_float(wa[j])));
@@ -707,7 +707,7 @@ st_row16<WIDE>(dst, wa);
                     for (int j = 0; j < 16; ++j) M3[j] = fmaf(cbk, M3[j], __uint_as_float(ma[j]));
                     if (wr) {
                         float* dst = (last ? a.M3_final + head : ck2 + 5 * dh) + off3;
-st_row16<WIDE>(dst, M3);
+                        st_row16<WIDE>(dst, M3);
                     }
                     if (final_block) {
                         uint32_t wa[16];
@@ -719,7 +719,7 @@ st_row16<WIDE>(dst, M3);
                         st_slab16p(s.W3, row, 16 * g, p);
                         if (wr) {
                             float* dst = (last ? a.W3_final + head : ck2 + 2 * dh) + off3;
-st_row16<WIDE>(dst, wa);
+                            st_row16<WIDE>(dst, wa);
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(fmaf(cmn2, M3[j], cwn2 * __uint_as_float(wa[j])));
@@ -743,7 +743,7 @@ st_row16<WIDE>(dst, wa);
                 st_two_term(s.W12[col >> 6], s.W12lo[col >> 6], row, col & 63, wa);
                 if (last || save_ck) {
                     float* dst = (last ? (row < 64 ? a.W1_final : a.W2_final) + head : ckn + (row < 64 ? 0 : dh)) + off12 + 16 * b;
-st_row16<WIDE>(dst, wa);
+                    st_row16<WIDE>(dst, wa);
                 }
 #pragma unroll
                 for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(cwn * __uint_as_float(wa[j]));
@@ -760,7 +760,7 @@ st_row16<WIDE>(dst, wa);
                 for (int j = 0; j < 16; ++j) M12[16 * b + j] = fmaf(cb, M12[16 * b + j], __uint_as_float(ma[j]));
                 if (last || save_ck) {
                     float* dst = (last ? (row < 64 ? a.M1_final : a.M2_final) + head : ckn + (row < 64 ? 3 : 4) * dh) + off12 + 16 * b;
-st_row16<WIDE>(dst, M12 + 16 * b);
+                    st_row16<WIDE>(dst, M12 + 16 * b);
                 }
             }
             tmem_wait_st();
@@ -781,7 +781,7 @@ st_row16<WIDE>(dst, M12 + 16 * b);
                 st_slab16p(s.W3, row, 16 * g, p);
                 if (last || save_ck) {
                     float* dst = (last ? a.W3_final + head : ckn + 2 * dh) + off3;
-st_row16<WIDE>(dst, wa);
+                    st_row16<WIDE>(dst, wa);
                 }
 #pragma unroll
                 for (int j = 0; j < 16; ++j) wa[j] = __float_as_uint(cwn * __uint_as_float(wa[j]));
@@ -793,7 +793,7 @@ st_row16<WIDE>(dst, wa);
                 for (int j = 0; j < 16; ++j) M3[j] = fmaf(cb, M3[j], __uint_as_float(ma[j]));
                 if (last || save_ck) {
                     float* dst = (last ? a.M3_final + head : ckn + 5 * dh) + off3;
-st_row16<WIDE>(dst, M3);
+                    st_row16<WIDE>(dst, M3);
                 }
             }
             tmem_wait_st();
