@@ -300,9 +300,10 @@ __device__ __forceinline__ float reduce16(const float (&v)[16], int lane) {
 
 // ---- activations ---------------------------------------------------------------------------------------------------------------
 // The epilogues evaluate them for every token and hidden unit, and were bound by the instructions of erff, expf and the division.
-// Normal distribution function and density: erfc(x) = t exp(P(t) - x^2), t = 1 / (1 + x / 2), P a Chebyshev fit of degree 9 to
-// log(exp(x^2) erfc(x) / t) on t in [0.15, 1], error 6e-8 (beyond, at |z| > 16, the tail is 0 in fp32); the distribution function is
-// within 2.4e-7, where the products that follow round to 16 bits of mantissa.
+// Normal distribution function and density: erfc(x) = t exp(P(t) - x^2), t = 1 / (1 + x / 2), the form of Press et al., Numerical Recipes
+// (erfc by Chebyshev fitting), with a fit of its own: P of degree 9 to log(exp(x^2) erfc(x) / t) on t in [0.15, 1], error 6e-8 (beyond,
+// at |z| > 16, the tail is 0 in fp32).  The distribution function is within 2.6e-7 in fp32, to which the hardware's exponential (3 ulp)
+// and division (2 ulp) may add 3e-7; the products that follow round to 16 bits of mantissa.  The reverse pass recomputes the activations with erff (tile_rec.cuh); the two are as far apart.
 __device__ __forceinline__ void normal_dist(float z, float& cdf, float& pdf) {
     const float x = 0.70710678118f * fabsf(z), x2 = x * x;
     const float t = __fdividef(1.0f, fmaf(0.5f, x, 1.0f));
