@@ -20,6 +20,17 @@ def _inputs(N, L, d, h, C, kind, **kw):
     return inputs.generate(r, **kw), dict(d=d, h=h, C=C, kind=kind, io="bf16")
 
 
+def check_fp32(got, ref, what):
+    """What is returned in fp32.  Every product takes both operands as two bf16 terms (2^-17 of a value is left over); over the few chunks
+    here that comes to 1e-4 at most, where an operand without its second term is off by 2^-9 and shows as 4e-3."""
+    errs = {}
+    for n in ("W", "M", "dW", "dM", "drow_norm", "deta", "dbeta", "dgamma"):
+        if n in got:
+            pairs = zip(got[n], ref[n]) if isinstance(got[n], list) else [(got[n], ref[n])]
+            errs.update({f"{n}{i}": util.rel_l2(a, b) for i, (a, b) in enumerate(pairs)})
+    assert all(e <= 1e-3 for e in errs.values()), f"{what}: {errs}"
+
+
 @pytest.mark.parametrize("normed", [False, True], ids=["plain", "normed"])
 @pytest.mark.parametrize("kind", [MLP, SWIGLU])
 @pytest.mark.parametrize("d,h,C,L", [
@@ -35,14 +46,22 @@ def test_block_tiled_edges(d, h, C, L, kind, normed):
     if normed:
         tgt = targets(x)
         got = gpu_forward_normed(x, tgt, impl=E.E2TTT_IMPL_TILED, **shape)
-        check_forward(got, oracle_fwd(x, tgt, C, kind), TOL_BF16, "block-tiled normed forward")
+        ref = oracle_fwd(x, tgt, C, kind)
+        check_forward(got, ref, TOL_BF16, "block-tiled normed forward")
+        check_fp32(got, ref, "block-tiled normed forward")
         got = gpu_backward_normed(x, tgt, impl=E.E2TTT_IMPL_TILED, via_saved_states=True, **shape)
-        check_backward(got, oracle_bwd(x, tgt, C, kind), 2 * TOL_BF16, "block-tiled normed backward")
+        ref = oracle_bwd(x, tgt, C, kind)
+        check_backward(got, ref, 2 * TOL_BF16, "block-tiled normed backward")
+        check_fp32(got, ref, "block-tiled normed backward")
     else:
         got, hd = util.gpu_forward(x, impl=E.E2TTT_IMPL_TILED, **shape)
         assert E.e2ttt_device_status(hd["ws"]) == 0
-        check_forward(got, util.oracle_forward(x, C, kind), TOL_BF16, "block-tiled forward")
-        check_backward(util.gpu_backward(x, impl=E.E2TTT_IMPL_TILED, **shape), util.oracle_backward(x, C, kind), 2 * TOL_BF16, "block-tiled backward")
+        ref = util.oracle_forward(x, C, kind)
+        check_forward(got, ref, TOL_BF16, "block-tiled forward")
+        check_fp32(got, ref, "block-tiled forward")
+        got, ref = util.gpu_backward(x, impl=E.E2TTT_IMPL_TILED, **shape), util.oracle_backward(x, C, kind)
+        check_backward(got, ref, 2 * TOL_BF16, "block-tiled backward")
+        check_fp32(got, ref, "block-tiled backward")
 
 
 @pytest.mark.parametrize("N,ckpt", [(1, 0), (1, 5), (40, 0), (40, 5)])
@@ -52,6 +71,24 @@ def test_block_tiled_reverse_over_groups_of_chunks(N, ckpt):
     got = util.gpu_backward(x, impl=E.E2TTT_IMPL_TILED, via_saved_states=ckpt > 0, ckpt_every=ckpt, **shape)
     ref = util.gpu_backward(x, impl=E.E2TTT_IMPL_SIMT, **shape)
     check_backward(got, ref, TOL_BF16, f"groups N={N} ckpt={ckpt}")
+    check_fp32(got, ref, f"groups N={N} ckpt={ckpt}")
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("d,h", [(64, 192), (128, 1088)], ids=["chain", "wide"])
+@pytest.mark.parametrize("how", ["plain", "checkpoints", "normed"])
+def test_both_reverse_chains_pass_their_state_from_group_to_group(how, d, h, kind):
+    """11 chunks, groups of 9 at most: the adjoints of the state, those of the row targets (summed over all chunks) and dk's last shares go from
+    one launch to the next, for up to 1024 hidden units and for more; with checkpoints the launches are segments of 4 chunks."""
+    x, shape = _inputs(1, 11 * 16 - 3, d, h, 16, kind, with_d_o=True, with_dstate=True)
+    if how == "normed":
+        tgt = targets(x)
+        got, ref = (gpu_backward_normed(x, tgt, impl=i, via_saved_states=True, **shape) for i in (E.E2TTT_IMPL_TILED, E.E2TTT_IMPL_SIMT))
+    else:
+        ckpt = 4 if how == "checkpoints" else 0
+        got, ref = (util.gpu_backward(x, impl=i, via_saved_states=True, ckpt_every=ckpt, **shape) for i in (E.E2TTT_IMPL_TILED, E.E2TTT_IMPL_SIMT))
+    check_backward(got, ref, TOL_BF16, how)
+    check_fp32(got, ref, how)
 
 
 @pytest.mark.parametrize("normed", [False, True], ids=["plain", "normed"])
