@@ -94,7 +94,7 @@ int other_cluster(const e2ttt_params* p) {  // CTAs per sequence there; 0 if the
 // C = 16 0.80, C = 32 0.96).  The SwiGLU network, with two more products per block, gains everywhere.
 bool tile_forward(const e2ttt_params* p) {
     if (!can_tile(p)) return false;
-    if (p->kind != E2TTT_MLP_GELU) return true;
+    if (p->kind != E2TTT_MLP_GELU || p->h > 1024) return true;  // (h > 1024: see bwd_common)
     const int N = p->B * p->H, dh = p->d * p->h, cl = other_cluster(p);
     if (p->h <= 64 && (cl == 8 ? p->C > 128 : cl == 4 && p->C > 384)) return false;
     if (N > 148) return !((p->C <= 4 && dh <= 16384) || (p->C <= 16 && dh <= 12288) || (p->C <= 32 && dh <= 9216 && p->h <= 256));
@@ -366,7 +366,11 @@ static int bwd_common(const e2ttt_params* p, const void* q, const void* k, const
     const int nchunks = (p->L + p->C - 1) / p->C;
     const int seg = row_norm ? 0 : segment_chunks(p);
     const SimtLayout lay = layout_of(p, true, true, row_norm != nullptr);
-    const bool tile = impl != E2TTT_IMPL_SIMT && tile_backward(p);  // the recomputing forwards too: both keep blocks in one region
+    // States are recomputed by the kernels of the forward, so that every memory plan gives the same bits.  Between the launches of a
+    // checkpointed call the two kinds may alternate: only T and S pass from launch to launch, except in the block-tiled chain for
+    // h > 1024, which leaves operand blocks where the other kernels' intermediates would go (tile_forward).
+    const bool tile = impl != E2TTT_IMPL_SIMT && tile_backward(p);
+    const bool tile_states = impl != E2TTT_IMPL_SIMT && tile_forward(p);
 
     void* ws_data = static_cast<char*>(workspace) + kStatusBytes;
     if (cudaMemsetAsync(workspace, 0, sizeof(int), reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) {
@@ -456,7 +460,7 @@ static int bwd_common(const e2ttt_params* p, const void* q, const void* k, const
             f.row_norm[i] = row_norm ? row_norm[i] : nullptr;
         }
         f.norm_eps = norm_eps;
-        return tile ? tile_fwd_launch(f, p->kind, stream) : simt_fwd_launch(f, p->kind, p->io_dtype, stream);
+        return tile_states ? tile_fwd_launch(f, p->kind, stream) : simt_fwd_launch(f, p->kind, p->io_dtype, stream);
     };
     // The reverse sweep over chunks [first_chunk, first_chunk + n), whose start states sit in lay.ckpt slots 0 .. n-1.
     auto reverse = [&](int first_chunk, int n, bool carry_in, bool carry_out) -> int {

@@ -178,9 +178,12 @@ def test_few_hidden_units_or_tokens(N, d, h, C, L):
     assert E.e2ttt_device_status(hd["ws"]) == 0
     check_forward({n: cut(a) for n, a in got.items()}, util.oracle_forward(x, C, MLP), TOL_BF16, "forward")
     ref = util.oracle_backward(x, C, MLP)
-    for ckpt in (0, 2):
-        got = util.gpu_backward(xs, impl=E.E2TTT_IMPL_TILED, via_saved_states=True, ckpt_every=ckpt, **shape)
-        check_backward({n: cut(a) for n, a in got.items()}, ref, 2 * TOL_BF16, f"backward, checkpoints {ckpt}")
+    plans = [util.gpu_backward(xs, impl=E.E2TTT_IMPL_TILED, via_saved_states=saved, ckpt_every=ckpt, **shape)
+             for saved, ckpt in ((True, 0), (True, 2), (False, 0), (False, 2))]
+    check_backward({n: cut(a) for n, a in plans[0].items()}, ref, 2 * TOL_BF16, "backward")
+    for got in plans[1:]:  # every memory plan: the same bits
+        for n, a in got.items():
+            assert all(np.array_equal(v, w) for v, w in (zip(a, plans[0][n]) if isinstance(a, list) else [(a, plans[0][n])])), n
 
 
 @pytest.mark.parametrize("kind,N,h,C,L", [(SWIGLU, 2, 384, 128, 200), (MLP, 2, 512, 96, 100), (SWIGLU, 2, 384, 256, 256)])
