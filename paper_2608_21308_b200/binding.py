@@ -138,6 +138,7 @@ def _io_torch_dtype(p):
 # ctypes table types are looked up once per (kind, d, h), pointers travel as plain integers, and the current stream
 # is asked for by its handle.  The checks of every argument stay (about 0.4 us per tensor).
 _F32 = torch.float32
+_Tensor = torch.Tensor
 _shape_cache = {}
 
 
@@ -157,7 +158,7 @@ def _state_shapes(p):
 def _ptr(t, dtype, shape, name):
     if t is None:
         return None
-    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.is_contiguous() and (shape is None or t.shape == shape):
+    if isinstance(t, _Tensor) and t.is_cuda and t.dtype is dtype and t.is_contiguous() and (shape is None or t.shape == shape):
         return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name}: expected a CUDA tensor")
