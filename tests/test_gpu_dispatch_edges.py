@@ -186,6 +186,20 @@ def test_few_hidden_units_or_tokens(N, d, h, C, L):
             assert all(np.array_equal(v, w) for v, w in (zip(a, plans[0][n]) if isinstance(a, list) else [(a, plans[0][n])])), n
 
 
+@pytest.mark.parametrize("saved", [True, False], ids=["saved", "recomputed"])
+@pytest.mark.parametrize("d,h,C,L", [(64, 64, 129, 260), (64, 128, 257, 520), (48, 64, 400, 450)], ids=["forward", "reverse", "both"])
+def test_normed_calls_off_the_block_tiled_kernels(d, h, C, L, saved):
+    """Forward, reverse pass or both on the other kernels: the row norms and the states pass from one kind to the other."""
+    x, shape = _inputs(2, L, d, h, C, MLP, with_d_o=True, with_dstate=True)
+    tgt = targets(x)
+    got, ref = gpu_forward_normed(x, tgt, impl=E.E2TTT_IMPL_TILED, **shape), oracle_fwd(x, tgt, C, MLP)
+    check_forward(got, ref, TOL_BF16, "normed forward")
+    check_fp32(got, ref, "normed forward")
+    got, ref = gpu_backward_normed(x, tgt, impl=E.E2TTT_IMPL_TILED, via_saved_states=saved, **shape), oracle_bwd(x, tgt, C, MLP)
+    check_backward(got, ref, 2 * TOL_BF16, "normed backward")
+    check_fp32(got, ref, "normed backward")
+
+
 @pytest.mark.parametrize("kind,N,h,C,L", [(SWIGLU, 2, 384, 128, 200), (MLP, 2, 512, 96, 100), (SWIGLU, 2, 384, 256, 256)])
 def test_noalloc_forward_where_the_block_tiled_layout_does_not_fit(kind, N, h, C, L):
     """The last one fits neither layout and is refused.  The others run on the kernels for wider heads: the same two-term products and fp32
