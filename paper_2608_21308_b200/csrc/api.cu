@@ -115,7 +115,8 @@ bool tile_backward(const e2ttt_params* p) {
 SimtLayout layout_of(const e2ttt_params* p, bool save_states, bool backward, bool normed, bool allow_tile = true) {
     const int nchunks = (p->L + p->C - 1) / p->C;
     const bool tile = allow_tile && can_tile(p) && (save_states || backward || p->impl != E2TTT_IMPL_SIMT);
-    return simt_layout(p->d, p->h, p->C, nmat_of(p->kind), nchunks, save_states, backward, normed ? 0 : segment_chunks(p), tile, p->B * p->H);
+    return simt_layout(p->d, p->h, p->C, nmat_of(p->kind), nchunks, save_states, backward, normed ? 0 : segment_chunks(p), tile, p->B * p->H,
+                       p->io_dtype == E2TTT_F32);
 }
 
 size_t simt_bytes(const e2ttt_params* p, bool save_states, bool backward, bool normed, bool allow_tile = true) {

@@ -160,7 +160,9 @@ __device__ void chunk_scalars_warp(const float* eta, const float* beta, const fl
 
 // ---- launch of an any-shape kernel: N clusters of a.cl CTAs -------------------------------------
 // `state`, per device: 0 nothing known, 1 the shared-memory limit is set, 8 or 16 the largest cluster the device grants
-template <typename K, typename A> int simt_launch(K kernel, A a, int threads, size_t smem, std::atomic<int> (&state)[64], cudaStream_t st) {
+// `more`: the kernel's further arguments
+template <typename K, typename A, typename... Args>
+int simt_launch(K kernel, A a, int threads, size_t smem, std::atomic<int> (&state)[64], cudaStream_t st, Args... more) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
@@ -201,7 +203,7 @@ template <typename K, typename A> int simt_launch(K kernel, A a, int threads, si
     }
     if (keep && known > state[dev].load()) state[dev] = known;
     of(a.cl);
-    e = cudaLaunchKernelEx(&cfg, kernel, a);
+    e = cudaLaunchKernelEx(&cfg, kernel, a, more...);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaGetLastError();
 }

@@ -276,8 +276,7 @@ static int launch_fwd(const SimtFwdArgs& a, cudaStream_t st) {
 
 int simt_fwd_launch(const SimtFwdArgs& a, int kind, int io_dtype, void* stream) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (io_dtype == 0)
-        return kind == 0 ? launch_fwd<double, float, 0, false>(a, st) : launch_fwd<double, float, 1, false>(a, st);
+    if (io_dtype == 0) return f64_fwd_launch(a, kind, stream);
     if (a.tc)
         return kind == 0 ? launch_fwd<float, __nv_bfloat16, 0, true>(a, st) : launch_fwd<float, __nv_bfloat16, 1, true>(a, st);
     return kind == 0 ? launch_fwd<float, __nv_bfloat16, 0, false>(a, st) : launch_fwd<float, __nv_bfloat16, 1, false>(a, st);

@@ -8,6 +8,67 @@
 
 namespace e2ttt {
 
+// ---- fp64 kernels (f64_fwd.cu, f64_bwd.cu; fp32 I/O) -----------------------------------------------------------------------
+// A [tokens x d] result of a contraction over hidden units has few tiles and is cut along k; the parts are added by whoever reads it.
+// From 32 tiles of 16 x 16 on there is work enough for a cluster without.
+constexpr int kF64Parts = 4;
+#ifdef __CUDACC__
+#define E2TTT_HD __host__ __device__
+#else
+#define E2TTT_HD
+#endif
+E2TTT_HD inline int f64_tiles(int M, int N, int T) { return ((M + T - 1) / T) * ((N + T - 1) / T); }
+// 32 x 32 tiles (half the loads per product) where a cluster of 16 has one for every CTA, else 16 x 16
+E2TTT_HD inline int f64_wide(int M, int N) { return M > 16 && N > 16 && f64_tiles(M, N, 16) >= 64; }
+E2TTT_HD inline int f64_parts(int C, int d, int h) {
+    const int n = (h + 63) / 64;
+    return f64_tiles(C, d, 16) >= 32 ? 1 : n < kF64Parts ? n : kF64Parts;
+}
+constexpr size_t kF64SlotBytes = (size_t)64 << 20;  // room for the slots of one call, where one slot per sequence does not take more
+
+struct F64Layout {
+    int G;  // chunks that the reverse pass prepares at a time (slots)
+    // forward: one chunk
+    size_t fK[2], fQ[2], fA, fAq, fc1, fc2, fUk, fUq, fPu, fPuW, fPuM, fPzW[2], fPzM[2];  // fK, fQ: the tokens, by the chunk's parity
+    // reverse pass, chain
+    size_t phb, zb[2], X2, Y2, Pub, Kb, dk, Eb, Ukb, nUkb, kwp;
+    // reverse pass, slots: offsets inside a slot
+    size_t slot, slot_stride;
+    size_t sK, sQ, sAk, sAq, sc1, sc2, se1, se2, szq[2], sPz[2], sPzW[2], sPzM[2], sUk, sUq, sY, sPu, sPuW, sPuM, sUqb, sr, smey, ssc, skwb, sdots;
+};
+
+inline size_t f64_layout(F64Layout& f, size_t o, int N, int d, int h, int C, int nmat, bool backward, int chunks) {
+    auto take = [&](size_t n) { size_t r = o; o += (n + 31) / 32 * 32; return r; };
+    const size_t Ch = (size_t)C * h, Cd = (size_t)C * d, sw = nmat == 3, parts = (size_t)f64_parts(C, d, h);
+    const size_t begin = o;
+    for (int i = 0; i < 2; ++i) { f.fK[i] = take(Cd); f.fQ[i] = take(Cd); }
+    f.fA = take(Ch); f.fAq = take(Ch); f.fc1 = take(Ch); f.fc2 = take(sw * Ch);
+    f.fUk = take(parts * Cd); f.fUq = take(parts * Cd); f.fPu = take(Cd); f.fPuW = take(Cd); f.fPuM = take(Cd);
+    for (int i = 0; i < nmat - 1; ++i) { f.fPzW[i] = take(Ch); f.fPzM[i] = take(Ch); }
+    const size_t end_fwd = o;
+    f.G = 0;
+    if (!backward) return end_fwd;
+    o = begin;
+    f.phb = take(Ch); f.zb[0] = take(Ch); f.zb[1] = take(sw * Ch);
+    f.X2 = take(parts * Cd); f.Y2 = take(parts * Cd); f.Pub = take(parts * Cd); f.Kb = take(parts * Cd); f.dk = take(parts * Cd);
+    f.Eb = take(Cd); f.Ukb = take(Cd); f.nUkb = take(Cd);
+    f.kwp = take((size_t)2 * ((h + 15) / 16) * C);
+    f.slot = o;
+    o = 0;
+    f.sK = take(Cd); f.sQ = take(Cd);
+    f.sAk = take(Ch); f.sAq = take(Ch); f.sc1 = take(Ch); f.sc2 = take(sw * Ch); f.se1 = take(Ch); f.se2 = take(sw * Ch);
+    for (int i = 0; i < nmat - 1; ++i) { f.szq[i] = take(Ch); f.sPz[i] = take(Ch); f.sPzW[i] = take(Ch); f.sPzM[i] = take(Ch); }
+    f.sUk = take(parts * Cd); f.sUq = take(parts * Cd); f.sY = take(Cd);
+    f.sPu = take(Cd); f.sPuW = take(Cd); f.sPuM = take(Cd); f.sUqb = take(Cd);
+    f.sr = take(C); f.smey = take(C); f.ssc = take((size_t)2 * C + 8); f.skwb = take((size_t)2 * C);
+    f.sdots = take((size_t)nmat * f64_tiles(h, d, f64_wide(h, d) ? 32 : 16) * 8 * 3);
+    f.slot_stride = o;
+    const size_t fit = kF64SlotBytes / (o * sizeof(double) * (size_t)N);
+    f.G = fit < 1 ? 1 : fit < (size_t)chunks ? (int)fit : chunks;
+    o = f.slot + f.slot_stride * (size_t)f.G;
+    return o > end_fwd ? o : end_fwd;
+}
+
 struct SimtLayout {
     // running state
     size_t W[3], M[3];
@@ -28,11 +89,14 @@ struct SimtLayout {
     int seg;             // chunks per segment (e2ttt_params.ckpt_every >= 2); 0 = the state of every chunk is kept
     size_t per_seq;      // elements per sequence
     TileLayout tl;       // region of the block-tiled kernels, when `tile`
+    F64Layout fl;        // region of the fp64 kernels, when `f64`
 };
 
 // tile != 0: a call may run on the block-tiled kernels (bf16 I/O, d <= 128): their region shares the space of the SIMT
 // kernels' intermediates (a call uses one of the two), behind the state that both kinds leave for each other.
-inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool save_states, bool backward, int seg = 0, int tile = 0, int N = 1) {
+// f64 != 0: fp32 I/O, which the fp64 kernels serve; their region follows the states.
+inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool save_states, bool backward, int seg = 0, int tile = 0, int N = 1,
+                              int f64 = 0) {
     SimtLayout l{};
     size_t o = 0;
     const size_t dh = (size_t)d * h;
@@ -48,6 +112,11 @@ inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool s
     } else {
         l.ckpt = take(save_states ? (size_t)(nchunks + 1) * 2 * nmat * dh : 0);
         l.cck = 0;
+    }
+    const int chunks = l.seg > 0 && l.seg < nchunks ? l.seg : nchunks;  // of a launch sequence of the reverse pass
+    if (f64) {
+        l.per_seq = f64_layout(l.fl, o, N, d, h, C, nmat, backward, chunks);
+        return l;
     }
     const size_t begin = o;
     l.Z1 = take((size_t)2 * C * h); l.Z2 = take((size_t)2 * C * h); l.A = take((size_t)2 * C * h);
@@ -67,7 +136,7 @@ inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool s
     }
     l.splitk = take((size_t)2 * 8 * 128 * 64);
     if (tile) {
-        const size_t end = tile_layout(l.tl, begin, N, d, h, C, nmat, backward, l.seg > 0 && l.seg < nchunks ? l.seg : nchunks);
+        const size_t end = tile_layout(l.tl, begin, N, d, h, C, nmat, backward, chunks);
         if (end > o) o = end;
     }
     l.per_seq = o;
@@ -139,6 +208,9 @@ template <typename Q> int simt_granted_cluster(int cl, Q active) { return cl > 8
 // launchers (simt_fwd.cu / simt_bwd.cu); return a cudaError_t value as int
 int simt_fwd_launch(const SimtFwdArgs& a, int kind, int io_dtype, void* stream);
 int simt_bwd_launch(const SimtBwdArgs& a, int kind, int io_dtype, void* stream);
+// fp32 I/O (f64_fwd.cu / f64_bwd.cu); the layout must have been made with `f64`
+int f64_fwd_launch(const SimtFwdArgs& a, int kind, void* stream);
+int f64_bwd_launch(const SimtBwdArgs& a, int kind, void* stream);
 // the same calls on the block-tiled kernels (tile_fwd.cu / tile_bwd.cu); the layout must have been made with `tile`
 int tile_fwd_launch(const SimtFwdArgs& a, int kind, void* stream);
 int tile_bwd_launch(const SimtBwdArgs& a, int kind, void* stream);
