@@ -1,6 +1,6 @@
 // Forward for fp32 I/O: Algorithm 1 chunk after chunk in fp64, any d, h, C and both networks.  A cluster of 1-16 CTAs per sequence, five
 // phases per chunk (f64_common.cuh): activations of the keys | u of the keys, activations of the queries | rows of the keys, the next
-// chunk's tokens and scalar kernels | adjoint of z, u of the queries | state transition, rows of the queries.
+// chunk's tokens and scalar kernels and the rows of the queries of the one before | adjoint of z, u of the queries | state transition.
 #include "f64_common.cuh"
 
 namespace e2ttt {
@@ -118,11 +118,23 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_fwd_kernel(const SimtFwdAr
 
     auto u_row = [&](size_t up, int m, int i) { return f64_parts_at(ws + up, (size_t)m * d + i, parts, pstride); };
     const double inv = 1.0 / d;
+    auto output_row = [&](int c, int m) {  // o = q + LN(u)
+        const size_t row = ((size_t)c * C + m) * d;
+        double su = 0.0;
+#pragma unroll 2
+        for (int i = lane; i < d; i += 32) su += u_row(fl.fUq, m, i);
+        const double mu = warp_sum(su) * inv;
+        double var = 0.0;
+#pragma unroll 2
+        for (int i = lane; i < d; i += 32) { const double x = u_row(fl.fUq, m, i) - mu; var += x * x; }
+        const double r = r_rsqrt(warp_sum(var) * inv + (double)a.eps);
+#pragma unroll 2
+        for (int i = lane; i < d; i += 32) o[row + i] = (float)((double)q[row + i] + (u_row(fl.fUq, m, i) - mu) * r);
+    };
     F64Ctx cx{};
     for (int c = 0; c < a.nchunks; ++c) {
         const int s = c * C, len = min(C, L - s);
         const float* kc = k + (size_t)s * d;
-        const float* qc = q + (size_t)s * d;
         const float* vc = v + (size_t)s * d;
         const ChunkScalars<double>& sc = sh.sc[c & 1];
         cx.len = len;
@@ -141,7 +153,11 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_fwd_kernel(const SimtFwdAr
             tokens(c + 1);
             scalars(c + 1);
         }
-        for (int m = rank + CL * warp; m < len; m += CL * kF64Warps) {
+        for (int m = rank + CL * warp; m < len + (a.o && c > 0 ? C : 0); m += CL * kF64Warps) {
+            if (m >= len) {  // rows of the queries of the chunk before
+                output_row(c - 1, m - len);
+                continue;
+            }
             double su = 0.0;
             double* pu = ws + fl.fPu + (size_t)m * d;
 #pragma unroll 2
@@ -179,20 +195,6 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_fwd_kernel(const SimtFwdAr
         else if (a.save_states == 2 && c + 1 < a.nchunks && (c + 1) % lay.seg == 0) slot = (c + 1) / lay.seg;
         cx.save = slot < 0 ? -1 : (long long)(slot * state_bytes);
         run(odd ? kFUpd1 : kFUpd, (odd ? kFUpd1 : kFUpd) + NMAT);
-        if (a.o)
-            for (int m = rank + CL * warp; m < len; m += CL * kF64Warps) {
-                double su = 0.0;
-#pragma unroll 2
-                for (int i = lane; i < d; i += 32) su += u_row(fl.fUq, m, i);
-                const double mu = warp_sum(su) * inv;
-                double var = 0.0;
-#pragma unroll 2
-                for (int i = lane; i < d; i += 32) { const double x = u_row(fl.fUq, m, i) - mu; var += x * x; }
-                const double r = r_rsqrt(warp_sum(var) * inv + (double)a.eps);
-#pragma unroll 2
-                for (int i = lane; i < d; i += 32)
-                    o[(size_t)(s + m) * d + i] = (float)((double)qc[(size_t)m * d + i] + (u_row(fl.fUq, m, i) - mu) * r);
-            }
         phase_sync(CL);
         // post-chunk normalisation (optional): every row w of every W_i becomes n w / (||w|| + eps_n); one warp per row
         if (normed) {
@@ -220,6 +222,8 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_fwd_kernel(const SimtFwdAr
             phase_sync(CL);
         }
     }
+    if (a.o)
+        for (int m = rank + CL * warp; m < L - (a.nchunks - 1) * C; m += CL * kF64Warps) output_row(a.nchunks - 1, m);
     for (int i = 0; i < NMAT; ++i) {
         if (!a.W_final[i]) continue;  // recomputation for the reverse pass: only the saved states matter
         float* wf = a.W_final[i] + (size_t)seq * dh;
