@@ -7,7 +7,7 @@ namespace e2ttt {
 
 namespace {
 
-enum { kFK, kFK1, kFQ, kFQ1, kFU, kFPz, kFUq, kFUpd, kFUpd1 = kFUpd + 3, kFJobs = kFUpd1 + 3 };
+enum { kFK, kFK1, kFU, kFQ, kFPz, kFUq, kFUpd, kFUpd1 = kFUpd + 3, kFJobs = kFUpd1 + 3 };
 struct F64FwdShared {
     F64Job job[kFJobs];
     ChunkScalars<double> sc[2];  // by the chunk's parity
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_fwd_kernel(const SimtFwdAr
     // a chunk's tokens -> fp64, for the products
     auto tokens = [&](int c) {
         const size_t e0 = (size_t)c * C * d, n = (size_t)min(C, L - c * C) * d;
-        double *kt = ws + fl.fK[c & 1], *qt = ws + fl.fQ[c & 1];
+        double *kt = ws + fl.fK[c & 1], *qt = ws + fl.fQ;
         for (size_t e = tid + (size_t)rank * kF64Threads; e < n; e += (size_t)kF64Threads * CL) {
             kt[e] = (double)k[e0 + e];
             qt[e] = (double)q[e0 + e];
@@ -81,8 +81,8 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_fwd_kernel(const SimtFwdAr
             act(j, fl.fK[b], fl.fA);
             f64_out(j, 1, f64_ptr(ws + fl.fc1));
             if (sw) f64_out(j, 2, f64_ptr(ws + fl.fc2));
-            act(sh.job[b ? kFQ1 : kFQ], fl.fQ[b], fl.fAq);
         }
+        act(sh.job[kFQ], fl.fQ, fl.fAq);
         auto to_u = [&](F64Job& j, size_t x, size_t out) {
             f64_make(j, kEpiStore, d, -1 - C, 1, 1, 1, d, sw, parts);
             f64_seg(j, h, f64_op(Wl, h, 1), f64_op(ws + x, h, 1));
@@ -145,8 +145,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_fwd_kernel(const SimtFwdAr
         const int odd = c & 1;
         run(kFK + odd, kFK + odd + 1);
         phase_sync(CL);
-        run(kFU, kFU + 1);
-        if (a.o) run(kFQ + odd, kFQ + odd + 1);
+        run(kFU, a.o ? kFQ + 1 : kFQ);
         phase_sync(CL);
         // Algorithm 1 line 3: layer norm, e = f(k) - v and pu = dL/du for the key rows; tokens and scalars of the next chunk
         if (c + 1 < a.nchunks) {

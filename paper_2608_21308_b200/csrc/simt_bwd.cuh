@@ -10,7 +10,7 @@
 //   GELU MLP : hidden a = gelu(z1)                 pz1 = ph gelu'(z1)
 //   SwiGLU   : hidden a = silu(z1) z2              pz1 = ph z2 silu'(z1),  pz2 = ph silu(z1)
 // The kernel is large (23 products, each with its own staging and epilogue), so every arithmetic has a file of its own: simt_bwd.cu
-// (fp32 FMAs and the dispatch), simt_bwd_f64.cu, simt_bwd_tc.cu.
+// (fp32 FMAs and the dispatch), simt_bwd_tc.cu; fp32 I/O has kernels of its own (f64_bwd.cu).
 #pragma once
 #include <type_traits>
 

@@ -29,7 +29,7 @@ constexpr size_t kF64SlotBytes = (size_t)64 << 20;  // room for the slots of one
 struct F64Layout {
     int G;  // chunks that the reverse pass prepares at a time (slots)
     // forward: one chunk
-    size_t fK[2], fQ[2], fA, fAq, fc1, fc2, fUk, fUq, fPu, fPuW, fPuM, fPzW[2], fPzM[2];  // fK, fQ: the tokens, by the chunk's parity
+    size_t fK[2], fQ, fA, fAq, fc1, fc2, fUk, fUq, fPu, fPuW, fPuM, fPzW[2], fPzM[2];  // fK: the keys, by the chunk's parity
     // reverse pass, chain
     size_t phb, zb[2], X2, Y2, Pub, Kb, dk, Eb, Ukb, nUkb, kwp;
     // reverse pass, slots: offsets inside a slot
@@ -41,10 +41,14 @@ inline size_t f64_layout(F64Layout& f, size_t o, int N, int d, int h, int C, int
     auto take = [&](size_t n) { size_t r = o; o += (n + 31) / 32 * 32; return r; };
     const size_t Ch = (size_t)C * h, Cd = (size_t)C * d, sw = nmat == 3, parts = (size_t)f64_parts(C, d, h);
     const size_t begin = o;
-    for (int i = 0; i < 2; ++i) { f.fK[i] = take(Cd); f.fQ[i] = take(Cd); }
+    f.fK[0] = take(Cd); f.fK[1] = take(Cd); f.fQ = take(Cd);
     f.fA = take(Ch); f.fAq = take(Ch); f.fc1 = take(Ch); f.fc2 = take(sw * Ch);
-    f.fUk = take(parts * Cd); f.fUq = take(parts * Cd); f.fPu = take(Cd); f.fPuW = take(Cd); f.fPuM = take(Cd);
-    for (int i = 0; i < nmat - 1; ++i) { f.fPzW[i] = take(Ch); f.fPzM[i] = take(Ch); }
+    f.fUk = take(parts * Cd); f.fUq = take(parts * Cd); f.fPu = take(Cd);
+    // (written element by element over what they are made of, so that a call without saved states needs little more than its state)
+    f.fPuW = f.fUk;
+    f.fPuM = parts > 1 ? f.fUk + Cd : take(Cd);
+    f.fPzW[0] = f.fc1; f.fPzW[1] = f.fc2;
+    for (int i = 0; i < nmat - 1; ++i) f.fPzM[i] = take(Ch);
     const size_t end_fwd = o;
     f.G = 0;
     if (!backward) return end_fwd;
@@ -94,7 +98,7 @@ struct SimtLayout {
 
 // tile != 0: a call may run on the block-tiled kernels (bf16 I/O, d <= 128): their region shares the space of the SIMT
 // kernels' intermediates (a call uses one of the two), behind the state that both kinds leave for each other.
-// f64 != 0: fp32 I/O, which the fp64 kernels serve; their region follows the states.
+// f64 != 0: fp32 I/O, which the fp64 kernels serve; their region lies in the same place.
 inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool save_states, bool backward, int seg = 0, int tile = 0, int N = 1,
                               int f64 = 0) {
     SimtLayout l{};
@@ -114,10 +118,6 @@ inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool s
         l.cck = 0;
     }
     const int chunks = l.seg > 0 && l.seg < nchunks ? l.seg : nchunks;  // of a launch sequence of the reverse pass
-    if (f64) {
-        l.per_seq = f64_layout(l.fl, o, N, d, h, C, nmat, backward, chunks);
-        return l;
-    }
     const size_t begin = o;
     l.Z1 = take((size_t)2 * C * h); l.Z2 = take((size_t)2 * C * h); l.A = take((size_t)2 * C * h);
     l.U = take((size_t)2 * C * d); l.Pu = take((size_t)C * d);
@@ -137,6 +137,10 @@ inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool s
     l.splitk = take((size_t)2 * 8 * 128 * 64);
     if (tile) {
         const size_t end = tile_layout(l.tl, begin, N, d, h, C, nmat, backward, chunks);
+        if (end > o) o = end;
+    }
+    if (f64) {
+        const size_t end = f64_layout(l.fl, begin, N, d, h, C, nmat, backward, chunks);
         if (end > o) o = end;
     }
     l.per_seq = o;

@@ -12,7 +12,7 @@
 //            128 registers per thread, does not: the batches made the reverse pass spill (d = 160: 5-10 % slower).
 // Output tiles are dealt round-robin to the `nranks` CTAs of the sequence's cluster; run() ends with phase_sync().
 //
-//   FmaGemm<Real> : CUDA-core FMAs in the kernel's own precision (fp64 for fp32 I/O, fp32 for bf16 I/O).
+//   FmaGemm<Real> : CUDA-core FMAs in fp32 (bf16 I/O, impl SIMT).
 //   TcGemm        : the 5th-generation tensor cores (tcgen05.mma, fp32 accumulation in tensor memory).  Every fp32
 //                   operand x is staged as two bf16 numbers, hi = bf16(x) and lo = bf16(x - hi), and a product is
 //                   three MMAs, hi*hi + hi*lo + lo*hi: the dropped lo*lo term and the residual of the split are

@@ -1,0 +1,58 @@
+"""fp32 I/O on the fp64 kernels (csrc/f64_*.cu) at the edges of their tiles, parts and groups of chunks, against the oracle."""
+import pytest
+
+from paper_2608_21308_b200 import binding as E
+from paper_2608_21308_b200 import inputs
+from tests import util
+from tests.test_gpu_normed import gpu_backward_normed, oracle_bwd, targets
+from tests.test_gpu_parity import check_backward, check_forward
+
+pytestmark = pytest.mark.gpu
+MLP, SWIGLU = inputs.KIND_MLP, inputs.KIND_SWIGLU
+# fp64 inside, rounded once to fp32 (2^-24 of a value); the oracle's sums are in another order, which in fp64 does not show
+TOL = 1e-6
+
+
+def _inputs(N, L, d, h, C, kind):
+    r = inputs.paper_regime(inputs.Recipe(B=N, H=1, L=L, d=d, h=h, C=C, kind=kind, io="f32", seed=17, m_std=0.002))
+    return inputs.generate(r, with_d_o=True, with_dstate=True), dict(d=d, h=h, C=C, kind=kind, io="f32")
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("N,d,h,C,L", [
+    (1, 1, 1, 1, 3),        # a value in every direction
+    (2, 16, 16, 16, 33),    # whole tiles; a chunk of one token
+    (8, 17, 33, 15, 40),    # one past a tile; clusters of 8
+    (1, 48, 336, 24, 31),   # 63 tiles of 16 x 16: the last with narrow tiles
+    (3, 64, 256, 16, 50),   # 64: wide tiles of the state, narrow ones of the tokens
+    (1, 40, 130, 65, 130),  # contractions of two slices and a remainder, in three parts
+    (75, 33, 70, 33, 66),   # one CTA per sequence
+    (1, 128, 136, 300, 310),# [tokens x d] results uncut
+    (9, 128, 384, 64, 300), # groups of three chunks (SwiGLU two), the last shorter
+])
+def test_forward_and_reverse_pass(N, d, h, C, L, kind):
+    x, shape = _inputs(N, L, d, h, C, kind)
+    got, hd = util.gpu_forward(x, **shape)
+    assert E.e2ttt_device_status(hd["ws"]) == 0
+    check_forward(got, util.oracle_forward(x, C, kind), TOL, "fp64 forward")
+    check_backward(util.gpu_backward(x, via_saved_states=True, **shape), util.oracle_backward(x, C, kind), TOL, "fp64 reverse pass")
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+def test_normalised_reverse_pass_over_groups_of_chunks(kind):
+    x, shape = _inputs(9, 5 * 64 - 20, 128, 384, 64, kind)
+    tgt = targets(x)
+    check_backward(gpu_backward_normed(x, tgt, impl=E.E2TTT_IMPL_AUTO, via_saved_states=True, **shape), oracle_bwd(x, tgt, 64, kind), 1e-5, "fp64 normed reverse pass")
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+def test_results_do_not_depend_on_the_cluster(kind):
+    """One sequence (a cluster of 16) and the same one among 80 (a CTA each): the same bits."""
+    import numpy as np
+
+    x, shape = _inputs(1, 70, 40, 130, 16, kind)
+    many = {n: [np.concatenate([w] * 80) for w in a] if isinstance(a, list) else np.concatenate([a] * 80) for n, a in x.items()}
+    one, all_ = util.gpu_backward(x, **shape), util.gpu_backward(many, **shape)
+    for n, a in one.items():
+        for p, q in zip(a, all_[n]) if isinstance(a, list) else [(a, all_[n])]:
+            assert np.array_equal(np.asarray(p)[0], np.asarray(q)[0]) and np.array_equal(np.asarray(p)[0], np.asarray(q)[79]), n

@@ -46,3 +46,33 @@ def test_a_short_training_call_asks_for_one_chunks_slots():
     """16 sequences of one chunk, d = 128, h = 512: 9.0 MB each, of which one slot is 1.83 MB (16 slots would make it 36.4 MB)."""
     p = E.make_params(1, 16, 64, 128, 512, 64, E.E2TTT_MLP_GELU, E.E2TTT_BF16, 1e-5, E.E2TTT_IMPL_AUTO)
     assert E.e2ttt_workspace_bytes(p, 1) < 16 * 9.5e6
+
+
+F64 = r"""
+#include "simt_layout.h"
+#include <initializer_list>
+using namespace e2ttt;
+int main() {
+    for (int N : {1, 13, 64, 2048})
+        for (int d : {1, 64, 128, 1024})
+            for (int h : {1, 256, 8192})
+                for (int C : {1, 16, 64, 512})
+                    for (int nmat : {2, 3})
+                        for (int nchunks : {1, 5, 300})
+                            for (int seg : {0, 4}) {
+                                const SimtLayout l = simt_layout(d, h, C, nmat, nchunks, true, true, seg, 0, N, 1);
+                                const F64Layout& f = l.fl;
+                                const int chunks = seg > 0 && seg < nchunks ? seg : nchunks;
+                                if (f.G < 1 || f.G > chunks) return 1;
+                                if (f.G > 1 && f.slot_stride * 8 * f.G * N > kF64SlotBytes) return 2;
+                                if (f.slot + f.slot_stride * f.G > l.per_seq) return 3;
+                            }
+    return 0;
+}
+"""
+
+
+def test_slots_of_the_fp64_reverse_pass_are_bounded(tmp_path):
+    (tmp_path / "f64.cpp").write_text(F64)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", str(CSRC), str(tmp_path / "f64.cpp"), "-o", str(tmp_path / "f64")], check=True)
+    assert subprocess.run([str(tmp_path / "f64")]).returncode == 0
