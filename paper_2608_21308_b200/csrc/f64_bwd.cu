@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_prepare_kernel(const F64Gr
     cx.len = len;
     cx.kW = sh.sc.kW;
     cx.kM = sh.sc.kM;
-    auto run = [&](int j0, int j1) { f64_jobs(sh.job, j0, j1, cx, rank, CL, f64_smem); };
+    auto run = [&](int j0, int j1) { f64_jobs<kF64Bwd>(sh.job, j0, j1, cx, rank, CL, f64_smem); };
     auto u_row = [&](size_t up, int m, int i) { return f64_parts_at(sl + up, (size_t)m * d + i, parts, pstride); };
     const double inv = 1.0 / d;
 
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) f64_chain_kernel(const F64Grou
     F64Ctx cx{};
     cx.kW = sh.kW;
     cx.kM = sh.kM;
-    auto run = [&](int j0, int j1) { f64_jobs(sh.job, j0, j1, cx, rank, CL, f64_smem); };
+    auto run = [&](int j0, int j1) { f64_jobs<kF64Bwd>(sh.job, j0, j1, cx, rank, CL, f64_smem); };
     auto dk_rows = [&](int c) {
         const int s = c * C, len = min(C, a.L - s);
         for (int t = rank + CL * warp; t < len; t += CL * kF64Warps)
@@ -501,15 +501,15 @@ int f64_bwd_launch(const SimtBwdArgs& a, int kind, void* stream) {
         // a cluster per chunk and sequence, as large as one wave allows
         ga.N = a.N * ga.ng;
         ga.cl = simt_cluster_size(ga.N, 1);
-        int rc = simt_launch(f64_prepare_kernel, ga, kF64Threads, prepare_smem, state[0], st, sw);
+        int rc = simt_launch(f64_prepare_kernel, ga, kF64Threads, prepare_smem, prepare_smem, state[0], st, sw);
         if (rc) return rc;
         ga.N = a.N;
         ga.cl = a.cl;
-        rc = simt_launch(f64_chain_kernel, ga, kF64Threads, chain_smem, state[1], st, sw);
+        rc = simt_launch(f64_chain_kernel, ga, kF64Threads, chain_smem, chain_smem, state[1], st, sw);
         if (rc) return rc;
         ga.N = a.N * ga.ng;
         ga.cl = 1;
-        rc = simt_launch(f64_gate_kernel, ga, kF64Threads, sizeof(F64GateShared), state[2], st, sw);
+        rc = simt_launch(f64_gate_kernel, ga, kF64Threads, sizeof(F64GateShared), sizeof(F64GateShared), state[2], st, sw);
         if (rc) return rc;
         end = ga.c0;
     }

@@ -43,18 +43,25 @@ struct F64Ctx {
     double cw, cm, cb;
     const double *kW, *kM;  // shared memory
     long long save;         // kEpiUpdate: bytes from results 2, 3 to the slot that takes the new state, -1: none
+    bool last;              // kEpiUpdate: the new state is the call's result: to 4, 5 (floats) instead of 0, 1
 };
 
 // Staging of one product: two stages.  Rows of ROW doubles per k: the fragments' loads (4 k x 4 neighbouring rows a half-warp) are free of
-// bank conflicts at ROW = 4 mod 16.  Four operands run in 16 x 16 tiles only
-template <int NA, int T> struct F64Smem {
+// bank conflicts at ROW = 4 mod 16.  Four operands run in 16 x 16 tiles only.  MODE: whose products, and with kF64FwdSmall (two CTAs on an SM) a
+// unit's sums lie over the slice that was multiplied last, a barrier later.
+enum { kF64Bwd, kF64Fwd, kF64FwdSmall };
+template <int NA, int T, int MODE> struct F64Smem {
+    static constexpr bool SMALL = MODE == kF64FwdSmall;
     static constexpr int KS = T == 16 ? 64 : 32, SPLIT = T == 16 ? 2 : 1, ROW = T + 4;
-    static constexpr int PRE = NA == 4 ? 6 : 4;
+    static constexpr int PRE = SMALL ? 2 : NA == 4 ? 6 : 4;
     double a[2][NA + 1][KS][ROW];  // b is the last
-    double part[NA][SPLIT][T * T];
+    double sums[SMALL ? 1 : NA * SPLIT][SMALL ? 1 : T * T];
     double pre[2][PRE][T * T];
+    __device__ __forceinline__ double* part(int stage, int i) { return SMALL ? &a[stage][0][0][0] + i * (T * T) : sums[i]; }
+    static_assert(!SMALL || NA * SPLIT * T * T <= (NA + 1) * KS * ROW);
 };
-constexpr size_t kF64TileSmem = sizeof(F64Smem<4, 16>) > sizeof(F64Smem<2, 32>) ? sizeof(F64Smem<4, 16>) : sizeof(F64Smem<2, 32>);
+constexpr size_t kF64TileSmem = sizeof(F64Smem<4, 16, kF64Bwd>) > sizeof(F64Smem<2, 32, kF64Bwd>) ? sizeof(F64Smem<4, 16, kF64Bwd>) : sizeof(F64Smem<2, 32, kF64Bwd>);
+static_assert(sizeof(F64Smem<2, 32, kF64Fwd>) <= kF64FwdTile && sizeof(F64Smem<2, 32, kF64FwdSmall>) <= f64_small_tile(true) && sizeof(F64Smem<2, 16, kF64FwdSmall>) <= f64_small_tile(false));
 
 __device__ __forceinline__ void f64_copy(uint32_t dst, const void* src, bool in) {  // 8 bytes; zeros where !in
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(in ? 8 : 0) : "memory");
@@ -96,8 +103,8 @@ static __device__ __noinline__ F64Act f64_act(int sw, int deriv, double z1, doub
 // T = 32: 32-deep slices.  The next slice is on its way (cp.async: no register holds it) while one is multiplied, by fp64 MMAs: they run
 // no faster than FMAs, but a shared-memory access feeds four times as many products (2 x 2 FMAs per thread took 70 cycles for each of
 // the 16 steps of a slice, all of it the port of shared memory).
-template <int NA, int T> static __device__ __noinline__ void f64_units(const F64Job& jb, const F64Ctx& cx, int first, int step, unsigned char* smem) {
-    using S = F64Smem<NA, T>;
+template <int NA, int T, int MODE> static __device__ __noinline__ void f64_units(const F64Job& jb, const F64Ctx& cx, int first, int step, unsigned char* smem) {
+    using S = F64Smem<NA, T, MODE>;
     constexpr int KS = S::KS, SPLIT = S::SPLIT, PER = T * KS / kF64Threads, EL = T * T / kF64Threads;
     constexpr int NT = T == 16 ? 1 : 2;  // 8 x 8 tiles per warp, below one another
     S& sm = *reinterpret_cast<S*>(smem);
@@ -206,6 +213,7 @@ template <int NA, int T> static __device__ __noinline__ void f64_units(const F64
             }
         }
         if (mcloses) {
+            if (S::SMALL) __syncthreads();
 #pragma unroll
             for (int a = 0; a < NA; ++a)
 #pragma unroll
@@ -213,13 +221,13 @@ template <int NA, int T> static __device__ __noinline__ void f64_units(const F64
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const int m = wm + 8 * t + (lane >> 2), n = wn + 2 * (lane & 3) + j;
-                        sm.part[a][wk][mf ? n * T + m : m * T + n] = acc[a][t][j];
+                        sm.part(ms, a * SPLIT + wk)[mf ? n * T + m : m * T + n] = acc[a][t][j];
                     }
             __syncthreads();
             // x(e, a): result of element e; P(e, i): what it combines with; put(e, i, v): result i
             auto x = [&](int e, int a) {
-                double s = sm.part[a][0][tid + e * kF64Threads];
-                if (SPLIT == 2) s += sm.part[a][SPLIT - 1][tid + e * kF64Threads];
+                double s = sm.part(ms, a * SPLIT)[tid + e * kF64Threads];
+                if (SPLIT == 2) s += sm.part(ms, a * SPLIT + 1)[tid + e * kF64Threads];
                 return s;
             };
             auto P = [&](int e, int i) { return sm.pre[ms][i][tid + e * kF64Threads]; };
@@ -263,13 +271,13 @@ template <int NA, int T> static __device__ __noinline__ void f64_units(const F64
                             }
                         }
                     }
-                } else if (epi == kEpiDq) {  // dq = d_o + ..
+                } else if (MODE == kF64Bwd && epi == kEpiDq) {  // dq = d_o + ..
                     float* o = reinterpret_cast<float*>(out(0));
                     const float* y = reinterpret_cast<const float*>(jb.ptr[kF64Aux].p);
 #pragma unroll
                     for (int e = 0; e < EL; ++e)
                         if (in(e)) o[off(e)] = (float)((double)y[off(e)] + x(e, 0));
-                } else if (epi == kEpiZ) {  // adjoint of z: what came through pz, and through the hidden activation (x is minus its adjoint)
+                } else if (MODE == kF64Bwd && epi == kEpiZ) {  // adjoint of z: what came through pz, and through the hidden activation (x is minus its adjoint)
 #pragma unroll 1
                     for (int i = 0; i < npre; i += 2) {
                         double* o = out(i / 2);
@@ -277,7 +285,7 @@ template <int NA, int T> static __device__ __noinline__ void f64_units(const F64
                         for (int e = 0; e < EL; ++e)
                             if (in(e)) o[off(e)] = P(e, i) - x(e, 0) * P(e, i + 1);
                     }
-                } else if (epi == kEpiT) {  // p: T, S, W, M of the chunk's start; the carries' adjoints
+                } else if (MODE == kF64Bwd && epi == kEpiT) {  // p: T, S, W, M of the chunk's start; the carries' adjoints
                     double d0 = 0.0, d1 = 0.0, d2 = 0.0;
                     double *ot = out(0), *os = out(1);
 #pragma unroll
@@ -297,7 +305,7 @@ template <int NA, int T> static __device__ __noinline__ void f64_units(const F64
                     }
                 }
             }
-            if constexpr (NA == 2) {
+            if constexpr (NA == 2 && MODE != kF64Bwd) {
                 if (epi == kEpiUpdate) {  // the state transition; G_t = -grad: the aggregations enter with a minus sign
                     double *ow = out(0), *om_ = out(1), *sw = nullptr, *sm_ = nullptr;
                     if (cx.save >= 0) {
@@ -308,14 +316,19 @@ template <int NA, int T> static __device__ __noinline__ void f64_units(const F64
                     for (int e = 0; e < EL; ++e)
                         if (in(e)) {
                             const double w = cx.cw * P(e, 0) + cx.cm * P(e, 1) - x(e, 0), mm = cx.cb * P(e, 1) - x(e, 1);
-                            ow[off(e)] = w;
-                            om_[off(e)] = mm;
+                            if (cx.last) {
+                                reinterpret_cast<float*>(out(4))[off(e)] = (float)w;
+                                reinterpret_cast<float*>(out(5))[off(e)] = (float)mm;
+                            } else {
+                                ow[off(e)] = w;
+                                om_[off(e)] = mm;
+                            }
                             if (sw) sw[off(e)] = w;
                             if (sm_) sm_[off(e)] = mm;
                         }
                 }
             }
-            if constexpr (NA >= 2) {
+            if constexpr (NA >= 2 && MODE == kF64Bwd) {
                 if (epi == kEpiXY) {  // x = T k, y = S k (first matrices): adjoint of pz, through pz = ph act'(z) to those of ph and z
                     // p: pz1, f1, ph f3 (, pz2, f2, ph f4)
 #pragma unroll
@@ -361,7 +374,7 @@ __device__ __forceinline__ int f64_job_units(const F64Job& jb, int len) {
     return ((M + T - 1) / T) * ((N + T - 1) / T) * jb.parts;
 }
 // Jobs [j0, j1) of one phase: their units are dealt to the cluster's CTAs in turn
-static __device__ void f64_jobs(const F64Job* jobs, int j0, int j1, const F64Ctx& cx, int rank, int nranks, unsigned char* smem) {
+template <int MODE> static __device__ void f64_jobs(const F64Job* jobs, int j0, int j1, const F64Ctx& cx, int rank, int nranks, unsigned char* smem) {
     int base = 0;
     for (int j = j0; j < j1; ++j) {
         const F64Job& jb = jobs[j];
@@ -369,12 +382,12 @@ static __device__ void f64_jobs(const F64Job* jobs, int j0, int j1, const F64Ctx
         base += n;
         if (first >= n) continue;
         if (jb.wide) {
-            if (jb.na == 1) f64_units<1, 32>(jb, cx, first, nranks, smem);
-            else f64_units<2, 32>(jb, cx, first, nranks, smem);
+            if (jb.na == 1) f64_units<1, 32, MODE>(jb, cx, first, nranks, smem);
+            else f64_units<2, 32, MODE>(jb, cx, first, nranks, smem);
         } else {
-            if (jb.na == 1) f64_units<1, 16>(jb, cx, first, nranks, smem);
-            else if (jb.na == 2) f64_units<2, 16>(jb, cx, first, nranks, smem);
-            else f64_units<4, 16>(jb, cx, first, nranks, smem);
+            if (jb.na == 1) f64_units<1, 16, MODE>(jb, cx, first, nranks, smem);
+            else if (MODE != kF64Bwd || jb.na == 2) f64_units<2, 16, MODE>(jb, cx, first, nranks, smem);
+            else f64_units<4, 16, kF64Bwd>(jb, cx, first, nranks, smem);
         }
     }
 }

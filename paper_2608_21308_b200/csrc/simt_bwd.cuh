@@ -592,7 +592,7 @@ static int launch_bwd(const SimtBwdArgs& a, cudaStream_t st) {
     using Engine = typename std::conditional<TC, TcGemmT<true>, FmaGemm<Real>>::type;
     constexpr size_t smem = Engine::kBytes + sizeof(ChunkScalars<Real>) + (16 + 8 * kMaxC) * sizeof(Real) + (TC ? 1024 : 0);
     static std::atomic<int> state[64];
-    return simt_launch(simt_bwd_kernel<Real, IO, KIND, TC>, a, Engine::kThreads, smem, state, st);
+    return simt_launch(simt_bwd_kernel<Real, IO, KIND, TC>, a, Engine::kThreads, smem, smem, state, st);
 }
 
 }  // namespace e2ttt

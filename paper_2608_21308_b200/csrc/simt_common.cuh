@@ -101,9 +101,10 @@ template <typename Real> struct ChunkScalars {
     Real cw, cm, cb;    // gt_0, bt_0 R_1 = beta_1 S_1, bt_0
 };
 
-// Executed by one warp.  eta/beta/gamma point at the chunk's first token; len <= 32 EPL tokens, EPL per lane.
-template <typename Real, int EPL>
-__device__ void chunk_scalars_scan(const float* eta, const float* beta, const float* gamma, int len, ChunkScalars<Real>* out) {
+// Executed by one warp.  eta/beta/gamma point at the chunk's first token; len <= 32 EPL tokens, EPL per lane.  Out: ChunkScalars<Real> or
+// a struct with the same names.
+template <typename Real, int EPL, typename Out>
+__device__ void chunk_scalars_scan(const float* eta, const float* beta, const float* gamma, int len, Out* out) {
     const int lane = threadIdx.x & 31;
     ScanMap<Real> local[EPL + 1];
     local[EPL].B = 1; local[EPL].G = 1; local[EPL].X = 0;
@@ -152,24 +153,25 @@ __device__ void chunk_scalars_scan(const float* eta, const float* beta, const fl
     }
 }
 // A lane's own tokens are a serial chain in front of the shuffles, so short chunks take fewer per lane.
-template <typename Real>
-__device__ void chunk_scalars_warp(const float* eta, const float* beta, const float* gamma, int len, ChunkScalars<Real>* out) {
+template <typename Real, typename Out>
+__device__ void chunk_scalars_warp(const float* eta, const float* beta, const float* gamma, int len, Out* out) {
     if (len <= 64) chunk_scalars_scan<Real, 2>(eta, beta, gamma, len, out);
     else chunk_scalars_scan<Real, kMaxC / 32>(eta, beta, gamma, len, out);
 }
 
 // ---- launch of an any-shape kernel: N clusters of a.cl CTAs -------------------------------------
 // `state`, per device: 0 nothing known, 1 the shared-memory limit is set, 8 or 16 the largest cluster the device grants
-// `more`: the kernel's further arguments
+// `smem`: of this launch, `most`: of any launch of the kernel (what is asked of the device once holds for all); `more`: the kernel's further
+// arguments
 template <typename K, typename A, typename... Args>
-int simt_launch(K kernel, A a, int threads, size_t smem, std::atomic<int> (&state)[64], cudaStream_t st, Args... more) {
+int simt_launch(K kernel, A a, int threads, size_t smem, size_t most, std::atomic<int> (&state)[64], cudaStream_t st, Args... more) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
     const bool keep = dev >= 0 && dev < 64;
     int known = keep ? state[dev].load() : 0;
     if (known == 0) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
         if (e != cudaSuccess) return (int)e;
         known = 1;
     }
@@ -179,7 +181,7 @@ int simt_launch(K kernel, A a, int threads, size_t smem, std::atomic<int> (&stat
     at[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
     cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = most;
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = 1;
@@ -203,6 +205,7 @@ int simt_launch(K kernel, A a, int threads, size_t smem, std::atomic<int> (&stat
     }
     if (keep && known > state[dev].load()) state[dev] = known;
     of(a.cl);
+    cfg.dynamicSmemBytes = smem;
     e = cudaLaunchKernelEx(&cfg, kernel, a, more...);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaGetLastError();

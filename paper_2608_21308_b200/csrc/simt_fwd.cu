@@ -271,7 +271,7 @@ static int launch_fwd(const SimtFwdArgs& a, cudaStream_t st) {
     using Engine = typename std::conditional<TC, TcGemmT<false>, FmaGemm<Real>>::type;
     constexpr size_t smem = Engine::kBytes + sizeof(ChunkScalars<Real>) + (TC ? 1024 : 0);
     static std::atomic<int> state[64];
-    return simt_launch(simt_fwd_kernel<Real, IO, KIND, TC>, a, Engine::kThreads, smem, state, st);
+    return simt_launch(simt_fwd_kernel<Real, IO, KIND, TC>, a, Engine::kThreads, smem, smem, state, st);
 }
 
 int simt_fwd_launch(const SimtFwdArgs& a, int kind, int io_dtype, void* stream) {

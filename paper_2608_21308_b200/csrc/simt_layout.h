@@ -24,6 +24,18 @@ E2TTT_HD inline int f64_parts(int C, int d, int h) {
     const int n = (h + 63) / 64;
     return f64_tiles(C, d, 16) >= 32 ? 1 : n < kF64Parts ? n : kF64Parts;
 }
+// Shared memory of the forward: staging (F64Smem, f64_common.cuh), the table of jobs, scalar kernels of two chunks.  More sequences than SMs
+// are bound by the latency of their phases: two CTAs share an SM, with no more than the shape needs (512 sequences of 64 tokens, d = h = 16,
+// C = 1: 3658 -> 2577 us; 300 of one token, d = 64, h = 256: 898 -> 680).  An SM for each is faster with all of its registers: 64 sequences
+// of 256 tokens, d = 128, h = 512 3.48 ms, on kernels with half of them 3.90.
+constexpr size_t kF64FwdTile = 137216, kF64FwdTable = 10 << 10;
+constexpr size_t f64_small_tile(bool wide) { return wide ? 88080 : 69648; }
+constexpr size_t f64_fwd_scalars(int C) { return 16 * (size_t)(5 * C + 8); }
+inline size_t f64_fwd_small(int d, int h, int C) {  // of one of two CTAs
+    return f64_small_tile(f64_wide(h, d) || f64_wide(h, C) || f64_wide(d, C)) + kF64FwdTable + f64_fwd_scalars(C);
+}
+// (an SM has 228 KB, of which 1 KB per CTA is the system's)
+inline bool f64_fwd_two(int N, int d, int h, int C) { return N > 148 && f64_fwd_small(d, h, C) <= (114 - 1) << 10; }
 constexpr size_t kF64SlotBytes = (size_t)64 << 20;  // room for the slots of one call, where one slot per sequence does not take more
 
 struct F64Layout {

@@ -1,4 +1,5 @@
 """fp32 I/O on the fp64 kernels (csrc/f64_*.cu) at the edges of their tiles, parts and groups of chunks, against the oracle."""
+import numpy as np
 import pytest
 
 from paper_2608_21308_b200 import binding as E
@@ -48,11 +49,30 @@ def test_normalised_reverse_pass_over_groups_of_chunks(kind):
 @pytest.mark.parametrize("kind", [MLP, SWIGLU])
 def test_results_do_not_depend_on_the_cluster(kind):
     """One sequence (a cluster of 16) and the same one among 80 (a CTA each): the same bits."""
-    import numpy as np
-
     x, shape = _inputs(1, 70, 40, 130, 16, kind)
     many = {n: [np.concatenate([w] * 80) for w in a] if isinstance(a, list) else np.concatenate([a] * 80) for n, a in x.items()}
     one, all_ = util.gpu_backward(x, **shape), util.gpu_backward(many, **shape)
     for n, a in one.items():
         for p, q in zip(a, all_[n]) if isinstance(a, list) else [(a, all_[n])]:
             assert np.array_equal(np.asarray(p)[0], np.asarray(q)[0]) and np.array_equal(np.asarray(p)[0], np.asarray(q)[79]), n
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("d,h,C,L", [
+    (40, 130, 16, 37),   # narrow tiles
+    (16, 16, 446, 450),  # the longest chunk with two CTAs on an SM, and the next one
+    (16, 16, 447, 450),
+    (64, 256, 215, 220), # the same with wide tiles
+    (64, 256, 216, 220),
+    (64, 256, 16, 1),    # a token
+])
+def test_forward_of_more_sequences_than_sms(d, h, C, L, kind):
+    """150 copies of a sequence on kernels that share an SM (f64_fwd_two): the bits of the one that has a cluster, which match the oracle."""
+    x, shape = _inputs(1, L, d, h, C, kind)
+    many = {n: [np.concatenate([w] * 150) for w in a] if isinstance(a, list) else np.concatenate([a] * 150) for n, a in x.items()}
+    one, _ = util.gpu_forward(x, **shape)
+    check_forward(one, util.oracle_forward(x, C, kind), TOL, "one sequence")
+    all_, _ = util.gpu_forward(many, **shape)
+    for n in ("o", "W", "M"):
+        for p, q in zip(one[n], all_[n]) if n != "o" else [(one[n], all_[n])]:
+            assert all(np.array_equal(p[0], q[i]) for i in (0, 75, 149)), n
