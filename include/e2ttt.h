@@ -277,19 +277,17 @@ E2TTT_API int e2ttt_device_status(const void* workspace, void* stream, int* stat
  * e2ttt_chunk_fwd asks for.
  *
  * Same arguments as e2ttt_chunk_fwd(save_states = 0), minus the workspace.  The scratch
- * is a fixed array of two and a half times E2TTT_NOALLOC_SCRATCH_BYTES inside the library's device image, so every
- * GPU that loads the library gives up that much memory until the process exits.  (What a call counts for is its
- * e2ttt_workspace_bytes(p, 0) - with fp32 I/O without what the fp64 kernels keep beside state and intermediates
- * where heads are wide and hidden units few; there the array is larger than the limit.)
- *   - A call whose count fits gives the results of e2ttt_chunk_fwd, bit for bit.
+ * is a fixed array of E2TTT_NOALLOC_SCRATCH_BYTES inside the library's device image, so every GPU
+ * that loads the library gives up that much memory until the process exits.
+ *   - A call whose e2ttt_workspace_bytes(p, 0) fits gives the results of e2ttt_chunk_fwd, bit for bit.
  *   - A bf16 call up to d = 128 on the any-shape kernels that does not fit, because the block-tiled kernels' operand
  *     blocks take more room than the intermediates of the kernels for wider heads, runs on the latter if those fit:
  *     the same arithmetic (operands as two bf16 terms, fp32 sums) in another order, so that the fp32 results agree to
  *     about 1e-4 and o to a unit in its last place.  (Two SwiGLU sequences, d = 128, h = 384, C = 128: 8.5 and
  *     6.6 MiB.)
  *   - Every other call returns E2TTT_ERR_WORKSPACE and launches nothing.  That includes every call with
- *     impl = E2TTT_IMPL_SIMT or fp32 I/O whose count exceeds E2TTT_NOALLOC_SCRATCH_BYTES.
- * With fp32 I/O the benchmark's tiny configuration, B*H = 1, d = 64, h = 256, C = 16, needs about 0.8 MiB.
+ *     impl = E2TTT_IMPL_SIMT or fp32 I/O whose e2ttt_workspace_bytes(p, 0) exceeds the scratch.
+ * With fp32 I/O the benchmark's tiny configuration, B*H = 1, d = 64, h = 256, C = 16, needs 1.8 MiB.
  * The call itself allocates and frees nothing.
  *
  * The first call on each device looks up the array's device address (one runtime query, with that

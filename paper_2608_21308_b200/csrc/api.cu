@@ -112,11 +112,11 @@ bool tile_backward(const e2ttt_params* p) {
 
 // A buffer with saved states has the block-tiled region whatever `impl` says: the forward and the backward of one training step may
 // be given different ones.
-SimtLayout layout_of(const e2ttt_params* p, bool save_states, bool backward, bool normed, bool allow_tile = true, bool allow_f64 = true) {
+SimtLayout layout_of(const e2ttt_params* p, bool save_states, bool backward, bool normed, bool allow_tile = true) {
     const int nchunks = (p->L + p->C - 1) / p->C;
     const bool tile = allow_tile && can_tile(p) && (save_states || backward || p->impl != E2TTT_IMPL_SIMT);
     return simt_layout(p->d, p->h, p->C, nmat_of(p->kind), nchunks, save_states, backward, normed ? 0 : segment_chunks(p), tile, p->B * p->H,
-                       allow_f64 && p->io_dtype == E2TTT_F32);
+                       p->io_dtype == E2TTT_F32);
 }
 
 size_t simt_bytes(const e2ttt_params* p, bool save_states, bool backward, bool normed, bool allow_tile = true) {
@@ -304,8 +304,6 @@ int e2ttt_chunk_fwd(const e2ttt_params* p, const void* q, const void* k, const v
 namespace e2ttt {
 size_t fixed_scratch_need(const e2ttt_params* p, size_t have) {  // of valid parameters
     size_t need = 0;
-    if (p->io_dtype == E2TTT_F32)  // by the state and intermediates of a call in fp64; the scratch has room for the kernels' further ones
-        return kStatusBytes + layout_of(p, false, false, false, true, false).per_seq * sizeof(double) * (size_t)p->B * p->H;
     if (e2ttt_workspace_bytes(p, 0, &need) == E2TTT_OK && need > have && p->impl != E2TTT_IMPL_TCGEN05) need = simt_bytes(p, false, false, false, false);
     return need;
 }

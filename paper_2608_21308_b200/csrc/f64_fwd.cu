@@ -1,6 +1,8 @@
 // Forward for fp32 I/O: Algorithm 1 chunk after chunk in fp64, any d, h, C and both networks.  A cluster of 1-16 CTAs per sequence, five
 // phases per chunk (f64_common.cuh): activations of the keys | u of the keys, activations of the queries | rows of the keys, the next
 // chunk's tokens and scalar kernels and the rows of the queries of the one before | adjoint of z, u of the queries | state transition.
+// With a compact layout (f64_compact) seven: activations of both | u of both | rows of both | adjoint of z | the keys' rows times K^M |
+// state transition | the next chunk's tokens.
 #include "f64_common.cuh"
 
 namespace e2ttt {
@@ -36,7 +38,7 @@ template <int PER_SM> __global__ void __launch_bounds__(kF64Threads, PER_SM) f64
     const float* gamma = a.gamma + (size_t)seq * a.Ls;
     const int parts = f64_parts(C, d, h);
     const size_t pstride = (size_t)C * d;
-    const bool normed = a.row_norm[0] != nullptr;
+    const bool normed = a.row_norm[0] != nullptr, compact = fl.compact;
     const size_t state_bytes = (size_t)2 * NMAT * dh * sizeof(double);
     double* saved = ws + (a.save_states == 2 ? lay.cck : lay.ckpt);
     // The last chunk's transition writes the final state itself, a pass over the state less.  With the table below built by all warps: one
@@ -159,19 +161,22 @@ template <int PER_SM> __global__ void __launch_bounds__(kF64Threads, PER_SM) f64
         // Algorithm 1 line 1: the network, keys first
         const int odd = c & 1;
         run(kFK + odd, kFK + odd + 1);
+        if (compact) run(kFQ, kFQ + 1);
         phase_sync(CL);
-        run(kFU, a.o ? kFQ + 1 : kFQ);
+        run(kFU, a.o && !compact ? kFQ + 1 : kFQ);
+        if (compact) run(kFUq, kFUq + 1);
         phase_sync(CL);
         // Algorithm 1 line 3: layer norm, e = f(k) - v and pu = dL/du for the key rows; tokens and scalars of the next chunk
         if (c + 1 < a.nchunks) {
-            tokens(c + 1);
+            if (!compact) tokens(c + 1);
             scalars(c + 1);
         }
-        for (int m = rank + CL * warp; m < len + (a.o && c > 0 ? C : 0); m += CL * kF64Warps) {
+        for (int m = rank + CL * warp; m < len + (a.o && c > 0 && !compact ? C : 0); m += CL * kF64Warps) {
             if (m >= len) {  // rows of the queries of the chunk before
                 output_row(c - 1, m - len);
                 continue;
             }
+            if (compact) output_row(c, m);  // (a lane writes pu where it alone read u of the query)
             double su = 0.0;
             double* pu = ws + fl.fPu + (size_t)m * d;
 #pragma unroll 2
@@ -196,13 +201,21 @@ template <int PER_SM> __global__ void __launch_bounds__(kF64Threads, PER_SM) f64
                 const double x = r * (e - se - y * sey);
                 pu[i] = x;
                 ws[fl.fPuW + (size_t)m * d + i] = x * sc.kW[m];
-                ws[fl.fPuM + (size_t)m * d + i] = x * sc.kM[m];
+                if (!compact) ws[fl.fPuM + (size_t)m * d + i] = x * sc.kM[m];
             }
         }
         phase_sync(CL);
         // back through the last matrix and the activation
-        run(kFPz, a.o ? kFUq + 1 : kFUq);
+        run(kFPz, a.o && !compact ? kFUq + 1 : kFUq);
         phase_sync(CL);
+        if (compact) {
+            for (int m = rank + CL * warp; m < len; m += CL * kF64Warps) {
+                double* pu = ws + fl.fPu + (size_t)m * d;
+#pragma unroll 4
+                for (int i = lane; i < d; i += 32) pu[i] *= sc.kM[m];
+            }
+            phase_sync(CL);
+        }
         // Algorithm 1 lines 4-7
         int slot = -1;  // the saved state that this chunk's end is
         if (a.save_states == 1 && (c + 1 < a.nchunks || normed)) slot = c + 1;
@@ -212,6 +225,10 @@ template <int PER_SM> __global__ void __launch_bounds__(kF64Threads, PER_SM) f64
         run(odd ? kFUpd1 : kFUpd, (odd ? kFUpd1 : kFUpd) + NMAT);
         if (cx.last) break;  // (nothing that follows reads it)
         phase_sync(CL);
+        if (compact && c + 1 < a.nchunks) {
+            tokens(c + 1);
+            phase_sync(CL);
+        }
         // post-chunk normalisation (optional): every row w of every W_i becomes n w / (||w|| + eps_n); one warp per row
         if (normed) {
             const int maxdim = d > h ? d : h;
@@ -238,7 +255,7 @@ template <int PER_SM> __global__ void __launch_bounds__(kF64Threads, PER_SM) f64
             phase_sync(CL);
         }
     }
-    if (a.o)
+    if (a.o && !compact)
         for (int m = rank + CL * warp; m < L - (a.nchunks - 1) * C; m += CL * kF64Warps) output_row(a.nchunks - 1, m);
     for (int i = 0; i < NMAT; ++i) {
         if (direct || !a.W_final[i]) continue;  // none: recomputation for the reverse pass, only the saved states matter

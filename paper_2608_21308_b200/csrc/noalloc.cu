@@ -8,10 +8,8 @@
 
 namespace {
 
-// Resident on every GPU that loads the library, for the life of the process.  Calls are accepted up to E2TTT_NOALLOC_SCRATCH_BYTES of
-// state and intermediates; the fp64 kernels keep up to 7 / 3 of that where heads are wide and hidden units few.
-constexpr size_t kScratchBytes = (size_t)E2TTT_NOALLOC_SCRATCH_BYTES / 2 * 5;
-static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
+// Resident on every GPU that loads the library, for the life of the process.
+static __device__ __align__(256) unsigned char g_static_scratch[E2TTT_NOALLOC_SCRATCH_BYTES];
 
 constexpr int kMaxDevices = 64;
 void* g_scratch_addr[kMaxDevices];  // device address of g_static_scratch, per device ordinal
@@ -72,5 +70,5 @@ extern "C" E2TTT_API int e2ttt_chunk_fwd_noalloc(const e2ttt_params* p, const vo
     rc = scratch_for_current_device(&scratch);
     if (rc != E2TTT_OK) return rc;
     return e2ttt::fwd_fixed_scratch(p, q, k, v, eta, beta, gamma, W_init, M_init, o, W_final, M_final, scratch,
-                                    p->io_dtype == E2TTT_F32 ? kScratchBytes : (size_t)E2TTT_NOALLOC_SCRATCH_BYTES, stream);
+                                    (size_t)E2TTT_NOALLOC_SCRATCH_BYTES, stream);
 }

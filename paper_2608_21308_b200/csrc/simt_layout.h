@@ -1,5 +1,5 @@
-// Workspace layout of the SIMT kernels (host and device).  Offsets are in elements of the kernel's
-// internal type (double for fp32 I/O, float for bf16 I/O), relative to the sequence's own slice.
+// Workspace layout of the any-shape kernels (host and device).  Offsets are in elements of the kernels' internal type (double for fp32 I/O:
+// the fp64 kernels; float for bf16 I/O: the SIMT and the block-tiled ones), relative to the sequence's own slice.
 #pragma once
 #include <stddef.h>
 #include <stdint.h>
@@ -38,7 +38,14 @@ inline size_t f64_fwd_small(int d, int h, int C) {  // of one of two CTAs
 inline bool f64_fwd_two(int N, int d, int h, int C) { return N > 148 && f64_fwd_small(d, h, C) <= (114 - 1) << 10; }
 constexpr size_t kF64SlotBytes = (size_t)64 << 20;  // room for the slots of one call, where one slot per sequence does not take more
 
+// Where a chunk's tokens outweigh what the network makes of them (heads wider than their hidden units) a forward without saved states
+// keeps them in three [tokens x d] places instead of seven, at two short phases more per chunk, so that no call needs more than its state,
+// 3 [tokens x d], 8 [tokens x h] and 1 MiB (simt_layout).  365 tokens, d = 832, h = 1: 7.0 MiB
+// instead of 16.3, 319 us instead of 317; 730 tokens 630 instead of 617.
+inline bool f64_compact(int d, int h, int C, int nmat) { return (size_t)C * d > 32000 + (size_t)C * h / (size_t)(nmat - 1); }
+
 struct F64Layout {
+    int compact;
     int G;  // chunks that the reverse pass prepares at a time (slots)
     // forward: one chunk
     size_t fK[2], fQ, fA, fAq, fc1, fc2, fUk, fUq, fPu, fPuW, fPuM, fPzW[2], fPzM[2];  // fK: the keys, by the chunk's parity
@@ -53,12 +60,13 @@ inline size_t f64_layout(F64Layout& f, size_t o, int N, int d, int h, int C, int
     auto take = [&](size_t n) { size_t r = o; o += (n + 31) / 32 * 32; return r; };
     const size_t Ch = (size_t)C * h, Cd = (size_t)C * d, sw = nmat == 3, parts = (size_t)f64_parts(C, d, h);
     const size_t begin = o;
-    f.fK[0] = take(Cd); f.fK[1] = take(Cd); f.fQ = take(Cd);
+    f.compact = !backward && f64_compact(d, h, C, nmat);  // (one part: from 128 tiles on)
+    f.fK[0] = take(Cd); f.fK[1] = f.compact ? f.fK[0] : take(Cd); f.fQ = take(Cd);
     f.fA = take(Ch); f.fAq = take(Ch); f.fc1 = take(Ch); f.fc2 = take(sw * Ch);
-    f.fUk = take(parts * Cd); f.fUq = take(parts * Cd); f.fPu = take(Cd);
+    f.fUk = take(parts * Cd); f.fUq = f.compact ? f.fQ : take(parts * Cd); f.fPu = f.compact ? f.fQ : take(Cd);
     // (written element by element over what they are made of, so that a call without saved states needs little more than its state)
     f.fPuW = f.fUk;
-    f.fPuM = parts > 1 ? f.fUk + Cd : take(Cd);
+    f.fPuM = f.compact ? f.fPu : parts > 1 ? f.fUk + Cd : take(Cd);
     f.fPzW[0] = f.fc1; f.fPzW[1] = f.fc2;
     for (int i = 0; i < nmat - 1; ++i) f.fPzM[i] = take(Ch);
     const size_t end_fwd = o;
@@ -110,7 +118,9 @@ struct SimtLayout {
 
 // tile != 0: a call may run on the block-tiled kernels (bf16 I/O, d <= 128): their region shares the space of the SIMT
 // kernels' intermediates (a call uses one of the two), behind the state that both kinds leave for each other.
-// f64 != 0: fp32 I/O, which the fp64 kernels serve; their region lies in the same place.
+// f64 != 0: fp32 I/O, which the fp64 kernels serve.  A training call has their region instead of the SIMT kernels' intermediates.  A forward
+// without saved states asks for as much as those would take, twice the bytes of a bf16 call: callers of the fixed scratch (noalloc.cu)
+// count by it.  The fp64 kernels' region is never larger (f64_compact).
 inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool save_states, bool backward, int seg = 0, int tile = 0, int N = 1,
                               int f64 = 0) {
     SimtLayout l{};
@@ -131,6 +141,14 @@ inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool s
     }
     const int chunks = l.seg > 0 && l.seg < nchunks ? l.seg : nchunks;  // of a launch sequence of the reverse pass
     const size_t begin = o;
+    size_t end64 = 0;
+    if (f64) {
+        end64 = f64_layout(l.fl, begin, N, d, h, C, nmat, backward, chunks);
+        if (backward) {
+            l.per_seq = end64;
+            return l;
+        }
+    }
     l.Z1 = take((size_t)2 * C * h); l.Z2 = take((size_t)2 * C * h); l.A = take((size_t)2 * C * h);
     l.U = take((size_t)2 * C * d); l.Pu = take((size_t)C * d);
     l.Pz1 = take((size_t)C * h); l.Pz2 = take((size_t)C * h);
@@ -151,11 +169,7 @@ inline SimtLayout simt_layout(int d, int h, int C, int nmat, int nchunks, bool s
         const size_t end = tile_layout(l.tl, begin, N, d, h, C, nmat, backward, chunks);
         if (end > o) o = end;
     }
-    if (f64) {
-        const size_t end = f64_layout(l.fl, begin, N, d, h, C, nmat, backward, chunks);
-        if (end > o) o = end;
-    }
-    l.per_seq = o;
+    l.per_seq = end64 > o ? end64 : o;
     return l;
 }
 

@@ -5,7 +5,7 @@ import pytest
 from paper_2608_21308_b200 import binding as E
 from paper_2608_21308_b200 import inputs
 from tests import util
-from tests.test_gpu_normed import gpu_backward_normed, oracle_bwd, targets
+from tests.test_gpu_normed import gpu_backward_normed, gpu_forward_normed, oracle_bwd, oracle_fwd, targets
 from tests.test_gpu_parity import check_backward, check_forward
 
 pytestmark = pytest.mark.gpu
@@ -55,6 +55,31 @@ def test_results_do_not_depend_on_the_cluster(kind):
     for n, a in one.items():
         for p, q in zip(a, all_[n]) if isinstance(a, list) else [(a, all_[n])]:
             assert np.array_equal(np.asarray(p)[0], np.asarray(q)[0]) and np.array_equal(np.asarray(p)[0], np.asarray(q)[79]), n
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("d,h,C,L", [
+    (828, 1, 365, 400),  # compact layout (f64_compact): the widest head of one hidden unit that fits the fixed scratch; a short last chunk
+    (256, 1, 126, 253),  # the first chunk length that takes it, a last chunk of one token
+    (256, 1, 125, 251),  # the last one that does not
+    (300, 40, 256, 512), # several tiles of hidden units
+])
+def test_wide_heads_with_few_hidden_units(d, h, C, L, kind):
+    import torch
+
+    x, shape = _inputs(1, L, d, h, C, kind)
+    got, hd = util.gpu_forward(x, **shape)
+    check_forward(got, util.oracle_forward(x, C, kind), TOL, "fp64 forward")
+    if h > 1:  # (a row of one weight is +-n: where the weight crosses zero, n w / (|w| + eps) magnifies its error by n / |w|)
+        tgt = targets(x)
+        check_forward(gpu_forward_normed(x, tgt, impl=E.E2TTT_IMPL_AUTO, **shape), oracle_fwd(x, tgt, C, kind), 1e-5, "fp64 normed forward")
+    # the same call in the fixed scratch: the same bits
+    o, Wf, Mf = torch.empty_like(hd["q"]), [torch.empty_like(w) for w in hd["W"]], [torch.empty_like(w) for w in hd["W"]]
+    E.e2ttt_chunk_fwd_noalloc(hd["p"], hd["q"], hd["k"], hd["v"], hd["eta"], hd["beta"], hd["gamma"], hd["W"], hd["M"], o, Wf, Mf)
+    torch.cuda.synchronize()
+    assert np.array_equal(o.cpu().numpy().reshape(1, L, d), got["o"])
+    for w, m, w0, m0 in zip(Wf, Mf, got["W"], got["M"]):
+        assert np.array_equal(w.cpu().numpy()[:, 0], w0) and np.array_equal(m.cpu().numpy()[:, 0], m0)
 
 
 @pytest.mark.parametrize("kind", [MLP, SWIGLU])
