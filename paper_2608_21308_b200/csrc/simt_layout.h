@@ -10,7 +10,9 @@ namespace e2ttt {
 
 // ---- fp64 kernels (f64_fwd.cu, f64_bwd.cu; fp32 I/O) -----------------------------------------------------------------------
 // A [tokens x d] result of a contraction over hidden units has few tiles and is cut along k; the parts are added by whoever reads it.
-// From 32 tiles of 16 x 16 on there is work enough for a cluster without.
+// From 32 tiles of 16 x 16 on there is work enough for a cluster without.  Forward and reverse pass, ms: 16 chunks of 16 tokens, d = 64,
+// h = 256, one sequence 0.95, in two parts 1.00, uncut 1.16 - but 16 sequences of 64 such chunks 13.6, 13.0, 13.8.  The line at 16 tiles:
+// one sequence of 512 tokens, C = 64, 0.93 -> 0.88, all else equal; at 64: 32 SwiGLU sequences of 512, d = 128, h = 384, 13.5 -> 14.7.
 constexpr int kF64Parts = 4;
 #ifdef __CUDACC__
 #define E2TTT_HD __host__ __device__
@@ -18,7 +20,9 @@ constexpr int kF64Parts = 4;
 #define E2TTT_HD
 #endif
 E2TTT_HD inline int f64_tiles(int M, int N, int T) { return ((M + T - 1) / T) * ((N + T - 1) / T); }
-// 32 x 32 tiles (half the loads per product) where a cluster of 16 has one for every CTA, else 16 x 16
+// 32 x 32 tiles (half the loads per product) where a cluster of 16 has one for every CTA, else 16 x 16.  From 128 tiles on: 16 chunks of
+// 16 tokens, d = 64, h = 256, one sequence 0.95 -> 1.23 ms.  From 32 on: one token of one sequence, d = 128, h = 512, 78 -> 94 us, but the
+// reverse pass of 32 SwiGLU sequences of 512 tokens, h = 384, 10.1 -> 8.1 ms.
 E2TTT_HD inline int f64_wide(int M, int N) { return M > 16 && N > 16 && f64_tiles(M, N, 16) >= 64; }
 E2TTT_HD inline int f64_parts(int C, int d, int h) {
     const int n = (h + 63) / 64;
@@ -36,7 +40,22 @@ inline size_t f64_fwd_small(int d, int h, int C) {  // of one of two CTAs
 }
 // (an SM has 228 KB, of which 1 KB per CTA is the system's)
 inline bool f64_fwd_two(int N, int d, int h, int C) { return N > 148 && f64_fwd_small(d, h, C) <= (114 - 1) << 10; }
-constexpr size_t kF64SlotBytes = (size_t)64 << 20;  // room for the slots of one call, where one slot per sequence does not take more
+// Chunks that the reverse pass prepares side by side (slots): at most 64 MB of them, or one per sequence; fewer sequences than SMs take no
+// more than one for every SM, or 32 MB of small ones.  ms / MB of workspace: 4096 tokens in chunks of 16, d = 64, h = 256, one sequence: 18
+// chunks 9.2 / 138, 74 8.4 / 159, 148 8.7 / 187, 163 (64 MB) 8.9 / 195; 64 sequences, d = h = 16, C = 1: 3 chunks 10.2 / 137, 4 MB 7.8 / 140,
+// 32 MB 7.3 / 168, 64 MB 7.5 / 200; one sequence, C = 512, d = 128, h = 512: one chunk 8.9 / 43, three of four (62 MB) 6.5 / 84; 4 SwiGLU
+// sequences, d = 72, h = 200, C = 64: 16 MB 1.53 / 49, 32 MB 1.47 / 64, 64 MB 1.22 / 95.
+constexpr int kF64SlotItems = 148;
+constexpr size_t kF64SlotFree = (size_t)32 << 20, kF64SlotBytes = (size_t)64 << 20;
+inline int f64_slots(int N, size_t slot_bytes, int chunks) {
+    const size_t all = slot_bytes * (size_t)N;
+    size_t g = kF64SlotBytes / all;
+    if (N < kF64SlotItems) {
+        const size_t each = (size_t)(kF64SlotItems + N - 1) / N, some = kF64SlotFree / all;
+        g = g < (each > some ? each : some) ? g : each > some ? each : some;
+    }
+    return g < 1 ? 1 : g < (size_t)chunks ? (int)g : chunks;
+}
 
 // Where a chunk's tokens outweigh what the network makes of them (heads wider than their hidden units) a forward without saved states
 // keeps them in three [tokens x d] places instead of seven, at two short phases more per chunk, so that no call needs more than its state,
@@ -87,8 +106,7 @@ inline size_t f64_layout(F64Layout& f, size_t o, int N, int d, int h, int C, int
     f.sr = take(C); f.smey = take(C); f.ssc = take((size_t)2 * C + 8); f.skwb = take((size_t)2 * C);
     f.sdots = take((size_t)nmat * f64_tiles(h, d, f64_wide(h, d) ? 32 : 16) * 8 * 3);
     f.slot_stride = o;
-    const size_t fit = kF64SlotBytes / (o * sizeof(double) * (size_t)N);
-    f.G = fit < 1 ? 1 : fit < (size_t)chunks ? (int)fit : chunks;
+    f.G = f64_slots(N, o * sizeof(double), chunks);
     o = f.slot + f.slot_stride * (size_t)f.G;
     return o > end_fwd ? o : end_fwd;
 }

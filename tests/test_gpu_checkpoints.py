@@ -117,3 +117,17 @@ def test_full_size_training_flow_memory_plans_agree(cfg):
     for n in GRADS:
         assert np.isfinite(a[n]).all(), n
     same_bits(a, b, "full size: every state kept vs checkpoints every 8")
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+def test_segments_of_several_groups_of_chunks_fp32(kind):
+    """d = 128, h = 384, 9 sequences: the fp64 reverse pass prepares two or three chunks at a time (its slots are bounded), so a segment of
+    four has two groups, and the adjoints of the state pass from group to group as well as from segment to segment: the bits of the plan that
+    keeps every state, saved or recomputed."""
+    r = inputs.paper_regime(inputs.Recipe(B=9, H=1, L=6 * 64 - 5, d=128, h=384, C=64, kind=kind, io="f32", seed=43, m_std=0.002))
+    x = inputs.generate(r, with_d_o=True, with_dstate=True)
+    shape = dict(d=128, h=384, C=64, kind=kind, io="f32")
+    full = util.gpu_backward(x, **shape)
+    check_backward(full, util.oracle_backward(x, 64, kind), 1e-6, "every chunk kept")
+    for saved in (False, True):
+        same_bits(util.gpu_backward(x, ckpt_every=4, via_saved_states=saved, **shape), full, f"groups in segments, saved={saved}")

@@ -76,3 +76,12 @@ def test_slots_of_the_fp64_reverse_pass_are_bounded(tmp_path):
     (tmp_path / "f64.cpp").write_text(F64)
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", str(CSRC), str(tmp_path / "f64.cpp"), "-o", str(tmp_path / "f64")], check=True)
     assert subprocess.run([str(tmp_path / "f64")]).returncode == 0
+
+
+def test_slots_stop_where_more_of_them_do_not_pay():
+    """fp32, one sequence of 4096 tokens in chunks of 16, d = 64, h = 256: 256 chunks, of which 148 are prepared at a time (187 MB; the 64 MB
+    that slots may take would make it 195).  64 sequences of chunks of one token, d = h = 16: 32 MB of slots."""
+    mb = lambda *a: E.e2ttt_workspace_bytes(E.make_params(*a, E.E2TTT_MLP_GELU, E.E2TTT_F32, 1e-5, E.E2TTT_IMPL_AUTO), 1) / 2**20
+    assert 185 < mb(1, 1, 4096, 64, 256, 16) < 189
+    assert mb(64, 1, 256, 16, 16, 1) < 170
+    assert mb(1, 1, 256, 64, 256, 16) < 16
