@@ -78,7 +78,7 @@ int pick_impl(const e2ttt_params* p, bool save_states, int* impl) {
 }
 
 // The block-tiled kernels serve the any-shape calls of bf16 I/O up to d = 128 (a head dimension in one accumulator tile);
-// wider heads and fp32 I/O run on the SIMT kernels.
+// wider heads run on the SIMT kernels, fp32 I/O on the fp64 ones.
 bool can_tile(const e2ttt_params* p) { return p->io_dtype == E2TTT_BF16 && p->d <= kTileMaxD; }
 
 // Where they do not pay, the any-shape kernels with tensor-core products (simt_fwd.cu, simt_bwd.cu) keep the call.  Both lose their time

@@ -9,7 +9,7 @@ int simt_bwd_launch(const SimtBwdArgs& a, int kind, int io_dtype, void* stream) 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (io_dtype == 0) return f64_bwd_launch(a, kind, stream);
     if (a.tc) return simt_bwd_launch_tc(a, kind, st);
-    return kind == 0 ? launch_bwd<float, __nv_bfloat16, 0, false>(a, st) : launch_bwd<float, __nv_bfloat16, 1, false>(a, st);
+    return kind == 0 ? launch_bwd<0, false>(a, st) : launch_bwd<1, false>(a, st);
 }
 
 }  // namespace e2ttt

@@ -4,7 +4,7 @@
 namespace e2ttt {
 
 int simt_bwd_launch_tc(const SimtBwdArgs& a, int kind, cudaStream_t st) {
-    return kind == 0 ? launch_bwd<float, __nv_bfloat16, 0, true>(a, st) : launch_bwd<float, __nv_bfloat16, 1, true>(a, st);
+    return kind == 0 ? launch_bwd<0, true>(a, st) : launch_bwd<1, true>(a, st);
 }
 
 }  // namespace e2ttt

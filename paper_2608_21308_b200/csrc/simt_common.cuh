@@ -1,5 +1,5 @@
 // Building blocks of the any-shape kernels (scans, layer norm, reductions, phase barrier, the FMA GEMM).
-// Real = double for fp32 I/O, float for bf16 I/O.
+// Real = double in the fp64 kernels (fp32 I/O), float in the others.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -257,30 +257,30 @@ __device__ __forceinline__ void phase_sync(int nranks) {
 //   64x64 tiles, 16-deep k slices, 4x4 results per thread: fewest loads per product, where there is a tile for every CTA;
 //   16x16 tiles, 64-deep k slices cut four ways inside the CTA, 2x2 results per thread, the next slice's loads in flight while one
 //   is multiplied: for the few tokens of a small problem.  A [32 x 64] result with 256 terms is one 64x64 tile - one CTA of
-//   eight, half of its rows unused, 16 exposed round trips to L2 (14 us in fp64) - but 8 small ones with 4 slices each.
-template <typename Real> struct __align__(2 * sizeof(Real)) Real2 { Real x, y; };
-
-template <typename Real> struct __align__(16) GemmSmem {
+//   eight, half of its rows unused, 16 exposed round trips to L2 - but 8 small ones with 4 slices each.  Forward and reverse pass
+//   (impl SIMT) of one sequence, large tiles alone -> both: 16 chunks of 16 tokens, d = 64, h = 256 5.53 -> 3.06 ms, 8 chunks of 64,
+//   d = 128, h = 512 6.60 -> 6.49.
+struct __align__(16) GemmSmem {
     union {
         struct {
-            Real A[2][kBK][kBM + 4];
-            Real B[kBK][kBN + 4];
+            float A[2][kBK][kBM + 4];
+            float B[kBK][kBN + 4];
         };
         struct {
-            Real2<Real> a[2][kSK][kSM / 2 + 1];  // pairs: one access per two values
-            Real2<Real> b[kSK][kSM / 2 + 1];
-            Real part[2][kSplit][kSM * kSM];
+            float2 a[2][kSK][kSM / 2 + 1];  // pairs: one access per two values
+            float2 b[kSK][kSM / 2 + 1];
+            float part[2][kSplit][kSM * kSM];
         } s;
     };
 };
 
-template <typename Real, int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FP, typename FE>
-__device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, GemmSmem<Real>* sm, int rank, int nranks) {
+template <int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FP, typename FE>
+__device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, GemmSmem* sm, int rank, int nranks) {
     const int tid = threadIdx.x;
     const int grp = tid / (kSimtThreads / kSplit), tx = tid & 7, ty = (tid >> 3) & 7;
     const int tn = (N + kSM - 1) / kSM, tiles = tn * ((M + kSM - 1) / kSM);
     constexpr int PER = kSM * kSK / kSimtThreads;
-    Real ra0[PER], ra1[PER], rb[PER], acc[NACC][2][2];
+    float ra0[PER], ra1[PER], rb[PER], acc[NACC][2][2];
     // the slice whose loads are in flight (the next one) and the slice in shared memory; divisions once per tile only
     int tile = rank, fm0 = (rank / tn) * kSM, fn0 = (rank % tn) * kSM, fk0 = 0;
     for (bool first = true;; first = false) {
@@ -295,9 +295,9 @@ __device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE e
                 const int am = A_KFAST ? idx / kSK : idx % kSM, ak = A_KFAST ? idx % kSK : idx / kSM;
                 const int bn = B_KFAST ? idx / kSK : idx % kSM, bk = B_KFAST ? idx % kSK : idx / kSM;
                 const bool ina = m0 + am < M && k0 + ak < K, inb = n0 + bn < N && k0 + bk < K;
-                reinterpret_cast<Real*>(sm->s.a[0][ak])[am] = ina ? ra0[r] : (Real)0;
-                if (NACC == 2) reinterpret_cast<Real*>(sm->s.a[1][ak])[am] = ina ? ra1[r] : (Real)0;
-                reinterpret_cast<Real*>(sm->s.b[bk])[bn] = inb ? rb[r] : (Real)0;
+                reinterpret_cast<float*>(sm->s.a[0][ak])[am] = ina ? ra0[r] : 0.0f;
+                if (NACC == 2) reinterpret_cast<float*>(sm->s.a[1][ak])[am] = ina ? ra1[r] : 0.0f;
+                reinterpret_cast<float*>(sm->s.b[bk])[bn] = inb ? rb[r] : 0.0f;
             }
             __syncthreads();
             fk0 += kSK;
@@ -334,10 +334,10 @@ __device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE e
         const int terms = min(kSK, K - k0);  // of this slice; dealt to the four groups in turn
 #pragma unroll 4
         for (int kk = grp; kk < terms; kk += kSplit) {
-            const Real2<Real> b = sm->s.b[kk][tx];
+            const float2 b = sm->s.b[kk][tx];
 #pragma unroll
             for (int a = 0; a < NACC; ++a) {
-                const Real2<Real> v = sm->s.a[a][kk][ty];
+                const float2 v = sm->s.a[a][kk][ty];
                 acc[a][0][0] += v.x * b.x; acc[a][0][1] += v.x * b.y;
                 acc[a][1][0] += v.y * b.x; acc[a][1][1] += v.y * b.y;
             }
@@ -350,7 +350,7 @@ __device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE e
 #pragma unroll
                     for (int j = 0; j < 2; ++j) sm->s.part[a][grp][(2 * ty + i) * kSM + 2 * tx + j] = acc[a][i][j];
             __syncthreads();
-            Real s[2] = {0, 0};
+            float s[2] = {0, 0};
 #pragma unroll
             for (int a = 0; a < NACC; ++a)
 #pragma unroll
@@ -361,13 +361,13 @@ __device__ void block_gemm_small(int M, int N, int K, FA fa, FB fb, FP pre, FE e
     }
 }
 
-template <typename Real, int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FP, typename FE>
-__device__ void block_gemm(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, GemmSmem<Real>* sm, int rank, int nranks) {
+template <int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FP, typename FE>
+__device__ void block_gemm(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, GemmSmem* sm, int rank, int nranks) {
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
     // fewer large tiles than CTAs, or a lone tile's row that is mostly padding: the small tiling keeps the cluster busy
     if (((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN) < nranks || 2 * M <= kBM || 2 * N <= kBN) {
-        block_gemm_small<Real, NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, pre, epi, sm, rank, nranks);
+        block_gemm_small<NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, pre, epi, sm, rank, nranks);
         phase_sync(nranks);
         return;
     }
@@ -375,7 +375,7 @@ __device__ void block_gemm(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, Ge
     for (int m0 = 0; m0 < M; m0 += kBM) {
         for (int n0 = 0; n0 < N; n0 += kBN, ++tile) {
             if (tile % nranks != rank) continue;
-            Real acc[NACC][4][4];
+            float acc[NACC][4][4];
 #pragma unroll
             for (int a = 0; a < NACC; ++a)
 #pragma unroll
@@ -389,7 +389,7 @@ __device__ void block_gemm(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, Ge
                     const int idx = tid + r * kSimtThreads;
                     const int mm = A_KFAST ? idx / kBK : idx % kBM;
                     const int kk = A_KFAST ? idx % kBK : idx / kBM;
-                    Real a0 = 0, a1 = 0;
+                    float a0 = 0, a1 = 0;
                     if (m0 + mm < M && k0 + kk < K) fa(m0 + mm, k0 + kk, a0, a1);
                     sm->A[0][kk][mm] = a0;
                     if (NACC == 2) sm->A[1][kk][mm] = a1;
@@ -399,21 +399,21 @@ __device__ void block_gemm(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, Ge
                     const int idx = tid + r * kSimtThreads;
                     const int nn = B_KFAST ? idx / kBK : idx % kBN;
                     const int kk = B_KFAST ? idx % kBK : idx / kBN;
-                    Real b = 0;
+                    float b = 0;
                     if (n0 + nn < N && k0 + kk < K) b = fb(n0 + nn, k0 + kk);
                     sm->B[kk][nn] = b;
                 }
                 __syncthreads();
 #pragma unroll
                 for (int kk = 0; kk < kBK; ++kk) {
-                    Real bv[4];
+                    float bv[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) bv[j] = sm->B[kk][tx * 4 + j];
 #pragma unroll
                     for (int a = 0; a < NACC; ++a) {
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const Real av = sm->A[a][kk][ty * 4 + i];
+                            const float av = sm->A[a][kk][ty * 4 + i];
 #pragma unroll
                             for (int j = 0; j < 4; ++j) acc[a][i][j] += av * bv[j];
                         }
@@ -435,7 +435,7 @@ __device__ void block_gemm(int M, int N, int K, FA fa, FB fb, FP pre, FE epi, Ge
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int m = m0 + ty * 4 + i, n = n0 + tx * 4 + j;
-                    if (m < M && n < N) epi(m, n, acc[0][i][j], NACC == 2 ? acc[NACC - 1][i][j] : (Real)0, p[i][j]);
+                    if (m < M && n < N) epi(m, n, acc[0][i][j], NACC == 2 ? acc[NACC - 1][i][j] : 0.0f, p[i][j]);
                 }
         }
     }

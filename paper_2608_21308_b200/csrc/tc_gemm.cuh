@@ -12,7 +12,7 @@
 //            128 registers per thread, does not: the batches made the reverse pass spill (d = 160: 5-10 % slower).
 // Output tiles are dealt round-robin to the `nranks` CTAs of the sequence's cluster; run() ends with phase_sync().
 //
-//   FmaGemm<Real> : CUDA-core FMAs in fp32 (bf16 I/O, impl SIMT).
+//   FmaGemm       : CUDA-core FMAs in fp32 (bf16 I/O, impl SIMT).
 //   TcGemm        : the 5th-generation tensor cores (tcgen05.mma, fp32 accumulation in tensor memory).  Every fp32
 //                   operand x is staged as two bf16 numbers, hi = bf16(x) and lo = bf16(x - hi), and a product is
 //                   three MMAs, hi*hi + hi*lo + lo*hi: the dropped lo*lo term and the residual of the split are
@@ -25,32 +25,32 @@
 
 namespace e2ttt {
 
-template <typename Real> struct FmaGemm {
+struct FmaGemm {
     static constexpr int kThreads = kSimtThreads;
-    static constexpr size_t kBytes = sizeof(GemmSmem<Real>);
-    GemmSmem<Real>* sm;
+    static constexpr size_t kBytes = sizeof(GemmSmem);
+    GemmSmem* sm;
     int rank, nranks;
     __device__ static unsigned char* align(unsigned char* raw) { return raw; }
     __device__ void setup(unsigned char* base, int* /*status*/, int rank_, int nranks_) {
-        sm = reinterpret_cast<GemmSmem<Real>*>(base);
+        sm = reinterpret_cast<GemmSmem*>(base);
         rank = rank_;
         nranks = nranks_;
     }
     __device__ void teardown() {}
-    __device__ void set_scratch(Real*) {}
+    __device__ void set_scratch(float*) {}
     template <int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FP, typename FE>
     __device__ void run_rmw(int M, int N, int K, FA fa, FB fb, FP pre, FE epi) {
-        block_gemm<Real, NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, pre, epi, sm, rank, nranks);
+        block_gemm<NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, pre, epi, sm, rank, nranks);
     }
     template <int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FE>
     __device__ void run(int M, int N, int K, FA fa, FB fb, FE epi) {
         run_rmw<NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, [](int, int) { return 0; },
-                                        [&](int m, int n, Real a0, Real a1, int) { epi(m, n, a0, a1); });
+                                        [&](int m, int n, float a0, float a1, int) { epi(m, n, a0, a1); });
     }
     template <int NACC, bool A_KFAST, bool B_KFAST, typename FA, typename FB, typename FT>
     __device__ void run_add(int M, int N, int K, FA fa, FB fb, FT at) {
         run_rmw<NACC, A_KFAST, B_KFAST>(M, N, K, fa, fb, [&](int m, int n) { return at(m, n); },
-                                        [&](int m, int n, Real acc, Real, Real old) { at(m, n) = old + acc; });
+                                        [&](int m, int n, float acc, float, float old) { at(m, n) = old + acc; });
     }
 };
 
