@@ -127,7 +127,8 @@ E2TTT_API int e2ttt_matrix_shape(int kind, int d, int h, int i, int* rows, int* 
 /* Bytes of caller-provided device workspace a call with these parameters needs.
  * save_states != 0: the size for a forward that also records the chunk-start states (every chunk's, or
  * the checkpoints p->ckpt_every selects plus room for one recomputed segment), and for the backward
- * that consumes them.  `bytes` is a host pointer. */
+ * that consumes them.  Beside the states the reverse pass keeps what it prepares of several chunks at a time: one chunk per
+ * sequence, and up to 64 MB for the whole call with fp32 I/O, 512 MB or twice that with bf16.  `bytes` is a host pointer. */
 E2TTT_API int e2ttt_workspace_bytes(const e2ttt_params* p, int save_states, size_t* bytes);
 
 /* Forward over all chunks of all sequences (Algorithm 1 applied chunk after chunk, Section 3.2).

@@ -5,7 +5,7 @@
 // same one), and little code.  With each product's loaders and epilogue inlined the reverse pass was 800 KB of machine code, walked
 // once per chunk: its phases waited for instructions, 6 us each.  Here a product is data - operands with strides, an epilogue number -
 // built once per launch in shared memory, and all products of a chunk go through the same few instantiations of f64_units(): 16 chunks
-// of 16 tokens, d = 64, h = 256, one sequence, forward and reverse pass 2806 -> 954 us.
+// of 16 tokens, d = 64, h = 256, one sequence, forward and reverse pass 2806 -> 948 us.
 //
 // A result does not depend on the cluster's size: tilings, the parts a contraction is cut into and all orders of summation follow from
 // the shape alone.
