@@ -261,6 +261,12 @@ int f64_fwd_launch(const SimtFwdArgs& a, int kind, void* stream);
 int f64_bwd_launch(const SimtBwdArgs& a, int kind, void* stream);
 // the same calls on the block-tiled kernels (tile_fwd.cu / tile_bwd.cu); the layout must have been made with `tile`
 int tile_fwd_launch(const SimtFwdArgs& a, int kind, void* stream);
+// Chunks of more than 64 tokens (tile_flow.cu, taken by tile_fwd_launch).  us, on clusters -> on work items: d = 128, h = 512, 64 sequences of 2048
+// tokens, C = 512 1521 -> 1001; one sequence 562 -> 290; C = 65, one sequence of 260 241 -> 212, 64 648 -> 507; SwiGLU, h = 384, 32 sequences,
+// C = 100 497 -> 295.  An item has all hidden units of 64 tokens: two blocks of tokens and wide networks leave too few items (h = 1024, C = 128:
+// one sequence 258 -> 279, 64 1057 -> 1084; C = 512 322 -> 197).
+inline bool tile_flow_serves(const TileLayout& t) { return t.tb > 2 || (t.tb == 2 && t.hb <= 8); }
+int tile_flow_launch(const SimtFwdArgs& a, int kind, void* stream);
 int tile_bwd_launch(const SimtBwdArgs& a, int kind, void* stream);
 
 }  // namespace e2ttt

@@ -235,6 +235,24 @@ __device__ __forceinline__ void st_split16(unsigned char* blk, int row, int col0
                      : "memory");
     }
 }
+// 16 consecutive values of one row of a 64 x 64 block in shared memory (hi; lo `lo` bytes behind)
+__device__ __forceinline__ void sts_split16(uint32_t blk, uint32_t lo, int row, int col0, const float (&v)[16]) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float x = v[8 * c + 2 * j], y = v[8 * c + 2 * j + 1];
+            const __nv_bfloat162 hh = __floats2bfloat162_rn(x, y);
+            const float2 hf = __bfloat1622float2(hh);
+            h[j] = *reinterpret_cast<const uint32_t*>(&hh);
+            l[j] = pack_bf16(x - hf.x, y - hf.y);
+        }
+        const uint32_t at = blk + row * 128 + ((((col0 >> 3) + c) ^ (row & 7)) << 4);
+        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
+        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at + lo), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
+    }
+}
 // hi + lo of 16 consecutive values
 __device__ __forceinline__ void ld_split16(const unsigned char* blk, int row, int col0, float (&v)[16]) {
     const bool sw = row & 1;

@@ -1,0 +1,35 @@
+"""The forward of chunks of more than 64 tokens on work items (csrc/tile_flow.cu) against the fp64 oracle, at the edges of its tiles: one block
+of hidden units and an odd number, one and two blocks of d, ragged chunks and blocks of tokens, several sets of sequences."""
+import numpy as np
+import pytest
+
+from paper_2608_21308_b200 import binding as E
+from paper_2608_21308_b200 import inputs
+from tests import util
+
+pytestmark = pytest.mark.gpu
+MLP, SWIGLU = inputs.KIND_MLP, inputs.KIND_SWIGLU
+# Operands are hi + lo of bf16: what a product drops is 2^-16 of it, the state sums up to 512 of them and carries them over three chunks
+# that amplify a perturbation by up to 1.8 each (GELU) or, with the product of two projections, twice that
+TOL = {MLP: 6 * 2.0**-16 * 5, SWIGLU: 40 * 2.0**-16 * 5}
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("d,h,C,L,N", [(8, 8, 65, 131, 1), (64, 64, 128, 300, 2), (72, 200, 200, 450, 3), (128, 384, 512, 1100, 2), (128, 128, 65, 66, 150),
+                                       (16, 16, 80, 250, 170)])
+def test_states_and_outputs(kind, d, h, C, L, N):
+    r = inputs.paper_regime(inputs.Recipe(B=N, H=1, L=L, d=d, h=h, C=C, kind=kind, io="bf16", seed=7, m_std=0.002))
+    x = inputs.generate(r)
+    heads = sorted({0, N // 2, N - 1})
+    ref = util.oracle_forward({k: [m[heads] for m in v] if isinstance(v, list) else v[heads] for k, v in x.items() if v is not None}, C, kind)
+    got, hd = util.gpu_forward(x, d=d, h=h, C=C, kind=kind, io="bf16", impl=E.E2TTT_IMPL_TILED)
+    assert E.e2ttt_device_status(hd["ws"]) == 0
+    errs = {"o": util.rel_err(got["o"][heads], ref["o"])}
+    assert errs["o"] <= 1e-2  # bf16 outputs
+    for name in ("W", "M"):
+        for i, m in enumerate(ref[name]):
+            errs[f"{name}{i + 1}"] = util.rel_err(got[name][i][heads], m)
+    bad = {k: v for k, v in errs.items() if k != "o" and not v <= TOL[kind]}
+    assert not bad, errs
+    again, _ = util.gpu_forward(x, d=d, h=h, C=C, kind=kind, io="bf16", impl=E.E2TTT_IMPL_TILED)
+    assert all(np.array_equal(a, b) for a, b in zip([got["o"], *got["W"], *got["M"]], [again["o"], *again["W"], *again["M"]]))
