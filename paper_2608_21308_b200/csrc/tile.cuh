@@ -72,7 +72,9 @@ struct Engine {
     __device__ void setup(unsigned char* ring_ptr, Sync* s, int* status, int rank_, int nranks_) {
         ring = smem_u32(ring_ptr);
         sy = s;
-        warp = threadIdx.x >> 5;
+        // From lane 0: the compiler then knows that it is the same for the warp, and keeps what follows from it - the MMAs' descriptors - in
+        // uniform registers
+        warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
         lane = threadIdx.x & 31;
         rank = rank_;
         nranks = nranks_;
@@ -89,7 +91,7 @@ struct Engine {
         tc_fence_before_sync();
         __syncthreads();
         tc_fence_after_sync();
-        tmem = s->tmem;
+        tmem = __shfl_sync(0xffffffffu, s->tmem, 0);
         wc.dead = &s->dead;
         wc.status = status;
     }
@@ -253,6 +255,36 @@ __device__ __forceinline__ void sts_split16(uint32_t blk, uint32_t lo, int row, 
         asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at + lo), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
     }
 }
+// 8 consecutive floats, 32-byte aligned
+__device__ __forceinline__ void st_f8(float* p, const float (&v)[8]) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void ld_f8(const float* p, float (&v)[8]) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void st_f16(float* p, const float (&v)[16]) {
+    float a[2][8];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) a[j >> 3][j & 7] = v[j];
+    st_f8(p, a[0]);
+    st_f8(p + 8, a[1]);
+}
+__device__ __forceinline__ void ld_f16(const float* p, float (&v)[16]) {
+    float a[2][8];
+    ld_f8(p, a[0]);
+    ld_f8(p + 8, a[1]);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = a[j >> 3][j & 7];
+}
+// Where the 16 values of hidden unit `row` of block bl and tokens tok .. of block tk are (tok a multiple of 16) in an fp32 [hidden x tokens]
+// intermediate.  An epilogue thread's values are neighbours: two accesses of 32 bytes instead of sixteen of 4
+__device__ __forceinline__ size_t f16_of(int bl, int tb, int tk, int tok, int row) {
+    return (((size_t)bl * tb + tk) * 4 + (tok >> 4)) * 1024 + (row & 63) * 16;
+}
 // hi + lo of 16 consecutive values
 __device__ __forceinline__ void ld_split16(const unsigned char* blk, int row, int col0, float (&v)[16]) {
     const bool sw = row & 1;
@@ -285,6 +317,16 @@ template <bool LO> __device__ __forceinline__ void st_split4(unsigned char* blk,
     }
 }
 
+__device__ __forceinline__ void acc8(uint32_t t, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(t)
+                 : "memory");
+    tmem_wait_ld();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
+}
 __device__ __forceinline__ void acc16(uint32_t t, float (&v)[16]) {
     uint32_t r[16];
     tmem_ld16(t, r);

@@ -25,6 +25,10 @@ using namespace tile;
 
 namespace {
 
+// GELU network: two more warps make up the copy and MMA warps' warpgroup, so that setmaxnreg can give the epilogues their registers (104,
+// and nothing spills: 64 sequences of 64 chunks 9.07 -> 8.40 ms).  The SwiGLU epilogues spill either way, and the copy and MMA warps of
+// that network as well with 64 (one chunk of 512 tokens, 32 sequences 559 -> 582 us)
+constexpr int chain_threads(int kind) { return kind == 0 ? 640 : kThreads; }
 constexpr int kCells = 6;                        // operand ring, cells of 16 KB; a load takes one or two neighbouring ones
 constexpr uint32_t kCell = 2 * kHalf;
 constexpr int kLoads = 8;                        // loads in flight at most
@@ -63,6 +67,7 @@ template <int NSET> struct Chain {
     uint32_t load_no = 0, cell = 0;           // ring: next load, next free cell
     uint32_t flying = 0, used = 0, feet = 0;  // copy warp: loads not known to be consumed, their cells, footprints (2 bits each)
     uint32_t job = 0;
+    bool own_T = false;
 
     __device__ bool epi() const { return warp < 16; }
     __device__ bool copier() const { return warp == 16; }
@@ -72,7 +77,7 @@ template <int NSET> struct Chain {
         resident = smem_u32(smem);
         ring = resident + kResident;
         sh = s;
-        warp = threadIdx.x >> 5;
+        warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // (as in Engine: uniform for the compiler)
         lane = threadIdx.x & 31;
         nranks = nranks_;
         if (threadIdx.x == 0) {
@@ -89,7 +94,7 @@ template <int NSET> struct Chain {
         tc_fence_before_sync();
         __syncthreads();
         tc_fence_after_sync();
-        tmem = s->tmem;
+        tmem = __shfl_sync(0xffffffffu, s->tmem, 0);
         wc.dead = &s->dead;
         wc.status = status;
     }
@@ -116,8 +121,12 @@ template <int NSET> struct Chain {
         tc_fence_after_sync();
         fence_proxy_async_all();
     }
-    __device__ void signal(uint64_t* bar) {  // epilogue warps: this warp's part of what `bar` stands for is written
-        fence_proxy_async_all();
+    // Epilogue warps: this warp's part of what `bar` stands for is written.  A fence of global memory waits for all stores under way
+    // (2-3 thousand cycles of a chunk each).  The blocks of the new S, behind `scaled`, are loaded after the chunk's cluster barriers, whose
+    // fence is in time for them; `ops` needs none where all of T's blocks are in shared memory (`own_T`)
+    __device__ void signal(uint64_t* bar) {
+        if (bar == &sh->ops && own_T) fence_proxy_async_smem();
+        else if (bar != &sh->scaled) fence_proxy_async_all();
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar);
@@ -255,7 +264,7 @@ __device__ __forceinline__ void acc_st16(uint32_t t, const float (&v)[16]) {
 
 // BESIDE: the launch has CTAs for the next group; without them the chain keeps the registers that its code costs (2 % of the time).
 // One sequence of 8192 tokens x 16 heads, training step: 12.8 -> 11.9 ms
-template <int KIND, bool NORMED, bool BESIDE> __global__ void __launch_bounds__(kThreads, 1)
+template <int KIND, bool NORMED, bool BESIDE> __global__ void __launch_bounds__(chain_threads(KIND), 1)
 tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
     constexpr int NMAT = (KIND == 0) ? 2 : 3, LAST = NMAT - 1;
     constexpr bool SW = KIND == 1;
@@ -287,6 +296,16 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
 
     if (!G.epi()) {
         // ================================================================= copy and MMA warps
+        if (!SW) asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        if (warp > 17) {  // the barriers of all threads
+#pragma unroll 1
+            for (int g = 0; g < ga.ng * (NORMED ? 3 : 2) + 1; ++g) {
+                G.cluster_arrive_all();
+                G.cluster_wait_all();
+            }
+            G.teardown();
+            return;
+        }
         // blocks of a [hidden x d] family in the workspace, own hidden units: hidden units on the lanes (MN-major where the rows are d),
         // contraction over d; and d on the lanes, contraction over the hidden units
         auto w_by_h = [&](const unsigned char* m, bool rows_d) {
@@ -465,6 +484,7 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
     }
 
     // ===================================================================== epilogue warps
+    if (!SW) asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
     const int q4 = warp & 3, grp = warp >> 2, row = 32 * q4 + lane;
     const bool on_h = row < 64 || two;      // lane of a product with hidden units on the lanes
     const int bl = b0 + (row >> 6);         // its hidden block
@@ -547,6 +567,7 @@ tile_chain_kernel(const GroupArgs ga, const NextGroup next) {
         }
         tmem_wait_st();
         if (!NORMED) G.signal(&sh.ops);
+        G.own_T = nres == NMAT;
     }
 
     // One row of dk of a chunk = its e-adjoint + the CTAs' partial sums, in CTA order
@@ -952,7 +973,7 @@ template <int KIND, bool NORMED, bool BESIDE> int launch(const GroupArgs& ga, co
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(ga.a.N * ga.a.cl + rec_ctas));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(chain_threads(KIND));
     cfg.dynamicSmemBytes = kChainSmem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];

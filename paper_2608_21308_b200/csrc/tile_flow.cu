@@ -114,27 +114,6 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-// 8 consecutive floats, 32-byte aligned
-__device__ __forceinline__ void st_row8(float* p, const float (&v)[8]) {
-    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
-                 : "memory");
-}
-__device__ __forceinline__ void ld_row8(const float* p, float (&v)[8]) {
-    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-                 : "l"(p)
-                 : "memory");
-}
-__device__ __forceinline__ void acc8(uint32_t t, float (&v)[8]) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(t)
-                 : "memory");
-    tmem_wait_ld();
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
-}
 // 8 consecutive values of one row of a 64 x 64 block in shared memory (hi; lo `lo` bytes behind)
 __device__ __forceinline__ void sts_split8(uint32_t blk, uint32_t lo, int row, int col0, const float (&v)[8]) {
     uint32_t h[4], l[4];
@@ -633,8 +612,8 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
                                 }
                                 if (live) {
                                     const size_t e0 = ((size_t)bl * tb + it.part) * 4096 + (grp * 64 + (row & 63)) * 16 + 8 * e;
-                                    st_row8(ws + tl.fc1 + e0, c1);
-                                    if (SW) st_row8(ws + tl.fc2 + e0, c2);
+                                    st_f8(ws + tl.fc1 + e0, c1);
+                                    if (SW) st_f8(ws + tl.fc2 + e0, c2);
                                 }
                                 if (e == 0 && b > 0) await(&sh.a_empty, bit(kA) ^ 1, 525);
                             } else {
@@ -775,8 +754,8 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
                     const bool live = bl < hb;
                     const float* cf = ws + (i == 0 ? tl.fc1 : tl.fc2) + (size_t)(live ? bl : b0) * tb * 4096 + (grp * 64 + (row & 63)) * 16;
                     float cv[2][8];
-                    ld_row8(cf, cv[0]);
-                    ld_row8(cf + 8, cv[1]);
+                    ld_f8(cf, cv[0]);
+                    ld_f8(cf + 8, cv[1]);
                     float* kb = sh.kb[warp];
                     const float* kx = (lane < 16 ? sc.kW : sc.kM) + 16 * grp + (lane & 15);
                     auto ld_k = [&](int tk) { return tk * 64 + 16 * grp + (lane & 15) < len ? kx[tk * 64] : 0.0f; };
@@ -800,8 +779,8 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
                         }
                         release(&sh.ph_empty[set]);
                         if (tk + 1 < tbn) {
-                            ld_row8(cf + (size_t)(tk + 1) * 4096, cv[0]);
-                            ld_row8(cf + (size_t)(tk + 1) * 4096 + 8, cv[1]);
+                            ld_f8(cf + (size_t)(tk + 1) * 4096, cv[0]);
+                            ld_f8(cf + (size_t)(tk + 1) * 4096 + 8, cv[1]);
                         }
 #pragma unroll 1
                         for (int m = 0; m < 2; ++m) {
