@@ -969,13 +969,17 @@ template <int KIND> int launch(const SimtFwdArgs& a, cudaStream_t st) {
     f.n2 = NMAT * f.ns;
     f.n3 = a.row_norm[0] ? (NMAT - 1) * f.ns + tl.db : 0;
     f.slots = tl.tb + f.n2 + f.n3;
-    // Half a set's items lie between dependent ones: as many as the GPU has in work
-    const int enough = (2 * 160 + f.slots - 1) / f.slots;
+    // How long the items take (thousand cycles, measured), and with it how many sequences keep the GPU busy while each waits for its own
+    // chain of items, with a third to spare; fewer sequences at a time are better for L2.  A sequence's weights and norm items are put off by as much as
+    // what they depend on takes
+    const double t1 = 20 + (KIND == 0 ? 11 : 14) * f.ns, t2 = 15 + 7.5 * tl.tb, t2last = 15 + 3.5 * tl.tb, t3 = f.n3 ? 10 : 0;
+    const double chain = t1 + t2 + t3, work = tl.tb * t1 + f.ns * ((NMAT - 1) * t2 + t2last) + f.n3 * t3;
+    const int enough = (int)(1.33 * 148 * chain / work) + 1;
     f.sets = a.N / enough < 1 ? 1 : a.N / enough;
     f.gs = (a.N + f.sets - 1) / f.sets;
     f.sets = (a.N + f.gs - 1) / f.gs;
-    f.off2 = f.n3 ? f.gs / 3 : f.gs / 2;
-    f.off3 = f.n3 ? 2 * f.gs / 3 : 0;
+    f.off2 = (int)(f.gs * t1 / chain);
+    f.off3 = f.n3 ? (int)(f.gs * (t1 + t2) / chain) : 0;
     f.steps = a.nchunks * f.gs + (f.off3 > f.off2 ? f.off3 : f.off2);
     const int per = (296 + a.N - 1) / a.N;
     tile_flow_init_kernel<NMAT><<<dim3(a.N, per < 16 ? per : 16), 256, 0, st>>>(a);

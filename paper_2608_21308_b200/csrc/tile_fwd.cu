@@ -468,7 +468,7 @@ template <int KIND> int launch(const SimtFwdArgs& a, cudaStream_t st) {
 
 int tile_fwd_launch(const SimtFwdArgs& a, int kind, void* stream) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (tile_flow_serves(a.lay.tl)) return tile_flow_launch(a, kind, stream);
+    if (tile_flow_serves(a.lay.tl, a.N)) return tile_flow_launch(a, kind, stream);
     return kind == 0 ? launch<0>(a, st) : launch<1>(a, st);
 }
 
