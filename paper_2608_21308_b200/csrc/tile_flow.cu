@@ -2,7 +2,7 @@
 //
 // A cluster per sequence (tile_fwd.cu) walks five phases per chunk, each ending in a barrier, and everything a phase leaves for the next -
 // 20 MB per chunk of 512 tokens at d = 128, h = 512 - is stored by threads at 18-31 B/clk and SM and read back through L2 and HBM.  All tokens
-// of a chunk see the same weights, so the chunk is cut twice instead (64 sequences of 4096 tokens: 2981 -> 1870 us):
+// of a chunk see the same weights, so the chunk is cut twice instead (64 sequences of 4096 tokens: 2990 -> 1750 us):
 //   tokens item  (sequence, chunk, 64 tokens)            z, activations, u, layer norm, outputs, pu.  All hidden units, 128 at a time: the
 //                                                        activations go from tensor memory to a shared-memory tile that the second
 //                                                        product reads; u never leaves tensor memory.  What is left for the other
@@ -14,6 +14,10 @@
 // an order in which every item comes after those it depends on, so the earliest unfinished item can always run, however many CTAs there are.
 // Sequences are taken in sets and, inside a set, out of step with each other: while one is at its tokens another is at its weights, and
 // as many items lie between dependent ones as the GPU has in work (steps, below).
+//
+// What bounds it now: a tokens item of 128 x 512 takes 75 thousand cycles, 46 of them on the activations - their instructions, half of it, and waits
+// for products and for the tile between them - a weights item of 512 tokens 77 (first matrices) and 45 (last).  An SM stores 32 B/clk, threads or bulk
+// copies alike, but 16 where a warp's lanes write 32 bytes of 32 lines (st_split16): tiles that are in shared memory anyway leave by bulk copies.
 //
 // 20 warps: 0-15 epilogues (warp w: lanes 32 (w & 3).., group w >> 2 of the columns), 16 copies operand blocks, 17 issues MMAs and the
 // bulk stores of the tiles that it reads, 18 reports finished items.  setmaxnreg gives the epilogues the control warps' registers.

@@ -1,4 +1,5 @@
-// Forward on the block-tiled engine (tile.cuh): Algorithm 1 chunk after chunk, bf16 I/O, d <= 128, any h and C, both networks.
+// Forward on the block-tiled engine (tile.cuh): Algorithm 1 chunk after chunk, bf16 I/O, d <= 128, any h and C, both networks; a few sequences of wide
+// networks (tile_flow_serves, simt_layout.h: the others run on work items, tile_flow.cu).
 //
 // A cluster of up to 8 CTAs works on one sequence; CTA r owns a slice of the hidden units - its rows of the first matrices, its
 // columns of the last - and computes everything that lives on hidden units for its slice alone.  What is summed over hidden

@@ -22,7 +22,8 @@ struct TileLayout {
     int cl;          // most CTAs per sequence
     // reverse pass, kept from launch to launch: operand blocks of the adjoints T, S of the chunk-end state
     size_t Tb[3], Sb[3];
-    // forward: operand blocks of W; tokens of two chunks; intermediates of one chunk
+    // forward: operand blocks of W; tokens of two chunks; intermediates of one chunk.  tile_flow.cu keeps the last matrix' blocks of odd chunks at fPzW[0]
+    // (and on into fPzM[0]: 2 hb tb blocks, db hb needed), scalar kernels of two chunks at fslot, its counters at fred
     size_t Wb[3], fK[2], fQ[2], fA, fAq, fc1, fc2, fslot, fPu, fPuW, fPuM, fPzW[2], fPzM[2], fred;
     // reverse pass, intermediates of one chunk
     size_t bPhb, bZk[2], bUk, bakb, bz0[2], bslot, bdk[2], bEb[2], bred;

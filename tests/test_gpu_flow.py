@@ -1,5 +1,5 @@
-"""The forward of chunks of more than 64 tokens on work items (csrc/tile_flow.cu) against the fp64 oracle, at the edges of its tiles: one block
-of hidden units and an odd number, one and two blocks of d, ragged chunks and blocks of tokens, several sets of sequences."""
+"""The forward on work items (csrc/tile_flow.cu) against the fp64 oracle, at the edges of its tiles and of its dispatch: one block of hidden units
+and an odd number, one and two blocks of d and of tokens, ragged chunks, several sets of sequences."""
 import numpy as np
 import pytest
 
@@ -16,7 +16,7 @@ TOL = {MLP: 6 * 2.0**-16 * 5, SWIGLU: 40 * 2.0**-16 * 5}
 
 @pytest.mark.parametrize("kind", [MLP, SWIGLU])
 @pytest.mark.parametrize("d,h,C,L,N", [(8, 8, 65, 131, 1), (64, 64, 128, 300, 2), (72, 200, 200, 450, 3), (128, 384, 512, 1100, 2), (128, 128, 65, 66, 150),
-                                       (16, 16, 80, 250, 170)])
+                                       (16, 16, 80, 250, 170), (96, 296, 64, 150, 3), (128, 520, 24, 60, 16)])
 def test_states_and_outputs(kind, d, h, C, L, N):
     r = inputs.paper_regime(inputs.Recipe(B=N, H=1, L=L, d=d, h=h, C=C, kind=kind, io="bf16", seed=7, m_std=0.002))
     x = inputs.generate(r)
