@@ -16,7 +16,8 @@ TOL = {MLP: 6 * 2.0**-16 * 5, SWIGLU: 40 * 2.0**-16 * 5}
 
 @pytest.mark.parametrize("kind", [MLP, SWIGLU])
 @pytest.mark.parametrize("d,h,C,L,N", [(8, 8, 65, 131, 1), (64, 64, 128, 300, 2), (72, 200, 200, 450, 3), (128, 384, 512, 1100, 2), (128, 128, 65, 66, 150),
-                                       (16, 16, 80, 250, 170), (96, 296, 64, 150, 3), (128, 520, 24, 60, 16)])
+                                       (16, 16, 80, 250, 170), (96, 296, 64, 150, 3), (128, 520, 24, 60, 16), (33, 50, 70, 150, 2),
+                                       (127, 131, 65, 70, 1)])
 def test_states_and_outputs(kind, d, h, C, L, N):
     r = inputs.paper_regime(inputs.Recipe(B=N, H=1, L=L, d=d, h=h, C=C, kind=kind, io="bf16", seed=7, m_std=0.002))
     x = inputs.generate(r)
