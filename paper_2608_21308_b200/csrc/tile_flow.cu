@@ -36,6 +36,11 @@ constexpr uint32_t kCell = 32768;
 // Shared memory: tile of activations (tokens) or of the scaled pz (weights) | tokens' rows (tokens) or the last matrix (weights) | ring
 constexpr uint32_t kTileBytes = 65536, kSideBytes = 65536;
 constexpr uint32_t kU = 256, kPh = 256;  // tensor-memory columns of u (two sums of 128) and of ph (two of 64); z and the aggregates: 0..255
+// u is summed over 8 x 128 hidden units at a time: every MMA truncates the sum it adds to.  The sums are added in fp32, by the threads that will
+// need them, in the workspace (where other kernels keep the queries' activations).  Error of the chunk-end states against 64 bits after two chunks of
+// 64 tokens, d = 128, in one sum -> this way: h = 8192 8.9e-6 -> 4.9e-6, 3072 5.5e-6 -> 4.9e-6 (operands of two bf16 terms alone: 4.4e-6).  33
+// sequences of two chunks, h = 2048: 376 -> 384 us.  Up to 1024 hidden units there is one sum, and the kernel is compiled without this
+constexpr int kUSteps = 8;
 
 struct FlowArgs {
     SimtFwdArgs a;
@@ -153,7 +158,8 @@ __device__ __forceinline__ void unpack8(const uint4& r, float (&v)[8]) {
     }
 }
 
-template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow_kernel(const FlowArgs f) {
+// WIDE: more than kUSteps slices of 128 hidden units
+template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow_kernel(const FlowArgs f) {
     constexpr int NMAT = (KIND == 0) ? 2 : 3, LAST = NMAT - 1;
     constexpr bool SW = KIND == 1;
     constexpr uint32_t NZ = SW ? 1 : 2;  // accumulators of z
@@ -398,7 +404,7 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
 #pragma unroll
                             for (int ks = 0; ks < 4; ++ks) {
                                 const uint64_t ah = a0 + ks * (2048 >> 4), wh = w0 + ks * (2048 >> 4);
-                                const bool acc = b > 1 || j > 0 || ks > 0;
+                                const bool acc = (WIDE ? (b - 1) % kUSteps != 0 : b > 1) || j > 0 || ks > 0;
                                 // the small terms in a sum of their own: every MMA truncates the sum it adds to
                                 umma_bf16_elect(tmem + kU + 128, ah + (B >> 4), wh, idesc, acc, issue);
                                 umma_bf16_elect(tmem + kU + 128, ah, wh + (B >> 4), idesc, true, issue);
@@ -407,7 +413,7 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
                             umma_commit_elect(&sh.empty[u], issue);
                         }
                         umma_commit_elect(&sh.a_empty, issue);
-                        if (b == ns) umma_commit_elect(&sh.u_full, issue);
+                        if (b == ns || (WIDE && b % kUSteps == 0)) umma_commit_elect(&sh.u_full, issue);
                         if (issue) {
                             bulk_wait_read();
                             mbar_arrive(&sh.a_empty);
@@ -533,7 +539,7 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
             arrive1(bar);
         };
         // parities of the waits, a bit each (registers are short: a spilled value comes from L2)
-        enum { kZ = 1, kA = 4, kUB = 8, kP = 16, kPz = 64, kAcc = 128, };  // kZ, kP: two bits, accumulator and parity
+        enum { kZ = 1, kA = 4, kUB = 8, kP = 16, kPz = 64, kAcc = 128, kSt = 256 };  // kZ, kP: two bits, accumulator and parity
         uint32_t par = 0;
         auto bit = [&](uint32_t b) { return (par & b) != 0 ? 1u : 0u; };
         for (uint32_t n = 0;; ++n) {
@@ -552,6 +558,7 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
             ChunkScalars<float>* scs = reinterpret_cast<ChunkScalars<float>*>(ws + tl.fslot);
             const ChunkScalars<float>& sc = scs[c & 1];
             const size_t tok0 = ((size_t)seq * a.Ls + s) * d;
+            auto u_sum = [&](int tk, int i) { return ws + tl.fAq + ((size_t)(tk * 4 + i) * 512 + threadIdx.x) * 8; };  // 8 of this thread's 32 columns
             if (it.type == kTokens) {
                 const int tk = it.part;
                 // ---- rows of the keys (0-63) and queries (64-127) -> operand slabs
@@ -636,6 +643,26 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
                         }
                     }
                     par ^= kA;
+                    if (WIDE && b > 0 && b % kUSteps == 0) {  // the MMAs that start the next sum wait for a_full
+                        await(&sh.u_full, bit(kUB), 536);
+                        par ^= kUB;
+                        if (32 * grp < dp)
+#pragma unroll 1
+                            for (int i = 0; i < 4; ++i) {
+                                float x[8], y[8];
+                                acc8(lanes + kU + 32 * grp + 8 * i, x);
+                                acc8(lanes + kU + 128 + 32 * grp + 8 * i, y);
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) x[j] += y[j];
+                                if (b > kUSteps) {
+                                    ld_f8(u_sum(it.part, i), y);
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j) x[j] += y[j];
+                                }
+                                st_f8(u_sum(it.part, i), x);
+                            }
+                        tc_fence_before_sync();
+                    }
                     signal(&sh.a_full);
                 }
                 // ---- rows: token `row` (keys 0-63, queries 64-127), 32 columns; sums over the four groups of warps through what the
@@ -648,6 +675,7 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
                 const float kw = key && live ? sc.kW[t] : 0.0f, km = key && live ? sc.kM[t] : 0.0f;
                 float u[32];
                 await(&sh.u_full, bit(kUB), 526);
+                par ^= kUB;
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
                     float x[16], y[16];
@@ -657,6 +685,14 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
                     for (int j = 0; j < 16; ++j) u[16 * i + j] = live && c0 + 16 * i + j < d ? x[j] + y[j] : 0.0f;
                 }
                 release(&sh.acc_free);
+                if (WIDE && c0 < dp)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float y[8];
+                        ld_f8(u_sum(tk, i), y);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) u[8 * i + j] += c0 + 8 * i + j < d ? y[j] : 0.0f;  // (nothing of a row past the end is used)
+                    }
                 float* red = reinterpret_cast<float*>(flow_smem + kHalf) + row;
                 auto total = [&](int which, float x) {  // over the groups, in their order
                     red[which * 512 + grp * 128] = x;
@@ -741,8 +777,8 @@ template <int KIND> __global__ void __launch_bounds__(kFlowThreads, 1) tile_flow
                     }
                 }
                 arrive1(&sh.side_free);
-                await(&sh.stored, bit(kUB), 527);
-                par ^= kUB;
+                await(&sh.stored, bit(kSt), 527);
+                par ^= kSt;
                 arrive1(&sh.tile_free);
             } else if (it.type == kWeights) {
                 const int i = it.part / ns, b0 = 2 * (it.part % ns);
@@ -956,13 +992,13 @@ template <int NMAT> __global__ void __launch_bounds__(256) tile_flow_init_kernel
     }
 }
 
-template <int KIND> int launch(const SimtFwdArgs& a, cudaStream_t st) {
+template <int KIND, bool WIDE> int launch(const SimtFwdArgs& a, cudaStream_t st) {
     constexpr int NMAT = KIND == 0 ? 2 : 3;
     static bool attr_done[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return (int)cudaGetLastError();
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(tile_flow_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFlowSmem);
+        cudaError_t e = cudaFuncSetAttribute(tile_flow_kernel<KIND, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFlowSmem);
         if (e != cudaSuccess) return (int)e;
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
@@ -988,7 +1024,7 @@ template <int KIND> int launch(const SimtFwdArgs& a, cudaStream_t st) {
     const int per = (296 + a.N - 1) / a.N;
     tile_flow_init_kernel<NMAT><<<dim3(a.N, per < 16 ? per : 16), 256, 0, st>>>(a);
     const long long items = (long long)a.N * f.slots;
-    tile_flow_kernel<KIND><<<items < 148 ? (int)items : 148, kFlowThreads, kFlowSmem, st>>>(f);
+    tile_flow_kernel<KIND, WIDE><<<items < 148 ? (int)items : 148, kFlowThreads, kFlowSmem, st>>>(f);
     return (int)cudaGetLastError();
 }
 
@@ -996,7 +1032,8 @@ template <int KIND> int launch(const SimtFwdArgs& a, cudaStream_t st) {
 
 int tile_flow_launch(const SimtFwdArgs& a, int kind, void* stream) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    return kind == 0 ? launch<0>(a, st) : launch<1>(a, st);
+    if (a.lay.tl.hb > 2 * kUSteps) return kind == 0 ? launch<0, true>(a, st) : launch<1, true>(a, st);
+    return kind == 0 ? launch<0, false>(a, st) : launch<1, false>(a, st);
 }
 
 }  // namespace e2ttt

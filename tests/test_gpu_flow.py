@@ -34,3 +34,28 @@ def test_states_and_outputs(kind, d, h, C, L, N):
     assert not bad, errs
     again, _ = util.gpu_forward(x, d=d, h=h, C=C, kind=kind, io="bf16", impl=E.E2TTT_IMPL_TILED)
     assert all(np.array_equal(a, b) for a, b in zip([got["o"], *got["W"], *got["M"]], [again["o"], *again["W"], *again["M"]]))
+
+
+def copies_of_two(d, h, C, L, N, kind, change=lambda x: None):
+    """N sequences, copies of two: all copies equal.  Returns the result and the oracle's for the two."""
+    x = inputs.generate(inputs.paper_regime(inputs.Recipe(B=2, H=1, L=L, d=d, h=h, C=C, kind=kind, io="bf16", seed=11, m_std=0.002)))
+    change(x)
+    ref = util.oracle_forward(x, C, kind)
+    rep = lambda a: np.concatenate([a] * ((N + 1) // 2))[:N]
+    xs = {n: [rep(w) for w in a] if isinstance(a, list) else rep(a) for n, a in x.items() if a is not None}
+    got, hd = util.gpu_forward(xs, d=d, h=h, C=C, kind=kind, io="bf16", impl=E.E2TTT_IMPL_TILED)
+    assert E.e2ttt_device_status(hd["ws"]) == 0
+    for a in [got["o"], *got["W"], *got["M"]]:
+        assert all(np.array_equal(a[n], a[n % 2]) for n in range(N))
+    assert util.rel_err(got["o"][:2], ref["o"]) <= 1e-2  # bf16 outputs
+    return got, ref
+
+
+# A product's operands, two bf16 terms each, are off by 2^-17 / sqrt 3 = 4.4e-6 of their size (rms).  An MMA truncates the sum it adds to, by 2^-24 of it on
+# average and always towards zero: 64 of them, one sum of u over 1024 hidden units, come to less than 64 * 2^-24 = 3.8e-6 of u.  Chunk-end states
+# of two chunks: within sqrt(4.4^2 + 3.8^2) = 5.8e-6, a fifth more for the second chunk.  512 MMAs in one sum (8192 hidden units): 9e-6 measured
+@pytest.mark.parametrize("d,h,C,L,N", [(128, 8192, 64, 128, 40), (64, 1160, 64, 100, 40), (128, 2048, 24, 48, 40), (72, 3200, 64, 128, 40)])
+def test_u_of_many_hidden_units_is_as_exact_as_that_of_few(d, h, C, L, N):
+    got, ref = copies_of_two(d, h, C, L, N, MLP)
+    errs = {f"{name}{i + 1}": util.rel_l2(got[name][i][:2], m) for name in ("W", "M") for i, m in enumerate(ref[name])}
+    assert all(e <= 7e-6 for e in errs.values()), errs
