@@ -261,12 +261,6 @@ int f64_fwd_launch(const SimtFwdArgs& a, int kind, void* stream);
 int f64_bwd_launch(const SimtBwdArgs& a, int kind, void* stream);
 // the same calls on the block-tiled kernels (tile_fwd.cu / tile_bwd.cu); the layout must have been made with `tile`
 int tile_fwd_launch(const SimtFwdArgs& a, int kind, void* stream);
-// Whether the kernel of work items (tile_flow.cu) serves a call of tile_fwd_launch, or a cluster per sequence.  us, on clusters -> on work items:
-// d = 128, h = 512, C = 512, 64 sequences of 2048 tokens 1521 -> 1000, one 562 -> 281; C = 40, 64 sequences of 320 949 -> 598; h = 1024, C = 64, 64
-// sequences of 512 1460 -> 948; SwiGLU, h = 384, C = 64, normalised, 128 sequences of 512 2421 -> 1889.  An item has all hidden units of
-// 64 tokens: few sequences of wide networks and few blocks of tokens have a longer way through it than through eight CTAs (h = 1024, C = 64, 8
-// sequences 380 -> 521, 16 589 -> 569; C = 128, 8 260 -> 294; h = 512, C = 40, 8 344 -> 369; h = 384, C = 64, 8 334 -> 325).
-inline bool tile_flow_serves(const TileLayout& t, int N) { return t.hb <= 6 * t.tb || N > tile_clusters_fit(kTileMaxCl); }
 int tile_flow_launch(const SimtFwdArgs& a, int kind, void* stream);
 int tile_bwd_launch(const SimtBwdArgs& a, int kind, void* stream);
 

@@ -13,7 +13,7 @@
 // Items depend on earlier items of the same sequence: counters per sequence, waited for by the copy warp.  The queue hands items out in
 // an order in which every item comes after those it depends on, so the earliest unfinished item can always run, however many CTAs there are.
 // Sequences are taken in sets and, inside a set, out of step with each other: while one is at its tokens another is at its weights, and
-// as many items lie between dependent ones as the GPU has in work (steps, below).
+// as many items lie between dependent ones as the GPU has in work (flow_plan, tile_flow.h).
 //
 // What bounds it now: a tokens item of 128 x 512 takes 75 thousand cycles, 46 of them on the activations - their instructions, half of it, and waits
 // for products and for the tile between them - a weights item of 512 tokens 77 (first matrices) and 45 (last).  An SM stores 32 B/clk, threads or bulk
@@ -21,8 +21,8 @@
 //
 // 20 warps: 0-15 epilogues (warp w: lanes 32 (w & 3).., group w >> 2 of the columns), 16 copies operand blocks, 17 issues MMAs and the
 // bulk stores of the tiles that it reads, 18 reports finished items.  setmaxnreg gives the epilogues the control warps' registers.
-#include "simt_layout.h"
 #include "tile.cuh"
+#include "tile_flow.h"
 
 namespace e2ttt {
 using namespace tile;
@@ -44,9 +44,7 @@ constexpr int kUSteps = 8;
 
 struct FlowArgs {
     SimtFwdArgs a;
-    int sets, gs, off2, off3;   // sets of gs sequences; a sequence's weights (norm) items come off2 (off3) steps after its tokens
-    int steps, slots;           // steps of a set, items of a step
-    int ns, n2, n3;             // slices of 128 hidden units; weights items, norm items of a chunk
+    FlowPlan p;
 };
 
 struct FlowShared {
@@ -72,30 +70,6 @@ struct Counters {
     unsigned tokens, weights, norms, pad;
     unsigned long long queue;
 };
-
-enum { kNone, kTokens, kWeights, kNorm, kEnd };
-struct Item {
-    int type, seq, c, part;
-};
-
-__device__ __forceinline__ Item decode(const FlowArgs& f, long long id) {
-    const SimtFwdArgs& a = f.a;
-    const long long per = (long long)f.steps * f.slots;
-    const int set = (int)(id / per);
-    if (set >= f.sets) return {kEnd, 0, 0, 0};
-    const long long r = id - set * per;
-    const int step = (int)(r / f.slots), slot = (int)(r - (long long)step * f.slots), tb = a.lay.tl.tb;
-    Item it;
-    int j = step;
-    if (slot < tb) { it.type = kTokens; it.part = slot; }
-    else if (slot < tb + f.n2) { it.type = kWeights; it.part = slot - tb; j -= f.off2; }
-    else { it.type = kNorm; it.part = slot - tb - f.n2; j -= f.off3; }
-    if (j < 0 || j >= a.nchunks * f.gs) return {kNone, 0, 0, 0};
-    it.c = j / f.gs;
-    it.seq = set * f.gs + j - it.c * f.gs;
-    if (it.seq >= a.N || (it.type == kTokens && it.part * 64 >= a.L - it.c * a.C)) it.type = kNone;
-    return it;
-}
 
 // The order in which copy and MMA warps go through the cells, and the parity of a cell's next load
 struct Cells {
@@ -196,7 +170,7 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
 
     const SimtLayout& lay = a.lay;
     const TileLayout& tl = lay.tl;
-    const int d = a.d, h = a.h, db = tl.db, hb = tl.hb, tb = tl.tb, dp = db * 64, ns = f.ns;
+    const int d = a.d, h = a.h, db = tl.db, hb = tl.hb, tb = tl.tb, dp = db * 64, ns = f.p.ns;
     const size_t dh = (size_t)d * h;
     const bool normed = a.row_norm[0] != nullptr, queries = a.o != nullptr;
     auto ws_of = [&](int seq) { return reinterpret_cast<float*>(a.ws) + (size_t)seq * lay.per_seq; };
@@ -210,7 +184,7 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
     };
     auto item_of = [&](uint32_t n) {
         const int4 x = sh.id[n & 1];
-        return Item{__shfl_sync(0xffffffffu, x.x, 0), __shfl_sync(0xffffffffu, x.y, 0), __shfl_sync(0xffffffffu, x.z, 0), __shfl_sync(0xffffffffu, x.w, 0)};
+        return FlowItem{__shfl_sync(0xffffffffu, x.x, 0), __shfl_sync(0xffffffffu, x.y, 0), __shfl_sync(0xffffffffu, x.z, 0), __shfl_sync(0xffffffffu, x.w, 0)};
     };
     auto cell_at = [&](uint32_t u) { return u < kCells ? ring0 + u * kCell : tile0 + (u - kCells) * kCell; };
     auto given_up = [&] { return __any_sync(0xffffffffu, *wc.dead != 0); };
@@ -250,23 +224,23 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
         unsigned long long* queue = &counters(0)->queue;
         for (uint32_t n = 0;; ++n) {
             if (n >= 2) mbar_wait(&sh.fin[n & 1], ((n >> 1) - 1) & 1, wc, 502);
-            Item it;
+            FlowItem it;
             do {
                 unsigned long long x = 0;
                 if (lane == 0) x = atomicAdd(queue, 1ull);
-                it = decode(f, (long long)__shfl_sync(0xffffffffu, x, 0));
-            } while (it.type == kNone);
+                it = flow_item(f.p, (long long)__shfl_sync(0xffffffffu, x, 0));
+            } while (it.type == kFlowNone);
             if (lane == 0) sh.id[n & 1] = make_int4(it.type, it.seq, it.c, it.part);
             arrive1(&sh.item[n & 1]);
-            if (it.type == kEnd || given_up()) break;
+            if (it.type == kFlowEnd || given_up()) break;
             const int c = it.c, tbn = (tokens_of(c) + 63) / 64;
             float* ws = ws_of(it.seq);
             auto blk = [&](size_t off) { return reinterpret_cast<const unsigned char*>(ws + off); };
             {   // what the item depends on
                 const Counters* cn = counters(it.seq);
-                const unsigned* p = it.type == kTokens ? (normed ? &cn->norms : &cn->weights) : it.type == kWeights ? &cn->tokens : &cn->weights;
-                const unsigned need = it.type == kTokens ? (unsigned)c * (normed ? f.n3 : f.n2)
-                                      : it.type == kWeights ? (unsigned)(c * tb + tbn) : (unsigned)(c + 1) * f.n2;
+                const unsigned* p = it.type == kFlowTokens ? (normed ? &cn->norms : &cn->weights) : it.type == kFlowWeights ? &cn->tokens : &cn->weights;
+                const unsigned need = it.type == kFlowTokens ? (unsigned)c * (normed ? f.p.n3 : f.p.n2)
+                                      : it.type == kFlowWeights ? (unsigned)(c * tb + tbn) : (unsigned)(c + 1) * f.p.n2;
                 if (need && ld_acquire(p) < need && !*wc.dead) {
                     const long long t0 = clock64();
                     while (ld_acquire(p) < need) {
@@ -283,7 +257,7 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
                 fence_proxy_async_all();
                 arrive1(&sh.go[n & 1]);
             }
-            if (it.type == kTokens) {
+            if (it.type == kFlowTokens) {
                 const unsigned char* wl = blk(wb_of(LAST, c));
                 for (int b = 0; b <= ns; ++b) {
                     if (b < ns)
@@ -299,7 +273,7 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
                             load(p, db == 2 ? p + B : nullptr);
                         }
                 }
-            } else if (it.type == kWeights) {
+            } else if (it.type == kFlowWeights) {
                 const int i = it.part / ns, b0 = 2 * (it.part % ns);
                 const bool two = b0 + 1 < hb;
                 if (i < LAST) {
@@ -347,13 +321,13 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
         };
         for (uint32_t n = 0;; ++n) {
             await(&sh.item[n & 1], n >> 1, 512);
-            const Item it = item_of(n);
-            if (it.type == kEnd || given_up()) break;
+            const FlowItem it = item_of(n);
+            if (it.type == kFlowEnd || given_up()) break;
             if (n >= 1) await(&sh.acc_free, n - 1, 513);
             const int c = it.c, tbn = (tokens_of(c) + 63) / 64;
             float* ws = ws_of(it.seq);
             auto blk = [&](size_t off) { return reinterpret_cast<unsigned char*>(ws + off); };
-            if (it.type == kTokens) {
+            if (it.type == kFlowTokens) {
                 const int tk = it.part;
                 await(&sh.x_full, nx++, 514);
                 await(&sh.go[n & 1], n >> 1, 535);  // the chunk before has been read
@@ -428,7 +402,7 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
                     mbar_arrive(&sh.stored);
                 }
                 __syncwarp();
-            } else if (it.type == kWeights && it.part / ns < LAST) {
+            } else if (it.type == kFlowWeights && it.part / ns < LAST) {
                 const int b0 = 2 * (it.part % ns);
                 const bool two = b0 + 1 < hb;
                 await(&sh.w_full, nw++, 517);
@@ -477,7 +451,7 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
                 }
                 arrive1(&sh.side_free);
                 umma_commit_elect(&sh.acc_full, issue);
-            } else if (it.type == kWeights) {
+            } else if (it.type == kFlowWeights) {
                 const uint32_t ida = make_idesc(128, db == 2 ? 128 : 64, false, true);
                 cells.all(true);
 #pragma unroll 1
@@ -513,13 +487,13 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
         // and by bulk copies.  A warp of its own: the fence waits for all of the item's stores
         for (uint32_t n = 0;; ++n) {
             mbar_wait(&sh.item[n & 1], (n >> 1) & 1, wc, 541);
-            const Item it = item_of(n);
-            if (it.type == kEnd || given_up()) break;
+            const FlowItem it = item_of(n);
+            if (it.type == kFlowEnd || given_up()) break;
             mbar_wait(&sh.written[n & 1], (n >> 1) & 1, wc, 542);
             if (lane == 0) {
                 Counters* cn = counters(it.seq);
                 __threadfence();
-                atomicAdd(it.type == kTokens ? &cn->tokens : it.type == kWeights ? &cn->weights : &cn->norms, 1u);
+                atomicAdd(it.type == kFlowTokens ? &cn->tokens : it.type == kFlowWeights ? &cn->weights : &cn->norms, 1u);
             }
             arrive1(&sh.fin[n & 1]);
         }
@@ -549,8 +523,8 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
             }
             epi_sync();
             if (!sh.cur[n & 1]) break;
-            const Item it = item_of(n);
-            if (it.type == kEnd) break;
+            const FlowItem it = item_of(n);
+            if (it.type == kFlowEnd) break;
             const int c = it.c, seq = it.seq, s = c * a.C, len = tokens_of(c), tbn = (len + 63) / 64;
             const bool last_chunk = c + 1 == a.nchunks;
             float* ws = ws_of(seq);
@@ -559,7 +533,7 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
             const ChunkScalars<float>& sc = scs[c & 1];
             const size_t tok0 = ((size_t)seq * a.Ls + s) * d;
             auto u_sum = [&](int tk, int i) { return ws + tl.fAq + ((size_t)(tk * 4 + i) * 512 + threadIdx.x) * 8; };  // 8 of this thread's 32 columns
-            if (it.type == kTokens) {
+            if (it.type == kFlowTokens) {
                 const int tk = it.part;
                 // ---- rows of the keys (0-63) and queries (64-127) -> operand slabs
                 if (n >= 1) await(&sh.side_free, n - 1, 522);
@@ -791,7 +765,7 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
                 await(&sh.stored, bit(kSt), 527);
                 par ^= kSt;
                 arrive1(&sh.tile_free);
-            } else if (it.type == kWeights) {
+            } else if (it.type == kFlowWeights) {
                 const int i = it.part / ns, b0 = 2 * (it.part % ns);
                 const bool two = b0 + 1 < hb;
                 await(&sh.go[n & 1], n >> 1, 528);
@@ -1013,28 +987,10 @@ template <int KIND, bool WIDE> int launch(const SimtFwdArgs& a, cudaStream_t st)
         if (e != cudaSuccess) return (int)e;
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
-    const TileLayout& tl = a.lay.tl;
-    FlowArgs f{};
-    f.a = a;
-    f.ns = (tl.hb + 1) / 2;
-    f.n2 = NMAT * f.ns;
-    f.n3 = a.row_norm[0] ? (NMAT - 1) * f.ns + tl.db : 0;
-    f.slots = tl.tb + f.n2 + f.n3;
-    // How long the items take (thousand cycles, measured), and with it how many sequences keep the GPU busy while each waits for its own
-    // chain of items, with a third to spare; fewer sequences at a time are better for L2.  A sequence's weights and norm items are put off by as much as
-    // what they depend on takes
-    const double t1 = 20 + (KIND == 0 ? 11 : 14) * f.ns, t2 = 15 + 7.5 * tl.tb, t2last = 15 + 3.5 * tl.tb, t3 = f.n3 ? 10 : 0;
-    const double chain = t1 + t2 + t3, work = tl.tb * t1 + f.ns * ((NMAT - 1) * t2 + t2last) + f.n3 * t3;
-    const int enough = (int)(1.33 * 148 * chain / work) + 1;
-    f.sets = a.N / enough < 1 ? 1 : a.N / enough;
-    f.gs = (a.N + f.sets - 1) / f.sets;
-    f.sets = (a.N + f.gs - 1) / f.gs;
-    f.off2 = (int)(f.gs * t1 / chain);
-    f.off3 = f.n3 ? (int)(f.gs * (t1 + t2) / chain) : 0;
-    f.steps = a.nchunks * f.gs + (f.off3 > f.off2 ? f.off3 : f.off2);
+    const FlowArgs f{a, flow_plan(a.lay.tl, a.N, a.L, a.C, NMAT, a.row_norm[0] != nullptr)};
     const int per = (296 + a.N - 1) / a.N;
     tile_flow_init_kernel<NMAT><<<dim3(a.N, per < 16 ? per : 16), 256, 0, st>>>(a);
-    const long long items = (long long)a.N * f.slots;
+    const long long items = (long long)a.N * f.p.slots;
     tile_flow_kernel<KIND, WIDE><<<items < 148 ? (int)items : 148, kFlowThreads, kFlowSmem, st>>>(f);
     return (int)cudaGetLastError();
 }

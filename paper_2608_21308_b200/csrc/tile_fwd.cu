@@ -1,5 +1,5 @@
 // Forward on the block-tiled engine (tile.cuh): Algorithm 1 chunk after chunk, bf16 I/O, d <= 128, any h and C, both networks; a few sequences of wide
-// networks (tile_flow_serves, simt_layout.h: the others run on work items, tile_flow.cu).
+// networks (tile_flow_serves, tile_flow.h: the others run on work items, tile_flow.cu).
 //
 // A cluster of up to 8 CTAs works on one sequence; CTA r owns a slice of the hidden units - its rows of the first matrices, its
 // columns of the last - and computes everything that lives on hidden units for its slice alone.  What is summed over hidden
@@ -7,8 +7,8 @@
 // the parts of its share of the rows in CTA order and runs the layer norm and its adjoint on them.
 // State: fp32, row-major, in the workspace (or directly in the slots of the saved states), updated by the aggregation's epilogue, which
 // also writes the operand blocks of the next chunk's weights.
-#include "simt_layout.h"
 #include "tile.cuh"
+#include "tile_flow.h"
 
 namespace e2ttt {
 using namespace tile;
@@ -469,7 +469,7 @@ template <int KIND> int launch(const SimtFwdArgs& a, cudaStream_t st) {
 
 int tile_fwd_launch(const SimtFwdArgs& a, int kind, void* stream) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (tile_flow_serves(a.lay.tl, a.N)) return tile_flow_launch(a, kind, stream);
+    if (tile_flow_serves(a.lay.tl, a.N, a.C, a.Ls, kind == 0 ? 2 : 3, a.row_norm[0] != nullptr)) return tile_flow_launch(a, kind, stream);
     return kind == 0 ? launch<0>(a, st) : launch<1>(a, st);
 }
 
