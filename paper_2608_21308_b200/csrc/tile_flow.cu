@@ -674,30 +674,18 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
                     const float* p = red + which * 512;
                     return (p[0] + p[128]) + (p[256] + p[384]);
                 };
-                // Pairwise: pu is free of a common part and of one along y only as far as these sums are exact, and weights of one sign bring it out.
-                // Error of the first matrix' momentum against 64 bits with all weights positive, C = 512, d = 128, h = 512: 3.7e-5 with one value after
-                // the other, 3.0e-5 this way and on clusters; no difference in time
-                auto pairs = [](const float (&v)[8]) { return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])); };
-                float x[4], y[4];
+                float x = 0.0f, y = 0.0f;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float v[8];
+                for (int j = 0; j < 32; ++j) x += u[j];
+                const float mu = total(0, x) / (float)d;
+                x = 0.0f;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) v[j] = u[8 * i + j];
-                    x[i] = pairs(v);
+                for (int j = 0; j < 32; ++j) {
+                    u[j] = c0 + j < d ? u[j] - mu : 0.0f;
+                    x += u[j] * u[j];
                 }
-                const float mu = total(0, (x[0] + x[1]) + (x[2] + x[3])) / (float)d;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float v[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        u[8 * i + j] = c0 + 8 * i + j < d ? u[8 * i + j] - mu : 0.0f;
-                        v[j] = u[8 * i + j] * u[8 * i + j];
-                    }
-                    x[i] = pairs(v);
-                }
-                const float r = r_rsqrt(total(1, (x[0] + x[1]) + (x[2] + x[3])) / (float)d + a.eps);
+                const float r = r_rsqrt(total(1, x) / (float)d + a.eps);
+                x = 0.0f;
                 auto error = [&](int i, float (&e)[8]) {  // k + y - v, of 8 columns; of a query: its output
                     float vv[8];
                     const int at = ((((c0 >> 3) + i) ^ row) & 7) * 16;
@@ -713,13 +701,14 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
 #pragma unroll
                     for (int j = 0; j < 8; ++j) u[8 * i + j] *= r;
                     error(i, e);
-                    x[i] = pairs(e);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) e[j] *= u[8 * i + j];
-                    y[i] = pairs(e);
+                    for (int j = 0; j < 8; ++j) {
+                        x += e[j];
+                        y += e[j] * u[8 * i + j];
+                    }
                 }
-                red[3 * 512 + grp * 128] = (y[0] + y[1]) + (y[2] + y[3]);
-                const float se = total(2, (x[0] + x[1]) + (x[2] + x[3])) / (float)d;
+                red[3 * 512 + grp * 128] = y;
+                const float se = total(2, x) / (float)d;
                 const float* py = red + 3 * 512;
                 const float sey = ((py[0] + py[128]) + (py[256] + py[384])) / (float)d;
                 if (key) {
