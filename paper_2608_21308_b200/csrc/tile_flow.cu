@@ -114,6 +114,11 @@ __device__ __forceinline__ void sts_split8(uint32_t blk, uint32_t lo, int row, i
 // 8 values of a token's row at column c, 0 beyond d
 __device__ __forceinline__ uint4 ld_row8(const __nv_bfloat16* row, int c, int d) {
     if ((d & 7) == 0) return c < d ? *reinterpret_cast<const uint4*>(row + c) : make_uint4(0u, 0u, 0u, 0u);
+    if ((d & 3) == 0) {  // rows of 8 bytes' alignment
+        const uint2 x = c < d ? *reinterpret_cast<const uint2*>(row + c) : make_uint2(0u, 0u);
+        const uint2 y = c + 4 < d ? *reinterpret_cast<const uint2*>(row + c + 4) : make_uint2(0u, 0u);
+        return make_uint4(x.x, x.y, y.x, y.y);
+    }
     uint32_t w[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -743,6 +748,11 @@ template <int KIND, bool WIDE> __global__ void __launch_bounds__(kFlowThreads, 1
                         if ((d & 7) == 0) {
                             if (c0 + 8 * i < d)
                                 *reinterpret_cast<uint4*>(o + c0 + 8 * i) = make_uint4(pack_bf16(e[0], e[1]), pack_bf16(e[2], e[3]), pack_bf16(e[4], e[5]), pack_bf16(e[6], e[7]));
+                        } else if ((d & 3) == 0) {
+#pragma unroll
+                            for (int j = 0; j < 8; j += 4)
+                                if (c0 + 8 * i + j < d)
+                                    *reinterpret_cast<uint2*>(o + c0 + 8 * i + j) = make_uint2(pack_bf16(e[j], e[j + 1]), pack_bf16(e[j + 2], e[j + 3]));
                         } else {
 #pragma unroll
                             for (int j = 0; j < 8; ++j)

@@ -59,3 +59,14 @@ def test_u_of_many_hidden_units_is_as_exact_as_that_of_few(d, h, C, L, N):
     got, ref = copies_of_two(d, h, C, L, N, MLP)
     errs = {f"{name}{i + 1}": util.rel_l2(got[name][i][:2], m) for name in ("W", "M") for i, m in enumerate(ref[name])}
     assert all(e <= 7e-6 for e in errs.values()), errs
+
+
+# Operands are off by 2^-17 / sqrt 3 = 4.4e-6 (rms) in each of the four products from a chunk's keys to its aggregates, 9e-6 together; two more chunks that
+# amplify it by up to 2 each stay below 1e-4.  An operand without its second term is off by 2^-9 / sqrt 3 = 1.1e-3
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("d,h,C,L", [(4, 8, 64, 70), (36, 144, 40, 75), (68, 72, 65, 130), (100, 400, 64, 129), (124, 64, 128, 200)])
+def test_rows_of_8_bytes_alignment(d, h, C, L, kind):
+    """Head dimensions that are multiples of four and not of eight; the bound as above, two chunks of several at most."""
+    got, ref = copies_of_two(d, h, C, L, 3, kind)
+    errs = {f"{name}{i + 1}": util.rel_l2(got[name][i][:2], m) for name in ("W", "M") for i, m in enumerate(ref[name])}
+    assert all(e <= 1e-4 for e in errs.values()), errs
