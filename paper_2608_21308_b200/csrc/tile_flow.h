@@ -10,27 +10,32 @@ inline int flow_blocks(int C, int Ls) { return ((Ls < C ? Ls : C) + 63) / 64; }
 
 // Whether the kernel of work items serves a call of tile_fwd_launch, or a cluster per sequence.  A tokens item has all hidden units of 64 tokens, one after the
 // other, so that wide networks have a longer way through it than through the eight, six or four CTAs that up to 15, 22 or 33 sequences get; several
-// blocks of tokens are items side by side but a loop to a cluster, more chunks leave items of other sequences to fill the gaps with, and more CTAs
-// in clusters share the way to L2.  us, on clusters -> on work items (d = 128 and the GELU network where not said):
-//   one chunk of one block    8 sequences, h = 256 49 -> 48, 384 51 -> 53, 512 51 -> 56, 2048 96 -> 135; 22, d = 64, h = 448 49 -> 62; 33, h = 1024 129 -> 140;
-//                             34 153 -> 143; 64 217 -> 206; SwiGLU, h = 384, 15 sequences 70 -> 62, 20 76 -> 72
-//   one chunk of two, three   128 tokens, 4 sequences, h = 768 70 -> 71, 1024 68 -> 79; 24, h = 1536 181 -> 173; 28, d = 64, h = 1024 125 -> 144;
-//                             192 tokens, 4 sequences, h = 1536 135 -> 105, 22 180 -> 211
-//   eight chunks of one       8 sequences, h = 384 319 -> 308, 640 354 -> 383, 1024 358 -> 503; 16, h = 512 366 -> 352, 768 385 -> 451, SwiGLU 718 -> 574;
-//                             20, h = 768 586 -> 490, 2048 946 -> 1011; 24, h = 1024 848 -> 636, 4096 1951 -> 1842; d = 64: 22, h = 640 336 -> 377,
-//                             24, h = 768 508 -> 435
-//   four chunks of two        8 sequences, h = 768 242 -> 233, 1024 237 -> 270; 16, h = 1024 403 -> 338, 4096 1055 -> 949
-//   normalised                four chunks of one: 8 sequences, h = 384 1.06, 24, h = 1024 .94, 2048 934 -> 1239 (a norm item has 64 whole rows of the last matrix);
-//                             one chunk, 192 of 512 tokens, 15 sequences, h = 1024 152 -> 184
-// Chunks of 512, h = 512, 64 sequences of 2048 tokens 1521 -> 1000
+// blocks of tokens are items side by side but a loop to a cluster, and more CTAs in clusters share the way to L2.  It does not go by the number of chunks, so that
+// a sequence given in several calls of whole chunks has the same bits as in one; single chunks are the worse for work items (a queue filled and
+// drained at once), and the lines lie where calls of one and of four chunks balance.  Time on work items / on clusters, one chunk, four chunks (d = 128 and
+// the GELU network where not said; 7000 calls measured):
+//   one block     8 sequences, h = 256 .96 .87, 384 1.06 .98, 512 1.12 1.10, 1024 1.39 1.40; d = 64, 33, h = 512 1.17 1.04; 22, h = 512 1.08 .87, 640 1.17 .86, 768 1.12 .84,
+//                 1024 1.17 .96; 23, h = 512 .96 .87, 1024 1.03 .78, 2048 1.12 .96; 28, h = 2048 1.10 .85; SwiGLU: 16, h = 512 .90 .86, 768 1.07 .86, 1024 1.13 .97
+//   two blocks    15 sequences, h = 768 .92 .76, 1024 1.12 .87; 16, h = 1024 .94 .81, 1536 1.05 .85, 2048 1.06 .91; 22, h = 2048 1.08 .90
+//   three, four   8 sequences, h = 1536 .91 .76, 2048 1.00 .87 | .93 .80; 15, h = 2048 1.09 .87 | .99 .79; 22 1.14 .79 | .98 .72; 64, h = 512 .77 .60 | .74 .60
+//   normalised    (a norm item has 64 whole rows of the last matrix)  one block: 8 sequences, h = 384 1.03 1.05, 22, h = 640 1.15 .94, 33, h = 1024 1.16 1.00, 64, h = 2048
+//                 1.06 1.09; d = 64: 33, h = 512 1.06 1.12, SwiGLU 22 .89 .99; two: d = 64, 22, h = 640 .98 .92, 768 1.18 1.08; four: 22, h = 2048 1.11 1.06, 23 .95 .93
+// Chunks of 512, h = 512, 64 sequences of 2048 tokens 1521 -> 1000 us
 inline bool tile_flow_serves(const TileLayout& t, int N, int C, int Ls, int nmat, bool normed) {
-    const int tb = flow_blocks(C, Ls);
-    const bool one = Ls <= C;
-    if (normed && t.hb > 16 && tb <= 3 && N <= 74) return false;
-    if (t.hb <= (tb > 2 && N <= 16 ? (normed ? 5 : 8) : 6) * tb) return !((one || normed) && tb == 1 && nmat == 2 && t.hb > 4 && N <= 22);
-    if (tb > 3 || (tb > 1 && !one)) return N > 15;
-    if (one) return N > 33 || (N > 22 && (tb == 3 || (tb == 2 && t.db == 2)));
-    return N > 22 || (N > 18 && t.db == 2 && t.hb <= 16) || (N > 15 && nmat == 3 && t.hb <= 24);
+    const int tb = flow_blocks(C, Ls), hb = t.hb;
+    const bool wide = t.db == 2, sw = nmat == 3;
+    if (normed && hb > 16 && tb <= 3 && N <= 74) return false;
+    if (tb > 2) return hb <= (normed ? 5 : 8) * tb || N > (normed && hb > 24 ? 22 : 15);
+    if (tb == 2) return hb <= (wide ? 12 : normed ? 6 : 10) || N > (hb > 24 || (normed && hb > 8) ? 22 : 15);
+    if (hb <= 4) return true;
+    if (normed) {
+        if (hb <= 6) return N > 22 || (sw && wide);
+        return N > (hb <= 8 && (wide || sw) ? 15 : hb <= 12 && (wide || sw) ? 22 : 33);
+    }
+    if (hb <= 6) return true;
+    if (hb > 16) return N > 24;
+    if (sw) return N > (wide && hb <= 12 ? 15 : 22);
+    return N > (wide ? (hb <= 8 ? 20 : 18) : hb <= 8 ? 33 : 24);
 }
 
 struct FlowPlan {

@@ -101,3 +101,29 @@ int main() {
 
 def test_calls_take_the_kernel_that_measured_the_faster(tmp_path):
     run(tmp_path, LINES)
+
+
+SPLIT = r"""
+int main() {
+    for (int N : {1, 2, 8, 15, 16, 19, 22, 23, 25, 33, 34, 64, 75, 148})
+        for (int d : {64, 128})
+            for (int hb = 1; hb <= 80; ++hb)
+                for (int C : {16, 64, 100, 128, 192, 256, 512})
+                    for (int nmat : {2, 3})
+                        for (int normed = 0; normed < 2; ++normed) {
+                            TileLayout tl{};
+                            tl.db = d / 64; tl.hb = hb; tl.tb = (C + 63) / 64;
+                            const bool one = tile_flow_serves(tl, N, C, C, nmat, normed);
+                            for (int Ls : {C + 1, 2 * C, 4 * C, 31 * C + 3})
+                                if (tile_flow_serves(tl, N, C, Ls, nmat, normed) != one) {
+                                    std::printf("N=%d d=%d hb=%d C=%d Ls=%d nmat=%d normed=%d\n", N, d, hb, C, Ls, nmat, normed);
+                                    return 1;
+                                }
+                        }
+    return 0;
+}
+"""
+
+
+def test_a_sequence_in_several_calls_takes_the_kernel_of_one(tmp_path):
+    run(tmp_path, SPLIT)

@@ -70,3 +70,23 @@ def test_rows_of_8_bytes_alignment(d, h, C, L, kind):
     got, ref = copies_of_two(d, h, C, L, 3, kind)
     errs = {f"{name}{i + 1}": util.rel_l2(got[name][i][:2], m) for name in ("W", "M") for i, m in enumerate(ref[name])}
     assert all(e <= 1e-4 for e in errs.values()), errs
+
+
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("N,d,h,C", [(8, 128, 384, 64), (16, 64, 320, 48), (24, 128, 1024, 16), (19, 128, 768, 64), (16, 128, 1600, 128), (3, 128, 512, 512)])
+def test_a_sequence_in_several_calls_has_the_bits_of_one(N, d, h, C, kind):
+    """Chunk by chunk, and in calls of one and two chunks, on either side of the lines between work items and clusters."""
+    L = 3 * C
+    x = inputs.generate(inputs.paper_regime(inputs.Recipe(B=2, H=1, L=L, d=d, h=h, C=C, kind=kind, io="bf16", seed=13, m_std=0.002)))
+    rep = lambda a: np.concatenate([a] * ((N + 1) // 2))[:N]
+    x = {n: [rep(w) for w in a] if isinstance(a, list) else rep(a) for n, a in x.items() if a is not None}
+    run = lambda y: util.gpu_forward(y, d=d, h=h, C=C, kind=kind, io="bf16", impl=E.E2TTT_IMPL_TILED)[0]
+    whole = run(x)
+    for cuts in ((0, C, 2 * C, L), (0, C, L)):
+        W, M, o = x["W"], x["M"], []
+        for a, b in zip(cuts, cuts[1:]):
+            part = run({**{n: np.ascontiguousarray(v[:, a:b]) for n, v in x.items() if n not in ("W", "M")}, "W": W, "M": M})
+            W, M = part["W"], part["M"]
+            o.append(part["o"])
+        assert np.array_equal(np.concatenate(o, 1), whole["o"])
+        assert all(np.array_equal(a, b) for a, b in zip([*W, *M], [*whole["W"], *whole["M"]]))
