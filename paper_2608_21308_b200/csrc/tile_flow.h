@@ -65,6 +65,13 @@ inline FlowPlan flow_plan(const TileLayout& tl, int N, int L, int C, int nmat, b
     f.sets = (N + f.gs - 1) / f.gs;
     f.off2 = (int)(f.gs * t1 / chain);
     f.off3 = f.n3 ? (int)(f.gs * (t1 + t2) / chain) : 0;
+    if (f.nchunks == 1 && N * f.tb <= 148 && N * f.slots > 148) {
+        // One chunk, a CTA for every tokens item but not for every item: tokens first, or the last of them wait for CTAs that wait for the first (64 sequences
+        // of 64 tokens, d = 64, h = 192 62 -> 54 us, on clusters 56; 148, h = 64 68 -> 56, 59)
+        f.sets = 1;
+        f.gs = f.off2 = N;
+        f.off3 = f.n3 ? 2 * N : 0;
+    }
     f.steps = f.nchunks * f.gs + (f.off3 > f.off2 ? f.off3 : f.off2);
     return f;
 }

@@ -127,3 +127,34 @@ int main() {
 
 def test_a_sequence_in_several_calls_takes_the_kernel_of_one(tmp_path):
     run(tmp_path, SPLIT)
+
+
+FIRST = r"""
+int main() {
+    int few = 0;
+    for (int N : {1, 5, 34, 64, 74, 100, 148, 149})
+        for (int h : {64, 192, 512})
+            for (int C : {16, 64, 128, 512})
+                for (int nmat : {2, 3})
+                    for (int normed = 0; normed < 2; ++normed) {
+                        TileLayout tl{};
+                        tl.db = 2; tl.hb = h / 64; tl.tb = (C + 63) / 64;
+                        const FlowPlan f = flow_plan(tl, N, C, C, nmat, normed);
+                        if (N * f.tb > 148 || N * f.slots <= 148) continue;
+                        ++few;
+                        long long tokens = 0, id = 0;
+                        for (FlowItem it = flow_item(f, 0); it.type != kFlowEnd; it = flow_item(f, ++id)) {
+                            if (it.type == kFlowTokens) ++tokens;
+                            if (it.type == kFlowWeights && tokens < (long long)N * f.tb) {
+                                std::printf("N=%d h=%d C=%d nmat=%d normed=%d\n", N, h, C, nmat, normed);
+                                return 1;
+                            }
+                        }
+                    }
+    return few > 40 ? 0 : 2;
+}
+"""
+
+
+def test_single_chunks_start_with_their_tokens(tmp_path):
+    run(tmp_path, FIRST)
