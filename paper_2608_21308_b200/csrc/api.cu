@@ -5,6 +5,7 @@
 #include "apply.h"
 #include "prepare.h"
 #include "simt_layout.h"
+#include "tile_flow.h"
 #include "tc_fwd.h"
 #include "tc_swiglu.h"
 
@@ -88,16 +89,11 @@ int other_cluster(const e2ttt_params* p) {  // CTAs per sequence there; 0 if the
     const int N = p->B * p->H, cl = simt_cluster_size(N, E2TTT_BF16);
     return N <= tile_clusters_fit(cl) ? cl : 0;
 }
-// Forward, GELU network.  Small states and chunks of a few tokens: a block of 64 is then mostly padding, and both kinds have one CTA per sequence.
-// us, there -> here: 148 sequences of 8 tokens, d = h = 64, C = 1 298 -> 350, C = 4 165 -> 198 (C = 16 196 -> 197; d = 128, h = 96, C = 4 245 -> 231);
-// 100 sequences 291 -> 278; 149, two waves there, 549 -> 351; 2000 sequences, d = h = 64, C = 1 3948 -> 4164, C = 4 2080 -> 2125, C = 16 2211 -> 2127,
-// d = h = 16, C = 16 1941 -> 2081; 600 sequences, d = h = 64, C = 1 1364 -> 1286.  The SwiGLU network, with two more products per block, gains everywhere.
+// Forward (the rule with both sides' times: tile_flow.h).  The SwiGLU network, with two more products per block, gains everywhere.
 bool tile_forward(const e2ttt_params* p) {
     if (!can_tile(p)) return false;
     if (p->kind != E2TTT_MLP_GELU || p->h > 1024) return true;  // (h > 1024: see bwd_common)
-    const int N = p->B * p->H, dh = p->d * p->h;
-    if (N > 100 && N <= 148) return !(p->C <= 4 && dh <= 4096);
-    return !(N > 600 && dh <= (p->C <= 4 ? 4096 : p->C <= 16 ? 1024 : 0));
+    return !flow_pads_too_much(p->B * p->H, p->d, p->h, p->C);
 }
 // Reverse pass.  At most 128 hidden units (one CTA per sequence in the chain) and long chunks: d = h = 64, 8 sequences, C = 512 0.60 of the
 // block-tiled time, C = 320 0.81 (256: 0.99); 15 sequences C = 448 0.70.  States of a few hundred values, up to 33 sequences: d = 16,

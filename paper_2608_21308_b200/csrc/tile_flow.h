@@ -38,6 +38,24 @@ inline bool tile_flow_serves(const TileLayout& t, int N, int C, int Ls, int nmat
     return N > (wide ? (hb <= 8 ? 20 : 18) : hb <= 8 ? 33 : 24);
 }
 
+// Many sequences of small states in chunks of a few tokens (GELU network, at most 1024 hidden units): a block of 64 tokens is then mostly padding, and
+// simt_fwd.cu, one CTA per sequence, can be the faster.  Its time goes by waves of 148 sequences; work items go to any CTA, so that theirs goes by
+// sequences, and a call fills and drains their queue once.  us of a wave and of 148 sequences per chunk, fitted to 5700 calls of 76 to 2000 sequences on both
+// kernels (within 5 % of what is measured).  It does not go by the number of chunks, so that a sequence given in several calls has the same bits as
+// in one: the line is where calls of two chunks break even.  us, there -> on work items, one chunk / four:
+//   C = 1   148 sequences, d = h = 64 43 -> 69 / 144 -> 176; 8 x 600 135 -> 196 / 499 -> 560; 64 x 192 105 -> 91 / 279 -> 271; 128 x 128 119 -> 97 / 269 -> 219
+//           100, d = h = 16 38 -> 53 / 128 -> 139; 64 x 72 49 -> 57 / 160 -> 148;  149, 64 x 64, two waves, 80 -> 70 / 270 -> 176;  592, 64 x 64 181 -> 190 / 588 -> 635
+//   C = 16  888, d = h = 16 231 -> 258 / 830 -> 917; 64 x 64 307 -> 276 / 952 -> 948; 128 x 16 315 -> 300 / 1121 -> 993;  C = 32  888, 8 x 8 255 -> 253 / 926 -> 907
+inline bool flow_pads_too_much(int N, int d, int h, int C) {
+    const int dh = d * h;
+    if (N <= 74 || dh > (C <= 4 ? 16384 : C <= 16 ? 12288 : C <= 32 && h <= 256 ? 9216 : 0) || (N <= 148 && C > 4)) return false;
+    const float waves = (float)((N + 147) / 148), tiles = (float)((h + 127) / 128), more = d > 64 ? 1.0f : 0.0f;
+    const float there = 5.0f + 23.0f * tiles + (h <= 64 ? 3.0f : h <= 128 ? 8.0f : 0.0f) + 9.0f * more + 1.2e-3f * dh + (dh > 8192 ? 1.5e-3f * (dh - 8192) : 0.0f) +
+                        (C > 4 ? (0.13f + 0.06f * tiles + 2e-5f * dh) * C : 0.0f);
+    const float here = 13.5f + 24.5f * tiles + 2.5f * more + 2e-4f * dh, once = 18.0f - 3.0f * waves;
+    return waves * there < here * N / 148.0f + (once > 0.0f ? once : 0.0f);
+}
+
 struct FlowPlan {
     int N, L, C, nchunks;       // the launch
     int tb;                     // blocks of 64 tokens of a chunk

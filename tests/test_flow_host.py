@@ -158,3 +158,24 @@ int main() {
 
 def test_single_chunks_start_with_their_tokens(tmp_path):
     run(tmp_path, FIRST)
+
+
+PADDING = r"""
+struct Call { int N, d, h, C; bool off; };
+int main() {
+    int bad = 0;
+    for (const Call& c : {  // calls of one and of four chunks were measured on both kernels; the faster one (where the two differ: over both)
+             Call{148, 8, 8, 1, true}, Call{148, 64, 64, 4, true}, Call{148, 64, 72, 4, true}, Call{148, 40, 104, 1, true}, Call{148, 32, 160, 4, true}, Call{148, 16, 300, 1, true},
+             Call{148, 8, 600, 1, true}, Call{120, 64, 64, 1, true}, Call{100, 16, 16, 4, true}, Call{100, 32, 32, 1, true}, Call{296, 64, 64, 1, true}, Call{296, 16, 300, 4, true},
+             Call{590, 16, 16, 16, true}, Call{592, 64, 64, 4, true}, Call{592, 24, 48, 16, true}, Call{888, 8, 130, 4, true}, Call{2000, 8, 130, 8, true}, Call{2000, 16, 16, 4, true},
+             Call{74, 8, 8, 1, false}, Call{76, 64, 64, 4, false}, Call{93, 128, 64, 1, false}, Call{148, 128, 96, 1, false}, Call{148, 64, 256, 4, false}, Call{148, 64, 64, 5, false},
+             Call{149, 8, 8, 1, false}, Call{149, 64, 64, 4, false}, Call{180, 64, 64, 16, false}, Call{297, 16, 16, 4, false}, Call{593, 64, 64, 16, false}, Call{888, 128, 64, 1, false},
+             Call{2000, 64, 64, 16, false}, Call{2000, 64, 128, 4, false}, Call{2000, 16, 16, 32, false}, Call{2000, 128, 128, 1, false}})
+        if (flow_pads_too_much(c.N, c.d, c.h, c.C) != c.off && bad++ < 9) std::printf("N=%d d=%d h=%d C=%d\n", c.N, c.d, c.h, c.C);
+    return bad != 0;
+}
+"""
+
+
+def test_many_small_sequences_take_the_kernel_that_measured_the_faster(tmp_path):
+    run(tmp_path, PADDING)

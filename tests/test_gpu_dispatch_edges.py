@@ -223,3 +223,36 @@ def test_noalloc_forward_where_the_block_tiled_layout_does_not_fit(kind, N, h, C
     for a, b in zip(Wf + Mf, ref["W"] + ref["M"]):
         assert util.rel_l2(a.cpu().numpy()[:, 0], b) <= 1e-4
     assert util.rel_l2(o.float().cpu().numpy()[:, 0], ref["o"]) <= 1e-3  # bf16: a few values round to the other neighbour
+
+
+# (The ids and comments of test_few_hidden_units_or_tokens name lines of the forward as they were before it ran on work items: of its rows the
+# forwards are all block-tiled now, the reverse passes on either side.)
+@pytest.mark.parametrize("normed", [False, True], ids=["plain", "normed"])
+@pytest.mark.parametrize("N,d,h,C", [(79, 64, 64, 4), (80, 64, 64, 4), (148, 64, 64, 4), (148, 64, 64, 5), (149, 64, 64, 4), (228, 64, 64, 4), (229, 64, 64, 4), (100, 64, 72, 4),
+                                     (101, 64, 72, 4), (148, 8, 512, 1), (122, 128, 64, 4), (123, 128, 64, 4), (221, 16, 16, 16), (222, 16, 16, 16), (243, 8, 8, 32),
+                                     (601, 16, 64, 17)])
+def test_many_sequences_of_short_chunks(N, d, h, C, normed):
+    """Either side of the lines that take a forward of many small sequences off the block-tiled kernels; its states and row norms pass to their
+    reverse pass.  Six chunks, checkpoints of two."""
+    x, shape = _inputs(2, 5 * C + 1, d, h, C, MLP, with_d_o=True, with_dstate=True)
+    rep = lambda a: np.concatenate([a] * ((N + 1) // 2))[:N]
+    xs = {n: [rep(w) for w in a] if isinstance(a, list) else rep(a) for n, a in x.items()}
+    cut = lambda got: {n: [w[:2] for w in a] if isinstance(a, list) else a[:2] for n, a in got.items()}
+    if normed:
+        tgt = targets(x)
+        got, ref = gpu_forward_normed(xs, [rep(t) for t in tgt], impl=E.E2TTT_IMPL_TILED, **shape), oracle_fwd(x, tgt, C, MLP)
+        refb = oracle_bwd(x, tgt, C, MLP)
+        plans = [gpu_backward_normed(xs, [rep(t) for t in tgt], impl=E.E2TTT_IMPL_TILED, via_saved_states=saved, **shape) for saved in (True, False)]
+    else:
+        got, ref, refb = util.gpu_forward(xs, impl=E.E2TTT_IMPL_TILED, **shape)[0], util.oracle_forward(x, C, MLP), util.oracle_backward(x, C, MLP)
+        plans = [util.gpu_backward(xs, impl=E.E2TTT_IMPL_TILED, via_saved_states=saved, ckpt_every=ckpt, **shape)
+                 for saved, ckpt in ((True, 0), (True, 2), (False, 0), (False, 2))]
+    for a in [got["o"], *got["W"], *got["M"]]:
+        assert all(np.array_equal(a[n], a[n % 2]) for n in range(N))
+    check_forward(cut(got), ref, TOL_BF16, "forward")
+    check_fp32(cut(got), ref, "forward")
+    check_backward(cut(plans[0]), refb, 2 * TOL_BF16, "backward")
+    check_fp32(cut(plans[0]), refb, "backward")
+    for got in plans[1:]:  # every memory plan: the same bits
+        for n, a in got.items():
+            assert all(np.array_equal(v, w) for v, w in (zip(a, plans[0][n]) if isinstance(a, list) else [(a, plans[0][n])])), n
