@@ -225,6 +225,31 @@ def test_noalloc_forward_where_the_block_tiled_layout_does_not_fit(kind, N, h, C
     assert util.rel_l2(o.float().cpu().numpy()[:, 0], ref["o"]) <= 1e-3  # bf16: a few values round to the other neighbour
 
 
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("N,d,h,C,L", [
+    (1, 72, 840, 65, 131), (15, 128, 1088, 128, 257),   # two blocks of tokens, the second of one token and full; a chunk of one token
+    (2, 128, 1600, 130, 261), (1, 64, 2112, 200, 450),  # three and four blocks, the last ones ragged
+])
+def test_wide_networks_on_clusters_with_several_blocks_of_tokens(N, d, h, C, L, kind):
+    """Few sequences of wide networks stay off the work items; their chunks have several blocks of tokens.  Plain, with saved states, normalised."""
+    U = min(N, 2)
+    x, shape = _inputs(U, L, d, h, C, kind)
+    rep = lambda a: np.concatenate([a] * ((N + U - 1) // U))[:N]
+    xs = {n: [rep(w) for w in a] if isinstance(a, list) else rep(a) for n, a in x.items() if a is not None}
+    cut = lambda got: {n: [w[:U] for w in a] if isinstance(a, list) else a[:U] for n, a in got.items()}
+    got, hd = util.gpu_forward(xs, impl=E.E2TTT_IMPL_TILED, **shape)
+    assert E.e2ttt_device_status(hd["ws"]) == 0
+    ref = util.oracle_forward(x, C, kind)
+    check_forward(cut(got), ref, TOL_BF16, "forward on clusters")
+    check_fp32(cut(got), ref, "forward on clusters")
+    saved, _ = util.gpu_forward(xs, impl=E.E2TTT_IMPL_TILED, save_states=True, **shape)
+    assert all(np.array_equal(a, b) for a, b in zip([got["o"], *got["W"], *got["M"]], [saved["o"], *saved["W"], *saved["M"]]))
+    tgt = targets(x)
+    got, ref = gpu_forward_normed(xs, [rep(t) for t in tgt], impl=E.E2TTT_IMPL_TILED, **shape), oracle_fwd(x, tgt, C, kind)
+    check_forward(cut(got), ref, TOL_BF16, "normed forward on clusters")
+    check_fp32(cut(got), ref, "normed forward on clusters")
+
+
 # (The ids and comments of test_few_hidden_units_or_tokens name lines of the forward as they were before it ran on work items: of its rows the
 # forwards are all block-tiled now, the reverse passes on either side.)
 @pytest.mark.parametrize("normed", [False, True], ids=["plain", "normed"])

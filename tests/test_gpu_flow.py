@@ -6,6 +6,9 @@ import pytest
 from paper_2608_21308_b200 import binding as E
 from paper_2608_21308_b200 import inputs
 from tests import util
+from tests.test_gpu_dispatch_edges import check_fp32
+from tests.test_gpu_normed import gpu_backward_normed, gpu_forward_normed, oracle_bwd, oracle_fwd, targets
+from tests.test_gpu_parity import TOL_BF16, check_backward
 
 pytestmark = pytest.mark.gpu
 MLP, SWIGLU = inputs.KIND_MLP, inputs.KIND_SWIGLU
@@ -63,6 +66,27 @@ def test_u_of_many_hidden_units_is_as_exact_as_that_of_few(d, h, C, L, N):
 
 # Operands are off by 2^-17 / sqrt 3 = 4.4e-6 (rms) in each of the four products from a chunk's keys to its aggregates, 9e-6 together; two more chunks that
 # amplify it by up to 2 each stay below 1e-4.  An operand without its second term is off by 2^-9 / sqrt 3 = 1.1e-3
+@pytest.mark.parametrize("normed", [False, True], ids=["plain", "normed"])
+@pytest.mark.parametrize("kind", [MLP, SWIGLU])
+@pytest.mark.parametrize("d,h,C,L,N", [(128, 384, 512, 1025, 67), (72, 200, 512, 1100, 101), (64, 64, 512, 600, 131)])
+def test_sequences_in_several_sets_of_which_the_last_is_short(d, h, C, L, N, kind, normed):
+    """Tokens, weights and norm items of several sequences and sets in work at a time; the last set has places without a sequence."""
+    if not normed:
+        got, ref = copies_of_two(d, h, C, L, N, kind)
+    else:
+        x = inputs.generate(inputs.paper_regime(inputs.Recipe(B=2, H=1, L=L, d=d, h=h, C=C, kind=kind, io="bf16", seed=12, m_std=0.002)))
+        tgt = targets(x)
+        ref = oracle_fwd(x, tgt, C, kind)
+        rep = lambda a: np.concatenate([a] * ((N + 1) // 2))[:N]
+        xs = {n: [rep(w) for w in a] if isinstance(a, list) else rep(a) for n, a in x.items() if a is not None}
+        got = gpu_forward_normed(xs, [rep(t) for t in tgt], d=d, h=h, C=C, kind=kind, io="bf16", impl=E.E2TTT_IMPL_TILED)
+        for a in [got["o"], *got["W"], *got["M"]]:
+            assert all(np.array_equal(a[n], a[n % 2]) for n in range(N))
+        assert util.rel_err(got["o"][:2], ref["o"]) <= 1e-2  # bf16 outputs
+    errs = {f"{name}{i + 1}": util.rel_l2(got[name][i][:2], m) for name in ("W", "M") for i, m in enumerate(ref[name])}
+    assert all(e <= 1e-4 for e in errs.values()), errs
+
+
 @pytest.mark.parametrize("kind", [MLP, SWIGLU])
 @pytest.mark.parametrize("d,h,C,L", [(4, 8, 64, 70), (36, 144, 40, 75), (68, 72, 65, 130), (100, 400, 64, 129), (124, 64, 128, 200)])
 def test_rows_of_8_bytes_alignment(d, h, C, L, kind):
@@ -90,3 +114,17 @@ def test_a_sequence_in_several_calls_has_the_bits_of_one(N, d, h, C, kind):
             o.append(part["o"])
         assert np.array_equal(np.concatenate(o, 1), whole["o"])
         assert all(np.array_equal(a, b) for a, b in zip([*W, *M], [*whole["W"], *whole["M"]]))
+
+
+def test_normalised_swiglu_training_step_of_four_long_chunks():
+    """2048 tokens in chunks of 512, d = 128, h = 384, saved states.  The bound as above for what is returned in fp32 of the state and its adjoints."""
+    shape = dict(d=128, h=384, C=512, kind=SWIGLU, io="bf16", impl=E.E2TTT_IMPL_TILED)
+    x = inputs.generate(inputs.paper_regime(inputs.Recipe(B=2, H=1, L=2048, d=128, h=384, C=512, kind=SWIGLU, io="bf16", seed=14, m_std=0.002)), with_d_o=True, with_dstate=True)
+    tgt = targets(x)
+    got, ref = gpu_forward_normed(x, tgt, **shape), oracle_fwd(x, tgt, 512, SWIGLU)
+    gotb, refb = gpu_backward_normed(x, tgt, via_saved_states=True, **shape), oracle_bwd(x, tgt, 512, SWIGLU)
+    assert util.rel_err(got["o"], ref["o"]) <= 1e-2  # bf16 outputs
+    errs = {f"{n}{i + 1}": util.rel_l2(a, b) for g, r, names in ((got, ref, ("W", "M")), (gotb, refb, ("dW", "dM"))) for n in names for i, (a, b) in enumerate(zip(g[n], r[n]))}
+    assert all(e <= 1e-4 for e in errs.values()), errs
+    check_backward(gotb, refb, 2 * TOL_BF16, "backward")
+    check_fp32(gotb, refb, "backward")
