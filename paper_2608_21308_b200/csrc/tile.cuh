@@ -266,25 +266,6 @@ __device__ __forceinline__ void ld_f8(const float* p, float (&v)[8]) {
                  : "l"(p)
                  : "memory");
 }
-__device__ __forceinline__ void st_f16(float* p, const float (&v)[16]) {
-    float a[2][8];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) a[j >> 3][j & 7] = v[j];
-    st_f8(p, a[0]);
-    st_f8(p + 8, a[1]);
-}
-__device__ __forceinline__ void ld_f16(const float* p, float (&v)[16]) {
-    float a[2][8];
-    ld_f8(p, a[0]);
-    ld_f8(p + 8, a[1]);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = a[j >> 3][j & 7];
-}
-// Where the 16 values of hidden unit `row` of block bl and tokens tok .. of block tk are (tok a multiple of 16) in an fp32 [hidden x tokens]
-// intermediate.  An epilogue thread's values are neighbours: two accesses of 32 bytes instead of sixteen of 4
-__device__ __forceinline__ size_t f16_of(int bl, int tb, int tk, int tok, int row) {
-    return (((size_t)bl * tb + tk) * 4 + (tok >> 4)) * 1024 + (row & 63) * 16;
-}
 // hi + lo of 16 consecutive values
 __device__ __forceinline__ void ld_split16(const unsigned char* blk, int row, int col0, float (&v)[16]) {
     const bool sw = row & 1;

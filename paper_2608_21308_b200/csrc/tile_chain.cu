@@ -15,7 +15,8 @@
 // to T has an epilogue of its own, which adds it to the master; after a matrix's last one T's operand blocks are written anew.
 // Everything else streams from the slots that tile_prep and tile_rec filled.
 //
-// 18 warps: 0-15 epilogues (warp w: lanes 32 (w & 3).., group w >> 2 of the columns), 16 copies operand blocks, 17 issues MMAs.
+// 18 warps: 0-15 epilogues (warp w: lanes 32 (w & 3).., group w >> 2 of the columns), 16 copies operand blocks, 17 issues MMAs; with the GELU
+// network two more, for the barriers alone (chain_threads).
 #include <type_traits>
 
 #include "tile_rec.cuh"
