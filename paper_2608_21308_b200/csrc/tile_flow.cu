@@ -15,8 +15,8 @@
 // Sequences are taken in sets and, inside a set, out of step with each other: while one is at its tokens another is at its weights, and
 // as many items lie between dependent ones as the GPU has in work (flow_plan, tile_flow.h).
 //
-// What bounds it now: a tokens item of 128 x 512 takes 75 thousand cycles, 46 of them on the activations - their instructions, half of it, and waits
-// for products and for the tile between them - a weights item of 512 tokens 77 (first matrices) and 45 (last).  An SM stores 32 B/clk, threads or bulk
+// What bounds it now: a tokens item of 128 x 512 takes 79 thousand cycles, 46 of them on the activations - their instructions, half of it, and waits
+// for products and for the tile between them - a weights item of 512 tokens 71 (first matrices) and 40 (last).  An SM stores 32 B/clk, threads or bulk
 // copies alike, but 16 where a warp's lanes write 32 bytes of 32 lines (st_split16): tiles that are in shared memory anyway leave by bulk copies.
 //
 // 20 warps: 0-15 epilogues (warp w: lanes 32 (w & 3).., group w >> 2 of the columns), 16 copies operand blocks, 17 issues MMAs and the

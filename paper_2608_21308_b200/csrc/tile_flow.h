@@ -40,8 +40,8 @@ inline bool tile_flow_serves(const TileLayout& t, int N, int C, int Ls, int nmat
 
 // Many sequences of small states in chunks of a few tokens (GELU network, at most 1024 hidden units): a block of 64 tokens is then mostly padding, and
 // simt_fwd.cu, one CTA per sequence, can be the faster.  Its time goes by waves of 148 sequences; work items go to any CTA, so that theirs goes by
-// sequences, and a call fills and drains their queue once.  us of a wave and of 148 sequences per chunk, fitted to 5700 calls of 76 to 2000 sequences on both
-// kernels (within 5 % of what is measured).  It does not go by the number of chunks, so that a sequence given in several calls has the same bits as
+// sequences, and a call fills and drains their queue once.  The sums below are us of a wave and of 148 sequences per chunk, after 5700 calls of 76 to 2000
+// sequences on both kernels.  It does not go by the number of chunks, so that a sequence given in several calls has the same bits as
 // in one: the line is where calls of two chunks break even.  us, there -> on work items, one chunk / four:
 //   C = 1   148 sequences, d = h = 64 43 -> 69 / 144 -> 176; 8 x 600 135 -> 196 / 499 -> 560; 64 x 192 105 -> 91 / 279 -> 271; 128 x 128 119 -> 97 / 269 -> 219
 //           100, d = h = 16 38 -> 53 / 128 -> 139; 64 x 72 49 -> 57 / 160 -> 148;  149, 64 x 64, two waves, 80 -> 70 / 270 -> 176;  592, 64 x 64 181 -> 190 / 588 -> 635
