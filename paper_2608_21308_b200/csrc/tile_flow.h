@@ -19,23 +19,24 @@ inline int flow_blocks(int C, int Ls) { return ((Ls < C ? Ls : C) + 63) / 64; }
 //   two blocks    15 sequences, h = 768 .92 .76, 1024 1.12 .87; 16, h = 1024 .94 .81, 1536 1.05 .85, 2048 1.06 .91; 22, h = 2048 1.08 .90
 //   three, four   8 sequences, h = 1536 .91 .76, 2048 1.00 .87 | .93 .80; 15, h = 2048 1.09 .87 | .99 .79; 22 1.14 .79 | .98 .72; 64, h = 512 .77 .60 | .74 .60
 //   normalised    (a norm item has 64 whole rows of the last matrix)  one block: 8 sequences, h = 384 1.03 1.05, 22, h = 640 1.15 .94, 33, h = 1024 1.16 1.00, 64, h = 2048
-//                 1.06 1.09; d = 64: 33, h = 512 1.06 1.12, SwiGLU 22 .89 .99; two: d = 64, 22, h = 640 .98 .92, 768 1.18 1.08; four: 22, h = 2048 1.11 1.06, 23 .95 .93
-// Chunks of 512, h = 512, 64 sequences of 2048 tokens 1521 -> 1000 us
+//                 1.06 1.09; d = 64: 33, h = 512 1.06 1.12, SwiGLU 22 .89 .99; two: SwiGLU, 15, h = 640 .88 .90, 768 1.05 .88; d = 64, 22, h = 640 .98 .92, 768 1.18 1.08; four: 22, h = 2048 1.11 1.06, 23 .95 .93
+// What clusters take changes from GPU to GPU, with where they fit: 16 sequences, h = 512, one block 54 and 67 us (four chunks 183, 195), on work items 57 (184); normalised,
+// h = 384 1.03 and .85.  Chunks of 512, h = 512, 64 sequences of 2048 tokens 1521 -> 1000 us
 inline bool tile_flow_serves(const TileLayout& t, int N, int C, int Ls, int nmat, bool normed) {
     const int tb = flow_blocks(C, Ls), hb = t.hb;
     const bool wide = t.db == 2, sw = nmat == 3;
     if (normed && hb > 16 && tb <= 3 && N <= 74) return false;
     if (tb > 2) return hb <= (normed ? 5 : 8) * tb || N > (normed && hb > 24 ? 22 : 15);
-    if (tb == 2) return hb <= (wide ? 12 : normed ? 6 : 10) || N > (hb > 24 || (normed && hb > 8) ? 22 : 15);
+    if (tb == 2) return hb <= (wide || (normed && sw) ? 12 : normed ? 6 : 10) || N > (hb > 24 || (normed && hb > 8) ? 22 : 15);
     if (hb <= 4) return true;
     if (normed) {
-        if (hb <= 6) return N > 22 || (sw && wide);
-        return N > (hb <= 8 && (wide || sw) ? 15 : hb <= 12 && (wide || sw) ? 22 : 33);
+        if (hb <= 6) return N > (wide ? 15 : 22) || sw;
+        return N > (sw && hb <= (wide ? 12 : 8) ? 15 : hb <= 8 && wide ? 15 : hb <= 12 && (wide || sw) ? 22 : 33);
     }
     if (hb <= 6) return true;
     if (hb > 16) return N > 24;
-    if (sw) return N > (wide && hb <= 12 ? 15 : 22);
-    return N > (wide ? (hb <= 8 ? 20 : 18) : hb <= 8 ? 33 : 24);
+    if (sw) return N > (hb <= (wide ? 12 : 8) ? 15 : 22);
+    return N > (wide ? (hb <= 8 ? 15 : 18) : hb <= 8 ? 33 : 24);
 }
 
 // Many sequences of small states in chunks of a few tokens (GELU network, at most 1024 hidden units): a block of 64 tokens is then mostly padding, and
